@@ -327,7 +327,8 @@ fh_status fh_synthesize_sing(int J, double W, int j_c, int K, const double *d_s,
  * (1/L) sum_p C_p^{(gamma)} B_p e^{2 pi i beta n p / L} for n = n0 - L/2 ..
  * n0 + L/2 - 1: C^{(gamma)} the gamma-fractional DFT of c zero-padded to L, B
  * the DFT of b at the integers -L/2 .. L/2-1, each fractional DFT by the chirp
- * factorisation as a circular convolution of radix-2 FFTs.  d_d receives
+ * factorisation as a circular convolution by FFTs (one FFT where the transform
+ * is an ordinary DFT of a power-of-two length).  d_d receives
  * batch*L complex (device).  L even, M <= L <= 2^24.  Work space as for
  * fh_synthesize_sing.  The error of the approximation is O(L^-2) for P > 2A. */
 fh_status fh_scaled_convolution(const double *d_c, int M, int batch, double beta, double gamma,

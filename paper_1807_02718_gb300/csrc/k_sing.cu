@@ -1,5 +1,5 @@
 // The 2D synthesis with the low-frequency split (Sec. 4.2; Sec. 5 steps
-// T1b-T2d) and the FFT-accelerated scaled convolution (Sec. 4.1.2).
+// T1b-T2d).
 //
 // Split synthesis.  For each window k and target x the inverse transform of
 // F_k(w) = B_k^slow(w) V(x, w) over [-W, W] is, by F(-w) = conj F(w),
@@ -26,20 +26,12 @@
 // D_p(t') = sum_m K_m(t') E[m][p] with E = (shifted DFT) o (FC extension) and
 // K_m(t') = e^{-i delta t'} 2A sinc((2A/P)(alpha t' - m)), alpha = P / (2 pi);
 // for the singular samples the FCC weights.
-//
-// Scaled convolution.  d_n = sum_m c_m b(beta n - gamma m) (eqs. conv_sum,
-// conv_sum_2 with the index reading of eq. discConv) is approximated by eq.
-// approx_conv_sum: C^{(gamma)}_p (gamma-fractional DFT of c zero-padded to
-// L), B_p (DFT of b at the integers -L/2..L/2-1) and the inverse
-// beta-fractional DFT of C B.  Each fractional DFT of length L is computed by
-// the chirp factorisation 2mp = m^2 + p^2 - (p - m)^2 as one circular
-// convolution of length Nf >= 2L (a power of two) by radix-2 FFTs.
 #include <cmath>
-#include <vector>
 
 #include "dfloat.cuh"
 #include "fc_gram_table.h"
 #include "fh_internal.h"
+#include "scratch.cuh"
 
 namespace fh {
 namespace {
@@ -88,27 +80,6 @@ __device__ __forceinline__ double2 expi_pi_ratio(long long num, long long den) {
     if (r < 0) r += 2 * den;
     double s, c;
     sincospi((double)r / (double)den, &s, &c);
-    return make_double2(c, s);
-}
-
-// (a N / D) mod 2 for integers N, D > 0: N = q D + r exactly, a q as an
-// exact two-term product, reduced modulo 2 before the small terms are added,
-// so that the phase pi a N / D keeps its accuracy for large N.
-__device__ __forceinline__ double mulmod2(double a, long long N, long long D) {
-    long long q = N / D, r = N - q * D;
-    if (r < 0) {
-        r += D;
-        --q;
-    }
-    const double hi = a * (double)q;
-    const double lo = fma(a, (double)q, -hi);
-    double v = fmod(hi, 2.0) + lo + a * (double)r / (double)D;
-    v = fmod(v, 2.0);
-    return v < 0.0 ? v + 2.0 : v;
-}
-__device__ __forceinline__ double2 expi_pi(double r) {   // e^{i pi r}
-    double s, c;
-    sincospi(r, &s, &c);
     return make_double2(c, s);
 }
 
@@ -290,123 +261,9 @@ __global__ void stack_fields_kernel(int n, int n_x, int j_c, const double2 *__re
     Vp[(long long)p * n_x + x] = p < n ? V[(long long)(j_c + p) * n_x + x] : Vs[(long long)(p - n) * n_x + x];
 }
 
-// ---- radix-2 FFT (Stockham, out of place), batched over rows of length Nf ----
-
-__global__ void fft_stage_kernel(int Nf, int half_len, int batch, const double2 *__restrict__ in,
-                                 double2 *__restrict__ out, double sign) {
-    // stage with butterflies of span Ls = 2 * half_len: element index j in [0, Nf/2)
-    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int halfN = Nf / 2;
-    if (g >= (long long)halfN * batch) return;
-    const int b = (int)(g / halfN), j = (int)(g % halfN);
-    const int k = j % half_len;                 // position within the group
-    const int grp = j / half_len;
-    const double2 *src = in + (long long)b * Nf;
-    double2 *dst = out + (long long)b * Nf;
-    const double2 x0 = src[j], x1 = src[j + halfN];
-    double sw, cw;
-    sincospi(sign * (double)k / (double)half_len, &sw, &cw);   // e^{sign i pi k / half_len}
-    const double2 t = cmul(x1, make_double2(cw, sw));
-    const int o = grp * 2 * half_len + k;
-    dst[o] = make_double2(x0.x + t.x, x0.y + t.y);
-    dst[o + half_len] = make_double2(x0.x - t.x, x0.y - t.y);
-}
-
-// Bluestein input: y[b][m'] = x[b][m'] e^{-i pi alpha m^2 / L} (m = m' - L/2),
-// zero for m' >= L (rows of length Nf).
-__global__ void chirp_in_kernel(int L, int Nf, int batch, double alpha, const double2 *__restrict__ x,
-                                double2 *__restrict__ y) {
-    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= (long long)Nf * batch) return;
-    const int b = (int)(g / Nf), i = (int)(g % Nf);
-    double2 v = make_double2(0.0, 0.0);
-    if (i < L) {
-        const long long m = i - L / 2;
-        v = cmul(x[(long long)b * L + i], expi_pi(-mulmod2(alpha, m * m, L)));
-    }
-    y[g] = v;
-}
-
-// Chirp filter z[k] = e^{i pi alpha k^2 / L} at k and Nf - k, |k| < L.
-__global__ void chirp_filter_kernel(int L, int Nf, double alpha, double2 *__restrict__ z) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= Nf) return;
-    long long k = -1;
-    if (i < L) k = i;
-    else if (i > Nf - L) k = Nf - i;
-    z[i] = k >= 0 ? expi_pi(mulmod2(alpha, k * k, L)) : make_double2(0.0, 0.0);
-}
-
-// Y[b][i] *= Z[i] / Nf
-__global__ void pointwise_kernel(int Nf, int batch, double2 *__restrict__ Y, const double2 *__restrict__ Z) {
-    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= (long long)Nf * batch) return;
-    const double2 z = Z[g % Nf];
-    const double2 r = cmul(Y[g], z);
-    Y[g] = make_double2(r.x / Nf, r.y / Nf);
-}
-
-// X[b][p'] = e^{-i pi alpha p^2 / L} conv[b][p'] (p = p' - L/2), times the
-// extra factor e^{2 pi i beta n0 p / L} * B[p'] when B is given (the middle of
-// eq. approx_conv_sum) and the scale 1/L when scale_L is set.
-__global__ void chirp_out_kernel(int L, int Nf, int batch, double alpha, const double2 *__restrict__ conv,
-                                 double2 *__restrict__ X, const double2 *__restrict__ Bm, double beta,
-                                 long long n0, int scale_L) {
-    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= (long long)L * batch) return;
-    const int b = (int)(g / L), i = (int)(g % L);
-    const long long p = i - L / 2;
-    double2 v = cmul(conv[(long long)b * Nf + i], expi_pi(-mulmod2(alpha, p * p, L)));
-    if (Bm) {
-        v = cmul(v, Bm[i]);
-        const long long np = n0 * p;                 // e^{2 pi i beta n0 p / L}
-        const double ph = np >= 0 ? mulmod2(2.0 * beta, np, L) : -mulmod2(2.0 * beta, -np, L);
-        v = cmul(v, expi_pi(ph));
-    }
-    if (scale_L) v = make_double2(v.x / L, v.y / L);
-    X[g] = v;
-}
-
-// b at the integers -L/2 .. L/2 - 1 (one row)
-__global__ void kernel_samples_kernel(int L, double A, double P, double2 *__restrict__ bq) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= L) return;
-    const double y = (2.0 * A / P) * (double)(i - L / 2);
-    bq[i] = make_double2(2.0 * A * (y == 0.0 ? 1.0 : sinpi(y) / (kPi * y)), 0.0);
-}
-
 // ---- host helpers ----
 
 unsigned grid_of(long long n, int block) { return (unsigned)((n + block - 1) / block); }
-
-// Batched FFT of rows of length Nf (a power of two) in place in buf, using
-// tmp of the same size; sign -1 forward, +1 inverse (unscaled).
-void fft_rows(double2 *buf, double2 *tmp, int Nf, int batch, double sign, cudaStream_t st) {
-    double2 *in = buf, *out = tmp;
-    for (int h = 1; h < Nf; h *= 2) {
-        const long long work = (long long)(Nf / 2) * batch;
-        fft_stage_kernel<<<grid_of(work, 256), 256, 0, st>>>(Nf, h, batch, in, out, sign);
-        double2 *t = in;
-        in = out;
-        out = t;
-    }
-    if (in != buf) cudaMemcpyAsync(buf, in, (size_t)Nf * batch * sizeof(double2), cudaMemcpyDeviceToDevice, st);
-}
-
-// X = FRFT_alpha(x) for batch rows of length L (eq. approx_conv_sum's
-// fractional transforms), with the optional middle factor of chirp_out_kernel.
-void frft_rows(const double2 *x, double2 *X, int L, int batch, double alpha, double2 *y, double2 *tmp,
-               double2 *z, double2 *ztmp, int Nf, const double2 *Bm, double beta, long long n0,
-               int scale_L, cudaStream_t st) {
-    chirp_in_kernel<<<grid_of((long long)Nf * batch, 256), 256, 0, st>>>(L, Nf, batch, alpha, x, y);
-    fft_rows(y, tmp, Nf, batch, -1.0, st);
-    chirp_filter_kernel<<<grid_of(Nf, 256), 256, 0, st>>>(L, Nf, alpha, z);
-    fft_rows(z, ztmp, Nf, 1, -1.0, st);
-    pointwise_kernel<<<grid_of((long long)Nf * batch, 256), 256, 0, st>>>(Nf, batch, y, z);
-    fft_rows(y, tmp, Nf, batch, 1.0, st);
-    chirp_out_kernel<<<grid_of((long long)L * batch, 256), 256, 0, st>>>(L, Nf, batch, alpha, y, X, Bm, beta, n0,
-                                                                        scale_L);
-}
 
 // Gauss-Legendre nodes and weights on [-1, 1] (Newton's method on P_n).
 void gauss_legendre(int n, double *x, double *w) {
@@ -428,20 +285,6 @@ void gauss_legendre(int n, double *x, double *w) {
         w[i] = 2.0 / ((1.0 - z * z) * dp * dp);
     }
 }
-
-struct Scratch {
-    std::vector<void *> bufs;
-    cudaStream_t st;
-    template <class T> T *get(size_t count) {
-        void *p = nullptr;
-        if (cudaMallocAsync(&p, std::max<size_t>(count, 1) * sizeof(T), st) != cudaSuccess) return nullptr;
-        bufs.push_back(p);
-        return static_cast<T *>(p);
-    }
-    ~Scratch() {
-        for (void *p : bufs) cudaFreeAsync(p, st);
-    }
-};
 
 }  // namespace
 }  // namespace fh
@@ -513,46 +356,6 @@ extern "C" fh_status fh_synthesize_sing(int J, double W, int j_c, int K, const d
         stack_fields_kernel<<<dim3(grid_of(n_x, 128), ns), 128, 0, st>>>(
             n, n_x, j_c, reinterpret_cast<const double2 *>(d_V), reinterpret_cast<const double2 *>(d_Vs), Vp);
         launch_synth_contract(ns, n_x, n_T, Vp, Gr, Gm, d_u, st);
-        if (cudaGetLastError() != cudaSuccess) status = FH_ECUDA;
-    }
-    return status;
-}
-
-extern "C" fh_status fh_scaled_convolution(const double *d_c, int M, int batch, double beta, double gamma,
-                                           long long n0, int L, double A, double P, double *d_d, void *stream) {
-    if (M < 2 || (M & 1) || batch < 1 || L < M || (L & 1) || !(A > 0.0) || !(P > 0.0) || !d_c || !d_d ||
-        !std::isfinite(beta) || !std::isfinite(gamma) || L > (1 << 24))
-        return FH_EINVAL;
-    if (cudaPeekAtLastError() != cudaSuccess) return FH_ECUDA;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    int Nf = 1;
-    while (Nf < 2 * L) Nf *= 2;
-    fh_status status = FH_OK;
-    {
-        Scratch sc{{}, st};
-        double2 *x = sc.get<double2>((size_t)L * batch);       // c zero-padded to L
-        double2 *Cg = sc.get<double2>((size_t)L * batch);
-        double2 *y = sc.get<double2>((size_t)Nf * batch);
-        double2 *tmp = sc.get<double2>((size_t)Nf * batch);
-        double2 *z = sc.get<double2>((size_t)Nf);
-        double2 *ztmp = sc.get<double2>((size_t)Nf);
-        double2 *bq = sc.get<double2>((size_t)L);
-        double2 *Bm = sc.get<double2>((size_t)L);
-        if (!x || !Cg || !y || !tmp || !z || !ztmp || !bq || !Bm) {
-            cudaGetLastError();
-            return FH_ENOMEM;
-        }
-        cudaMemsetAsync(x, 0, (size_t)L * batch * sizeof(double2), st);
-        cudaMemcpy2DAsync(x + (L / 2 - M / 2), (size_t)L * sizeof(double2), d_c, (size_t)M * sizeof(double2),
-                          (size_t)M * sizeof(double2), batch, cudaMemcpyDeviceToDevice, st);
-        // B_p: DFT of b at the integers (alpha = 1)
-        kernel_samples_kernel<<<grid_of(L, 256), 256, 0, st>>>(L, A, P, bq);
-        frft_rows(bq, Bm, L, 1, 1.0, y, tmp, z, ztmp, Nf, nullptr, 0.0, 0, 0, st);
-        // C^{(gamma)}_p, times B_p e^{2 pi i beta n0 p / L}
-        frft_rows(x, Cg, L, batch, gamma, y, tmp, z, ztmp, Nf, Bm, beta, n0, 0, st);
-        // the inverse beta-fractional transform: d_{n0+n'} = (1/L) sum_p (...) e^{2 pi i beta n' p / L}
-        frft_rows(Cg, reinterpret_cast<double2 *>(d_d), L, batch, -beta, y, tmp, z, ztmp, Nf, nullptr, 0.0, 0, 1,
-                  st);
         if (cudaGetLastError() != cudaSuccess) status = FH_ECUDA;
     }
     return status;
