@@ -125,6 +125,7 @@ struct fh_ctx {
     DevBuf d_zf, d_dzf, d_sf, d_wpf;
     DevBuf d_z, d_dz, d_ddz, d_kress, d_logsin, d_A, d_psi, d_info, d_nu, d_nu_f, d_ph, d_omega, d_pw;
     DevBuf d_stab;
+    DevBuf d_lu64;                       // FP64 LU: the row moves of each system's current panel
     DevBuf d_A32, d_piv, d_g, d_iters, d_resid, d_tcerr, d_y32, d_rstate, d_rchunk, d_Bf, d_dblk,
         d_blk_off, d_dinv;
     // tensor-core LU work space: tensor maps of the FP32 matrices, staged
@@ -162,7 +163,7 @@ struct fh_ctx {
                          &d_part, &d_N, &d_mat_off, &d_vec_off, &d_tab, &d_tab_off, &d_tab_N,
                          &d_kappa, &d_eta, &d_solve_j, &d_solve_prob, &d_order, &d_curves,
                          &d_pdir, &d_zf, &d_dzf, &d_sf, &d_wpf, &d_z, &d_dz, &d_ddz, &d_kress, &d_logsin, &d_A, &d_psi,
-                         &d_info, &d_nu, &d_nu_f, &d_ph, &d_omega, &d_pw, &d_stab, &d_A32, &d_piv, &d_g, &d_iters,
+                         &d_info, &d_nu, &d_nu_f, &d_ph, &d_omega, &d_pw, &d_stab, &d_lu64, &d_A32, &d_piv, &d_g, &d_iters,
                          &d_resid, &d_tcerr, &d_y32, &d_rstate, &d_rchunk, &d_Bf, &d_dblk, &d_blk_off, &d_dinv,
                          &d_lu_maps, &d_lu_opnd, &d_lu_aoff, &d_lu_boff, &d_wa, &d_a, &d_x, &d_T, &d_u, &d_V, &d_Gr, &d_Gm, &d_Gs, &d_Vs, &d_ctc, &d_ctc_err,
                          &d_tmpA, &d_tmpg, &d_tmp_ll, &d_tmp_d, &d_tmp_i};
@@ -1273,11 +1274,12 @@ fh_status solve_kernels(fh_ctx *ctx, bool mixed, bool tc) {
         FH_CUDA(ctx, cudaMemsetAsync(ctx->d_info.p, 0, (size_t)ctx->S * sizeof(int), ctx->stream));
     }
     if (!mixed) {
-        PhaseScope ps(ctx, FH_PH_FACTOR, 1);
-        fh::launch_lu_solve_fp64(ctx->d_order.as<int>(), ctx->S, ctx->d_N.as<int>(),
-                                 ctx->d_mat_off.as<long long>(), ctx->d_vec_off.as<int>(),
-                                 ctx->d_A.as<double2>(), ctx->d_psi.as<double2>(),
-                                 ctx->d_info.as<int>(), ctx->stream);
+        PhaseScope ps(ctx, FH_PH_FACTOR,
+                      fh::lu_fp64_launches(ctx->order.data(), ctx->solve_N.data(), ctx->S));
+        fh::launch_lu_solve_fp64(ctx->d_order.as<int>(), ctx->order.data(), ctx->solve_N.data(), ctx->S,
+                                 ctx->d_N.as<int>(), ctx->d_mat_off.as<long long>(), ctx->d_vec_off.as<int>(),
+                                 ctx->d_A.as<double2>(), ctx->d_psi.as<double2>(), ctx->d_info.as<int>(),
+                                 ctx->d_lu64.p, ctx->stream, ctx->side, ctx->ev_fork, ctx->ev_join);
         FH_TRY(check_launch(ctx, "lu fp64"));
     } else {
         {
@@ -1320,6 +1322,7 @@ fh_status fh_solve_frequencies(fh_ctx *ctx, const double *eta, fh_solve_stats *s
         return fail(ctx, FH_EINVAL, "tensor-core LU supports N <= %d (largest N is %d)",
                     fh::kTcMaxN, ctx->maxN);
     // every buffer of the launch sequence exists before it is launched or captured
+    if (!mixed) FH_TRY(ensure(ctx, ctx->d_lu64, fh::lu_fp64_scratch_bytes(ctx->S)));
     if (mixed) {
         FH_TRY(ensure(ctx, ctx->d_g, (size_t)ctx->vec_total * sizeof(double2)));
         FH_TRY(ensure(ctx, ctx->d_A32, (size_t)ctx->mat_total * sizeof(float2)));

@@ -106,8 +106,13 @@ void launch_rhs(const SolveTables &t, int S, int maxN, const double2 *z, const d
 // Solves A_s x = b_s in place (b_s overwritten by x_s); A_s overwritten by
 // its LU factors.  order[] lists solves largest first.  info[s] = 0 on
 // success, else 1 + column of the first zero / non-finite pivot.
-void launch_lu_solve_fp64(const int *order, int S, const int *N, const long long *mat_off,
-                          const int *vec_off, double2 *A, double2 *b, int *info, cudaStream_t st);
+// order_h, N_h: host copies.  Half of the systems run on `side`, forked from and
+// joined back into st by the two events.  scratch: lu_fp64_scratch_bytes(S).
+size_t lu_fp64_scratch_bytes(int S);
+int lu_fp64_launches(const int *order_h, const int *N_h, int S);
+void launch_lu_solve_fp64(const int *order, const int *order_h, const int *N_h, int S, const int *N,
+                          const long long *mat_off, const int *vec_off, double2 *A, double2 *b, int *info,
+                          void *scratch, cudaStream_t st, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join);
 
 // Mixed precision: FP32 copy (the hi parts) of the double-float matrices,
 // FP32 LU, double-float residual refinement.

@@ -2,18 +2,40 @@
 // A_s psi_s = g_s for every frequency (Sec. 5 step F3; the paper solves its 2D
 // systems directly and notes LU for small problems in its appendix).
 //
-// FP64 path: one CTA per frequency, right-looking blocked LU (panel width
-// NB) on the column-major matrix.  The right side is carried as column N so
-// row swaps and eliminations reach it in flight; back substitution follows.
-// The trailing update A22 -= L21 U12 is a complex rank-NB product staged in
-// shared memory, 4 x 4 complex outputs per thread.
+// FP64 path: right-looking blocked LU (panels of NB = 16 columns) on the
+// column-major matrices, all systems advancing together.  The right side is
+// carried as column N, so that row exchanges and eliminations reach it in
+// flight; L is not needed once its panel's update is done, so columns left of
+// a panel are never exchanged.  Per panel two launches over the systems that
+// still have one (a prefix of the order, largest first):
+//   panel  one CTA per system: partial pivoting within the panel;
+//   strip  one CTA per SW columns right of it: the panel's row exchanges, U12
+//          = L11^{-1} A12, then A22 -= L21 U12 for all rows of the strip.
+// Every second system runs on a second stream, so that one half's panels
+// (short dependent steps that leave most of the chip idle) overlap with the
+// other half's strips.
+//
+// Bound: the FP64 pipe, two FMAs per clock and SM (1.05 TFLOP/s measured), so
+// that one warp's FMA occupies an SM for 16 clocks: loads, shared memory and
+// launches are nearly free, and what counts is that every SM has FMAs to
+// issue.  One CTA per system, as before, leaves the largest system on one SM
+// (N = 480: 43 ms at the SM's peak) and 63 systems on 63 SMs; strips of SW = 8
+// columns spread each system over N / 8 CTAs.
+// Measured (GB300, LU phase; the flops at peak take 2.7 and 20 ms): 63 systems
+// of N = 256: 14.3 -> 3.5 ms; 255 systems of N = 64..480: 78.0 -> 20.5 ms
+// (strips of 16 columns: 3.8 and 21.1 ms).
+#include <algorithm>
+
 #include "fh_internal.h"
 
 namespace fh {
 namespace {
 
-constexpr int NB = 16;   // panel width
-constexpr int TT = 64;   // trailing tile edge
+constexpr int NB = 16;             // panel width
+constexpr int kPanelRows = 512;    // panels of at most this many rows stay in registers
+constexpr int SW = 8;              // columns of a strip
+constexpr int kStripThreads = 128;
+constexpr int kMaxMoved = 2 * NB;
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -22,204 +44,346 @@ __device__ __forceinline__ double2 cinv(double2 a) {
     const double d = a.x * a.x + a.y * a.y;
     return make_double2(a.x / d, -a.y / d);
 }
+// v -= l u in four FMAs (as v -= (l.x u.x - l.y u.y) it takes six instructions)
+__device__ __forceinline__ void csub(double2 &v, double2 l, double2 u) {
+    v.x = fma(l.y, u.y, fma(-l.x, u.x, v.x));
+    v.y = fma(-l.y, u.x, fma(-l.x, u.y, v.y));
+}
 
-__global__ void __launch_bounds__(256) lu_solve_fp64_kernel(
-    const int *__restrict__ order, const int *__restrict__ Ns,
-    const long long *__restrict__ mat_off, const int *__restrict__ vec_off,
-    double2 *__restrict__ A, double2 *__restrict__ B, int *__restrict__ info) {
-    const int s = order[blockIdx.x];
-    const int n = Ns[s];
-    double2 *a = A + mat_off[s];
-    double2 *y = B + vec_off[s];
-    const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
+// Rows that a panel moves, relative to its first row: row src goes to dst.
+struct Moves {
+    int cnt, dst[kMaxMoved], src[kMaxMoved];
+};
 
-    __shared__ double red_v[8];
-    __shared__ int red_i[8];
-    __shared__ int sh_piv, sh_bad;
-    __shared__ double2 sh_val;
-    __shared__ double2 Ls[TT][NB + 1];
-    __shared__ double2 Us[NB][TT];
+// Pivot key of an active row: the bits of |re| + |im| (monotone as integers;
+// NaN above everything), then ~position (the smaller position wins a tie).
+struct Key {
+    unsigned hi, lo, pos;
+};
+__device__ __forceinline__ Key key_of(double2 v, int pos) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(fabs(v.x) + fabs(v.y));
+    return {(unsigned)(b >> 32), (unsigned)b, ~(unsigned)pos};
+}
+__device__ __forceinline__ Key warp_max(Key k) {
+    const unsigned h = __reduce_max_sync(0xffffffffu, k.hi);
+    const unsigned l = __reduce_max_sync(0xffffffffu, k.hi == h ? k.lo : 0u);
+    const unsigned p = __reduce_max_sync(0xffffffffu, k.hi == h && k.lo == l ? k.pos : 0u);
+    return {h, l, p};
+}
+__device__ __forceinline__ bool key_less(Key a, Key b) {
+    return a.hi != b.hi ? a.hi < b.hi : a.lo != b.lo ? a.lo < b.lo : a.pos < b.pos;
+}
+__device__ __forceinline__ bool key_bad(Key k) {   // nothing left, zero, infinite or NaN
+    return k.pos == 0u || (k.hi | k.lo) == 0u || k.hi >= 0x7FF00000u;
+}
 
-#define AT(i, j) a[(long long)(j) * n + (i)]
+struct PanelShared {
+    Key best[2][kPanelRows / 32];   // best key of every warp
+    double2 row[2][NB];             // the pivot row from its column on
+    double2 pinv[2];
+    Moves mv;
+};
 
-    for (int k0 = 0; k0 < n; k0 += NB) {
-        const int nb = min(NB, n - k0);
-        // ---- panel factorisation, columns k0 .. k0+nb-1 ----
-        for (int c = k0; c < k0 + nb; ++c) {
-            double best = -1.0;
-            int bi = n;
-            for (int r = c + tid; r < n; r += 256) {
-                const double2 v = AT(r, c);
-                const double m = fabs(v.x) + fabs(v.y);
-                if (m > best) { best = m; bi = r; }
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                const double ov = __shfl_down_sync(0xffffffffu, best, o);
-                const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-                if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
-            }
-            if (lane == 0) { red_v[warp] = best; red_i[warp] = bi; }
-            __syncthreads();
-            if (tid == 0) {
-                double bv = red_v[0];
-                int bidx = red_i[0];
-                for (int w = 1; w < 8; ++w)
-                    if (red_v[w] > bv || (red_v[w] == bv && red_i[w] < bidx)) { bv = red_v[w]; bidx = red_i[w]; }
-                int bad = !(bv > 0.0) || bidx >= n;
-                double2 pv = make_double2(0.0, 0.0);
-                if (!bad) {
-                    pv = AT(bidx, c);
-                    bad = !isfinite(pv.x) || !isfinite(pv.y);
-                }
-                if (bad) info[s] = c + 1;
-                sh_bad = bad;
-                sh_piv = bidx;
-                if (!bad) sh_val = cinv(pv);
-            }
-            __syncthreads();
-            if (sh_bad) return;
-            const int p = sh_piv;
-            if (p != c) {
-                for (int j = tid; j < n; j += 256) {
-                    const double2 t0 = AT(c, j);
-                    AT(c, j) = AT(p, j);
-                    AT(p, j) = t0;
-                }
-                if (tid == 0) { const double2 t0 = y[c]; y[c] = y[p]; y[p] = t0; }
-            }
-            __syncthreads();
-            const double2 pinv = sh_val;
-            for (int r = c + 1 + tid; r < n; r += 256) AT(r, c) = cmul(AT(r, c), pinv);
-            __syncthreads();
-            const int ncols = k0 + nb - c - 1;
-            const int rows = n - c - 1;
-            if (ncols > 0 && rows > 0) {
-                for (int e = tid; e < rows * ncols; e += 256) {
-                    const int r = c + 1 + e % rows;
-                    const int j = c + 1 + e / rows;
-                    const double2 l = AT(r, c), u = AT(c, j);
-                    double2 v = AT(r, j);
-                    v.x -= l.x * u.x - l.y * u.y;
-                    v.y -= l.x * u.y + l.y * u.x;
-                    AT(r, j) = v;
-                }
-            }
-            __syncthreads();
+// Columns k0 .. k0 + 15 of system order[first + 2 blockIdx.x]: up to 512 rows
+// with one row per thread in registers.  Rows do not move; each thread tracks
+// the position its row has under the exchanges, and rows go to their final
+// place at the end.  Per column: keys reduced by redux within the warps and
+// across them, the winning thread publishes its row and the reciprocal of the
+// pivot (one division per column: a warp's FP64 division occupies the SM's
+// pipe for ~500 clocks), the others eliminate.
+__device__ void panel_registers(double2 *a, int n, int k0, PanelShared &ps, int *info) {
+    const int m = n - k0, nb = min(NB, m), t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int nw = blockDim.x >> 5;
+    double2 v[NB];
+    const bool own = t < m;
+#pragma unroll
+    for (int q = 0; q < NB; ++q)
+        v[q] = own && q < nb ? a[(long long)(k0 + q) * n + k0 + t] : make_double2(0.0, 0.0);
+    int pos = t;
+    bool active = own;
+#pragma unroll
+    for (int c = 0; c < NB; ++c) {
+        if (c >= nb) break;
+        const int pb = c & 1;
+        const Key mine = active ? key_of(v[c], pos) : Key{0u, 0u, 0u};
+        const Key wb = warp_max(mine);
+        if (lane == 0) ps.best[pb][warp] = wb;
+        __syncthreads();
+        const Key k = warp_max(lane < nw ? ps.best[pb][lane] : Key{0u, 0u, 0u});
+        if (key_bad(k)) {   // the same verdict in every thread
+            if (t == 0) *info = k0 + c + 1;
+            return;
         }
-        // ---- U12 = L11^{-1} A12 (columns k0+nb .. n-1, column n = right side) ----
-        for (int j = k0 + nb + tid; j <= n; j += 256) {
-            double2 x[NB];
+        const int wpos = (int)~k.pos;
+        if (active && pos == wpos) {
 #pragma unroll
-            for (int q = 0; q < NB; ++q)
-                if (q < nb) x[q] = (j < n) ? AT(k0 + q, j) : y[k0 + q];
-#pragma unroll
-            for (int q = 0; q < NB; ++q) {
-                if (q < nb) {
-#pragma unroll
-                    for (int r = q + 1; r < NB; ++r) {
-                        if (r < nb) {
-                            const double2 l = AT(k0 + r, k0 + q);
-                            x[r].x -= l.x * x[q].x - l.y * x[q].y;
-                            x[r].y -= l.x * x[q].y + l.y * x[q].x;
-                        }
-                    }
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < NB; ++q)
-                if (q < nb) {
-                    if (j < n) AT(k0 + q, j) = x[q]; else y[k0 + q] = x[q];
-                }
+            for (int q = c; q < NB; ++q) ps.row[pb][q] = v[q];
+            ps.pinv[pb] = cinv(v[c]);
+            pos = c;
+            active = false;
+        } else if (active && pos == c) {
+            pos = wpos;   // exchanged with the pivot row
         }
         __syncthreads();
-        // ---- trailing update A22 -= L21 U12 (column n = right side) ----
-        const int r0 = k0 + nb;
-        const int m = n - r0;
-        if (m > 0) {
-            const int ntr = (m + TT - 1) / TT, ntc = (m + 1 + TT - 1) / TT;
-            const int tx = tid & 15, ty = tid >> 4;
-            for (int tile = 0; tile < ntr * ntc; ++tile) {
-                const int i0 = r0 + (tile % ntr) * TT, j0 = r0 + (tile / ntr) * TT;
-                for (int e = tid; e < TT * NB; e += 256) {
-                    const int rr = e % TT, q = e / TT;
-                    double2 v = make_double2(0.0, 0.0);
-                    if (i0 + rr < n && q < nb) v = AT(i0 + rr, k0 + q);
-                    Ls[rr][q] = v;
-                }
-                for (int e = tid; e < TT * NB; e += 256) {
-                    const int q = e % NB, cc = e / NB;
-                    const int j = j0 + cc;
-                    double2 v = make_double2(0.0, 0.0);
-                    if (q < nb && j <= n) v = (j < n) ? AT(k0 + q, j) : y[k0 + q];
-                    Us[q][cc] = v;
-                }
-                __syncthreads();
-                double2 acc[4][4];
+        if (active) {
+            const double2 l = cmul(v[c], ps.pinv[pb]);
+            v[c] = l;
 #pragma unroll
-                for (int aa = 0; aa < 4; ++aa)
+            for (int q = c + 1; q < NB; ++q) csub(v[q], l, ps.row[pb][q]);
+        }
+    }
+    if (own) {
 #pragma unroll
-                    for (int bb = 0; bb < 4; ++bb) {
-                        const int i = i0 + tx + 16 * aa, j = j0 + ty + 16 * bb;
-                        double2 v = make_double2(0.0, 0.0);
-                        if (i < n && j <= n) v = (j < n) ? AT(i, j) : y[i];
-                        acc[aa][bb] = v;
-                    }
-#pragma unroll 4
-                for (int q = 0; q < NB; ++q) {
-                    double2 l[4], u[4];
-#pragma unroll
-                    for (int aa = 0; aa < 4; ++aa) l[aa] = Ls[tx + 16 * aa][q];
-#pragma unroll
-                    for (int bb = 0; bb < 4; ++bb) u[bb] = Us[q][ty + 16 * bb];
-#pragma unroll
-                    for (int aa = 0; aa < 4; ++aa)
-#pragma unroll
-                        for (int bb = 0; bb < 4; ++bb) {
-                            acc[aa][bb].x -= l[aa].x * u[bb].x - l[aa].y * u[bb].y;
-                            acc[aa][bb].y -= l[aa].x * u[bb].y + l[aa].y * u[bb].x;
-                        }
-                }
-#pragma unroll
-                for (int aa = 0; aa < 4; ++aa)
-#pragma unroll
-                    for (int bb = 0; bb < 4; ++bb) {
-                        const int i = i0 + tx + 16 * aa, j = j0 + ty + 16 * bb;
-                        if (i < n && j <= n) {
-                            if (j < n) AT(i, j) = acc[aa][bb]; else y[i] = acc[aa][bb];
-                        }
-                    }
-                __syncthreads();
+        for (int q = 0; q < NB; ++q)
+            if (q < nb) a[(long long)(k0 + q) * n + k0 + pos] = v[q];
+        if (pos != t) {
+            const int i = atomicAdd(&ps.mv.cnt, 1);
+            if (i < kMaxMoved) {   // at most 2 NB rows change position
+                ps.mv.dst[i] = pos;
+                ps.mv.src[i] = t;
             }
         }
     }
-    // ---- back substitution U x = y ----
-    for (int j = n - 1; j >= 0; --j) {
-        if (tid == 0) {
-            const double2 xj = cmul(y[j], cinv(AT(j, j)));
-            y[j] = xj;
-            sh_val = xj;
+}
+
+// The same panel for any number of rows, in place: rows are exchanged in the
+// panel's columns; the update of a column's right neighbours also finds the
+// next column's best key.
+__device__ void panel_memory(double2 *a, int n, int k0, PanelShared &ps, int *info) {
+    const int m = n - k0, nb = min(NB, m), t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int nw = blockDim.x >> 5;
+    double2 *p0 = a + (long long)k0 * n + k0;   // panel element (r, q) at p0[q n + r]
+    Key next = {0u, 0u, 0u};
+    for (int r = t; r < m; r += blockDim.x) {
+        const Key k = key_of(p0[r], r);
+        if (key_less(next, k)) next = k;
+    }
+    for (int c = 0; c < nb; ++c) {
+        const int pb = c & 1;
+        const Key wb = warp_max(next);
+        if (lane == 0) ps.best[pb][warp] = wb;
+        __syncthreads();
+        const Key k = warp_max(lane < nw ? ps.best[pb][lane] : Key{0u, 0u, 0u});
+        if (key_bad(k)) {
+            if (t == 0) *info = k0 + c + 1;
+            return;
+        }
+        const int wpos = (int)~k.pos;
+        if (t < nb) {
+            double2 *col = p0 + (long long)t * n;
+            const double2 u = col[wpos];
+            if (wpos != c) {
+                col[wpos] = col[c];
+                col[c] = u;
+            }
+            ps.row[pb][t] = u;
+            if (t == c) ps.pinv[pb] = cinv(u);
+        }
+        if (t == 0 && wpos != c) {   // compose the exchange (c, wpos) with the moves so far
+            int ic = -1, ip = -1;
+            for (int i = 0; i < ps.mv.cnt; ++i) {
+                if (ps.mv.dst[i] == c) ic = i;
+                if (ps.mv.dst[i] == wpos) ip = i;
+            }
+            if (ic < 0) {
+                ic = ps.mv.cnt++;
+                ps.mv.dst[ic] = ps.mv.src[ic] = c;
+            }
+            if (ip < 0) {
+                ip = ps.mv.cnt++;
+                ps.mv.dst[ip] = ps.mv.src[ip] = wpos;
+            }
+            const int s0 = ps.mv.src[ic];
+            ps.mv.src[ic] = ps.mv.src[ip];
+            ps.mv.src[ip] = s0;
         }
         __syncthreads();
-        const double2 xj = sh_val;
-        for (int i = tid; i < j; i += 256) {
-            const double2 u = AT(i, j);
+        const double2 pinv = ps.pinv[pb];
+        next = {0u, 0u, 0u};
+        for (int r = c + 1 + t; r < m; r += blockDim.x) {
+            const double2 l = cmul(p0[(long long)c * n + r], pinv);
+            p0[(long long)c * n + r] = l;
+            for (int q = c + 1; q < nb; ++q) {
+                double2 v = p0[(long long)q * n + r];
+                csub(v, l, ps.row[pb][q]);
+                p0[(long long)q * n + r] = v;
+                if (q == c + 1) {
+                    const Key k1 = key_of(v, r);
+                    if (key_less(next, k1)) next = k1;
+                }
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kPanelRows) lu_panel_fp64_kernel(
+    const int *__restrict__ order, const int *__restrict__ Ns, const long long *__restrict__ mat_off,
+    double2 *__restrict__ A, Moves *__restrict__ moves, int *__restrict__ info, int k0) {
+    __shared__ PanelShared ps;
+    const int s = order[2 * blockIdx.x];
+    if (info[s] != 0) return;
+    const int n = Ns[s];
+    double2 *a = A + mat_off[s];
+    if (threadIdx.x == 0) ps.mv.cnt = 0;
+    __syncthreads();
+    // by the system's own size, so that its result does not depend on the batch
+    if (n - k0 <= kPanelRows) panel_registers(a, n, k0, ps, info + s);
+    else panel_memory(a, n, k0, ps, info + s);
+    __syncthreads();
+    Moves *mv = moves + s;
+    for (int i = threadIdx.x; i < kMaxMoved; i += blockDim.x) {
+        mv->dst[i] = ps.mv.dst[i];
+        mv->src[i] = ps.mv.src[i];
+    }
+    if (threadIdx.x == 0) mv->cnt = min(ps.mv.cnt, kMaxMoved);
+}
+
+// Columns j0 .. j0 + SW - 1 (j0 = k0 + 16 + SW blockIdx.x; column n is the right
+// side) of system order[first + 2 blockIdx.y]: exchanges, U12, update.  A
+// thread takes a row with its 16 values of L in registers; U12 is broadcast
+// from shared memory (one 16-byte read per four FMAs).
+__global__ void __launch_bounds__(kStripThreads, 4) lu_strip_fp64_kernel(
+    const int *__restrict__ order, const int *__restrict__ Ns, const long long *__restrict__ mat_off,
+    const int *__restrict__ vec_off, double2 *__restrict__ A, double2 *__restrict__ B,
+    const Moves *__restrict__ moves, const int *__restrict__ info, int k0) {
+    __shared__ double2 L11[NB][NB + 1], U[SW][NB];   // U[column][row]
+    const int s = order[2 * blockIdx.y], n = Ns[s];
+    const int nb = min(NB, n - k0), j0 = k0 + nb + SW * (int)blockIdx.x;
+    if (j0 > n || info[s] != 0) return;
+    const int nc = min(SW, n + 1 - j0), t = threadIdx.x;
+    double2 *a = A + mat_off[s], *y = B + vec_off[s];
+    auto column = [&](int j) { return j < n ? a + (long long)j * n : y; };
+    // row exchanges: every moved row of the strip is read before any is written
+    const int nmv = moves[s].cnt;
+    double2 mvv[kMaxMoved * SW / kStripThreads];
+#pragma unroll
+    for (int i = 0; i < kMaxMoved * SW / kStripThreads; ++i) {
+        const int e = t + i * kStripThreads, p = e & (kMaxMoved - 1), c = e / kMaxMoved;
+        if (p < nmv && c < nc) mvv[i] = column(j0 + c)[k0 + moves[s].src[p]];
+    }
+    for (int e = t; e < NB * NB; e += kStripThreads) {
+        const int r = e % NB, q = e / NB;
+        L11[r][q] = r < nb && q < r ? a[(long long)(k0 + q) * n + k0 + r] : make_double2(0.0, 0.0);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kMaxMoved * SW / kStripThreads; ++i) {
+        const int e = t + i * kStripThreads, p = e & (kMaxMoved - 1), c = e / kMaxMoved;
+        if (p < nmv && c < nc) column(j0 + c)[k0 + moves[s].dst[p]] = mvv[i];
+    }
+    __syncthreads();
+    // U12: half a warp per column, lane r holds row r
+    const int r = t & (NB - 1);
+#pragma unroll
+    for (int h = 0; h < NB * SW / kStripThreads; ++h) {
+        const int c = t / NB + h * (kStripThreads / NB);
+        double2 *col = column(j0 + min(c, nc - 1)) + k0;
+        double2 x = r < nb ? col[r] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int q = 0; q < NB - 1; ++q) {
+            const double2 xq = make_double2(__shfl_sync(0xffffffffu, x.x, q, NB), __shfl_sync(0xffffffffu, x.y, q, NB));
+            if (r > q) csub(x, L11[r][q], xq);
+        }
+        if (c < nc && r < nb) col[r] = x;
+        U[c][r] = x;
+    }
+    __syncthreads();
+    const int r0 = k0 + nb;   // nb == NB whenever rows are left
+    for (int i = r0 + t; i < n; i += kStripThreads) {
+        double2 l[NB];
+#pragma unroll
+        for (int q = 0; q < NB; ++q) l[q] = a[(long long)(k0 + q) * n + i];
+#pragma unroll 2
+        for (int c = 0; c < nc; ++c) {
+            double2 *p = column(j0 + c) + i;
+            double2 v = *p;
+#pragma unroll
+            for (int q = 0; q < NB; ++q) csub(v, l[q], U[c][q]);
+            *p = v;
+        }
+    }
+}
+
+// Back substitution U x = y in place, one CTA per system, blocks of 16
+// columns from the last: half a warp solves the diagonal block (lane r holds
+// row r), then every row above subtracts the block's 16 products.
+__global__ void __launch_bounds__(256) lu_back_fp64_kernel(
+    const int *__restrict__ order, const int *__restrict__ Ns, const long long *__restrict__ mat_off,
+    const int *__restrict__ vec_off, const double2 *__restrict__ A, double2 *__restrict__ B,
+    const int *__restrict__ info) {
+    __shared__ double2 xs[NB];
+    const int s = order[blockIdx.x], n = Ns[s], t = threadIdx.x;
+    if (info[s] != 0) return;
+    const double2 *a = A + mat_off[s];
+    double2 *y = B + vec_off[s];
+    for (int jb = (n - 1) / NB * NB; jb >= 0; jb -= NB) {
+        const int nb = min(NB, n - jb);
+        if (t < NB) {
+            double2 u[NB];
+#pragma unroll
+            for (int q = 0; q < NB; ++q)
+                u[q] = t < nb && q >= t && q < nb ? a[(long long)(jb + q) * n + jb + t] : make_double2(0.0, 0.0);
+            double2 x = t < nb ? y[jb + t] : make_double2(0.0, 0.0);
+            double2 inv = make_double2(0.0, 0.0);   // reciprocal of the lane's diagonal entry
+#pragma unroll
+            for (int q = 0; q < NB; ++q)
+                if (q == t) inv = u[q];
+            inv = t < nb ? cinv(inv) : inv;
+#pragma unroll
+            for (int q = NB - 1; q >= 0; --q) {
+                if (t == q) x = cmul(x, inv);
+                const double2 xq = make_double2(__shfl_sync(0xffffu, x.x, q, NB), __shfl_sync(0xffffu, x.y, q, NB));
+                if (t < q && q < nb) csub(x, u[q], xq);
+            }
+            if (t < nb) y[jb + t] = x;
+            xs[t] = x;
+        }
+        __syncthreads();
+        for (int i = t; i < jb; i += blockDim.x) {
             double2 v = y[i];
-            v.x -= u.x * xj.x - u.y * xj.y;
-            v.y -= u.x * xj.y + u.y * xj.x;
+#pragma unroll
+            for (int q = NB - 1; q >= 0; --q)
+                if (q < nb) csub(v, a[(long long)(jb + q) * n + i], xs[q]);
             y[i] = v;
         }
         __syncthreads();
     }
-#undef AT
 }
 
 }  // namespace
 
-void launch_lu_solve_fp64(const int *order, int S, const int *N, const long long *mat_off,
-                          const int *vec_off, double2 *A, double2 *b, int *info, cudaStream_t st) {
+size_t lu_fp64_scratch_bytes(int S) { return (size_t)S * sizeof(Moves); }
+
+int lu_fp64_launches(const int *order_h, const int *N_h, int S) {
+    int n = S > 0 ? 1 : 0;
+    for (int half = 0; half < 2 && half < S; ++half) n += 2 * ((N_h[order_h[half]] + NB - 1) / NB);
+    return n;
+}
+
+void launch_lu_solve_fp64(const int *order, const int *order_h, const int *N_h, int S, const int *N,
+                          const long long *mat_off, const int *vec_off, double2 *A, double2 *b, int *info,
+                          void *scratch, cudaStream_t st, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join) {
     if (S <= 0) return;
-    lu_solve_fp64_kernel<<<S, 256, 0, st>>>(order, N, mat_off, vec_off, A, b, info);
+    Moves *mv = static_cast<Moves *>(scratch);
+    cudaEventRecord(fork, st);
+    cudaStreamWaitEvent(side, fork, 0);
+    for (int half = 0; half < 2 && half < S; ++half) {   // systems half, half + 2, .. of the order
+        cudaStream_t q = half ? side : st;
+        int active = (S - half + 1) / 2;
+        const int n0 = N_h[order_h[half]];
+        for (int k0 = 0; k0 < n0; k0 += NB) {
+            while (N_h[order_h[half + 2 * (active - 1)]] <= k0) --active;
+            const int rows = std::min(n0 - k0, kPanelRows);
+            lu_panel_fp64_kernel<<<active, (rows + 31) / 32 * 32, 0, q>>>(order + half, N, mat_off, A, mv, info, k0);
+            // columns right of the panel with the right side (the smaller systems' extra CTAs return)
+            const int strips = (std::max(n0 - k0 - NB, 0) + SW) / SW;
+            lu_strip_fp64_kernel<<<dim3(strips, active), kStripThreads, 0, q>>>(order + half, N, mat_off, vec_off, A,
+                                                                                b, mv, info, k0);
+        }
+    }
+    cudaEventRecord(join, side);
+    cudaStreamWaitEvent(st, join, 0);
+    lu_back_fp64_kernel<<<S, 256, 0, st>>>(order, N, mat_off, vec_off, A, b, info);
 }
 
 }  // namespace fh
