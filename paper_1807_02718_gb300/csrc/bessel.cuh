@@ -119,15 +119,15 @@ __device__ __forceinline__ void pq_horner(const PQShared &tb, double x, double r
     }
 }
 
-// Small-argument branch (x < 8) of the joint routine.
-__device__ __forceinline__ void bessel_small(double x, double &J0, double &Y0, double &J1,
-                                             double &Y1) {
+// Small-argument branch (x < 8) with ln(x/2) given (shared by a frequency group).
+__device__ __forceinline__ void bessel_small_ln(double x, double lnh, double &J0, double &Y0, double &J1,
+                                                double &Y1) {
     const double t = x * x * (1.0 / 32.0) - 1.0;
     J0 = clenshaw<kA0_N>(kA0, t);
     const double a1 = clenshaw<kA1_N>(kA1, t);
     const double a2 = clenshaw<kA2_N>(kA2, t);
     const double a3 = clenshaw<kA3_N>(kA3, t);
-    const double L = kTwoOverPi * log(0.5 * x);
+    const double L = kTwoOverPi * lnh;
     Y0 = fma(L, J0, a1);
     J1 = x * a2;
     Y1 = fma(L, J1, fma(x, a3, -kTwoOverPi / x));

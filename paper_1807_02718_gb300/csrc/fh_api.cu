@@ -397,12 +397,11 @@ void split_groups(fh_ctx *ctx, int gmax, std::vector<int2> &sg, std::vector<doub
     }
 }
 
-// Assembly CTAs of one matrix order n (tiles of 32 x 32): all nt^2 tiles for
-// the FP64 kernel, the nt (nt + 1) / 2 tiles of the upper triangle for the
-// double-float kernel (which writes both entries of each node pair).
-long long assembly_tiles(const fh_ctx *ctx, int n) {
+// Assembly CTAs of one matrix order n: the nt (nt + 1) / 2 tiles of 32 x 32 of
+// the upper triangle (the kernels write both entries of each node pair).
+long long assembly_tiles(int n) {
     const long long nt = (n + 31) / 32;
-    return ctx->precision == FH_FP64 ? nt * nt : nt * (nt + 1) / 2;
+    return nt * (nt + 1) / 2;
 }
 
 // Work lists of the assembly and target-field kernels under ctx->tune
@@ -434,7 +433,7 @@ fh_status build_schedules(fh_ctx *ctx) {
     long long gt = 0;
     for (const int2 &g : ctx->sg) {
         ctx->sg_tile_off.push_back(gt);
-        gt += assembly_tiles(ctx, ctx->solve_N[g.x]);
+        gt += assembly_tiles(ctx->solve_N[g.x]);
         for (int j = 0; j < g.y; ++j) ctx->order.push_back(g.x + j);
     }
     ctx->sg_tile_off.push_back(gt);
@@ -1546,7 +1545,7 @@ fh_status fh_assemble_matrix(fh_ctx *ctx, int j, double eta_j, double *A, double
     eta[s] = eta_j;
     FH_TRY(upload(ctx, ctx->d_eta, eta));
     std::vector<int2> sg1 = {sgv};
-    std::vector<long long> to1 = {0, assembly_tiles(ctx, n)};
+    std::vector<long long> to1 = {0, assembly_tiles(n)};
     std::vector<double> dk1 = {ctx->sg_dk[gi]};
     FH_TRY(upload(ctx, ctx->d_tmp_sg, sg1));
     FH_TRY(upload(ctx, ctx->d_tmp_ll, to1));

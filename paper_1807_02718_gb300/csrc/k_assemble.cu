@@ -14,11 +14,11 @@
 // Diagonal limits: M1 = -s/4pi, M2 = [i/4 - C/2pi - ln(kappa s/2)/2pi] s,
 // L1 = 0, L2 = (z1'' z2' - z2'' z1') / (4 pi s^2).
 //
-// One CTA assembles one 32 x 32 tile for up to kGroup frequencies; tiles of
-// all frequencies (of all problems of a batch) form one flat launch (prefix
-// offsets tile_off).  Each warp writes 32 consecutive rows of a column:
-// column-major stores of 512 B (the double-float kernel also writes the
-// transposed entries, 16 B per row, which meet in L2).
+// One CTA assembles one 32 x 32 tile of the upper triangle, and its mirror
+// image, for up to kGroup frequencies; tiles of all frequencies (of all
+// problems of a batch) form one flat launch (prefix offsets tile_off).  Each
+// warp writes 32 consecutive rows of a column (512 B) and the transposed
+// entries, 16 B per row, which meet in L2.
 #include "bessel.cuh"
 #include "dfloat.cuh"
 #include "fh_internal.h"
@@ -38,12 +38,32 @@ __device__ __forceinline__ int find_solve(const long long *__restrict__ off, int
     return lo;
 }
 
-// Grouped assembly: one CTA per 32 x 32 tile of a frequency subgroup (up to
-// kGroup consecutive frequencies with the same N, hence the same nodes).  The
-// geometry of each entry (r, N_il, Kress weight, log kernel, speeds) and the
-// phase e^{i(kappa_0 r - pi/4)} with its step e^{i dkappa r} are computed once;
-// each frequency then evaluates the P/Q series and writes its own matrix.
-__global__ void __launch_bounds__(256) assemble_group_kernel(
+// Upper-triangle tile of flat index lt: lt = tc (tc + 1) / 2 + tr, 0 <= tr <= tc.
+__device__ __forceinline__ void triangle_tile(long long lt, int &tr, int &tc) {
+    int c = (int)((sqrtf(8.f * (float)lt + 1.f) - 1.f) * 0.5f);
+    while (c > 0 && (long long)c * (c + 1) / 2 > lt) --c;
+    while ((long long)(c + 1) * (c + 2) / 2 <= lt) ++c;
+    tc = c;
+    tr = (int)(lt - (long long)c * (c + 1) / 2);
+}
+
+// FP64 assembly.  Per node pair and frequency, with
+//   g4 = N_il s_l / (4 s_i r),  s4 = s_l / 4,  W = (pi/n) ln(4 sin^2) - R,
+//   A1 = g4 W/pi, B1 = g4 pi/n, C1 = s4 pi/n, D1 = s4 W/pi,
+//   Re A = kappa (A1 J1 - B1 Y1) + eta C1 J0,  Im A = kappa B1 J1 + eta (C1 Y0 - D1 J0)
+// (the combination of M, M1, M2, L, L1, L2 above).  r, the Bessel values and W
+// (even in i - l) are those of A(l, i) too, so a CTA takes a 32 x 32 tile of
+// the upper triangle for up to kGroup frequencies of one N and writes both
+// entries of every pair, the second one with its own geometry factors (N_li,
+// s_i and s_l exchanged).  Once per pair: the geometry factors, the phase
+// e^{i(kappa_0 r - pi/4)} with the amplitude sqrt(2 / (pi r)), the step e^{i
+// dkappa r}, and ln r where the small-argument series will need it.
+// Bound by the FP64 pipe (2 FMAs per clock and SM): about 100 FP64 instructions
+// per entry, the small-argument series of the near-diagonal warps included,
+// against 168 for one thread per entry with M1, M2, L1, L2 formed separately.
+// Measured (GB300): 255 systems of N 64..480: 5.75 -> 3.56 ms; 63 systems of N =
+// 256: 1.77 -> 1.10 ms.
+__global__ void __launch_bounds__(256, 2) assemble_group_kernel(
     SolveTables t, Subgroups grp, int n_groups, const double2 *__restrict__ z,
     const double2 *__restrict__ dz, const double2 *__restrict__ ddz,
     const double *__restrict__ kress, const double *__restrict__ logsin,
@@ -53,10 +73,9 @@ __global__ void __launch_bounds__(256) assemble_group_kernel(
     const int2 sgv = grp.sg[g];
     const int s0 = sgv.x, cnt = sgv.y;
     const int N = t.N[s0];
-    const int nt = (N + kTile - 1) / kTile;
-    const long long lt = b - grp.tile_off[g];
-    const int tr = (int)(lt % nt), tc = (int)(lt / nt);
-    __shared__ double kap[kGroup], eta[kGroup], ikap[kGroup], isqk[kGroup], corr[kGroup];
+    int tr, tc;
+    triangle_tile(b - grp.tile_off[g], tr, tc);
+    __shared__ double kap[kGroup], eta[kGroup], ikap8[kGroup], sqk[kGroup], eqk[kGroup], lnk2[kGroup], corr[kGroup];
     __shared__ long long moff[kGroup];
     __shared__ PQShared pqt;
     pq_stage(pqt);
@@ -64,10 +83,13 @@ __global__ void __launch_bounds__(256) assemble_group_kernel(
     if (threadIdx.x < kGroup) {
         const int j = threadIdx.x;
         const double k = (j < cnt) ? t.kappa[s0 + j] : 1.0;
+        const double e = (j < cnt) ? t.eta[s0 + j] : 0.0;
         kap[j] = k;
-        eta[j] = (j < cnt) ? t.eta[s0 + j] : 0.0;
-        ikap[j] = 1.0 / k;
-        isqk[j] = 1.0 / sqrt(k);
+        eta[j] = e;
+        ikap8[j] = 8.0 / k;
+        sqk[j] = sqrt(k);
+        eqk[j] = e / sqrt(k);
+        lnk2[j] = log(0.5 * k);
         moff[j] = ((j < cnt) ? t.mat_off[s0 + j] : 0) + out_shift;
     }
     __syncthreads();
@@ -81,16 +103,16 @@ __global__ void __launch_bounds__(256) assemble_group_kernel(
     const double2 zi = z[vo + i], dzi = dz[vo + i];
     const double si = sqrt(dzi.x * dzi.x + dzi.y * dzi.y);
     const double inv4pi = 1.0 / (4.0 * kPi);
+    const double isi = 1.0 / si, si4 = 0.25 * si, C2 = si4 * pin;
 
     for (int q = threadIdx.x >> 5; q < kTile; q += 8) {
         const int l = tc * kTile + q;
         if (l >= N) break;
+        if (tr == tc && l < i) continue;   // each pair once on a diagonal tile
         int d = i - l;
         if (d < 0) d += N;
         const double Rw = kress[to + d];
-        const double2 dzl = dz[vo + l];
-        const double sl = sqrt(dzl.x * dzl.x + dzl.y * dzl.y);
-        const long long e_off = (long long)l * N + i;
+        const long long e_il = (long long)l * N + i, e_li = (long long)i * N + l;
         if (l == i) {
             const double2 dd = ddz[vo + i];
             const double M1 = -si * inv4pi;
@@ -100,55 +122,59 @@ __global__ void __launch_bounds__(256) assemble_group_kernel(
                 const double M2i = 0.25 * si;
                 const double ar = 0.5 + pin * (L2r + eta[j] * M2i);
                 const double ai = Rw * (-eta[j] * M1) + pin * (0.0 - eta[j] * M2r);
-                A[moff[j] + e_off] = make_double2(ar, ai);
+                A[moff[j] + e_il] = make_double2(ar, ai);
             }
             continue;
         }
-        const double2 zl = z[vo + l];
+        const double2 zl = z[vo + l], dzl = dz[vo + l];
         const double d1 = zl.x - zi.x, d2 = zl.y - zi.y;
         const double r = sqrt(d1 * d1 + d2 * d2);
         const double ir = 1.0 / r;
-        const double Nil = dzi.y * d1 - dzi.x * d2;
-        const double ls = logsin[to + d];
-        const double gg = Nil * sl / (si * r);
+        const double sl = sqrt(dzl.x * dzl.x + dzl.y * dzl.y);
+        const double sl4 = 0.25 * sl;
+        const double Wp = fma(pin, logsin[to + d], -Rw) * (1.0 / kPi);   // W / pi
+        const double g4 = (dzi.y * d1 - dzi.x * d2) * sl4 * isi * ir;     // N_il s_l / (4 s_i r)
+        const double h4 = (dzl.x * d2 - dzl.y * d1) * si4 / sl * ir;      // N_li s_i / (4 s_l r)
+        const double A1 = g4 * Wp, B1 = g4 * pin, C1 = sl4 * pin, D1 = sl4 * Wp;
+        const double A2 = h4 * Wp, B2 = h4 * pin, D2 = si4 * Wp;
         const double amp = sqrt(kTwoOverPi * ir);
         double sn, cs, ss, sc;
         sincos(kap[0] * r, &sn, &cs);
         sincos(dk * r, &ss, &sc);
-        double c0 = (cs + sn) * kSqrtHalf, s0v = (sn - cs) * kSqrtHalf;   // e^{i(x0 - pi/4)}
-#pragma unroll
-        for (int j = 0; j < kGroup; ++j) {
-            if (j < cnt) {
-                const double kappa = kap[j];
-                const double x = kappa * r;
-                double J0, Y0, J1, Y1;
-                if (x >= 8.0) {
-                    const double dl = corr[j] * r;
-                    const double c = c0 - dl * s0v, sv = s0v + dl * c0;
-                    double P0, Q0, P1, Q1;
-                    pq_horner<true>(pqt, x, 8.0 * ir * ikap[j], P0, Q0, P1, Q1);
-                    const double Am = amp * isqk[j];
-                    J0 = Am * (P0 * c - Q0 * sv);
-                    Y0 = Am * (P0 * sv + Q0 * c);
-                    J1 = Am * (P1 * sv + Q1 * c);
-                    Y1 = Am * (Q1 * sv - P1 * c);
-                } else {
-                    bessel_small(x, J0, Y0, J1, Y1);
-                }
-                const double Mr = -0.25 * Y0 * sl, Mi = 0.25 * J0 * sl;
-                const double M1 = -J0 * sl * inv4pi;
-                const double M2r = Mr - M1 * ls;
-                const double Lr = -0.25 * kappa * Y1 * gg, Li = 0.25 * kappa * J1 * gg;
-                const double L1 = -kappa * inv4pi * J1 * gg;
-                const double L2r = Lr - L1 * ls;
-                const double et = eta[j];
-                const double ar = Rw * L1 + pin * (L2r + et * Mi);
-                const double ai = Rw * (-et * M1) + pin * (Li - et * M2r);
-                A[moff[j] + e_off] = make_double2(ar, ai);
-                const double cn = c0 * sc - s0v * ss;
-                s0v = s0v * sc + c0 * ss;
-                c0 = cn;
+        const double ah = amp * kSqrtHalf;
+        double c0 = (cs + sn) * ah, s0v = (sn - cs) * ah;   // amp e^{i(x0 - pi/4)}
+        const double lnr = kap[0] * r < 8.0 ? log(r) : 0.0;   // shared by the group
+#pragma unroll 1
+        for (int j = 0; j < cnt; ++j) {
+            const double x = kap[j] * r;
+            double J0, Y0, J1, Y1;   // times sqrt(kappa_j)
+            if (x >= 8.0) {
+                const double dl = corr[j] * r;
+                const double c = fma(-dl, s0v, c0), sv = fma(dl, c0, s0v);
+                double P0, Q0, P1, Q1;
+                pq_horner<true>(pqt, x, ir * ikap8[j], P0, Q0, P1, Q1);
+                J0 = fma(P0, c, -Q0 * sv);
+                Y0 = fma(P0, sv, Q0 * c);
+                J1 = fma(P1, sv, Q1 * c);
+                Y1 = fma(Q1, sv, -P1 * c);
+            } else {
+                bessel_small_ln(x, lnk2[j] + lnr, J0, Y0, J1, Y1);
+                const double f = sqk[j];
+                J0 *= f;
+                Y0 *= f;
+                J1 *= f;
+                Y1 *= f;
             }
+            J0 *= eqk[j];
+            Y0 *= eqk[j];
+            J1 *= sqk[j];
+            Y1 *= sqk[j];
+            double2 *Aj = A + moff[j];
+            Aj[e_il] = make_double2(fma(A1, J1, fma(C1, J0, -B1 * Y1)), fma(B1, J1, fma(C1, Y0, -D1 * J0)));
+            Aj[e_li] = make_double2(fma(A2, J1, fma(C2, J0, -B2 * Y1)), fma(B2, J1, fma(C2, Y0, -D2 * J0)));
+            const double cn = fma(c0, sc, -s0v * ss);
+            s0v = fma(s0v, sc, c0 * ss);
+            c0 = cn;
         }
     }
 }
@@ -191,11 +217,8 @@ __global__ void __launch_bounds__(256, 3) assemble_group_df_kernel(
     const int2 sgv = grp.sg[g];
     const int s0 = sgv.x, cnt = sgv.y;
     const int N = t.N[s0];
-    const long long lt = b - grp.tile_off[g];
-    int tc = (int)((sqrtf(8.f * (float)lt + 1.f) - 1.f) * 0.5f);
-    while (tc > 0 && (long long)tc * (tc + 1) / 2 > lt) --tc;
-    while ((long long)(tc + 1) * (tc + 2) / 2 <= lt) ++tc;
-    const int tr = (int)(lt - (long long)tc * (tc + 1) / 2);   // 0 <= tr <= tc < ceil(N / 32)
+    int tr, tc;
+    triangle_tile(b - grp.tile_off[g], tr, tc);   // 0 <= tr <= tc < ceil(N / 32)
     __shared__ double kap[kGroup];
     __shared__ float kapf[kGroup], corrf[kGroup];
     __shared__ dfv kapd[kGroup], ikap8[kGroup], sqk[kGroup], eqk[kGroup], lnk2[kGroup];
