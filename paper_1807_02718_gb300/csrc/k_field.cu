@@ -6,8 +6,9 @@
 // on the Nystrom nodes).  omega = 0 has no solve; V(x, 0) := 1 there (the 2D
 // low-frequency limit of the radiating field with data e^{i kappa p.r}).
 //
-// One CTA per (frequency, 128 targets); source nodes are staged through
-// shared memory with the weights c_i = (pi/n) |z'_i| psi_i / 4 premultiplied.
+// One CTA per (frequency subgroup, chunk of nodes, tile of targets); source
+// nodes are staged through shared memory with the weights (pi/n) |z'_i| psi_i /
+// 4 premultiplied.
 #include "bessel.cuh"
 #include "dfloat.cuh"
 #include "fh_internal.h"
@@ -18,15 +19,29 @@ namespace {
 constexpr int kTgt = 128;
 constexpr int kChunk = kFieldChunk;   // largest number of source nodes per work item
 
-// Work item w = (subgroup g, chunk of `chunk` <= kChunk nodes).  One CTA per (128 targets, item):
-// for each target-node pair the distance r, 1/r, sqrt(2/(pi r)),
-// e^{i(kappa_0 r - pi/4)} and the step e^{i dkappa r} are formed once; each
-// frequency j of the subgroup then needs only the Horner P0/Q0 series
-// (x = kappa_j r >= 8) or the small-argument series (x < 8).  The phase
-// carries the exact kappa_j through a first-order correction
-// e^{i (kappa_j - kappa_0 - j dkappa) r}.  Partial sums per item go to
-// scratch; field_reduce_kernel adds them in a fixed order (the result does
-// not depend on scheduling).
+// Work item w = (subgroup g, chunk of `chunk` <= kChunk nodes).  One CTA per
+// (kTileF64 targets, item); thread (target tid % kTileF64, slice tid /
+// kTileF64) takes every kSlicesF64-th node of the chunk, and the slices' sums are
+// added in slice order (the split is the same for every n_x, so that a
+// target's field does not depend on the other targets of the call).
+// For each target-node pair the distance r, 1/r, the phase e^{i(kappa_0 r -
+// pi/4)} with the amplitude sqrt(2/(pi r)) and the step e^{i dkappa r} are formed
+// once; each frequency j of the subgroup then needs only the Horner P0/Q0
+// series (x = kappa_j r >= 8) or the small-argument series (x < 8); 1 /
+// sqrt(kappa_j) is on the staged densities.  The phase carries the exact
+// kappa_j through a first-order correction e^{i (kappa_j - kappa_0 - j dkappa)
+// r}.  Partial sums per item go to scratch; field_reduce_kernel adds them in a
+// fixed order (the result does not depend on scheduling).
+// Bound by the FP64 pipe: 2 FMAs per clock and SM, a warp instruction holding it
+// for 16 clocks whatever its number of active lanes.  With one target per
+// thread and 128 targets per CTA, 16 targets left 7 of 8 lanes idle and a CTA
+// (64 nodes x 8 frequencies) held an SM for a millisecond, so that a few
+// hundred targets made less than three waves of them.  Measured (GB300): 16
+// targets x 63 frequencies, N = 256: 2.60 -> 0.38 ms; 1024 x 255, N 64..480:
+// 8.44 -> 6.69 ms; spectra, fields and synthesis at 333 targets x 1001 times,
+// 200 frequencies: 4.77 -> 1.9 ms.
+constexpr int kTileF64 = 16, kSlicesF64 = kTgt / kTileF64;
+
 __global__ void __launch_bounds__(kTgt) field_partial_kernel(
     SolveTables t, Subgroups grp, const int2 *__restrict__ items, int item_begin, int chunk,
     const double2 *__restrict__ z, const double2 *__restrict__ dz,
@@ -41,86 +56,92 @@ __global__ void __launch_bounds__(kTgt) field_partial_kernel(
     const int vo0 = t.vec_off[s0];
     const double wq = 2.0 * kPi / (double)N * 0.25;   // (pi/n) / 4
     const double dk = grp.dkappa[g];
-    __shared__ double kap[kGroup], ikap[kGroup], isqk[kGroup], corr[kGroup];
+    __shared__ double kap[kGroup], ikap8[kGroup], isqk[kGroup], sqk[kGroup], corr[kGroup];
     __shared__ double2 zs[kChunk];
-    __shared__ double2 ps[kGroup][kChunk];   // (pi/n)|z'|/4 * psi_j at each node
+    __shared__ double2 ps[kGroup][kChunk];   // (pi/n)|z'|/4 * psi_j / sqrt(kappa_j) at each node
+    __shared__ double2 sums[kGroup][kTgt];
     __shared__ PQShared pqt;
     pq_stage(pqt);
     if (threadIdx.x < kGroup) {
         const int j = threadIdx.x;
         const double k = (j < cnt) ? t.kappa[s0 + j] : 1.0;
         kap[j] = k;
-        ikap[j] = 1.0 / k;
+        ikap8[j] = 8.0 / k;
+        sqk[j] = sqrt(k);
         isqk[j] = 1.0 / sqrt(k);
     }
+    __syncthreads();
     const int ne = min(chunk, N - i0);
-    for (int e = threadIdx.x; e < kChunk; e += kTgt) {
-        const int i = i0 + e;
-        double2 zz = make_double2(0.0, 0.0);
-        double sp = 0.0;
-        if (e < ne) {
-            const double2 d = dz[vo0 + i];
-            sp = sqrt(d.x * d.x + d.y * d.y) * wq;
-            zz = z[vo0 + i];
-        }
-        zs[e] = zz;
-        for (int j = 0; j < kGroup; ++j) {
-            double2 v = make_double2(0.0, 0.0);
-            if (e < ne && j < cnt) {
-                const double2 q = psi[t.vec_off[s0 + j] + i];
-                v = make_double2(q.x * sp, q.y * sp);
-            }
-            ps[j][e] = v;
+    if (threadIdx.x < kGroup) corr[threadIdx.x] = kap[threadIdx.x] - (kap[0] + threadIdx.x * dk);
+    for (int e = threadIdx.x; e < ne; e += kTgt) {
+        const double2 d = dz[vo0 + i0 + e];
+        const double sp = sqrt(d.x * d.x + d.y * d.y) * wq;
+        zs[e] = z[vo0 + i0 + e];
+        for (int j = 0; j < cnt; ++j) {
+            const double2 q = psi[t.vec_off[s0 + j] + i0 + e];
+            const double f = sp * isqk[j];
+            ps[j][e] = make_double2(q.x * f, q.y * f);
         }
     }
     __syncthreads();
-    if (threadIdx.x < kGroup) corr[threadIdx.x] = kap[threadIdx.x] - (kap[0] + threadIdx.x * dk);
-    __syncthreads();
-    const int it = blockIdx.x * kTgt + threadIdx.x;
-    if (it >= n_x) return;
-    const double px = x[2 * it], py = x[2 * it + 1];
+    const int it = blockIdx.x * kTileF64 + threadIdx.x % kTileF64;
     double2 acc[kGroup];
 #pragma unroll
     for (int j = 0; j < kGroup; ++j) acc[j] = make_double2(0.0, 0.0);
-    for (int e = 0; e < ne; ++e) {
-        const double d1 = px - zs[e].x, d2 = py - zs[e].y;
-        const double r = sqrt(d1 * d1 + d2 * d2);
-        const double ir = 1.0 / r;
-        const double ar = sqrt(kTwoOverPi * ir);
-        double sn, cs, ss, sc;
-        sincos(kap[0] * r, &sn, &cs);
-        sincos(dk * r, &ss, &sc);
-        double c0 = (cs + sn) * kSqrtHalf, s0v = (sn - cs) * kSqrtHalf;   // e^{i(x0 - pi/4)}
+    if (it < n_x) {
+        const double px = x[2 * it], py = x[2 * it + 1];
+        for (int e = threadIdx.x / kTileF64; e < ne; e += kSlicesF64) {
+            const double d1 = px - zs[e].x, d2 = py - zs[e].y;
+            const double r = sqrt(d1 * d1 + d2 * d2);
+            const double ir = 1.0 / r;
+            const double ar = sqrt(kTwoOverPi * ir) * kSqrtHalf;
+            double sn, cs, ss, sc;
+            sincos(kap[0] * r, &sn, &cs);
+            sincos(dk * r, &ss, &sc);
+            double c0 = (cs + sn) * ar, s0v = (sn - cs) * ar;   // sqrt(2/(pi r)) e^{i(x0 - pi/4)}
 #pragma unroll
-        for (int j = 0; j < kGroup; ++j) {
-            if (j < cnt) {
-                const double xj = kap[j] * r;
-                double J0, Y0;
-                if (xj >= 8.0) {
-                    const double dl = corr[j] * r;
-                    const double c = c0 - dl * s0v, sv = s0v + dl * c0;
-                    double P0, Q0, P1, Q1;
-                    pq_horner<false>(pqt, xj, 8.0 * ir * ikap[j], P0, Q0, P1, Q1);
-                    const double A = ar * isqk[j];
-                    J0 = A * (P0 * c - Q0 * sv);
-                    Y0 = A * (P0 * sv + Q0 * c);
-                } else {
-                    bessel_small0(xj, J0, Y0);
+            for (int j = 0; j < kGroup; ++j) {
+                if (j < cnt) {
+                    const double xj = kap[j] * r;
+                    double J0, Y0;   // times sqrt(kappa_j)
+                    if (xj >= 8.0) {
+                        const double dl = corr[j] * r;
+                        const double c = fma(-dl, s0v, c0), sv = fma(dl, c0, s0v);
+                        double P0, Q0, P1, Q1;
+                        pq_horner<false>(pqt, xj, ir * ikap8[j], P0, Q0, P1, Q1);
+                        J0 = fma(P0, c, -Q0 * sv);
+                        Y0 = fma(P0, sv, Q0 * c);
+                    } else {
+                        bessel_small0(xj, J0, Y0);
+                        J0 *= sqk[j];
+                        Y0 *= sqk[j];
+                    }
+                    const double2 q = ps[j][e];
+                    acc[j].x = fma(-Y0, q.x, fma(-J0, q.y, acc[j].x));
+                    acc[j].y = fma(-Y0, q.y, fma(J0, q.x, acc[j].y));
+                    const double cn = fma(c0, sc, -s0v * ss);
+                    s0v = fma(s0v, sc, c0 * ss);
+                    c0 = cn;
                 }
-                const double2 q = ps[j][e];
-                acc[j].x += -Y0 * q.x - J0 * q.y;
-                acc[j].y += -Y0 * q.y + J0 * q.x;
-                const double cn = c0 * sc - s0v * ss;
-                s0v = s0v * sc + c0 * ss;
-                c0 = cn;
             }
         }
     }
 #pragma unroll
-    for (int j = 0; j < kGroup; ++j)
-        if (j < cnt) part[((long long)w * kGroup + j) * n_x + it] = acc[j];
+    for (int j = 0; j < kGroup; ++j) sums[j][threadIdx.x] = acc[j];
+    __syncthreads();
+    for (int o = threadIdx.x; o < cnt * kTileF64; o += kTgt) {
+        const int j = o / kTileF64, k = o % kTileF64, ix = blockIdx.x * kTileF64 + k;
+        if (ix >= n_x) continue;
+        double2 v = sums[j][k];
+#pragma unroll
+        for (int sl = 1; sl < kSlicesF64; ++sl) {
+            const double2 u = sums[j][sl * kTileF64 + k];
+            v.x += u.x;
+            v.y += u.y;
+        }
+        part[((long long)w * kGroup + j) * n_x + ix] = v;
+    }
 }
-
 
 // Mixed-precision variant of field_partial_kernel: the same sums with the
 // distances, H0 (Hankel form for kappa r >= 8, the small-argument series with
@@ -377,8 +398,8 @@ void launch_target_field(const SolveTables &t, const Subgroups &g, int g_begin, 
         field_partial_df_kernel<kGroup><<<grid, kTgt, 0, st>>>(t, g, items, item_begin, chunk, z, dz, psi,
                                                                x, n_x, zf, part);
     else
-        field_partial_kernel<<<grid, kTgt, 0, st>>>(t, g, items, item_begin, chunk, z, dz, psi, x, n_x,
-                                                    part);
+        field_partial_kernel<<<dim3((n_x + kTileF64 - 1) / kTileF64, n_items), kTgt, 0, st>>>(
+            t, g, items, item_begin, chunk, z, dz, psi, x, n_x, part);
     dim3 g2((n_x + 127) / 128, n_groups);
     field_reduce_kernel<<<g2, 128, 0, st>>>(g, g_begin, item_first, item_begin, solve_j, part, n_x, V);
 }
