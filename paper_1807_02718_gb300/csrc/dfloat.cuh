@@ -302,6 +302,135 @@ __device__ __forceinline__ void df_hankel(const GShared &tb, float xf, dfv r8, d
     }
 }
 
+// ---- two double-float values at once ----
+// The packed binary32 instructions (two FMAs, products or sums on a register
+// pair) leave the FMA pipe's rate as it is (measured: 75 against 74 TFLOP/s)
+// but take one issue slot for two operations, and issue is what bounds the
+// kernels below.  Each function is the scalar one applied to both halves.
+struct df2 {
+    float2 h, l;
+};
+
+__device__ __forceinline__ float2 p2(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ float2 p2_neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 p2_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 p2_sub(float2 a, float2 b) { return __fadd2_rn(a, p2_neg(b)); }
+__device__ __forceinline__ float2 p2_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 p2_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+__device__ __forceinline__ df2 df2_make(dfv a, dfv b) { return {p2(a.hi, b.hi), p2(a.lo, b.lo)}; }
+__device__ __forceinline__ dfv df2_x(df2 a) { return {a.h.x, a.l.x}; }
+__device__ __forceinline__ dfv df2_y(df2 a) { return {a.h.y, a.l.y}; }
+__device__ __forceinline__ df2 df2_swap(df2 a) { return {p2(a.h.y, a.h.x), p2(a.l.y, a.l.x)}; }
+
+__device__ __forceinline__ df2 df2_quick(float2 s, float2 e) {   // |s| >= |e|
+    const float2 h = p2_add(s, e);
+    return {h, p2_sub(e, p2_sub(h, s))};
+}
+
+__device__ __forceinline__ float2 p2_two_sum_err(float2 a, float2 b, float2 s) {   // s = a + b
+    const float2 bb = p2_sub(s, a);
+    return p2_add(p2_sub(a, p2_sub(s, bb)), p2_sub(b, bb));
+}
+
+__device__ __forceinline__ df2 df2_add(df2 a, df2 b) {
+    const float2 s = p2_add(a.h, b.h);
+    return df2_quick(s, p2_add(p2_two_sum_err(a.h, b.h, s), p2_add(a.l, b.l)));
+}
+
+__device__ __forceinline__ df2 df2_add_f(df2 a, float2 b) {
+    const float2 s = p2_add(a.h, b);
+    return df2_quick(s, p2_add(p2_two_sum_err(a.h, b, s), a.l));
+}
+
+// a b as the rounded product and its error with the cross terms
+__device__ __forceinline__ float2 p2_prod(df2 a, df2 b, float2 &e) {
+    const float2 p = p2_mul(a.h, b.h);
+    e = p2_fma(a.h, b.h, p2_neg(p));
+    e = p2_fma(a.h, b.l, e);
+    e = p2_fma(a.l, b.h, e);
+    return p;
+}
+
+__device__ __forceinline__ df2 df2_mul(df2 a, df2 b) {
+    float2 e;
+    const float2 p = p2_prod(a, b, e);
+    return df2_quick(p, e);
+}
+
+__device__ __forceinline__ df2 df2_dot2(df2 a, df2 b, df2 c, df2 d) {   // a b + c d
+    float2 e, f;
+    const float2 p = p2_prod(a, b, e), q = p2_prod(c, d, f), s = p2_add(p, q);
+    return df2_quick(s, p2_add(p2_two_sum_err(p, q, s), p2_add(e, f)));
+}
+
+__device__ __forceinline__ void df2_acc(float2 &sh, float2 &sl, df2 a, df2 b) {   // as df_acc
+    float2 e;
+    const float2 p = p2_prod(a, b, e), t = p2_add(sh, p);
+    sl = p2_add(sl, p2_add(p2_two_sum_err(sh, p, t), e));
+    sh = t;
+}
+
+// Remainder polynomials of the Hankel form for two functions at a time (which
+// two: PQ0 = P0 with Q0; PP = P0 with P1 and QQ = Q0 with Q1), coefficients
+// interleaved: (c1 c1' c2 c2'), (c3 c3' c4 c4'), (c5 c5' c0.hi c0'.hi), (c0.lo
+// c0'.lo centre 1/half-width), so that a pair is four 16-byte loads.
+template <int kPairs> struct GPair {
+    float4 v[kPQ_NI][kPairs][4];
+};
+
+template <int kPairs>
+__device__ __forceinline__ void g_stage_pairs(GPair<kPairs> &tb, const int (&fa)[kPairs], const int (&fb)[kPairs]) {
+    for (int e = threadIdx.x; e < kPQ_NI * kPairs; e += blockDim.x) {
+        const int k = e / kPairs, q = e % kPairs;
+        const float *a = kG + (k * 4 + fa[q]) * kG_TERMS, *b = kG + (k * 4 + fb[q]) * kG_TERMS;
+        const float *a0 = kG0DF + 2 * (k * 4 + fa[q]), *b0 = kG0DF + 2 * (k * 4 + fb[q]);
+        tb.v[k][q][0] = make_float4(a[1], b[1], a[2], b[2]);
+        tb.v[k][q][1] = make_float4(a[3], b[3], a[4], b[4]);
+        tb.v[k][q][2] = make_float4(a[5], b[5], a0[0], b0[0]);
+        tb.v[k][q][3] = make_float4(a0[1], b0[1], kPQ_UCf[k], kPQ_IUHf[k]);
+    }
+}
+
+__device__ __forceinline__ int g_interval(float xf) {
+    return (xf >= 10.f) + (xf >= 13.f) + (xf >= 18.f) + (xf >= 28.f) + (xf >= 60.f);
+}
+
+// u k + u^2 G for both functions (as pq_rem; the constant term and the Hankel
+// term dominate what is added to them, so that a sum's error takes three
+// operations; u2 = u^2 need not be renormalised).
+__device__ __forceinline__ df2 pq_rem_pair(const float4 *g, float uhi, dfv u, float2 k, dfv u2) {
+    const float4 g0 = g[0], g1 = g[1], g2 = g[2], g3 = g[3];
+    const float tv = (uhi - g3.z) * g3.w;
+    const float2 t = p2(tv, tv), uh = p2(u.hi, u.hi), ul = p2(u.lo, u.lo);
+    float2 a = p2_fma(p2(g2.x, g2.y), t, p2(g1.z, g1.w));
+    a = p2_fma(a, t, p2(g1.x, g1.y));
+    a = p2_fma(a, t, p2(g0.z, g0.w));
+    a = p2_mul(p2_fma(a, t, p2(g0.x, g0.y)), t);
+    const float2 c0 = p2(g2.z, g2.w), gh = p2_add(c0, a);
+    const float2 gl = p2_add(p2_sub(a, p2_sub(gh, c0)), p2(g3.x, g3.y));
+    const float2 p = p2_mul(uh, k);
+    const float2 pe = p2_fma(ul, k, p2_fma(uh, k, p2_neg(p)));
+    float2 qe;
+    const float2 q = p2_prod({p2(u2.hi, u2.hi), p2(u2.lo, u2.lo)}, {gh, gl}, qe);
+    const float2 s = p2_add(p, q);
+    return df2_quick(s, p2_add(p2_sub(q, p2_sub(s, p)), p2_add(pe, qe)));
+}
+
+// Hankel-form (J0, Y0) at x = kappa r >= 8 (as df_hankel): r8 = 8 / x, cs = a
+// (cos, sin)(x - pi/4), sc its halves exchanged.
+__device__ __forceinline__ df2 df2_hankel0(const GPair<1> &tb, float xf, dfv r8, df2 cs, df2 sc) {
+    const dfv u = df_mul(r8, r8);
+    const float p = u.hi * u.hi;
+    const dfv u2 = {p, fmaf(u.hi, u.lo + u.lo, fmaf(u.hi, u.hi, -p))};
+    const df2 rem = pq_rem_pair(tb.v[g_interval(xf)][0], u.hi, u, p2(-9.0f / 8192.0f, 75.0f / 524288.0f), u2);
+    const float sq = rem.h.y - 1.0f / 64.0f;   // Q0 = r8 (rem - 1/64)
+    const dfv Q0 = df_mul(r8, {sq, rem.l.y + (rem.h.y - (sq + 1.0f / 64.0f))});
+    const df2 dP = {p2(rem.h.x, rem.h.x), p2(rem.l.x, rem.l.x)};
+    // J0 = c + dP0 c - Q0 s, Y0 = s + dP0 s + Q0 c
+    return df2_add(cs, df2_dot2(dP, cs, {p2(-Q0.hi, Q0.hi), p2(-Q0.lo, Q0.lo)}, sc));
+}
+
 // ---- small arguments (x < 8) ----
 // With t = x^2/32 - 1 (the A&S 9.1.10-9.1.11 ascending series with the
 // logarithmic parts taken out, as in the FP64 routine):
