@@ -1,14 +1,16 @@
 // J0, Y0, J1, Y1 in FP64 for x > 0, evaluated together (one sincos, one log).
 //
-//   x < 8:  J0 = A0(t), Y0 = (2/pi) ln(x/2) J0 + A1(t), J1 = x A2(t),
-//           Y1 = (2/pi) ln(x/2) J1 - 2/(pi x) + x A3(t),   t = x^2/32 - 1
+//   x < 8:  J0 = A0, Y0 = (2/pi) ln(x/2) J0 + A1, J1 = x A2,
+//           Y1 = (2/pi) ln(x/2) J1 - 2/(pi x) + x A3
 //           (A0..A3 are entire in x^2: the ascending series of A&S 9.1.10-9.1.11
-//            with the logarithmic parts taken out);
+//            with the logarithmic parts taken out; ten Horner terms on each of 16
+//            intervals of x^2, a third of the FP64 instructions of one Clenshaw
+//            sum of 17 Chebyshev terms over [0, 8));
 //   x >= 8: H_nu(x) = sqrt(2/(pi x)) (P_nu + i Q_nu) e^{i (x - (2 nu + 1) pi/4)},
 //           P0 = B0, Q0 = (8/x) B1, P1 = B2, Q1 = (8/x) B3 as functions of
 //           u = (x0/x)^2 on [8, 20] and [20, inf)  (Hankel's form, A&S 9.2.5-9.2.6).
-// Each A_k / B_k is a Chebyshev series (bessel_cheb.h, made by
-// gen_bessel_cheb.py) summed by Clenshaw's recurrence.  Absolute error is
+// Each B_k is a Chebyshev series (bessel_cheb.h, made by gen_bessel_cheb.py)
+// summed by Clenshaw's recurrence.  Absolute error is
 // ~2e-16 for O(1) values (see the GPU test against reference tables).
 #pragma once
 
@@ -106,9 +108,10 @@ __device__ __forceinline__ double horner8(const double *c, double t) {
 }
 
 template <bool want1>
-__device__ __forceinline__ void pq_horner(const PQShared &tb, double x, double r8, double &P0,
+__device__ __forceinline__ void pq_horner(const PQShared &tb, float xf, double r8, double &P0,
                                           double &Q0, double &P1, double &Q1) {
-    const int k = (x >= 10.0) + (x >= 13.0) + (x >= 18.0) + (x >= 28.0) + (x >= 60.0);
+    // (the interval from binary32 comparisons: FP64 ones would take five issues of the FP64 pipe)
+    const int k = (xf >= 10.f) + (xf >= 13.f) + (xf >= 18.f) + (xf >= 28.f) + (xf >= 60.f);
     const double t = (r8 * r8 - tb.uc[k]) * tb.iuh[k];
     const double *c = tb.c + k * 4 * kPQ_TERMS;
     P0 = horner8(c, t);
@@ -119,39 +122,47 @@ __device__ __forceinline__ void pq_horner(const PQShared &tb, double x, double r
     }
 }
 
-// Small-argument branch (x < 8) with ln(x/2) given (shared by a frequency group).
-__device__ __forceinline__ void bessel_small_ln(double x, double lnh, double &J0, double &Y0, double &J1,
-                                                double &Y1) {
-    const double t = x * x * (1.0 / 32.0) - 1.0;
-    J0 = clenshaw<kA0_N>(kA0, t);
-    const double a1 = clenshaw<kA1_N>(kA1, t);
-    const double a2 = clenshaw<kA2_N>(kA2, t);
-    const double a3 = clenshaw<kA3_N>(kA3, t);
-    const double L = kTwoOverPi * lnh;
-    Y0 = fma(L, J0, a1);
-    J1 = x * a2;
-    Y1 = fma(L, J1, fma(x, a3, -kTwoOverPi / x));
+// A0..A3 at x < 8 (the first kF of them; order A0, A1, A2, A3), tab = kAS or a
+// copy of it in shared memory.
+template <int kF>
+__device__ __forceinline__ void small_series(const double *tab, double x, double (&a)[kF]) {
+    const double v = x * x;
+    const int k = min((int)((float)v * 0.25f), kAS_NI - 1);
+    const double t = fma(v, 0.5, -(double)(2 * k + 1));
+    const double *c = tab + k * 4 * kAS_TERMS;
+#pragma unroll
+    for (int f = 0; f < kF; ++f) {
+        double s = c[f * kAS_TERMS + kAS_TERMS - 1];
+#pragma unroll
+        for (int p = kAS_TERMS - 2; p >= 0; --p) s = fma(s, t, c[f * kAS_TERMS + p]);
+        a[f] = s;
+    }
 }
 
-__device__ __forceinline__ void bessel_small0(double x, double &J0, double &Y0) {
-    const double t = x * x * (1.0 / 32.0) - 1.0;
-    J0 = clenshaw<kA0_N>(kA0, t);
-    const double a1 = clenshaw<kA1_N>(kA1, t);
-    Y0 = fma(kTwoOverPi * log(0.5 * x), J0, a1);
+// Small-argument branch (x < 8) with lnh = ln(x/2) and r8 = 8/x given (both
+// shared by a frequency group).
+__device__ __forceinline__ void bessel_small_ln(const double *tab, double x, double r8, double lnh, double &J0,
+                                                double &Y0, double &J1, double &Y1) {
+    double a[4];
+    small_series(tab, x, a);
+    const double L = kTwoOverPi * lnh;
+    J0 = a[0];
+    Y0 = fma(L, J0, a[1]);
+    J1 = x * a[2];
+    Y1 = fma(L, J1, fma(x, a[3], -0.125 * kTwoOverPi * r8));
+}
+
+__device__ __forceinline__ void bessel_small0_ln(const double *tab, double x, double lnh, double &J0, double &Y0) {
+    double a[2];
+    small_series(tab, x, a);
+    J0 = a[0];
+    Y0 = fma(kTwoOverPi * lnh, J0, a[1]);
 }
 
 __device__ __forceinline__ void bessel_j0y0j1y1(double x, double &J0, double &Y0, double &J1,
                                                 double &Y1) {
     if (x < 8.0) {
-        const double t = x * x * (1.0 / 32.0) - 1.0;
-        J0 = clenshaw<kA0_N>(kA0, t);
-        const double a1 = clenshaw<kA1_N>(kA1, t);
-        const double a2 = clenshaw<kA2_N>(kA2, t);
-        const double a3 = clenshaw<kA3_N>(kA3, t);
-        const double L = kTwoOverPi * log(0.5 * x);
-        Y0 = fma(L, J0, a1);
-        J1 = x * a2;
-        Y1 = fma(L, J1, fma(x, a3, -kTwoOverPi / x));
+        bessel_small_ln(kAS, x, 8.0 / x, log(0.5 * x), J0, Y0, J1, Y1);
     } else {
         double s, c;
         sincos(x, &s, &c);
@@ -169,10 +180,7 @@ __device__ __forceinline__ void bessel_j0y0j1y1(double x, double &J0, double &Y0
 
 __device__ __forceinline__ void bessel_j0y0(double x, double &J0, double &Y0) {
     if (x < 8.0) {
-        const double t = x * x * (1.0 / 32.0) - 1.0;
-        J0 = clenshaw<kA0_N>(kA0, t);
-        const double a1 = clenshaw<kA1_N>(kA1, t);
-        Y0 = fma(kTwoOverPi * log(0.5 * x), J0, a1);
+        bessel_small0_ln(kAS, x, log(0.5 * x), J0, Y0);
     } else {
         double s, c;
         sincos(x, &s, &c);

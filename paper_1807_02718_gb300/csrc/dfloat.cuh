@@ -220,88 +220,6 @@ __device__ __forceinline__ void df_expi_kr(float k1, float k2, float k3, dfv r, 
     else { c = sn; s = df_neg(cs); }
 }
 
-// Remainder polynomials staged in shared memory (threads of a warp may fall
-// into different x intervals).
-struct __align__(16) GShared {
-    float c[kPQ_NI * 4 * kG_TERMS];   // read as float4 pairs (kG_TERMS = 8)
-    float2 c0[kPQ_NI * 4];          // constant terms as (hi, lo)
-    float uc[kPQ_NI], iuh[kPQ_NI];
-};
-static_assert(kG_TERMS == 8, "g_poly reads each remainder polynomial as two float4");
-
-__device__ __forceinline__ void g_stage(GShared &tb) {
-    for (int i = threadIdx.x; i < kPQ_NI * 4 * kG_TERMS; i += blockDim.x) tb.c[i] = kG[i];
-    for (int i = threadIdx.x; i < kPQ_NI * 4; i += blockDim.x) tb.c0[i] = make_float2(kG0DF[2 * i], kG0DF[2 * i + 1]);
-    for (int i = threadIdx.x; i < kPQ_NI; i += blockDim.x) {
-        tb.uc[i] = kPQ_UCf[i];
-        tb.iuh[i] = kPQ_IUHf[i];
-    }
-}
-
-// The binary32 part of a remainder polynomial: G - c0 = t (c1 + c2 t + ...
-// + c5 t^4), its coefficients (c0 unused) as two 16-byte loads of the eight
-// table entries; c6 and c7 are zero on every interval (gen_bessel_cheb.py
-// checks that at most six terms are needed).
-__device__ __forceinline__ float g_poly(const float *c, float t) {
-    const float4 lo = reinterpret_cast<const float4 *>(c)[0], hi = reinterpret_cast<const float4 *>(c)[1];
-    float a = fmaf(hi.y, t, hi.x);
-    a = fmaf(a, t, lo.w);
-    a = fmaf(a, t, lo.z);
-    a = fmaf(a, t, lo.y);
-    return a * t;
-}
-
-// u k + u^2 G with G = c0 + at (c0 a df pair, at binary32, k an exact
-// binary32 coefficient): the Hankel terms of P or Q after the constant one,
-// summed with one renormalisation.
-__device__ __forceinline__ dfv pq_rem(dfv u, float k, dfv u2, float2 c0, float at) {
-    const dfv G = df_add_f(df_make(c0.x, c0.y), at);
-    const float p = u.hi * k;
-    const float e = fmaf(u.lo, k, fmaf(u.hi, k, -p));
-    const float q = u2.hi * G.hi;
-    float f = fmaf(u2.hi, G.hi, -q);
-    f = fmaf(u2.hi, G.lo, f);
-    f = fmaf(u2.lo, G.hi, f);
-    const float sm = p + q;
-    const float bb = sm - p;
-    return df_quick(sm, ((p - (sm - bb)) + (q - bb)) + (e + f));
-}
-
-// Hankel-form J0, Y0 (and J1, Y1 when want1) at x = kappa r >= 8, scaled by
-// the amplitude that the caller carries in the phase:
-//   r8 = 8 / x (df), (c, s) = a e^{i (x - pi/4)} for any real a;
-//   J0 = a' (P0 c - Q0 s), Y0 = a' (P0 s + Q0 c), and with e^{i (x - 3pi/4)}
-//   = (s, -c): J1 = a' (P1 s + Q1 c), Y1 = a' (Q1 s - P1 c), where
-//   a' = sqrt(2 / (pi x)) / a (a = sqrt(2 / (pi x)) gives J and Y themselves).
-// P = 1 + dP: each value is the phase component plus one two-product dot
-// product of the small corrections (|dP| <= 1.2e-3, |Q| <= 0.05).
-template <bool want1>
-__device__ __forceinline__ void df_hankel(const GShared &tb, float xf, dfv r8, dfv c, dfv s, dfv &J0,
-                                          dfv &Y0, dfv &J1, dfv &Y1) {
-    const dfv u = df_mul(r8, r8);
-    const int k = (xf >= 10.f) + (xf >= 13.f) + (xf >= 18.f) + (xf >= 28.f) + (xf >= 60.f);
-    const float t = (u.hi - tb.uc[k]) * tb.iuh[k];
-    const dfv u2 = df_mul(u, u);
-    const float *g = tb.c + k * 4 * kG_TERMS;
-    const float4 g01 = reinterpret_cast<const float4 *>(tb.c0)[2 * k];
-    // dP0 = P0 - 1, Q0 = r8 (-1/64 + 75 u / 524288 + u^2 G1)
-    const dfv dP0 = pq_rem(u, -9.0f / 8192.0f, u2, make_float2(g01.x, g01.y), g_poly(g, t));
-    const dfv Q0 = df_mul(r8, df_add_f(pq_rem(u, 75.0f / 524288.0f, u2, make_float2(g01.z, g01.w),
-                                              g_poly(g + kG_TERMS, t)),
-                                       -1.0f / 64.0f));
-    J0 = df_add(c, df_dot2(dP0, c, df_neg(Q0), s));
-    Y0 = df_add(s, df_dot2(dP0, s, Q0, c));
-    if (want1) {
-        const float4 g23 = reinterpret_cast<const float4 *>(tb.c0)[2 * k + 1];
-        const dfv dP1 = pq_rem(u, 15.0f / 8192.0f, u2, make_float2(g23.x, g23.y), g_poly(g + 2 * kG_TERMS, t));
-        const dfv Q1 = df_mul(r8, df_add_f(pq_rem(u, -105.0f / 524288.0f, u2, make_float2(g23.z, g23.w),
-                                                  g_poly(g + 3 * kG_TERMS, t)),
-                                           3.0f / 64.0f));
-        J1 = df_add(s, df_dot2(dP1, s, Q1, c));
-        Y1 = df_add(df_neg(c), df_dot2(Q1, s, df_neg(dP1), c));
-    }
-}
-
 // ---- two double-float values at once ----
 // The packed binary32 instructions (two FMAs, products or sums on a register
 // pair) leave the FMA pipe's rate as it is (measured: 75 against 74 TFLOP/s)
@@ -321,6 +239,7 @@ __device__ __forceinline__ float2 p2_fma(float2 a, float2 b, float2 c) { return 
 __device__ __forceinline__ df2 df2_make(dfv a, dfv b) { return {p2(a.hi, b.hi), p2(a.lo, b.lo)}; }
 __device__ __forceinline__ dfv df2_x(df2 a) { return {a.h.x, a.l.x}; }
 __device__ __forceinline__ dfv df2_y(df2 a) { return {a.h.y, a.l.y}; }
+__device__ __forceinline__ df2 df2_bcast(dfv a) { return {p2(a.hi, a.hi), p2(a.lo, a.lo)}; }
 __device__ __forceinline__ df2 df2_swap(df2 a) { return {p2(a.h.y, a.h.x), p2(a.l.y, a.l.x)}; }
 
 __device__ __forceinline__ df2 df2_quick(float2 s, float2 e) {   // |s| >= |e|
@@ -364,6 +283,13 @@ __device__ __forceinline__ df2 df2_dot2(df2 a, df2 b, df2 c, df2 d) {   // a b +
     return df2_quick(s, p2_add(p2_two_sum_err(p, q, s), p2_add(e, f)));
 }
 
+__device__ __forceinline__ df2 df2_dot3(df2 a, df2 b, df2 c, df2 d, df2 u, df2 v) {   // a b + c d + u v
+    float2 e, f, g;
+    const float2 p = p2_prod(a, b, e), q = p2_prod(c, d, f), w = p2_prod(u, v, g), s = p2_add(p, q), t = p2_add(s, w);
+    const float2 err = p2_add(p2_two_sum_err(p, q, s), p2_two_sum_err(s, w, t));
+    return df2_quick(t, p2_add(err, p2_add(p2_add(e, f), g)));
+}
+
 __device__ __forceinline__ void df2_acc(float2 &sh, float2 &sl, df2 a, df2 b) {   // as df_acc
     float2 e;
     const float2 p = p2_prod(a, b, e), t = p2_add(sh, p);
@@ -396,9 +322,12 @@ __device__ __forceinline__ int g_interval(float xf) {
     return (xf >= 10.f) + (xf >= 13.f) + (xf >= 18.f) + (xf >= 28.f) + (xf >= 60.f);
 }
 
-// u k + u^2 G for both functions (as pq_rem; the constant term and the Hankel
-// term dominate what is added to them, so that a sum's error takes three
-// operations; u2 = u^2 need not be renormalised).
+// u k + u^2 G with G = c0 + at (c0 a df pair, at binary32, k an exact binary32
+// coefficient) for both functions: the Hankel terms of P or Q after the
+// constant one.  The constant term of G and the Hankel term dominate what is
+// added to them, so that a sum's error takes three operations; u2 = u^2 need
+// not be renormalised.  c6 and c7 are zero on every interval
+// (gen_bessel_cheb.py checks that at most six terms are needed).
 __device__ __forceinline__ df2 pq_rem_pair(const float4 *g, float uhi, dfv u, float2 k, dfv u2) {
     const float4 g0 = g[0], g1 = g[1], g2 = g[2], g3 = g[3];
     const float tv = (uhi - g3.z) * g3.w;
@@ -417,49 +346,106 @@ __device__ __forceinline__ df2 pq_rem_pair(const float4 *g, float uhi, dfv u, fl
     return df2_quick(s, p2_add(p2_sub(q, p2_sub(s, p)), p2_add(pe, qe)));
 }
 
-// Hankel-form (J0, Y0) at x = kappa r >= 8 (as df_hankel): r8 = 8 / x, cs = a
-// (cos, sin)(x - pi/4), sc its halves exchanged.
+// u^2 of u = (8 / x)^2 as a double-float value (not renormalised)
+__device__ __forceinline__ dfv df_square(dfv u) {
+    const float p = u.hi * u.hi;
+    return {p, fmaf(u.hi, u.lo + u.lo, fmaf(u.hi, u.hi, -p))};
+}
+
+// Hankel form at x = kappa r >= 8, scaled by the amplitude that the caller
+// carries in the phase: r8 = 8 / x, cs = a (cos, sin)(x - pi/4) for any real a,
+// sc its halves exchanged; the values are a' times the Bessel functions, a' =
+// a / sqrt(2 / (pi x)) (a = sqrt(2 / (pi x)) gives J and Y themselves).  P = 1 +
+// dP: each value is the phase component plus one two-product dot product of
+// the small corrections (|dP| <= 1.2e-3, |Q| <= 0.05).
+// Order 0: (J0, Y0) = (c, s) + dP0 (c, s) + Q0 (-s, c).
 __device__ __forceinline__ df2 df2_hankel0(const GPair<1> &tb, float xf, dfv r8, df2 cs, df2 sc) {
     const dfv u = df_mul(r8, r8);
-    const float p = u.hi * u.hi;
-    const dfv u2 = {p, fmaf(u.hi, u.lo + u.lo, fmaf(u.hi, u.hi, -p))};
-    const df2 rem = pq_rem_pair(tb.v[g_interval(xf)][0], u.hi, u, p2(-9.0f / 8192.0f, 75.0f / 524288.0f), u2);
+    const df2 rem = pq_rem_pair(tb.v[g_interval(xf)][0], u.hi, u, p2(-9.0f / 8192.0f, 75.0f / 524288.0f), df_square(u));
     const float sq = rem.h.y - 1.0f / 64.0f;   // Q0 = r8 (rem - 1/64)
     const dfv Q0 = df_mul(r8, {sq, rem.l.y + (rem.h.y - (sq + 1.0f / 64.0f))});
     const df2 dP = {p2(rem.h.x, rem.h.x), p2(rem.l.x, rem.l.x)};
-    // J0 = c + dP0 c - Q0 s, Y0 = s + dP0 s + Q0 c
     return df2_add(cs, df2_dot2(dP, cs, {p2(-Q0.hi, Q0.hi), p2(-Q0.lo, Q0.lo)}, sc));
 }
 
-// ---- small arguments (x < 8) ----
-// With t = x^2/32 - 1 (the A&S 9.1.10-9.1.11 ascending series with the
-// logarithmic parts taken out, as in the FP64 routine):
-//   J0 = A0(t),  Y0 = (2/pi) ln(x/2) J0 + A1(t),
-//   J1 = x A2(t), Y1 = (2/pi) ln(x/2) J1 - 2/(pi x) + x A3(t),
-// A_k Chebyshev series in t (bessel_cheb.h).  Clenshaw's recurrence runs in
-// binary32 over the coefficients k >= kChebHead (all below 2^-24 of the
-// largest, |c_k| <= 2e-10) and in double-float over the rest.
-constexpr int kChebHead = 12;
+// Orders 0 and 1 together: J = (J0, J1) = (c, s) + dP (c, s) + Q m and N = -(Y0,
+// Y1) = m + dP m - Q (c, s), m = (-s, c) (e^{i (x - 3 pi/4)} = (s, -c)).
+__device__ __forceinline__ void df2_hankel01(const GPair<2> &tb, float xf, dfv r8, df2 cs, df2 sc, df2 &J, df2 &N) {
+    const dfv u = df_mul(r8, r8), u2 = df_square(u);
+    const float4 (*g)[4] = tb.v[g_interval(xf)];
+    const df2 dP = pq_rem_pair(g[0], u.hi, u, p2(-9.0f / 8192.0f, 15.0f / 8192.0f), u2);
+    const df2 rq = pq_rem_pair(g[1], u.hi, u, p2(75.0f / 524288.0f, -105.0f / 524288.0f), u2);
+    const float2 q0 = p2(-1.0f / 64.0f, 3.0f / 64.0f), sq = p2_add(rq.h, q0);   // Q = r8 (q0 + rem)
+    const df2 Q = df2_mul({p2(r8.hi, r8.hi), p2(r8.lo, r8.lo)},
+                          {sq, p2_add(rq.l, p2_sub(rq.h, p2_sub(sq, q0)))});
+    const df2 m = {p2(-sc.h.x, sc.h.y), p2(-sc.l.x, sc.l.y)};
+    J = df2_add(cs, df2_dot2(dP, cs, Q, m));
+    N = df2_add(m, df2_dot2(dP, m, {p2_neg(Q.h), p2_neg(Q.l)}, cs));
+}
 
-template <int N>
-__device__ __forceinline__ dfv df_clenshaw(const float *c, dfv t) {
-    const float t2f = 2.f * t.hi;
-    float f1 = 0.f, f2 = 0.f;
+// ---- small arguments (x < 8) ----
+// The A&S 9.1.10-9.1.11 ascending series with the logarithmic parts taken
+// out, as in the FP64 routine:
+//   J0 = A0,  Y0 = (2/pi) ln(x/2) J0 + A1,
+//   J1 = x A2, Y1 = (2/pi) ln(x/2) J1 - 2/(pi x) + x A3,
+// ten Horner terms in t = (x^2 - (4 k + 2)) / 2 on the interval k of x^2, two
+// functions at a time (tables kASJY0, kASJY01 of bessel_cheb.h): the four highest terms
+// (|c| <= 4e-8) in binary32, six in double-float.  About a quarter of the
+// instructions of one Clenshaw sum of 17 Chebyshev terms per function.
+constexpr int kASPair = 8;   // float4 per interval and pair
+
+// (A_a, A_b) at t from the pair's eight float4
+__device__ __forceinline__ df2 df2_small_series(const float4 *f, dfv t) {
+    const float2 th = p2(t.hi, t.hi);
+    const float4 f0 = f[0], f1 = f[1];
+    float2 a = p2_fma(p2(f0.x, f0.y), th, p2(f0.z, f0.w));
+    a = p2_fma(a, th, p2(f1.x, f1.y));
+    a = p2_fma(a, th, p2(f1.z, f1.w));
+    df2 s = {a, p2(0.f, 0.f)};
+    const df2 tt = {th, p2(t.lo, t.lo)};
 #pragma unroll
-    for (int k = N - 1; k >= kChebHead; --k) {
-        const float f0 = fmaf(t2f, f1, c[2 * k] - f2);
-        f2 = f1;
-        f1 = f0;
+    for (int k = 2; k < kASPair; ++k) {
+        const float4 c = f[k];
+        float2 e;
+        const float2 p = p2_prod(s, tt, e), ch = p2(c.x, c.y), h = p2_add(p, ch);
+        s = df2_quick(h, p2_add(p2_two_sum_err(p, ch, h), p2_add(e, p2(c.z, c.w))));
     }
-    dfv b1 = df_make(f1, 0.f), b2 = df_make(f2, 0.f);
-    const dfv t2 = df_make(2.f * t.hi, 2.f * t.lo);
-#pragma unroll
-    for (int k = kChebHead - 1; k >= 1; --k) {
-        const dfv b0 = df_add(df_mul(t2, b1), df_add(df_make(c[2 * k], c[2 * k + 1]), df_neg(b2)));
-        b2 = b1;
-        b1 = b0;
-    }
-    return df_add(df_mul(t, b1), df_add(df_make(c[0], c[1]), df_neg(b2)));
+    return s;
+}
+
+// Interval of x^2 and t on it.
+__device__ __forceinline__ int small_interval(dfv x, dfv &t) {
+    const dfv v = df_mul(x, x);
+    const int k = min((int)(v.hi * 0.25f), kAS_NI - 1);
+    const dfv d = df_add_f(v, -(float)(4 * k + 2));
+    t = df_make(0.5f * d.hi, 0.5f * d.lo);
+    return k;
+}
+
+// (J0, Y0) at 0 < x < 8 from x and lnh = ln(x/2); tab: kASJY0 or a copy.
+__device__ __forceinline__ df2 df2_bessel_small0(const float4 *tab, dfv x, dfv lnh) {
+    dfv t;
+    const int k = small_interval(x, t);
+    const df2 A = df2_small_series(tab + k * kASPair, t);
+    const dfv L = df_mul(df_make(kLogConstDF[2], kLogConstDF[3]), lnh);   // (2/pi) ln(x/2)
+    return df2_make(df2_x(A), df_mad(L, df2_x(A), df2_y(A)));
+}
+
+// J = (J0, J1) and N = -(Y0, Y1); r8 = 8 / x; tab: kASJY01 or a copy.
+__device__ __forceinline__ void df2_bessel_small01(const float4 *tab, dfv x, dfv r8, dfv lnh, df2 &J, df2 &N) {
+    dfv t;
+    const float4 *f = tab + 2 * kASPair * small_interval(x, t);
+    const df2 A = df2_small_series(f, t), B = df2_small_series(f + kASPair, t);   // (A0, A2), (A1, A3)
+    const dfv two_pi = df_make(kLogConstDF[2], kLogConstDF[3]);
+    const dfv L = df_mul(two_pi, lnh);
+    J = df2_make(df2_x(A), df_mul(x, df2_y(A)));
+    // x A3 - 2/(pi x)
+    const dfv tpx = df_mul(df_make(-0.125f * two_pi.hi, -0.125f * two_pi.lo), r8);
+    const df2 b = df2_make(df2_x(B), df_mad(x, df2_y(B), tpx));
+    float2 e;
+    const float2 p = p2_prod(df2_bcast(L), J, e), h = p2_add(p, b.h);
+    const df2 Y = df2_quick(h, p2_add(p2_two_sum_err(p, b.h, h), p2_add(e, b.l)));
+    N = {p2_neg(Y.h), p2_neg(Y.l)};
 }
 
 // ln a for a double-float a > 0 (normal): a = m 2^e with m in [1/sqrt2, sqrt2),
@@ -485,28 +471,8 @@ __device__ __forceinline__ dfv df_log(dfv a) {
     return df_add(df_mul_f(ln2, (float)e), df_mul(df_make(2.f * s.hi, 2.f * s.lo), p));
 }
 
-// J0, Y0 (and J1, Y1 when want1) at 0 < x < 8 from x and lnh = ln(x/2).
-template <bool want1>
-__device__ __forceinline__ void df_bessel_small(dfv x, dfv lnh, dfv &J0, dfv &Y0, dfv &J1, dfv &Y1) {
-    const dfv x2 = df_mul(x, x);
-    const dfv t = df_add_f(df_make(x2.hi * 0.03125f, x2.lo * 0.03125f), -1.f);
-    const dfv L = df_mul(df_make(kLogConstDF[2], kLogConstDF[3]), lnh);   // (2/pi) ln(x/2)
-    J0 = df_clenshaw<kA0_N>(kA0DF, t);
-    Y0 = df_add(df_mul(L, J0), df_clenshaw<kA1_N>(kA1DF, t));
-    if (want1) {
-        J1 = df_mul(x, df_clenshaw<kA2_N>(kA2DF, t));
-        const dfv tpx = df_mul(df_make(kLogConstDF[2], kLogConstDF[3]), df_rcp(x));   // 2/(pi x)
-        Y1 = df_add(df_add(df_mul(L, J1), df_neg(tpx)), df_mul(x, df_clenshaw<kA3_N>(kA3DF, t)));
-    }
-}
-
-// Out-of-line entry points for the rarely taken branches of the large kernels
-// (their code stays out of the instruction stream of the common path).
+// Out of line: a rarely taken branch of the large kernels (its code stays out
+// of the instruction stream of the common path).
 static __device__ __noinline__ void df_expi_cold(double x, dfv &c, dfv &s) { df_expi(x, c, s); }
-
-static __device__ __noinline__ void df_bessel_small0_cold(dfv x, dfv lnh, dfv &J0, dfv &Y0) {
-    dfv J1, Y1;
-    df_bessel_small<false>(x, lnh, J0, Y0, J1, Y1);
-}
 
 }  // namespace fh

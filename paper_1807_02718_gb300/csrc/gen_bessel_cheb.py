@@ -2,7 +2,8 @@
 
 The device routine (bessel.cuh) evaluates the four functions together:
 
-  x < 8 (variable t = x^2/32 - 1 in [-1, 1]; all four series are entire in x^2):
+  x < 8 (all four series are entire in v = x^2; 16 intervals of v of width 4, t in
+      [-1, 1] on each):
       J0(x)            = A0(t)
       Y0(x)            = (2/pi) J0(x) ln(x/2) + A1(t)
       J1(x)            = x A2(t)
@@ -41,27 +42,77 @@ def cheb(f, n=NPTS):
     return c[: last + 1]
 
 
-def x_small(t):
-    return mp.sqrt(32 * (t + 1))
+def a0(x):
+    return mp.besselj(0, x)
 
 
-def a0(t):
-    return mp.besselj(0, x_small(t))
-
-
-def a1(t):
-    x = x_small(t)
+def a1(x):
     return mp.bessely(0, x) - TWO_PI_INV * mp.besselj(0, x) * mp.log(x / 2)
 
 
-def a2(t):
-    x = x_small(t)
+def a2(x):
     return mp.besselj(1, x) / x
 
 
-def a3(t):
-    x = x_small(t)
+def a3(x):
     return (mp.bessely(1, x) - TWO_PI_INV * mp.besselj(1, x) * mp.log(x / 2) + 2 / (mp.pi * x)) / x
+
+
+AS_NI = 16      # intervals of x^2 in [0, 64)
+AS_TERMS = 10   # monomial terms of each (remainder below 1e-17)
+AS_DF = 6       # of these, double-float pairs on the double-float path; the others (<= 4e-8) binary32
+
+
+def small_table():
+    """Horner coefficients [interval][A0..A3][power of t], t = (x^2 - (4 k + 2)) / 2."""
+    rows = []
+    w = mp.mpf(64) / AS_NI
+    for k in range(AS_NI):
+        row = []
+        for f in (a0, a1, a2, a3):
+            def g(t, f=f, k=k):
+                v = w * k + w / 2 * (1 + t)
+                return f(mp.sqrt(v if v > 0 else mp.mpf("1e-30")))
+
+            c = cheb(g, 24)
+            if len(c) > AS_TERMS:
+                raise SystemExit(f"small-argument interval {k} needs {len(c)} terms")
+            c = cheb_to_monomial(c + [mp.mpf(0)] * (AS_TERMS - len(c)))
+            if max(abs(v) for v in c[AS_DF:]) > mp.mpf("4e-8"):
+                raise SystemExit(f"small-argument interval {k}: binary32 terms too large")
+            row.append(c)
+        rows.append(row)
+    return rows
+
+
+def emit_small(rows):
+    """kAS (FP64) and the pair tables of the double-float path: 32 floats per
+    interval and pair (a, b): a9 b9 a8 b8 a7 b7 a6 b6, then a_k.hi b_k.hi a_k.lo b_k.lo, k = 5 .. 0."""
+    flat = [v for row in rows for c in row for v in c]
+    wrap = lambda words, n: ",\n    ".join(", ".join(words[i:i + n]) for i in range(0, len(words), n))  # noqa: E731
+    body = wrap([mp.nstr(v, 20, min_fixed=-1, max_fixed=-1) for v in flat], 5)
+    out = ["// A0..A3 (x < 8): Horner coefficients [interval][function][power of t], t = (x^2 - (4 k + 2)) / 2",
+           f"constexpr int kAS_NI = {AS_NI}, kAS_TERMS = {AS_TERMS};",
+           f"static __device__ const double kAS[{len(flat)}] = {{\n    {body}}};"]
+    for name, pairs, text in (("kASJY0", ((0, 1),), "(A0, A1)"), ("kASJY01", ((0, 2), (1, 3)), "(A0, A2), (A1, A3)")):
+        vals = []
+        for row in rows:
+            for fa, fb in pairs:
+                a, b = row[fa], row[fb]
+                for p in range(AS_TERMS - 1, AS_DF - 1, -1):
+                    vals += [f32(a[p]), f32(b[p])]
+                for p in range(AS_DF - 1, -1, -1):
+                    ah, bh = f32(a[p]), f32(b[p])
+                    vals += [ah, bh, f32(a[p] - ah), f32(b[p] - bh)]
+        body = wrap([repr(float(v)) + "f" for v in vals], 8)
+        out.append(f"// the same for {text} on the double-float path [interval][pair][32]")
+        out.append(f"static __device__ const __align__(16) float {name}[{len(vals)}] = {{\n    {body}}};")
+    return out
+
+
+def f32(v):
+    import struct
+    return mp.mpf(struct.unpack("f", struct.pack("f", float(v)))[0])
 
 
 def pq(nu, x):
@@ -208,8 +259,7 @@ def main():
     out = ["// Generated by gen_bessel_cheb.py (Chebyshev interpolation with mpmath);",
            "// do not edit.  See that script and bessel.cuh for the definitions.",
            "#pragma once", ""]
-    for name, f in (("kA0", a0), ("kA1", a1), ("kA2", a2), ("kA3", a3)):
-        out.append(emit(name, cheb(f)))
+    out += emit_small(small_table())
     (b_lo, u0_lo) = large(mp.mpf(8), mp.mpf(20))
     (b_hi, u0_hi) = large(mp.mpf(20), mp.inf)
     out.append(f"constexpr double kBLoU0 = {mp.nstr(u0_lo, 20)};   // (8/20)^2")
@@ -237,9 +287,6 @@ def main():
     out.append("// (-1)^k / (2k+1)! and (-1)^k / (2k)! as double-float pairs, k = 0..8 (sine and cosine series)")
     out.append(df_consts("kSinDF", [(-1) ** k / mp.factorial(2 * k + 1) for k in range(9)]))
     out.append(df_consts("kCosDF", [(-1) ** k / mp.factorial(2 * k) for k in range(9)]))
-    out.append("// A0..A3 (x < 8) as double-float pairs [hi, lo] for the double-float path")
-    for name, f in (("kA0DF", a0), ("kA1DF", a1), ("kA2DF", a2), ("kA3DF", a3)):
-        out.append(df_consts(name, cheb(f)))
     out.append("// 1 / (2k + 1), k = 0..10 (ln m = 2 s sum_k s^2k / (2k + 1), s = (m - 1)/(m + 1)),")
     out.append("// ln 2, 2 / pi and ln(1/2) as double-float pairs")
     out.append(df_consts("kAtanhDF", [mp.mpf(1) / (2 * k + 1) for k in range(11)]))
@@ -247,8 +294,6 @@ def main():
     # Cody-Waite split of pi/2: C1 with 12 significant bits (k C1 exact in
     # binary32 for k < 2^12), C2 and C3 the next binary32 pieces
     c1 = mp.floor(mp.pi / 2 * 2 ** 11 + mp.mpf(1) / 2) / 2 ** 11
-    import struct
-    f32 = lambda v: mp.mpf(struct.unpack("f", struct.pack("f", float(v)))[0])
     c2 = f32(mp.pi / 2 - c1)
     c3 = f32(mp.pi / 2 - c1 - c2)
     out.append("// pi/2 = C1 + C2 + C3 (Cody-Waite, C1 with 12 significant bits) and pi/4 as a double-float pair")

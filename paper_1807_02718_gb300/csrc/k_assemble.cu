@@ -58,11 +58,12 @@ __device__ __forceinline__ void triangle_tile(long long lt, int &tr, int &tc) {
 // s_i and s_l exchanged).  Once per pair: the geometry factors, the phase
 // e^{i(kappa_0 r - pi/4)} with the amplitude sqrt(2 / (pi r)), the step e^{i
 // dkappa r}, and ln r where the small-argument series will need it.
-// Bound by the FP64 pipe (2 FMAs per clock and SM): about 100 FP64 instructions
+// Bound by the FP64 pipe (2 FMAs per clock and SM): about 75 FP64 instructions
 // per entry, the small-argument series of the near-diagonal warps included,
 // against 168 for one thread per entry with M1, M2, L1, L2 formed separately.
-// Measured (GB300): 255 systems of N 64..480: 5.75 -> 3.56 ms; 63 systems of N =
-// 256: 1.77 -> 1.10 ms.
+// Measured (GB300): 255 systems of N 64..480: 5.75 -> 2.55 ms (3.56 with Clenshaw
+// sums below x = 8 and FP64 interval comparisons); 63 systems of N = 256: 1.77
+// -> 0.65 ms.
 __global__ void __launch_bounds__(256, 2) assemble_group_kernel(
     SolveTables t, Subgroups grp, int n_groups, const double2 *__restrict__ z,
     const double2 *__restrict__ dz, const double2 *__restrict__ ddz,
@@ -76,6 +77,7 @@ __global__ void __launch_bounds__(256, 2) assemble_group_kernel(
     int tr, tc;
     triangle_tile(b - grp.tile_off[g], tr, tc);
     __shared__ double kap[kGroup], eta[kGroup], ikap8[kGroup], sqk[kGroup], eqk[kGroup], lnk2[kGroup], corr[kGroup];
+    __shared__ float kapf[kGroup];
     __shared__ long long moff[kGroup];
     __shared__ PQShared pqt;
     pq_stage(pqt);
@@ -85,6 +87,7 @@ __global__ void __launch_bounds__(256, 2) assemble_group_kernel(
         const double k = (j < cnt) ? t.kappa[s0 + j] : 1.0;
         const double e = (j < cnt) ? t.eta[s0 + j] : 0.0;
         kap[j] = k;
+        kapf[j] = (float)k;
         eta[j] = e;
         ikap8[j] = 8.0 / k;
         sqk[j] = sqrt(k);
@@ -143,22 +146,24 @@ __global__ void __launch_bounds__(256, 2) assemble_group_kernel(
         sincos(dk * r, &ss, &sc);
         const double ah = amp * kSqrtHalf;
         double c0 = (cs + sn) * ah, s0v = (sn - cs) * ah;   // amp e^{i(x0 - pi/4)}
-        const double lnr = kap[0] * r < 8.0 ? log(r) : 0.0;   // shared by the group
+        const float rf = (float)r;
+        const double lnr = kapf[0] * rf < 8.f ? log(r) : 0.0;   // shared by the group
 #pragma unroll 1
         for (int j = 0; j < cnt; ++j) {
-            const double x = kap[j] * r;
+            const float xf = kapf[j] * rf;
+            const double r8 = ir * ikap8[j];
             double J0, Y0, J1, Y1;   // times sqrt(kappa_j)
-            if (x >= 8.0) {
+            if (xf >= 8.f) {
                 const double dl = corr[j] * r;
                 const double c = fma(-dl, s0v, c0), sv = fma(dl, c0, s0v);
                 double P0, Q0, P1, Q1;
-                pq_horner<true>(pqt, x, ir * ikap8[j], P0, Q0, P1, Q1);
+                pq_horner<true>(pqt, xf, r8, P0, Q0, P1, Q1);
                 J0 = fma(P0, c, -Q0 * sv);
                 Y0 = fma(P0, sv, Q0 * c);
                 J1 = fma(P1, sv, Q1 * c);
                 Y1 = fma(Q1, sv, -P1 * c);
             } else {
-                bessel_small_ln(x, lnk2[j] + lnr, J0, Y0, J1, Y1);
+                bessel_small_ln(kAS, kap[j] * r, r8, lnk2[j] + lnr, J0, Y0, J1, Y1);
                 const double f = sqk[j];
                 J0 *= f;
                 Y0 *= f;
@@ -200,6 +205,14 @@ __global__ void __launch_bounds__(256, 2) assemble_group_kernel(
 // so that with J' = sqrt(kappa_j) J (what the Hankel form returns)
 //   Re A = sqrt(kappa) (A1 J1' - B1 Y1') + (eta / sqrt(kappa)) C1 J0',
 //   Im A = sqrt(kappa) B1 J1' + (eta / sqrt(kappa)) (C1 Y0' - D1 J0').
+// Bound by FP32 issue: the frequency loop works on pairs packed in one
+// instruction, (cos, sin) of the phase, (P0, P1) and (Q0, Q1), (J0, J1) and (Y0,
+// Y1), and the two entries (i, l), (l, i).  With 8 points per wavelength about
+// twenty entries of every row take the small-argument series (x < 8), whose
+// warps cost as much as the others only with short series.
+// Measured (GB300, band kernel and right sides included): 255 systems of N
+// 64..480: 0.84 -> 0.51 ms; 511 systems of N 64..1920: 11.7 -> 10.1 ms; 16 x 127
+// systems of N 64..832: 6.4 -> 4.1 ms.
 // r, the Bessel values, the phases and the Kress log weight (even in i - l)
 // are the same for A(i, l) and A(l, i): a CTA takes a tile (tr, tc) of the
 // upper triangle (flat index tc (tc + 1) / 2 + tr within the subgroup) and
@@ -210,7 +223,7 @@ __global__ void __launch_bounds__(256, 2) assemble_group_kernel(
 __global__ void __launch_bounds__(256, 3) assemble_group_df_kernel(
     SolveTables t, Subgroups grp, int n_groups, const double2 *__restrict__ dz,
     const float4 *__restrict__ zf, const float4 *__restrict__ dzf, const float2 *__restrict__ sf,
-    const float2 *__restrict__ wpf, float4 *__restrict__ A, float2 *__restrict__ A32, long long out_shift,
+    const float2 *__restrict__ wpf, float4 *__restrict__ A_out, float2 *__restrict__ A32, long long out_shift,
     long long tile_base) {
     const long long b = tile_base + blockIdx.x;
     const int g = find_solve(grp.tile_off, n_groups, b);
@@ -219,19 +232,23 @@ __global__ void __launch_bounds__(256, 3) assemble_group_df_kernel(
     const int N = t.N[s0];
     int tr, tc;
     triangle_tile(b - grp.tile_off[g], tr, tc);   // 0 <= tr <= tc < ceil(N / 32)
-    __shared__ double kap[kGroup];
-    __shared__ float kapf[kGroup], corrf[kGroup];
-    __shared__ dfv kapd[kGroup], ikap8[kGroup], sqk[kGroup], eqk[kGroup], lnk2[kGroup];
+    __shared__ double kap0;
+    __shared__ float kapf[kGroup], dcorr[kGroup];
+    __shared__ dfv kapd[kGroup], ikap8[kGroup], sqk[kGroup], lnk2[kGroup];
+    __shared__ df2 esq[kGroup];   // (eta / sqrt(kappa), sqrt(kappa))
     __shared__ long long moff[kGroup];
     __shared__ float k3s[3];   // kappa_0 as three binary32 pieces
-    __shared__ GShared gt;
-    g_stage(gt);
+    __shared__ GPair<2> gt;
+    __shared__ float4 as[kAS_NI * 2 * kASPair];
+    g_stage_pairs<2>(gt, {0, 1}, {2, 3});
+    for (int e = threadIdx.x; e < kAS_NI * 2 * kASPair; e += blockDim.x) as[e] = reinterpret_cast<const float4 *>(kASJY01)[e];
     const double dk = grp.dkappa[g];
     const dfv dkd = df_from(dk);
     const float dkf = (float)dk;
     if (threadIdx.x == 0) {
         const double k0 = t.kappa[s0];
         const float a = (float)k0, b = (float)(k0 - (double)a);
+        kap0 = k0;
         k3s[0] = a;
         k3s[1] = b;
         k3s[2] = (float)(k0 - (double)a - (double)b);
@@ -240,14 +257,15 @@ __global__ void __launch_bounds__(256, 3) assemble_group_df_kernel(
         const int j = threadIdx.x;
         const double k = (j < cnt) ? t.kappa[s0 + j] : 1.0;
         const double e = (j < cnt) ? t.eta[s0 + j] : 0.0;
-        kap[j] = k;
+        const double k0 = t.kappa[s0];
         kapf[j] = (float)k;
         kapd[j] = df_from(k);
         ikap8[j] = df_from(8.0 / k);
         sqk[j] = df_from(sqrt(k));
-        eqk[j] = df_from(e / sqrt(k));
+        esq[j] = df2_make(df_from(e / sqrt(k)), sqk[j]);
         lnk2[j] = df_from(log(0.5 * k));   // ln(kappa/2): ln(x/2) = ln(kappa/2) + ln r
-        corrf[j] = (float)(k - ((j < cnt ? t.kappa[s0] : 1.0) + j * dk));
+        // kappa_j - kappa_{j-1} - dkappa: the phase's correction beyond the step
+        dcorr[j] = (j > 0 && j < cnt) ? (float)((k - (k0 + j * dk)) - (t.kappa[s0 + j - 1] - (k0 + (j - 1) * dk))) : 0.f;
         moff[j] = ((j < cnt) ? t.mat_off[s0 + j] : 0) + out_shift;
     }
     __syncthreads();
@@ -290,52 +308,46 @@ __global__ void __launch_bounds__(256, 3) assemble_group_df_kernel(
         const dfv gg4 = df_mul(df_mul(Nil, sl), df_mul(ir, isi4));          // N_il s_l / (4 s_i r)
         const dfv gq4 = df_mul(df_mul(Nli, si4), df_mul(ir, df_rcp(sl)));   // N_li s_i / (4 s_l r)
         const dfv sl4 = df_mul_f(sl, 0.25f);
-        const dfv A1 = df_mul(gg4, Wp), B1 = df_mul(gg4, pind), C1 = df_mul(sl4, pind), D1 = df_mul(sl4, Wp);
-        const dfv A2 = df_mul(gq4, Wq), B2 = df_mul(gq4, pind), D2 = df_mul(si4, Wq);
+        // (entry (i, l), entry (l, i))
+        const df2 A = df2_mul(df2_make(gg4, gq4), df2_make(Wp, Wq)), B = df2_mul(df2_make(gg4, gq4), df2_bcast(pind));
+        const df2 C = df2_make(df_mul(sl4, pind), C2), D = df2_mul(df2_make(sl4, si4), df2_make(Wp, Wq));
         const dfv amp0 = df_sqrt(df_mul(ir, two_over_pi));
         dfv c, sv, sc, ss;
         if (kapf[0] * rd.hi < kExpiKrMax) df_expi_kr(k3s[0], k3s[1], k3s[2], rd, c, sv);
-        else df_expi_cold(kap[0] * df_to(rd) - 0.78539816339744830962, c, sv);   // e^{i (kappa_0 r - pi/4)}
+        else df_expi_cold(kap0 * df_to(rd) - 0.78539816339744830962, c, sv);   // e^{i (kappa_0 r - pi/4)}
         if (dkf * rd.hi < 3.1f) df_sincos_mid(df_mul(dkd, rd), ss, sc);   // e^{i dkappa r}, no FP64 reduction
         else df_expi_cold(dk * df_to(rd), sc, ss);
-        c = df_mul(c, amp0);
-        sv = df_mul(sv, amp0);
+        df2 cs = df2_mul(df2_make(c, sv), df2_bcast(amp0));
+        const df2 stc = df2_bcast(sc), sts = df2_make(df_neg(ss), ss);
         const dfv lnr = kapf[0] * rd.hi < 8.0f ? df_log(rd) : df_make(0.f, 0.f);   // shared by the group
 #pragma unroll 1   // not unrolled: half the registers, twice the occupancy
-        for (int j = 0; j < kGroup; ++j) {
-            if (j < cnt) {
-                const float xf = kapf[j] * rd.hi;
-                dfv J0, Y0, J1, Y1;   // each times sqrt(kappa_j)
-                if (xf >= 8.0f) {
-                    const float dl = corrf[j] * rd.hi;
-                    const dfv cj = df_add_f(c, -dl * sv.hi), sj = df_add_f(sv, dl * c.hi);
-                    df_hankel<true>(gt, xf, df_mul(ir, ikap8[j]), cj, sj, J0, Y0, J1, Y1);
-                } else {
-                    df_bessel_small<true>(df_mul(kapd[j], rd), df_add(lnr, lnk2[j]), J0, Y0, J1, Y1);
-                    const dfv q = sqk[j];
-                    J0 = df_mul(J0, q);
-                    Y0 = df_mul(Y0, q);
-                    J1 = df_mul(J1, q);
-                    Y1 = df_mul(Y1, q);
-                }
-                const dfv sq = sqk[j], eq = eqk[j];
-                const long long mo = moff[j];
-                {
-                    const dfv ar = df_dot2(sq, df_dot2(A1, J1, df_neg(B1), Y1), eq, df_mul(C1, J0));
-                    const dfv ai = df_dot2(sq, df_mul(B1, J1), eq, df_dot2(C1, Y0, df_neg(D1), J0));
-                    A[mo + e_il] = make_float4(ar.hi, ar.lo, ai.hi, ai.lo);
-                    if (A32) A32[mo + e_li] = make_float2(ar.hi, ai.hi);
-                }
-                {
-                    const dfv br = df_dot2(sq, df_dot2(A2, J1, df_neg(B2), Y1), eq, df_mul(C2, J0));
-                    const dfv bi = df_dot2(sq, df_mul(B2, J1), eq, df_dot2(C2, Y0, df_neg(D2), J0));
-                    A[mo + e_li] = make_float4(br.hi, br.lo, bi.hi, bi.lo);
-                    if (A32) A32[mo + e_il] = make_float2(br.hi, bi.hi);
-                }
-                const dfv cn = df_dot2(c, sc, df_neg(sv), ss);
-                sv = df_dot2(sv, sc, c, ss);
-                c = cn;
+        for (int j = 0; j < cnt; ++j) {
+            const float xf = kapf[j] * rd.hi, dl = dcorr[j] * rd.hi;
+            cs = df2_add_f(cs, p2(-dl * cs.h.y, dl * cs.h.x));
+            const df2 sw = df2_swap(cs);
+            const dfv r8 = df_mul(ir, ikap8[j]);
+            df2 J, Y;   // sqrt(kappa_j) (J0, J1) and -sqrt(kappa_j) (Y0, Y1)
+            if (xf >= 8.0f) {
+                df2_hankel01(gt, xf, r8, cs, sw, J, Y);
+            } else {
+                df2_bessel_small01(as, df_mul(kapd[j], rd), r8, df_add(lnr, lnk2[j]), J, Y);
+                const df2 q = df2_bcast(sqk[j]);
+                J = df2_mul(J, q);
+                Y = df2_mul(Y, q);
             }
+            J = df2_mul(J, esq[j]);   // (eta J0, kappa J1), and the same of -Y
+            Y = df2_mul(Y, esq[j]);
+            const df2 J0 = df2_bcast(df2_x(J)), J1 = df2_bcast(df2_y(J)), Y0 = df2_bcast(df2_x(Y)), Y1 = df2_bcast(df2_y(Y));
+            const df2 re = df2_dot3(A, J1, B, Y1, C, J0);
+            const df2 im = df2_dot3(B, J1, C, {p2_neg(Y0.h), p2_neg(Y0.l)}, D, {p2_neg(J0.h), p2_neg(J0.l)});
+            const long long mo = moff[j];
+            A_out[mo + e_il] = make_float4(re.h.x, re.l.x, im.h.x, im.l.x);
+            A_out[mo + e_li] = make_float4(re.h.y, re.l.y, im.h.y, im.l.y);
+            if (A32) {
+                A32[mo + e_li] = make_float2(re.h.x, im.h.x);
+                A32[mo + e_il] = make_float2(re.h.y, im.h.y);
+            }
+            cs = df2_dot2(cs, stc, sw, sts);   // c' = c cos - s sin, s' = s cos + c sin
         }
     }
 }

@@ -37,8 +37,8 @@ constexpr int kChunk = kFieldChunk;   // largest number of source nodes per work
 // thread and 128 targets per CTA, 16 targets left 7 of 8 lanes idle and a CTA
 // (64 nodes x 8 frequencies) held an SM for a millisecond, so that a few
 // hundred targets made less than three waves of them.  Measured (GB300): 16
-// targets x 63 frequencies, N = 256: 2.60 -> 0.38 ms; 1024 x 255, N 64..480:
-// 8.44 -> 6.69 ms; spectra, fields and synthesis at 333 targets x 1001 times,
+// targets x 63 frequencies, N = 256: 2.60 -> 0.20 ms; 1024 x 255, N 64..480:
+// 8.44 -> 5.61 ms; spectra, fields and synthesis at 333 targets x 1001 times,
 // 200 frequencies: 4.77 -> 1.9 ms.
 constexpr int kTileF64 = 16, kSlicesF64 = kTgt / kTileF64;
 
@@ -56,7 +56,8 @@ __global__ void __launch_bounds__(kTgt) field_partial_kernel(
     const int vo0 = t.vec_off[s0];
     const double wq = 2.0 * kPi / (double)N * 0.25;   // (pi/n) / 4
     const double dk = grp.dkappa[g];
-    __shared__ double kap[kGroup], ikap8[kGroup], isqk[kGroup], sqk[kGroup], corr[kGroup];
+    __shared__ double kap[kGroup], ikap8[kGroup], isqk[kGroup], sqk[kGroup], lnk2[kGroup], corr[kGroup];
+    __shared__ float kapf[kGroup];
     __shared__ double2 zs[kChunk];
     __shared__ double2 ps[kGroup][kChunk];   // (pi/n)|z'|/4 * psi_j / sqrt(kappa_j) at each node
     __shared__ double2 sums[kGroup][kTgt];
@@ -66,9 +67,11 @@ __global__ void __launch_bounds__(kTgt) field_partial_kernel(
         const int j = threadIdx.x;
         const double k = (j < cnt) ? t.kappa[s0 + j] : 1.0;
         kap[j] = k;
+        kapf[j] = (float)k;
         ikap8[j] = 8.0 / k;
         sqk[j] = sqrt(k);
         isqk[j] = 1.0 / sqrt(k);
+        lnk2[j] = log(0.5 * k);   // ln(x/2) = ln(kappa/2) + ln r
     }
     __syncthreads();
     const int ne = min(chunk, N - i0);
@@ -99,20 +102,22 @@ __global__ void __launch_bounds__(kTgt) field_partial_kernel(
             sincos(kap[0] * r, &sn, &cs);
             sincos(dk * r, &ss, &sc);
             double c0 = (cs + sn) * ar, s0v = (sn - cs) * ar;   // sqrt(2/(pi r)) e^{i(x0 - pi/4)}
+            const float rf = (float)r;
+            const double lnr = kapf[0] * rf < 8.f ? log(r) : 0.0;   // shared by the group
 #pragma unroll
             for (int j = 0; j < kGroup; ++j) {
                 if (j < cnt) {
-                    const double xj = kap[j] * r;
+                    const float xf = kapf[j] * rf;
                     double J0, Y0;   // times sqrt(kappa_j)
-                    if (xj >= 8.0) {
+                    if (xf >= 8.f) {
                         const double dl = corr[j] * r;
                         const double c = fma(-dl, s0v, c0), sv = fma(dl, c0, s0v);
                         double P0, Q0, P1, Q1;
-                        pq_horner<false>(pqt, xj, ir * ikap8[j], P0, Q0, P1, Q1);
+                        pq_horner<false>(pqt, xf, ir * ikap8[j], P0, Q0, P1, Q1);
                         J0 = fma(P0, c, -Q0 * sv);
                         Y0 = fma(P0, sv, Q0 * c);
                     } else {
-                        bessel_small0(xj, J0, Y0);
+                        bessel_small0_ln(kAS, kap[j] * r, lnk2[j] + lnr, J0, Y0);
                         J0 *= sqk[j];
                         Y0 *= sqk[j];
                     }
@@ -194,7 +199,9 @@ __global__ void __launch_bounds__(kTgt, 6) field_partial_df_kernel(
     // the frequency loop stays rolled (a small instruction footprint)
     __shared__ float2 accs[kG][2][kTgt];
     __shared__ GPair<1> gt;
+    __shared__ float4 as[kAS_NI * kASPair];
     g_stage_pairs<1>(gt, {0}, {1});
+    for (int e = threadIdx.x; e < kAS_NI * kASPair; e += kTgt) as[e] = reinterpret_cast<const float4 *>(kASJY0)[e];
     if (threadIdx.x == 0) {
         const double k0 = t.kappa[s0];
         const float a = (float)k0, b = (float)(k0 - (double)a);
@@ -247,8 +254,8 @@ __global__ void __launch_bounds__(kTgt, 6) field_partial_df_kernel(
             else df_expi_cold(kap0 * df_to(rd) - 0.78539816339744830962, c, sv);   // e^{i (kappa_0 r - pi/4)}
             if (dkf * rd.hi < 3.1f) df_sincos_mid(df_mul(dkd, rd), ss, sc);   // e^{i dkappa r}, no FP64 reduction
             else df_expi_cold(dk * df_to(rd), sc, ss);
-            df2 cs = df2_mul(df2_make(c, sv), df2_make(amp0, amp0));
-            const df2 stc = df2_make(sc, sc), sts = df2_make(df_neg(ss), ss);
+            df2 cs = df2_mul(df2_make(c, sv), df2_bcast(amp0));
+            const df2 stc = df2_bcast(sc), sts = df2_make(df_neg(ss), ss);
             const dfv lnr = kapf[0] * rd.hi < 8.0f ? df_log(rd) : df_make(0.f, 0.f);   // shared by the group
             const bool renorm = ((e / kSlicesDf) & 15) == 15;
 #pragma unroll 1
@@ -261,15 +268,13 @@ __global__ void __launch_bounds__(kTgt, 6) field_partial_df_kernel(
                 if (xf >= 8.0f) {
                     JY = df2_hankel0(gt, xf, df_mul(ir, ikap8[j]), cs, sw);
                 } else {
-                    dfv J0, Y0;
-                    df_bessel_small0_cold(df_mul(kapd[j], rd), df_add(lnr, lnk2[j]), J0, Y0);
-                    JY = df2_mul(df2_make(J0, Y0), df2_make(sqk[j], sqk[j]));
+                    JY = df2_mul(df2_bessel_small0(as, df_mul(kapd[j], rd), df_add(lnr, lnk2[j])), df2_bcast(sqk[j]));
                 }
                 // sums += Y0 (-qr, -qi) + J0 (-qi, qr)
                 const float4 qy = ps[j][e][0], qj = ps[j][e][1];
                 float2 h = accs[j][0][threadIdx.x], l = accs[j][1][threadIdx.x];
-                df2_acc(h, l, {p2(JY.h.y, JY.h.y), p2(JY.l.y, JY.l.y)}, {p2(qy.x, qy.y), p2(qy.z, qy.w)});
-                df2_acc(h, l, {p2(JY.h.x, JY.h.x), p2(JY.l.x, JY.l.x)}, {p2(qj.x, qj.y), p2(qj.z, qj.w)});
+                df2_acc(h, l, df2_bcast(df2_y(JY)), {p2(qy.x, qy.y), p2(qy.z, qy.w)});
+                df2_acc(h, l, df2_bcast(df2_x(JY)), {p2(qj.x, qj.y), p2(qj.z, qj.w)});
                 if (renorm) {   // every 16 nodes of the thread
                     const df2 v = df2_quick(h, l);
                     h = v.h;
@@ -341,36 +346,28 @@ __global__ void bessel_eval_kernel(const double *__restrict__ x, int n, double *
 // kernels (Hankel form for x >= 8, small-argument series with a double-float
 // logarithm below), for testing them.
 __global__ void bessel_eval_df_kernel(const double *__restrict__ x, int n, double *__restrict__ out) {
-    __shared__ GShared gt;
-    g_stage(gt);
+    __shared__ GPair<2> gt;
+    g_stage_pairs<2>(gt, {0, 1}, {2, 3});
     __syncthreads();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double xv = x[i];
-    double J0, Y0, J1, Y1;
+    const dfv r8 = df_from(8.0 / xv);
+    df2 J, N;
     if (xv >= 8.0) {
-        dfv c, s, j0, y0, j1, y1;
+        dfv c, s;
         df_expi(xv - 0.78539816339744830962, c, s);
-        const dfv amp = df_from(sqrt(kTwoOverPi / xv));   // carried by the phase
-        df_hankel<true>(gt, (float)xv, df_from(8.0 / xv), df_mul(c, amp), df_mul(s, amp), j0, y0, j1, y1);
-        J0 = df_to(j0);
-        Y0 = df_to(y0);
-        J1 = df_to(j1);
-        Y1 = df_to(y1);
+        const df2 cs = df2_mul(df2_make(c, s), df2_bcast(df_from(sqrt(kTwoOverPi / xv))));   // amplitude carried by the phase
+        df2_hankel01(gt, (float)xv, r8, cs, df2_swap(cs), J, N);
     } else {
         const dfv xd = df_from(xv);
         const dfv lnh = df_add(df_log(xd), df_make(kLogConstDF[4], kLogConstDF[5]));   // ln(x/2)
-        dfv j0, y0, j1, y1;
-        df_bessel_small<true>(xd, lnh, j0, y0, j1, y1);
-        J0 = df_to(j0);
-        Y0 = df_to(y0);
-        J1 = df_to(j1);
-        Y1 = df_to(y1);
+        df2_bessel_small01(reinterpret_cast<const float4 *>(kASJY01), xd, r8, lnh, J, N);
     }
-    out[4 * i + 0] = J0;
-    out[4 * i + 1] = Y0;
-    out[4 * i + 2] = J1;
-    out[4 * i + 3] = Y1;
+    out[4 * i + 0] = df_to(df2_x(J));
+    out[4 * i + 1] = -df_to(df2_x(N));
+    out[4 * i + 2] = df_to(df2_y(J));
+    out[4 * i + 3] = -df_to(df2_y(N));
 }
 
 }  // namespace
