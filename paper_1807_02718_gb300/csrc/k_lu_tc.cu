@@ -114,6 +114,12 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
+// v -= l u in four FMAs (written as v.x -= l.x u.x - l.y u.y it takes six instructions)
+__device__ __forceinline__ void csub(float2 &v, float2 l, float2 u) {
+    v.x = fmaf(l.y, u.y, fmaf(-l.x, u.x, v.x));
+    v.y = fmaf(-l.y, u.x, fmaf(-l.x, u.y, v.y));
+}
+
 __device__ __forceinline__ float tf32_round(float v) {
     uint32_t u = __float_as_uint(v);
     u = (u + 0x1000u) & 0xFFFFE000u;     // round the 13 dropped mantissa bits to nearest
@@ -169,7 +175,9 @@ struct PanelShared {
     uint32_t kh[2][kWarps], kl[2][kWarps];      // per-warp best keys
     float2 wrow[2][kWarps][NB];                 // cluster of one: warp winners' rows
     Cand cand[2][kMaxCluster];                  // cluster: every CTA's candidate
-    float2 l11[NB + 16][NB + 1];                // unit lower L11 of the current panel; rows NB.. stay zero
+    float2 lcol[2][NB];                         // diagonal block: the current column
+    float2 pinv[NB];                            // its pivots' reciprocals and keys
+    uint32_t kd[NB];
     int mv_dst[kMaxMoved], mv_src[kMaxMoved];
     int mv_cnt;
     uint64_t bar[2];
@@ -260,11 +268,8 @@ __device__ __forceinline__ void trsm_groups(float2 (&x)[NB], int g0, int g1, con
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int e = i + 1; e < kRows; ++e) {   // rows past the panel read zero rows of l11
-                const float2 l = L[e][i];
-                x[e].x -= l.x * x[i].x - l.y * x[i].y;
-                x[e].y -= l.x * x[i].y + l.y * x[i].x;
-            }
+            for (int e = i + 1; e < kRows; ++e)   // rows past the panel read zero rows of l11
+                csub(x[e], L[e][i], x[i]);
 #pragma unroll
         for (int i = 0; i < 4; ++i)
             if (q0 + i < nb) __stcg(col + (long long)(q0 + i) * n, x[i]);
@@ -338,12 +343,13 @@ __global__ void __launch_bounds__(kThreads, 1) lu_factor_tc_kernel(
     uint8_t *sC = sB + kBStages * LT::kBSlot;                           // stages x C tile (1 KiB aligned)
     float4 *gbuf = reinterpret_cast<float4 *>(sB);                      // row gather (B + C)
     constexpr int kGather = (kBStages * LT::kBSlot + kStages * kCTile) / 16;   // float4 in gbuf
-    // second panel of a pair: L21 of the first panel in the rows of the
-    // second's pivots (32 x 32), kept in the A space between the updates
-    float2 (*lpq)[NB + 2] = reinterpret_cast<float2 (*)[NB + 2]>(sA);
-    static_assert(NB * (NB + 2) * 8 <= LT::kASpace, "the pair's L block fits the A space");
-    static_assert(NB * (NB + 2) * 8 <= LT::kASpace && (NB * (NB + 2)) % 2 == 0,
-                  "the pivot-row table of the checked-pivot panel fits the A space as whole float4s");
+    // tables of the current panel in the A space, idle between the updates:
+    // the pivot rows U11; the unit lower L11, rows NB.. zero; for the second
+    // panel of a pair, L21 of the first panel in the rows of the second's pivots
+    float2 (*u11)[NB + 1] = reinterpret_cast<float2 (*)[NB + 1]>(sA);
+    float2 (*l11)[NB + 1] = u11 + NB;
+    float2 (*lpq)[NB + 1] = l11 + NB + 16;
+    static_assert((NB + (NB + 16) + NB) * (NB + 1) * 8 <= LT::kASpace, "the panel's tables fit the A space");
 
     const int cs = kMulti ? cs_arg : 1;
     const int rank = kMulti ? (int)cg::this_cluster().block_rank() : 0;
@@ -378,7 +384,6 @@ __global__ void __launch_bounds__(kThreads, 1) lu_factor_tc_kernel(
         pp.armed_a = pp.commits_a = 0;
         for (int b = 0; b < kStages; ++b) pp.commits[b] = 0;
     }
-    for (int i = tid; i < 16 * (NB + 1); i += kThreads) ps.l11[NB + i / (NB + 1)][i % (NB + 1)] = make_float2(0.f, 0.f);
     if (rank == 0)   // pv: factored position -> original row, while factoring
         for (int i = tid; i < n; i += kThreads) pv[i] = i;
     tc::fence_async_smem();
@@ -398,19 +403,31 @@ __global__ void __launch_bounds__(kThreads, 1) lu_factor_tc_kernel(
         role = role == 1 ? 2 : (LT::kPair && n - k0 > 2 * NB ? 1 : 0);
         const int nb = min(NB, n - k0), m = n - k0;
         if (tid == 0) ps.mv_cnt = 0;
-        const bool own = myslot < m;
         float2 v[NB];
-        {
-            const float4 *src = reinterpret_cast<const float4 *>(a + (long long)(k0 + (own ? myslot : 0)) * n + k0);
+        auto load_row = [&](bool on, int i) {   // the panel's part of row k0 + i
+            const float4 *src = reinterpret_cast<const float4 *>(a + (long long)(k0 + (on ? i : 0)) * n + k0);
 #pragma unroll
             for (int h = 0; h < NB / 2; ++h) {
-                const float4 t = (own && 2 * h < nb) ? __ldcg(src + h) : make_float4(0.f, 0.f, 0.f, 0.f);
+                const float4 t = (on && 2 * h < nb) ? __ldcg(src + h) : make_float4(0.f, 0.f, 0.f, 0.f);
                 v[2 * h] = make_float2(t.x, t.y);
                 v[2 * h + 1] = make_float2(t.z, t.w);
             }
-        }
-        int mypos = myslot;
-        bool active = own;
+        };
+        auto store_row = [&](int i) {
+            float4 *dst = reinterpret_cast<float4 *>(a + (long long)(k0 + i) * n + k0);
+#pragma unroll
+            for (int h = 0; h < NB / 2; ++h)
+                if (2 * h < nb) __stcg(dst + h, make_float4(v[2 * h].x, v[2 * h].y, v[2 * h + 1].x, v[2 * h + 1].y));
+        };
+        auto load_first = [&](int i) {   // row k0 + i of the pair's first panel (L21)
+            const float4 *lp = reinterpret_cast<const float4 *>(a + (long long)(k0 + i) * n + (k0 - NB));
+#pragma unroll
+            for (int h = 0; h < NB / 2; ++h) {
+                const float4 t = __ldcg(lp + h);
+                v[2 * h] = make_float2(t.x, t.y);
+                v[2 * h + 1] = make_float2(t.z, t.w);
+            }
+        };
 
         // 1a. Checked fast path.  Partial pivoting keeps the diagonal row
         // whenever, at every column, no row below it has a larger key (the
@@ -418,83 +435,45 @@ __global__ void __launch_bounds__(kThreads, 1) lu_factor_tc_kernel(
         // the smallest position, so it wins ties).  For the second-kind CFIE
         // systems that holds with a wide margin (the largest key below the
         // diagonal is ~1/4 of it), and then the per-column search and
-        // exchange across the cluster decide nothing.  So: the warp owning
-        // the panel's first rows (CTA 0, threads 0-31) eliminates the 32 x 32
-        // diagonal block, checking the keys among its rows and writing each
-        // pivot row and its reciprocal into u11 (the A staging space, idle
-        // during the panel); u11 goes to every CTA; every other row is
-        // eliminated against u11 with its own key checked; one verdict per
-        // panel.  The arithmetic is that of the search path below.  If any
-        // check fails (or a pivot is zero or not finite) the panel is
-        // reloaded and factored by the search path.
+        // exchange across the cluster decide nothing.  So every CTA of the
+        // cluster eliminates the panel's 32 x 32 diagonal block itself (two
+        // entries per thread, one barrier per column in a short rolled loop;
+        // the same bits in every CTA, so that nothing is exchanged), checking
+        // the keys among its rows and leaving U11 and L11 in the tables; the
+        // other rows, split evenly over the CTAs, one per thread, are
+        // eliminated against U11 with their own keys checked; one verdict per
+        // panel.  If any check fails (or a pivot is zero or not finite) the
+        // panel is reloaded and factored by the search path.
+        // What a panel costs (cycles of the 512-frequency kite's clusters of
+        // 3 and 4, per-phase clocks of an instrumented copy): 256 k when one
+        // warp eliminated the block, a row per lane, and copied its rows to
+        // the other CTAs (50 k), when rows belonged to CTAs by 512 (29 k) and
+        // when the write-back waited for the cluster (37 k); 197 k now: load
+        // 13, block 19, rows 14, verdict and staging 8, write-back 13, U12 38,
+        // update 82.  Shared-memory reads bound the rows and U12 (a
+        // warp-wide broadcast read takes a cycle per four bytes), so the
+        // complex product is four FMAs and one 8-byte read; packed pairs with
+        // 16-byte reads were slower (U12 37 -> 54 k).  Factor phase: 38.2 ->
+        // 29.3 ms (BF16, 511 systems of N 64..1920), 1.06 -> 0.88 ms (255, N to
+        // 480), 8.9 -> 7.2 ms (TF32, 16 x 127 systems of N 64..832).
         bool fast = false;
+        const int frows = nb == NB ? ((m - NB + cs - 1) / cs + 1) & ~1 : 0;   // rows below the block, per CTA
+        const int frow = rank * frows + tid;                                 // this thread's, relative to k0 + NB
+        const bool lrow = tid < frows && frow < m - NB;
         {
-            float2 (*u11)[NB + 2] = reinterpret_cast<float2 (*)[NB + 2]>(sA);   // [c][q]; pinv at [c][NB]
             uint32_t fail = 0u;
-            const bool dwarp = rank == 0 && warp == 0;     // rows 0-31: the diagonal block
-            const bool lrow = own && myslot >= nb;         // rows eliminated against u11
-            auto diag_step = [&](auto rows_c, const int q0) {
-                constexpr int kRows = decltype(rows_c)::value;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int c = q0 + i;
-                    if (c < nb) {
-                        if (lane == c) {
-#pragma unroll
-                            for (int e = i; e < kRows; ++e)
-                                if (q0 + e < NB) u11[c][q0 + e] = v[e];
-                        }
-                        __syncwarp();
-                        const float2 pvt = u11[c][c];
-                        const uint32_t kd = __float_as_uint(fabsf(pvt.x) + fabsf(pvt.y));
-                        const bool act = own && lane > c;
-                        const uint32_t kr = act ? __float_as_uint(fabsf(v[i].x) + fabsf(v[i].y)) : 0u;
-                        const uint32_t kmax = __reduce_max_sync(0xffffffffu, kr);
-                        if (kmax > kd || kd == 0u || kd >= 0x7F800000u) fail = 1u;
-                        const float rd = 1.f / (pvt.x * pvt.x + pvt.y * pvt.y);
-                        const float2 pinv = make_float2(pvt.x * rd, -pvt.y * rd);
-                        if (lane == 0) u11[c][NB] = pinv;
-                        if (act) {
-                            const float2 l = cmul(v[i], pinv);
-                            v[i] = l;
-#pragma unroll
-                            for (int e = i + 1; e < kRows; ++e)
-                                if (q0 + e < NB) {
-                                    const float2 u = u11[c][q0 + e];
-                                    v[e].x -= l.x * u.x - l.y * u.y;
-                                    v[e].y -= l.x * u.y + l.y * u.x;
-                                }
-                        }
-                        __syncwarp();
-                    }
-                }
-                float2 t[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) t[e] = v[e];
-#pragma unroll
-                for (int e = 0; e + 4 < NB; ++e) v[e] = v[e + 4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) v[NB - 4 + e] = t[e];
-            };
+            load_row(lrow, NB + frow);
             auto row_step = [&](auto rows_c, const int q0) {
                 constexpr int kRows = decltype(rows_c)::value;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int c = q0 + i;
-                    if (c < nb && lrow) {
-                        const float2 pvt = u11[c][c], pinv = u11[c][NB];
-                        const uint32_t kd = __float_as_uint(fabsf(pvt.x) + fabsf(pvt.y));
-                        if (__float_as_uint(fabsf(v[i].x) + fabsf(v[i].y)) > kd) fail = 1u;
-                        const float2 l = cmul(v[i], pinv);
-                        v[i] = l;
+                    if (__float_as_uint(fabsf(v[i].x) + fabsf(v[i].y)) > ps.kd[c]) fail = 1u;
+                    const float2 l = cmul(v[i], ps.pinv[c]);
+                    v[i] = l;
 #pragma unroll
-                        for (int e = i + 1; e < kRows; ++e)
-                            if (q0 + e < NB) {
-                                const float2 u = u11[c][q0 + e];
-                                v[e].x -= l.x * u.x - l.y * u.y;
-                                v[e].y -= l.x * u.y + l.y * u.x;
-                            }
-                    }
+                    for (int e = i + 1; e < kRows; ++e)
+                        if (q0 + e < NB) csub(v[e], l, u11[c][q0 + e]);
                 }
                 float2 t[4];
 #pragma unroll
@@ -504,21 +483,61 @@ __global__ void __launch_bounds__(kThreads, 1) lu_factor_tc_kernel(
 #pragma unroll
                 for (int e = 0; e < 4; ++e) v[NB - 4 + e] = t[e];
             };
-            if (dwarp) {
-#pragma unroll 1
-                for (int q0 = 0; q0 < NB / 2; q0 += 4) diag_step(std::integral_constant<int, NB>{}, q0);
-#pragma unroll 1
-                for (int q0 = NB / 2; q0 < NB; q0 += 4) diag_step(std::integral_constant<int, NB / 2>{}, q0);
-                if constexpr (kMulti) {   // u11 (pivot rows and reciprocals) to the other CTAs
-                    const float4 *src = reinterpret_cast<const float4 *>(&u11[0][0]);
-                    constexpr int kU4 = NB * (NB + 2) / 2;
-                    for (int r = 1; r < cs; ++r) {
-                        float4 *dst = reinterpret_cast<float4 *>(at_rank(&u11[0][0], cs, r));
-                        for (int e = lane; e < kU4; e += 32) dst[e] = src[e];
-                    }
+            {
+                const int r = tid >> 4, cl = tid & 15;   // entries (r, cl), (r, cl + 16)
+                const float2 *src = a + (long long)(k0 + r) * n + k0;
+                const float2 z = make_float2(0.f, 0.f);
+                float2 d0 = r < nb && cl < nb ? __ldcg(src + cl) : z;
+                float2 d1 = r < nb && cl + 16 < nb ? __ldcg(src + cl + 16) : z;
+                // the zero rows of l11; L21 of the pair's first panel in this panel's first rows
+                l11[NB + r / 2][16 * (r & 1) + cl] = z;
+                if (LT::kPair && role == 2) {
+                    lpq[r][cl] = __ldcg(src - NB + cl);
+                    lpq[r][cl + 16] = __ldcg(src - NB + cl + 16);
                 }
+                auto diag_half = [&](auto half_c) {
+                    constexpr int h = decltype(half_c)::value;
+#pragma unroll 1
+                    for (int cc = 0; cc < 16; ++cc) {
+                        const int c = 16 * h + cc;
+                        if (c >= nb) break;
+                        if (cl == cc) ps.lcol[c & 1][r] = h ? d1 : d0;
+                        if (r == c) {
+                            u11[c][cl] = d0;
+                            u11[c][cl + 16] = d1;
+                        }
+                        __syncthreads();
+                        const float2 pvt = ps.lcol[c & 1][c], lv = ps.lcol[c & 1][r];
+                        const uint32_t kd = __float_as_uint(fabsf(pvt.x) + fabsf(pvt.y));
+                        const bool act = r > c && r < nb;
+                        if (kd == 0u || kd >= 0x7F800000u ||
+                            (act && __float_as_uint(fabsf(lv.x) + fabsf(lv.y)) > kd))
+                            fail = 1u;
+                        const float rd = 1.f / (pvt.x * pvt.x + pvt.y * pvt.y);
+                        const float2 pinv = make_float2(pvt.x * rd, -pvt.y * rd);
+                        if (tid == 0) {
+                            ps.pinv[c] = pinv;
+                            ps.kd[c] = kd;
+                        }
+                        if (act) {
+                            const float2 l = cmul(lv, pinv);
+                            if (h == 0) {
+                                if (cl > cc) csub(d0, l, u11[c][cl]);
+                                else if (cl == cc) d0 = l;
+                                csub(d1, l, u11[c][cl + 16]);
+                            } else {
+                                if (cl > cc) csub(d1, l, u11[c][cl + 16]);
+                                else if (cl == cc) d1 = l;
+                            }
+                        }
+                    }
+                };
+                diag_half(std::integral_constant<int, 0>{});
+                diag_half(std::integral_constant<int, 1>{});
+                if (cl < r) l11[r][cl] = d0;
+                if (cl + 16 < r) l11[r][cl + 16] = d1;
             }
-            sys_sync(cs, false);   // u11 in every CTA
+            __syncthreads();   // the tables
             if (lrow) {
 #pragma unroll 1
                 for (int q0 = 0; q0 < NB / 2; q0 += 4) row_step(std::integral_constant<int, NB>{}, q0);
@@ -529,22 +548,30 @@ __global__ void __launch_bounds__(kThreads, 1) lu_factor_tc_kernel(
             if constexpr (kMulti) {
                 if (tid == 0)
                     for (int r = 0; r < cs; ++r) *at_rank(&ps.ffail[rank], cs, r) = any;
-                sys_sync(cs, false);
+                cg::this_cluster().barrier_arrive();
+            }
+            // the L21 rows to the staged A operand while the verdict arrives
+            // (the search path stages them again)
+            if (!any && lrow) {
+                if (role != 2) put_a_row<kKind, 1>(atiles, frow / TR, frow % TR, v, 0);
+                else put_a_row<kKind, 2>(atiles, frow / TR, frow % TR, v, 1);
+            }
+            if constexpr (kMulti) {
+                cg::this_cluster().barrier_wait();
                 int all = 0;
                 for (int r = 0; r < cs; ++r) all |= ps.ffail[r];
                 fast = all == 0;
             } else {
                 fast = any == 0;
             }
-            if (!fast) {   // the search path below, from the panel as loaded
-                const float4 *src = reinterpret_cast<const float4 *>(a + (long long)(k0 + (own ? myslot : 0)) * n + k0);
-#pragma unroll
-                for (int h = 0; h < NB / 2; ++h) {
-                    const float4 t = (own && 2 * h < nb) ? __ldcg(src + h) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    v[2 * h] = make_float2(t.x, t.y);
-                    v[2 * h + 1] = make_float2(t.z, t.w);
-                }
-            }
+        }
+        // the search path: thread t of CTA r owns panel row 512 r + t
+        const bool own = !fast && myslot < m;
+        int mypos = myslot;
+        bool active = own;
+        if (!fast) {
+            load_row(own, myslot);
+            sys_sync(cs, false);   // the tables are read and the staging stores issued everywhere
         }
 
         // 1. panel factorisation in registers, four columns per step of a
@@ -756,57 +783,68 @@ __global__ void __launch_bounds__(kThreads, 1) lu_factor_tc_kernel(
 
         // 2. panel to its final rows (and the L21 rows to the staged A
         // operand); L11 and the moved rows to every CTA
-        if (own) {
-            float4 *dst = reinterpret_cast<float4 *>(a + (long long)(k0 + mypos) * n + k0);
-#pragma unroll
-            for (int h = 0; h < NB / 2; ++h)
-                if (2 * h < nb) __stcg(dst + h, make_float4(v[2 * h].x, v[2 * h].y, v[2 * h + 1].x, v[2 * h + 1].y));
-            if (role != 2) {
-                if (mypos >= nb && nb == NB)
-                    put_a_row<kKind, 1>(atiles, (mypos - NB) / TR, (mypos - NB) % TR, v, 0);
-            } else if (mypos >= NB) {
-                put_a_row<kKind, 2>(atiles, (mypos - NB) / TR, (mypos - NB) % TR, v, 1);
+        if (fast) {
+            // no row moves: the diagonal block from the tables, the other rows
+            // from their threads, then slot 0 of the two-panel A tiles (the
+            // row's L21 of the first panel; v is done with).  What the other
+            // CTAs need is read after the barrier before the update.
+            if (rank == 0 && tid < NB * NB / 2) {
+                const int r = tid / (NB / 2), q = 2 * (tid % (NB / 2));
+                if (r < nb && q < nb) {
+                    const float2 e0 = q < r ? l11[r][q] : u11[r][q], e1 = q + 1 < r ? l11[r][q + 1] : u11[r][q + 1];
+                    __stcg(reinterpret_cast<float4 *>(a + (long long)(k0 + r) * n + k0 + q), make_float4(e0.x, e0.y, e1.x, e1.y));
+                }
             }
-            if (mypos < nb)
-                for (int r = 0; r < cs; ++r) {
-                    float2 *l = at_rank(&ps.l11[mypos][0], cs, r);
-#pragma unroll
-                    for (int q = 0; q < NB; ++q)
-                        if (q < mypos) l[q] = v[q];
+            if (lrow) {
+                store_row(NB + frow);
+                if (role == 2) {
+                    load_first(NB + frow);
+                    put_a_row<kKind, 2>(atiles, frow / TR, frow % TR, v, 0);
                 }
-            if (role == 2) {
-                // the row's L21 of the first panel (v is done with), from its
-                // place before the swaps of this panel: into slot 0 of the
-                // two-panel A tiles, or for a pivot row into row mypos of lpq
-                // at every CTA
-                const float4 *lp = reinterpret_cast<const float4 *>(a + (long long)(k0 + myslot) * n + (k0 - NB));
-#pragma unroll
-                for (int h = 0; h < NB / 2; ++h) {
-                    const float4 t = __ldcg(lp + h);
-                    v[2 * h] = make_float2(t.x, t.y);
-                    v[2 * h + 1] = make_float2(t.z, t.w);
+            }
+        } else {
+            if (own) {
+                store_row(mypos);
+                if (role != 2) {
+                    if (mypos >= nb && nb == NB)
+                        put_a_row<kKind, 1>(atiles, (mypos - NB) / TR, (mypos - NB) % TR, v, 0);
+                } else if (mypos >= NB) {
+                    put_a_row<kKind, 2>(atiles, (mypos - NB) / TR, (mypos - NB) % TR, v, 1);
                 }
-                if (mypos >= NB) {
-                    put_a_row<kKind, 2>(atiles, (mypos - NB) / TR, (mypos - NB) % TR, v, 0);
-                } else {
+                if (mypos < nb)
                     for (int r = 0; r < cs; ++r) {
-                        float4 *dst = reinterpret_cast<float4 *>(at_rank(&lpq[mypos][0], cs, r));
+                        float2 *l = at_rank(&l11[mypos][0], cs, r);
 #pragma unroll
-                        for (int h = 0; h < NB / 2; ++h)
-                            dst[h] = make_float4(v[2 * h].x, v[2 * h].y, v[2 * h + 1].x, v[2 * h + 1].y);
+                        for (int q = 0; q < NB; ++q)
+                            if (q < mypos) l[q] = v[q];
+                    }
+                if (role == 2) {
+                    // the row's L21 of the first panel (v is done with), from its
+                    // place before the swaps of this panel: into slot 0 of the
+                    // two-panel A tiles, or for a pivot row into row mypos of lpq
+                    // at every CTA
+                    load_first(myslot);
+                    if (mypos >= NB) {
+                        put_a_row<kKind, 2>(atiles, (mypos - NB) / TR, (mypos - NB) % TR, v, 0);
+                    } else {
+                        for (int r = 0; r < cs; ++r) {
+                            float2 *dst = at_rank(&lpq[mypos][0], cs, r);
+#pragma unroll
+                            for (int q = 0; q < NB; ++q) dst[q] = v[q];
+                        }
                     }
                 }
+                if (mypos != myslot)
+                    for (int r = 0; r < cs; ++r) {
+                        const int idx = atomicAdd(at_rank(&ps.mv_cnt, cs, r), 1);
+                        if (idx < kMaxMoved) {   // at most 2 nb rows change position
+                            *at_rank(&ps.mv_dst[idx], cs, r) = mypos;
+                            *at_rank(&ps.mv_src[idx], cs, r) = myslot;
+                        }
+                    }
             }
-            if (mypos != myslot)
-                for (int r = 0; r < cs; ++r) {
-                    const int idx = atomicAdd(at_rank(&ps.mv_cnt, cs, r), 1);
-                    if (idx < kMaxMoved) {   // at most 2 nb rows change position
-                        *at_rank(&ps.mv_dst[idx], cs, r) = mypos;
-                        *at_rank(&ps.mv_src[idx], cs, r) = myslot;
-                    }
-                }
+            sys_sync(cs, true);
         }
-        sys_sync(cs, true);
 
         // column ranges of this CTA outside the panel: an even share of the
         // columns left of it, [lc_lo, lc_hi), and of those right of it, columns
@@ -815,7 +853,7 @@ __global__ void __launch_bounds__(kThreads, 1) lu_factor_tc_kernel(
         const int WL = (((k0 + cs - 1) / cs) + 1) & ~1, WR = (((nr + cs - 1) / cs) + 1) & ~1;
         const int lc_lo = min(k0, rank * WL), lc_hi = min(k0, lc_lo + WL);
         const int rc_lo = k0 + min(nr, rank * WR), rc_hi = k0 + min(nr, rank * WR + WR);
-        const int nmv = min(ps.mv_cnt, kMaxMoved);
+        const int nmv = fast ? 0 : min(ps.mv_cnt, kMaxMoved);
         if (nmv > 0) {
             int t_perm = 0;
             if (rank == 0 && tid < nmv) t_perm = pv[k0 + ps.mv_src[tid]];
@@ -852,39 +890,28 @@ __global__ void __launch_bounds__(kThreads, 1) lu_factor_tc_kernel(
         // (second panel of a pair: first A12 -= L21(first panel) U12(first
         // panel) in these rows, the update the first panel left out)
         const BDest bd{btiles, b2tiles, role == 0 ? INT_MAX : role == 1 ? NB : 0, role == 2 ? 1 : 0};
-        // (U12 of the first panel over this CTA's columns, rows k0 - NB ..,
-        // into the gather space with coalesced loads: up[q][c - rc_lo])
-        float2 *up = reinterpret_cast<float2 *>(gbuf);
-        const int ncol = rc_hi - rc_lo;
-        // (at most 512 columns: a CTA owns 512 rows, so cs >= n / 512)
-        if (role == 2 && NB * ncol > 2 * kGather) failed = true;
-        if (role == 2 && !failed) {
-            for (int e = tid; e < NB * ncol; e += kThreads) {
-                const int q = e / ncol, c = e - q * ncol;
-                up[e] = __ldcg(a + (long long)(k0 - NB + q) * n + rc_lo + c + nb);
-            }
-            __syncthreads();
-        }
         for (int c = rc_lo + tid; c < rc_hi; c += kThreads) {
             float2 *col = a + (long long)k0 * n + c + nb;
             float2 x[NB];
 #pragma unroll
             for (int e = 0; e < NB; ++e)
                 x[e] = e < nb ? __ldcg(col + (long long)e * n) : make_float2(0.f, 0.f);
-            if (role == 2 && !failed) {
-#pragma unroll 2
-                for (int q = 0; q < NB; ++q) {
-                    const float2 u = up[q * ncol + (c - rc_lo)];
+            if (LT::kPair && role == 2) {
+                // (U12 of the first panel: the rows above, eight at a time)
+                const float2 *up = col - (long long)NB * n;
+#pragma unroll 1
+                for (int q0 = 0; q0 < NB; q0 += 8) {
+                    float2 u[8];
 #pragma unroll
-                    for (int e = 0; e < NB; ++e) {
-                        const float2 l = lpq[e][q];
-                        x[e].x -= l.x * u.x - l.y * u.y;
-                        x[e].y -= l.x * u.y + l.y * u.x;
-                    }
+                    for (int q = 0; q < 8; ++q) u[q] = __ldcg(up + (long long)(q0 + q) * n);
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+#pragma unroll
+                        for (int e = 0; e < NB; ++e) csub(x[e], lpq[e][q0 + q], u[q]);
                 }
             }
-            trsm_groups<kKind, NB>(x, 0, NB / 8, ps.l11, col, n, nb, bd, c - k0);
-            trsm_groups<kKind, NB / 2>(x, NB / 8, NB / 4, ps.l11, col, n, nb, bd, c - k0);
+            trsm_groups<kKind, NB>(x, 0, NB / 8, l11, col, n, nb, bd, c - k0);
+            trsm_groups<kKind, NB / 2>(x, NB / 8, NB / 4, l11, col, n, nb, bd, c - k0);
         }
         // the swaps, U12 and the staged operands (generic stores to global
         // memory) are read by the TMA engine below, which also overwrites the
