@@ -53,7 +53,7 @@ struct Problem {
     int K = 0;
     double H = 10.0;
     std::vector<double> s;
-    DevBuf d_s, d_B;
+    DevBuf d_s, d_B, d_Bf;   // window centres, spectra, spectra as double-float pairs
     int S() const { return J - 1; }
 };
 
@@ -126,7 +126,7 @@ struct fh_ctx {
     DevBuf d_z, d_dz, d_ddz, d_kress, d_logsin, d_A, d_psi, d_info, d_nu, d_nu_f, d_ph, d_omega, d_pw;
     DevBuf d_stab;
     DevBuf d_lu64;                       // FP64 LU: the row moves of each system's current panel
-    DevBuf d_A32, d_piv, d_g, d_iters, d_resid, d_tcerr, d_y32, d_rstate, d_rchunk, d_Bf, d_dblk,
+    DevBuf d_A32, d_piv, d_g, d_iters, d_resid, d_tcerr, d_y32, d_rstate, d_rchunk, d_dblk,
         d_blk_off, d_dinv;
     // tensor-core LU work space: tensor maps of the FP32 matrices, staged
     // operand tiles and their offsets; valid for (lu_key_ptr, lu_key_gen)
@@ -154,6 +154,7 @@ struct fh_ctx {
         for (Problem &pb : probs) {
             free_buf(pb.d_s);
             free_buf(pb.d_B);
+            free_buf(pb.d_Bf);
         }
         probs.clear();
     }
@@ -164,7 +165,7 @@ struct fh_ctx {
                          &d_kappa, &d_eta, &d_solve_j, &d_solve_prob, &d_order, &d_curves,
                          &d_pdir, &d_zf, &d_dzf, &d_sf, &d_wpf, &d_z, &d_dz, &d_ddz, &d_kress, &d_logsin, &d_A, &d_psi,
                          &d_info, &d_nu, &d_nu_f, &d_ph, &d_omega, &d_pw, &d_stab, &d_lu64, &d_A32, &d_piv, &d_g, &d_iters,
-                         &d_resid, &d_tcerr, &d_y32, &d_rstate, &d_rchunk, &d_Bf, &d_dblk, &d_blk_off, &d_dinv,
+                         &d_resid, &d_tcerr, &d_y32, &d_rstate, &d_rchunk, &d_dblk, &d_blk_off, &d_dinv,
                          &d_lu_maps, &d_lu_opnd, &d_lu_aoff, &d_lu_boff, &d_wa, &d_a, &d_x, &d_T, &d_u, &d_V, &d_Gr, &d_Gm, &d_Gs, &d_Vs, &d_ctc, &d_ctc_err,
                          &d_tmpA, &d_tmpg, &d_tmp_ll, &d_tmp_d, &d_tmp_i};
         for (DevBuf *b : all) free_buf(*b);
@@ -777,11 +778,12 @@ fh_status spectra_common(fh_ctx *ctx, Problem &pb, const double *d_a, int n_samp
     const size_t wa_bytes = (size_t)K * (size_t)(Q + 1) * sizeof(double);
     FH_TRY(ensure(ctx, ctx->d_wa, wa_bytes));
     FH_TRY(ensure(ctx, pb.d_B, (size_t)K * pb.J * sizeof(double2)));
+    FH_TRY(ensure(ctx, pb.d_Bf, (size_t)K * pb.J * sizeof(float4)));
     FH_TRY(upload(ctx, pb.d_s, s));
     PhaseScope ps(ctx, FH_PH_SPECTRA, 2);
     fh::launch_window_spectra(d_a, n_samples, start0, step, (int)Q, dt, H, K, pb.J,
                               ctx->d_omega.as<double>() + pb.omega_off, ctx->d_wa.as<double>(),
-                              pb.d_B.as<double2>(), ctx->stream);
+                              pb.d_B.as<double2>(), pb.d_Bf.as<float4>(), ctx->stream);
     FH_TRY(check_launch(ctx, "window spectra"));
     pb.K = K;
     pb.H = H;
@@ -810,7 +812,7 @@ fh_status synth_buffers(fh_ctx *ctx, Problem &pb, int n_x, int n_T) {
         FH_TRY(ensure(ctx, ctx->d_Gs, (size_t)2 * pb.J * fh::synth_pitch(n_T) * sizeof(float2)));
         FH_TRY(ensure(ctx, ctx->d_Vs, (size_t)2 * pb.J * fh::synth_pitch(n_x) * sizeof(float2)));
     }
-    return ensure(ctx, ctx->d_Bf, (size_t)pb.K * pb.J * sizeof(float4));
+    return FH_OK;
 }
 
 // Runs the enclosed launches on another stream of the context.
@@ -826,9 +828,9 @@ fh_status weights_kernels(fh_ctx *ctx, Problem &pb, const double *d_T, int n_T) 
     const bool tcc = use_contract_tc(ctx, pb);
     const bool mixed = ctx->precision != FH_FP64 && !tcc;   // double-float weights and contraction
     {
-        PhaseScope ps(ctx, FH_PH_WEIGHTS, 2);
+        PhaseScope ps(ctx, FH_PH_WEIGHTS, 1);
         fh::launch_synth_weights(pb.J, pb.M, pb.W, pb.K, pb.d_s.as<double>(), pb.d_B.as<double2>(),
-                                 ctx->d_Bf.as<float4>(), ctx->d_nu_f.as<float4>() + pb.nu_off,
+                                 pb.d_Bf.as<float4>(), ctx->d_nu_f.as<float4>() + pb.nu_off,
                                  ctx->d_ph.as<float4>() + pb.ph_off,
                                  pb.stab_off >= 0 ? ctx->d_stab.as<float4>() + pb.stab_off : nullptr, d_T, n_T,
                                  ctx->d_Gr.as<double>(), ctx->d_Gm.as<double>(),

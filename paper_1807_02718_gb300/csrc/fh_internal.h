@@ -171,9 +171,10 @@ void launch_lu_refine(bool row_major, const int *order, int S, const int *N,
                       double tol, int *iters, double *resid, int *info, int maxN, cudaStream_t st);
 
 // ---- window spectra (k_window.cu) ----
+// B[k * J + j], and Bf the same as double-float pairs (re hi, re lo, im hi, im lo).
 void launch_window_spectra(const double *a, int n_samples, long long start0, long long step,
                            int Q, double dt, double H, int K, int J, const double *omega,
-                           double *wa_scratch, double2 *B, cudaStream_t st);
+                           double *wa_scratch, double2 *B, float4 *Bf, cudaStream_t st);
 
 // ---- target fields (k_field.cu) ----
 // V[j * n_x + i] = V(x_i, omega_j); V[0 * n_x + i] = 1 (omega_0 = 0).
@@ -200,7 +201,7 @@ void launch_bessel_eval_df(const double *x, int n, double *out, cudaStream_t st)
 // ---- synthesis (k_synth.cu) ----
 // nu[r * J + p] = sum_{m=-h}^{h-1} (-1)^m T_r(m/h) e^{-2 pi i m p / M} (T_r
 // the Chebyshev polynomials, the r = 0 row halved; nu may be null), and nu_f
-// the same as double-float pairs (re hi, re lo, im hi, im lo); pw is scratch
+// the same as double-float pairs (re hi, im hi, re lo, im lo); pw is scratch
 // of M * kFarTerms doubles.  Far windows (|y| >= 1.25 h) need at most 48 terms.
 constexpr int kFarTerms = 64;
 void launch_far_table(int J, int M, double *pw, double2 *nu, float4 *nu_f, float4 *phase_tab,
@@ -208,11 +209,11 @@ void launch_far_table(int J, int M, double *pw, double2 *nu, float4 *nu_f, float
 // Gr/Gm: planes [p][t] with u(x,t) = sum_p Vr[p][x] Gr[p][t] + Vi[p][x] Gm[p][t].
 // Gs (optional; then Gr/Gm are not written): the same weights as double-float
 // pairs (hi, lo), rows p = Gr[p] and J + p = Gm[p], row pitch synth_pitch(n_T),
-// for launch_synth_contract_df.  Bf: optional scratch of K * J float4 for the
-// double-float copy of B (one extra launch); null splits B on the fly.
+// for launch_synth_contract_df.  Bf: the double-float copy of B; with sinc_tab
+// null it may be null too (B is split on the fly).  One launch.
 inline int synth_pitch(int n) { return (n + 3) & ~3; }
 void launch_synth_weights(int J, int M, double W, int K, const double *s, const double2 *B,
-                          float4 *Bf, const float4 *nu_f, const float4 *phase_tab,
+                          const float4 *Bf, const float4 *nu_f, const float4 *phase_tab,
                           const float4 *sinc_tab, const double *T, int n_T, double *Gr, double *Gm,
                           float2 *Gs, cudaStream_t st);
 // Dynamic shared memory launch_synth_weights needs for J frequencies and K
@@ -231,7 +232,7 @@ size_t synth_weights_smem(int J, int K, bool table);
 // window's Fourier transform is flat to 1.4e-15 on [-pi, pi] and its aliases
 // from [3 pi, inf) sum below 1.1e-15.  The table holds D_p(y_g) for |g| <= G =
 // ceil(2.5 h) + 24 (every near y, |y| < 1.25 h, with its 42 samples) as
-// double-float pairs (re hi, re lo, im hi, im lo), row g + G, column p:
+// double-float pairs (re hi, im hi, re lo, im lo), row g + G, column p:
 // integer rows are the phases themselves, half-integer rows the direct sums
 // in double-float.  Built for J <= kSincTabMaxJ (table size (2G + 1) J).
 constexpr int kSincTabMaxJ = 1025;

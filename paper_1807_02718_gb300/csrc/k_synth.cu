@@ -29,7 +29,9 @@
 // truncation error).  Its ratio |rho| is below the Taylor ratio h/|y| (0.5
 // against 0.8 at |y| = 1.25 h), hence fewer terms.  Near windows interpolate a
 // table of the direct sums or sum the M terms directly.
+#include "dfloat.cuh"
 #include "fh_internal.h"
+#include "sinc_interp.cuh"
 
 namespace fh {
 namespace {
@@ -112,7 +114,7 @@ __global__ void __launch_bounds__(128) far_table_kernel(int J, int M, const doub
     if (r < kFarTerms) {
         if (nu) nu[(long long)r * J + p] = make_double2(sr, si);
         const float rh = (float)sr, ih = (float)si;   // double-float copy for the far Horner
-        nu_f[(long long)r * J + p] = make_float4(rh, (float)(sr - (double)rh), ih, (float)(si - (double)ih));
+        nu_f[(long long)r * J + p] = make_float4(rh, ih, (float)(sr - (double)rh), (float)(si - (double)ih));
     }
 }
 
@@ -181,58 +183,6 @@ __device__ __forceinline__ void df_horner(float &ah, float &al, dfl r, float vh,
 }
 
 __device__ __forceinline__ dfl df_negq(dfl a) { return {-a.hi, -a.lo}; }
-
-// sqrt(a) in double-float (a > 0): s = sqrt(a.hi) in binary32, corrected by
-// (a - s^2) / (2 s) with s^2 exact through the FMA residual.
-__device__ __forceinline__ dfl df_sqrtq(dfl a) {
-    const float s = sqrtf(a.hi);
-    const float r = (fmaf(-s, s, a.hi) + a.lo) / (2.f * s);
-    const float h = s + r;
-    return {h, r - (h - s)};
-}
-
-// e^x in double-float for -88 < x <= 0: x = k ln2 + r with |r| <= ln2 / 2,
-// ln2 = L1 + L2 where L1 holds 16 significant bits (k L1 exact for |k| < 2^8);
-// e^r by its Taylor series at 0, the terms n = 8 .. 13 (below 6e-9 for
-// |r| <= 0.347) in binary32 and the rest in double-float; then e^x = 2^k e^r.
-constexpr double kLn2 = 0.69314718055994530942;
-constexpr float kLn2A = 0.693145751953125f;
-constexpr float kLn2B = (float)(kLn2 - 0.693145751953125);
-constexpr float kLn2C = (float)(kLn2 - 0.693145751953125 - (double)kLn2B);
-// 1/n! for n = 3 .. 7 as double-float pairs (1/0!, 1/1!, 1/2! are exact)
-#define FH_INV_FACT(n, v) \
-    constexpr float kIF##n##h = (float)(v); \
-    constexpr float kIF##n##l = (float)((v) - (double)(float)(v));
-FH_INV_FACT(3, 1.0 / 6.0)
-FH_INV_FACT(4, 1.0 / 24.0)
-FH_INV_FACT(5, 1.0 / 120.0)
-FH_INV_FACT(6, 1.0 / 720.0)
-FH_INV_FACT(7, 1.0 / 5040.0)
-#undef FH_INV_FACT
-
-__device__ __forceinline__ dfl df_expq(dfl x) {
-    const float k = rintf(x.hi * 1.4426950408889634f);
-    // r = x - k ln2: x.hi - k L1 is exact (Sterbenz), k L2 exact as a pair
-    const float kb = k * kLn2B, kbe = fmaf(k, kLn2B, -kb);
-    dfl r = df_addq({x.hi - k * kLn2A, x.lo}, {-kb, -fmaf(k, kLn2C, kbe)});
-    float tail = 1.f / 6227020800.f;   // 1/13!
-    tail = fmaf(tail, r.hi, 1.f / 479001600.f);
-    tail = fmaf(tail, r.hi, 1.f / 39916800.f);
-    tail = fmaf(tail, r.hi, 1.f / 3628800.f);
-    tail = fmaf(tail, r.hi, 1.f / 362880.f);
-    tail = fmaf(tail, r.hi, 1.f / 40320.f);
-    dfl q = {tail, 0.f};
-    q = df_addq(df_mulq(q, r), {kIF7h, kIF7l});
-    q = df_addq(df_mulq(q, r), {kIF6h, kIF6l});
-    q = df_addq(df_mulq(q, r), {kIF5h, kIF5l});
-    q = df_addq(df_mulq(q, r), {kIF4h, kIF4l});
-    q = df_addq(df_mulq(q, r), {kIF3h, kIF3l});
-    q = df_addq(df_mulq(q, r), {0.5f, 0.f});
-    q = df_addq(df_mulq(q, r), {1.f, 0.f});
-    q = df_addq(df_mulq(q, r), {1.f, 0.f});
-    const int ki = (int)k;
-    return {ldexpf(q.hi, ki), ldexpf(q.lo, ki)};
-}
 
 // Direct near-window sum, unscaled, for the thread's p (all threads of the CTA
 // call it; it begins and ends with a barrier):
@@ -325,7 +275,10 @@ __global__ void __launch_bounds__(kTabThreads) sinc_table_kernel(int J, int M, i
             const int g = e_first + 2 * (int)(idx / J);
             const int n = g / 2;
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (n >= -h && n < h) v = ph_g[(long long)(n + M) * pp % M];
+            if (n >= -h && n < h) {
+                const float4 e = ph_g[(long long)(n + M) * pp % M];
+                v = make_float4(e.x, e.z, e.y, e.w);
+            }
             tab[(long long)(g + G) * J + pp] = v;
         }
         return;
@@ -382,7 +335,7 @@ __global__ void __launch_bounds__(kTabThreads) sinc_table_kernel(int J, int M, i
         if (g > G) break;
         const float tr = ac[r][0] + ac[r][1], ti = ac[r][2] + ac[r][3];
         const dfl re = {tr, ac[r][1] - (tr - ac[r][0])}, im = {ti, ac[r][3] - (ti - ac[r][2])};
-        tab[(long long)(g + G) * J + p] = make_float4(re.hi, re.lo, im.hi, im.lo);
+        tab[(long long)(g + G) * J + p] = make_float4(re.hi, im.hi, re.lo, im.lo);
         // D_p(-y) = conj(D_p(y)) + (-1)^p (sinc(y - h) - sinc(y + h)): m and -m
         // swap, c_{-m} = conj(c_m), and the end terms m = -h, h differ; at
         // y = g/2, sinc(y -+ h) = (-1)^h sin(pi y) / (pi (y -+ h))
@@ -390,7 +343,7 @@ __global__ void __launch_bounds__(kTabThreads) sinc_table_kernel(int J, int M, i
         const double corr = ((h & 1) ? -sy : sy) * 2.0 * (double)h / (kPi * (y * y - (double)h * (double)h));
         const dfl c = df_split((p & 1) ? -corr : corr);
         const dfl rn = df_addq(re, c);
-        tab[(long long)(G - g) * J + p] = make_float4(rn.hi, rn.lo, -im.hi, -im.lo);
+        tab[(long long)(G - g) * J + p] = make_float4(rn.hi, -im.hi, rn.lo, -im.lo);
     }
 }
 
@@ -400,34 +353,186 @@ __host__ __device__ inline size_t weights_smem_head(int K) {
     return ((size_t)K * (2 * sizeof(double) + 3 * sizeof(float2) + 3 * sizeof(int)) + 15) & ~(size_t)15;
 }
 
-constexpr float kBetaUHi = (float)(kSincBeta / kSincU);
-constexpr float kBetaULo = (float)(kSincBeta / kSincU - (double)kBetaUHi);
-constexpr float k2PiHi = (float)(2.0 * kPi);
-constexpr float k2PiLo = (float)(2.0 * kPi - (double)k2PiHi);
 constexpr float kInv2PiHi = (float)(0.5 / kPi);
 constexpr float kInv2PiLo = (float)(0.5 / kPi - (double)kInv2PiHi);
 
-// One CTA per time t, thread p.  The per-window quantities that do not depend
-// on p (y, near or far, sin(pi y), the far ratio h/y and its truncation R)
-// are formed once per CTA.  Near windows: with the sampled table, 42 samples
-// around y weighted by sinc(2u) E(u) (weights formed once per window, FP64,
-// then split); without it, the direct M-term sums (near_sum).  Far windows:
-// Horner in double-float over the double-float copy of nu.
+// Far windows (|y| >= 1.25 h): the ratio rho and prefactor of the Chebyshev
+// expansion, its truncation R and the number R1 of leading terms taken in
+// double-float (from binary32 logarithms: term counts, not values).
+__device__ __forceinline__ void far_window(double y, int h, double scale, double &rho, double &f, int &R, int &R1) {
+    const double a = y / (double)h;
+    const double sq = copysign(sqrt((a - 1.0) * (a + 1.0)), a);
+    rho = 1.0 / (a + sq);
+    const float lr = -logf(fabsf((float)rho));
+    R = max(1, min((int)ceilf(48.f * 0.693147181f / lr), kFarTerms));
+    R1 = max(1, min((int)ceilf((25.f * 0.693147181f + logf((float)R)) / lr), R));
+    f = scale * sinpi(y) * 2.0 / (kPi * (double)h * sq);
+}
+
+// G = (mu_p / 2 pi) q, mu_p / 2 pi = 1/(2 pi) or 1/pi, in double-float; the planes
+// hold (Re G, -Im G).
+__device__ __forceinline__ void store_weight(int J, int p, int t, int n_T, int pitch_T, dfl q, dfl qi, double *Gr,
+                                             double *Gm, float2 *Gs) {
+    const bool edge = p == 0 || p == J - 1;
+    const dfl c = edge ? dfl{kInv2PiHi, kInv2PiLo} : dfl{2.f * kInv2PiHi, 2.f * kInv2PiLo};
+    const dfl a = df_mulq(q, c), b = df_negq(df_mulq(qi, c));
+    if (Gs) {
+        Gs[(long long)p * pitch_T + t] = make_float2(a.hi, a.lo);
+        Gs[(long long)(J + p) * pitch_T + t] = make_float2(b.hi, b.lo);
+    } else {
+        Gr[(long long)p * n_T + t] = (double)a.hi + (double)a.lo;
+        Gm[(long long)p * n_T + t] = (double)b.hi + (double)b.lo;
+    }
+}
+
+// Weights from the sampled near sums (J <= kSincTabMaxJ).  One CTA per time and
+// 256 columns p, in two groups of 128 threads with two columns each; group g
+// takes the windows k = g mod 2, and the groups' sums are added in order (a
+// fixed split, so that a time's weights do not depend on the other times).
+// Near windows: 42 samples around y, their weights (with 2W/M) formed by the
+// group's first threads; far windows: Horner's rule over the far table, the
+// terms past R1 in binary32.  (re, im) are one packed pair throughout.
+// Bound by FP32 issue with many times; with few, by the dependent steps of a
+// window (weights, barrier, loads from L2), which the groups take side by side.
+// (Four groups, 512 threads, were 4 % slower with many times: fewer CTAs hide
+// the FP64 set-up.)  Measured (GB300): 4096 times, J = 256, 29 windows: 0.63 ms before; 16
+// times, J = 128, 7 windows: 56 us before (one window after another, re and im
+// apart).
+constexpr int kWGroups = 2, kWCols = 128, kWChunk = 64;
+
+struct FarNear {
+    int R, R1;          // R = 0: near
+    SincPoint pt;       // near
+    dfv rho, f;         // far
+};
+
+__global__ void __launch_bounds__(kWGroups *kWCols, 4) weights_tab_kernel(
+    int J, int M, double W, int K, const double *__restrict__ s, const float4 *__restrict__ Bf,
+    const float4 *__restrict__ nu_f, const float4 *__restrict__ tab, int G, const double *__restrict__ T, int n_T,
+    double *__restrict__ Gr, double *__restrict__ Gm, float2 *__restrict__ Gs, int pitch_T) {
+    __shared__ FarNear win[kWChunk];
+    __shared__ float2 swt[kWGroups][kSincPts];
+    __shared__ float4 part[kWGroups - 1][2 * kWCols];
+    const int t = blockIdx.x, h = M / 2;
+    const int grp = threadIdx.x / kWCols, lane = threadIdx.x % kWCols;
+    const int p0 = blockIdx.y * 2 * kWCols + lane;
+    const bool two = blockIdx.y * 2 * kWCols + kWCols < J;      // the CTA has second columns
+    const int pa = min(p0, J - 1), pb = min(p0 + kWCols, J - 1);   // (columns past J - 1 are computed and dropped)
+    const double tt = T[t], scale = 2.0 * W / (double)M;
+    const dfv sc = df_from(scale);
+    float2 qh[2], ql[2];
+    qh[0] = qh[1] = ql[0] = ql[1] = p2(0.f, 0.f);
+    for (int k0 = 0; k0 < K; k0 += kWChunk) {
+        __syncthreads();
+        for (int k = threadIdx.x; k < min(kWChunk, K - k0); k += blockDim.x) {
+            FarNear w;
+            const double y = W * (tt - s[k0 + k]) * (1.0 / kPi);
+            w.R = w.R1 = 0;
+            w.rho = w.f = df_make(0.f, 0.f);
+            w.pt = SincPoint{0, 0, w.rho, w.rho};
+            if (fabs(y) < 1.25 * (double)h) {
+                w.pt = sinc_point(y);
+            } else {
+                double rho, f;
+                far_window(y, h, scale, rho, f, w.R, w.R1);
+                w.rho = df_from(rho);
+                w.f = df_from(f);
+            }
+            win[k] = w;
+        }
+        __syncthreads();
+        for (int k = k0 + grp; k < min(k0 + kWChunk, K); k += kWGroups) {
+            const FarNear &w = win[k - k0];
+            df2 d[2];
+            if (w.R == 0) {
+                asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(kWCols) : "memory");   // the last window's weights are read
+                if (lane < kSincPts) {
+                    const dfv v = df_mul(sinc_weight(w.pt, lane), sc);
+                    swt[grp][lane] = p2(v.hi, v.lo);
+                }
+                asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(kWCols) : "memory");
+                const float4 *row = tab + (long long)(w.pt.g0 + G) * J;
+                float2 ah = p2(0.f, 0.f), al = ah, bh = ah, bl = ah;
+#pragma unroll 6
+                for (int q = 0; q < kSincPts; ++q) {
+                    const float2 wt = swt[grp][q];
+                    const df2 ww = {p2(wt.x, wt.x), p2(wt.y, wt.y)};
+                    const float4 va = __ldg(row + (long long)q * J + pa);
+                    df2_acc(ah, al, ww, {p2(va.x, va.y), p2(va.z, va.w)});
+                    if (two) {
+                        const float4 vb = __ldg(row + (long long)q * J + pb);
+                        df2_acc(bh, bl, ww, {p2(vb.x, vb.y), p2(vb.z, vb.w)});
+                    }
+                }
+                d[0] = df2_quick(ah, al);
+                d[1] = df2_quick(bh, bl);
+            } else {
+                const float2 rh = p2(w.rho.hi, w.rho.hi), rl = p2(w.rho.lo, w.rho.lo);
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    if (c == 1 && !two) break;
+                    const float4 *col = nu_f + (c ? pb : pa);
+                    float2 a = p2(0.f, 0.f);
+#pragma unroll 4
+                    for (int r = w.R - 1; r >= w.R1; --r) {     // binary32 tail
+                        const float4 v = __ldg(col + (long long)r * J);
+                        a = p2_fma(a, rh, p2(v.x, v.y));
+                    }
+                    df2 f = {a, p2(0.f, 0.f)};
+#pragma unroll 4
+                    for (int r = w.R1 - 1; r >= 0; --r) {
+                        const float4 v = __ldg(col + (long long)r * J);
+                        float2 e;
+                        const float2 x = p2_prod(f, {rh, rl}, e), vh = p2(v.x, v.y), y = p2_add(x, vh);
+                        f = df2_quick(y, p2_add(p2_two_sum_err(x, vh, y), p2_add(e, p2(v.z, v.w))));
+                    }
+                    d[c] = df2_mul(f, df2_bcast(w.f));
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {   // q += b d (complex)
+                if (c == 1 && !two) break;
+                const float4 b4 = __ldg(Bf + (long long)k * J + (c ? pb : pa));
+                df2_acc(qh[c], ql[c], {p2(b4.x, b4.x), p2(b4.y, b4.y)}, d[c]);
+                df2_acc(qh[c], ql[c], {p2(-b4.z, b4.z), p2(-b4.w, b4.w)}, df2_swap(d[c]));
+            }
+        }
+    }
+    if (grp > 0) {
+#pragma unroll
+        for (int c = 0; c < 2; ++c) part[grp - 1][lane + c * kWCols] = make_float4(qh[c].x, qh[c].y, ql[c].x, ql[c].y);
+    }
+    __syncthreads();
+    if (grp > 0) return;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const int p = p0 + c * kWCols;
+        if (p >= J) break;
+        df2 q = df2_quick(qh[c], ql[c]);
+        for (int g = 0; g < kWGroups - 1; ++g) {
+            const float4 v = part[g][lane + c * kWCols];
+            q = df2_add(q, {p2(v.x, v.y), p2(v.z, v.w)});
+        }
+        store_weight(J, p, t, n_T, pitch_T, {q.h.x, q.l.x}, {q.h.y, q.l.y}, Gr, Gm, Gs);
+    }
+}
+
+// Weights without the sampled table (larger J, or no memory for it): one CTA
+// per time, thread p.  The per-window quantities that do not depend on p (y,
+// near or far, sin(pi y), the far ratio and its truncation R) are formed once
+// per CTA.  Near windows: the direct M-term sums (near_sum); far windows:
+// Horner's rule in double-float over the far table.
 __global__ void __launch_bounds__(256) weights_kernel(
     int J, int M, double W, int K, const double *__restrict__ s, const double2 *__restrict__ B,
     const float4 *__restrict__ Bf, const float4 *__restrict__ nu_f, const float4 *__restrict__ ph_g,
-    const float4 *__restrict__ tab, int G, const double *__restrict__ T, int n_T,
-    double *__restrict__ Gr, double *__restrict__ Gm, float2 *__restrict__ Gs, int pitch_T) {
+    const double *__restrict__ T, int n_T, double *__restrict__ Gr, double *__restrict__ Gm,
+    float2 *__restrict__ Gs, int pitch_T) {
     extern __shared__ __align__(16) double smd[];
-    __shared__ float2 swt[kSincPts];                          // interpolation weights, double-float
     double *wy = smd;                                        // K: y
-    double *wf = wy + K;                                     // K: sin(pi y) (near) or the far prefactor
+    double *wf = wy + K;                                     // K: sin(pi y) (near)
     float2 *wrho = reinterpret_cast<float2 *>(wf + K);       // K: rho (far) or 2W/M (near), double-float
-    float2 *wfd = wrho + K;                                  // K: far prefactor or sin(2 pi y), double-float
-    float2 *wu = wfd + K;                                    // K: u_c = y - g_c / 2 (near, table)
-    int *wR = reinterpret_cast<int *>(wu + K);               // K: far terms R | R1 << 16, 0 = near
-    int *wg = wR + K;                                        // K: first sample row g0 (near, table)
-    int *wgc = wg + K;                                       // K: nearest sample row g_c (near, table)
+    float2 *wfd = wrho + K;                                  // K: far prefactor, double-float
+    int *wR = reinterpret_cast<int *>(wfd + 2 * K);          // K: far terms R | R1 << 16, 0 = near
     float4 *ph4 = reinterpret_cast<float4 *>(reinterpret_cast<char *>(smd) + weights_smem_head(K));
     float4 *sc4 = ph4 + M;   // h: [0] = (S(y), S(y+h)), [j] = (S(y-j) + S(y+j), S(y-j) - S(y+j))
     const int t = blockIdx.x;
@@ -435,8 +540,7 @@ __global__ void __launch_bounds__(256) weights_kernel(
     const int h = M / 2;
     const double tt = T[t];
     const double scale = 2.0 * W / (double)M;
-    if (!tab)   // phases for the direct near sums
-        for (int q = threadIdx.x; q < M; q += blockDim.x) ph4[q] = ph_g[q];
+    for (int q = threadIdx.x; q < M; q += blockDim.x) ph4[q] = ph_g[q];   // phases for the direct near sums
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
         const double y = W * (tt - s[k]) * (1.0 / kPi);
         wy[k] = y;
@@ -444,35 +548,14 @@ __global__ void __launch_bounds__(256) weights_kernel(
             wR[k] = 0;
             const dfl sd = df_split(scale);
             wrho[k] = make_float2(sd.hi, sd.lo);
-            if (tab) {   // samples g0 .. g0 + 41 around y, sin(2 pi y)
-                // offsets from the nearest sample g_c: u_c = y - g_c / 2 is exact in FP64
-                // (|u_c| <= 1/4), so that sin(2 pi u) / u stays accurate as u -> 0
-                const int gc = (int)rint(2.0 * y);
-                const dfl uc = df_split(y - 0.5 * (double)gc);
-                double sn, cs;
-                sincospi(y, &sn, &cs);
-                const dfl s2 = df_split(2.0 * sn * cs);
-                wg[k] = (int)floor(2.0 * y) - (kSincPts / 2 - 1);
-                wgc[k] = gc;
-                wu[k] = make_float2(uc.hi, uc.lo);
-                wfd[k] = make_float2(s2.hi, s2.lo);
-            } else {
-                wf[k] = sinpi(y);
-            }
+            wf[k] = sinpi(y);
         } else {
-            const double sy = sinpi(y);
-            const double a = y / (double)h;
-            const double sq = copysign(sqrt((a - 1.0) * (a + 1.0)), a);
-            const double rho = 1.0 / (a + sq);
-            // truncation from binary32 logarithms (a term count, not a value)
-            const float lr = -logf(fabsf((float)rho));
-            const int R = max(1, min((int)ceilf(48.f * 0.693147181f / lr), kFarTerms));
-            const int R1 = max(1, min((int)ceilf((25.f * 0.693147181f + logf((float)R)) / lr), R));
+            double rho, f;
+            int R, R1;
+            far_window(y, h, scale, rho, f, R, R1);
             wR[k] = R | (R1 << 16);
-            const dfl rr = df_split(rho);
+            const dfl rr = df_split(rho), fd = df_split(f);
             wrho[k] = make_float2(rr.hi, rr.lo);
-            wf[k] = scale * sy * 2.0 / (kPi * (double)h * sq);
-            const dfl fd = df_split(wf[k]);
             wfd[k] = make_float2(fd.hi, fd.lo);
         }
     }
@@ -482,45 +565,7 @@ __global__ void __launch_bounds__(256) weights_kernel(
     for (int k = 0; k < K; ++k) {
         const int R = wR[k] & 0xffff, R1 = wR[k] >> 16;
         dfl dr = {0.f, 0.f}, di = {0.f, 0.f};
-        if (R == 0 && tab) {          // near window, sampled (the same branch in the whole CTA)
-            const int g0 = wg[k];
-            __syncthreads();          // previous window's weights read
-            if (threadIdx.x < kSincPts) {
-                // sinc(2u) E(u) at u = y - g/2 = u_c + (g_c - g)/2 in double-float:
-                // sin(2 pi u) = (-1)^g sin(2 pi y), E(u) = exp((beta/U) sqrt(U^2 - u^2) - beta)
-                const int i = (int)threadIdx.x;
-                const float2 uc2 = wu[k];
-                const dfl u = df_addq({uc2.x, uc2.y}, {0.5f * (float)(wgc[k] - g0 - i), 0.f});
-                dfl w = {1.f, 0.f};
-                if (u.hi != 0.f || u.lo != 0.f) {
-                    const dfl w2 = df_addq({(float)(kSincU * kSincU), 0.f}, df_negq(df_mulq(u, u)));
-                    w = {0.f, 0.f};
-                    if (w2.hi > 0.f) {
-                        const dfl arg = df_addq(df_mulq(df_sqrtq(w2), {kBetaUHi, kBetaULo}),
-                                                {(float)-kSincBeta, 0.f});
-                        const float2 s22 = wfd[k];
-                        const dfl s2 = ((g0 + i) & 1) ? dfl{-s22.x, -s22.y} : dfl{s22.x, s22.y};
-                        w = df_mulq(df_mulq(s2, df_expq(arg)), df_rcpq(df_mulq(u, {k2PiHi, k2PiLo})));
-                    }
-                }
-                swt[i] = make_float2(w.hi, w.lo);
-            }
-            __syncthreads();
-            if (p < J) {
-                const float4 *col = tab + (long long)(g0 + G) * J + p;
-                float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-#pragma unroll 6
-                for (int i = 0; i < kSincPts; ++i) {
-                    const float4 v = col[(long long)i * J];
-                    const float2 w = swt[i];
-                    df_mac(rh, rl, {w.x, w.y}, {v.x, v.y});
-                    df_mac(ih, il, {w.x, w.y}, {v.z, v.w});
-                }
-                const float2 sd = wrho[k];   // 2W/M
-                dr = df_mulq({rh, rl}, {sd.x, sd.y});
-                di = df_mulq({ih, il}, {sd.x, sd.y});
-            }
-        } else if (R == 0) {          // near window, direct sums
+        if (R == 0) {          // near window (the same branch in the whole CTA)
             float rh, rl, ih, il;
             near_sum(wy[k], df_split(wf[k] * (1.0 / kPi)), h, M, p, J, ph4, sc4, rh, rl, ih, il);
             if (p < J) {
@@ -535,13 +580,13 @@ __global__ void __launch_bounds__(256) weights_kernel(
             for (int r = R - 1; r >= R1; --r) {     // FP32 tail
                 const float4 v = nu_f[(long long)r * J + p];
                 ah = fmaf(ah, rho.hi, v.x);
-                bh = fmaf(bh, rho.hi, v.z);
+                bh = fmaf(bh, rho.hi, v.y);
             }
             float al = 0.f, bl = 0.f;
             for (int r = R1 - 1; r >= 0; --r) {
                 const float4 v = nu_f[(long long)r * J + p];
-                df_horner(ah, al, rho, v.x, v.y);
-                df_horner(bh, bl, rho, v.z, v.w);
+                df_horner(ah, al, rho, v.x, v.z);
+                df_horner(bh, bl, rho, v.y, v.w);
             }
             const float2 f2 = wfd[k];
             const dfl f = {f2.x, f2.y};
@@ -566,27 +611,7 @@ __global__ void __launch_bounds__(256) weights_kernel(
             df_mac(qih, qil, bi, dr);
         }
     }
-    if (p < J) {   // G = (mu_p / 2 pi) q, mu_p / 2 pi = 1/(2 pi) or 1/pi, in double-float
-        const bool edge = p == 0 || p == J - 1;
-        const dfl c = edge ? dfl{kInv2PiHi, kInv2PiLo} : dfl{2.f * kInv2PiHi, 2.f * kInv2PiLo};
-        const dfl a = df_mulq({qrh, qrl}, c), b = df_negq(df_mulq({qih, qil}, c));
-        if (Gs) {
-            Gs[(long long)p * pitch_T + t] = make_float2(a.hi, a.lo);
-            Gs[(long long)(J + p) * pitch_T + t] = make_float2(b.hi, b.lo);
-        } else {
-            Gr[(long long)p * n_T + t] = (double)a.hi + (double)a.lo;
-            Gm[(long long)p * n_T + t] = (double)b.hi + (double)b.lo;
-        }
-    }
-}
-
-// Split a complex FP64 table into double-float pairs (re hi, re lo, im hi, im lo).
-__global__ void split_df_kernel(const double2 *__restrict__ B, float4 *__restrict__ Bf, long long n) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double2 b = B[i];
-    const dfl r = df_split(b.x), m = df_split(b.y);
-    Bf[i] = make_float4(r.hi, r.lo, m.hi, m.lo);
+    if (p < J) store_weight(J, p, t, n_T, pitch_T, {qrh, qrl}, {qih, qil}, Gr, Gm, Gs);
 }
 
 constexpr int BM = 64, BN = 64, BK = 16;
@@ -802,21 +827,20 @@ size_t synth_weights_smem(int J, int K, bool table) {
 }
 
 void launch_synth_weights(int J, int M, double W, int K, const double *s, const double2 *B,
-                          float4 *Bf, const float4 *nu_f, const float4 *phase_tab,
+                          const float4 *Bf, const float4 *nu_f, const float4 *phase_tab,
                           const float4 *sinc_tab, const double *T, int n_T, double *Gr, double *Gm,
                           float2 *Gs, cudaStream_t st) {
     if (n_T <= 0) return;
-    const size_t smem = synth_weights_smem(J, K, sinc_tab != nullptr);
+    if (sinc_tab) {
+        weights_tab_kernel<<<dim3(n_T, (J + 2 * kWCols - 1) / (2 * kWCols)), kWGroups * kWCols, 0, st>>>(
+            J, M, W, K, s, Bf, nu_f, sinc_tab, sinc_tab_half(J), T, n_T, Gr, Gm, Gs, synth_pitch(n_T));
+        return;
+    }
+    const size_t smem = synth_weights_smem(J, K, false);
     static std::atomic<unsigned long long> attr{0};
     ensure_smem_attr((const void *)weights_kernel, (int)kWeightsMaxSmem, attr);
-    if (Bf) {
-        const long long n = (long long)K * J;
-        split_df_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(B, Bf, n);
-    }
-    dim3 grid(n_T, (J + 255) / 256);
-    weights_kernel<<<grid, 256, smem, st>>>(J, M, W, K, s, B, Bf, nu_f, phase_tab, sinc_tab,
-                                            sinc_tab ? sinc_tab_half(J) : 0, T, n_T, Gr, Gm, Gs,
-                                            synth_pitch(n_T));
+    weights_kernel<<<dim3(n_T, (J + 255) / 256), 256, smem, st>>>(J, M, W, K, s, B, Bf, nu_f, phase_tab, T, n_T, Gr, Gm,
+                                                                 Gs, synth_pitch(n_T));
 }
 
 void launch_synth_contract(int J, int n_x, int n_T, const double2 *V, const double *Gr,

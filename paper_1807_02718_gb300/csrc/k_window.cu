@@ -49,7 +49,7 @@ constexpr int kChunk = 1024;
 __global__ void __launch_bounds__(256) spectra_kernel(const double *__restrict__ wa, int Q,
                                                       double dt, double H, int K, int J,
                                                       const double *__restrict__ omega,
-                                                      double2 *__restrict__ B) {
+                                                      double2 *__restrict__ B, float4 *__restrict__ Bf) {
     const int j = blockIdx.x;
     const double w = omega[j];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -96,7 +96,12 @@ __global__ void __launch_bounds__(256) spectra_kernel(const double *__restrict__
                 si[s] += __shfl_down_sync(0xffffffffu, si[s], o);
             }
             const int k = kb + warp + 8 * s;
-            if (lane == 0 && k < K) B[(long long)k * J + j] = make_double2(dt * sr[s], dt * si[s]);
+            if (lane == 0 && k < K) {
+                const double2 b = make_double2(dt * sr[s], dt * si[s]);
+                const float rh = (float)b.x, ih = (float)b.y;   // double-float copy for the synthesis weights
+                B[(long long)k * J + j] = b;
+                Bf[(long long)k * J + j] = make_float4(rh, (float)(b.x - (double)rh), ih, (float)(b.y - (double)ih));
+            }
         }
     }
 }
@@ -105,11 +110,11 @@ __global__ void __launch_bounds__(256) spectra_kernel(const double *__restrict__
 
 void launch_window_spectra(const double *a, int n_samples, long long start0, long long step,
                            int Q, double dt, double H, int K, int J, const double *omega,
-                           double *wa, double2 *B, cudaStream_t st) {
+                           double *wa, double2 *B, float4 *Bf, cudaStream_t st) {
     if (K <= 0 || J <= 0) return;
     dim3 g1((Q + 1 + 255) / 256, K);
     windowed_samples_kernel<<<g1, 256, 0, st>>>(a, n_samples, start0, step, Q, dt, H, wa);
-    spectra_kernel<<<J, 256, 0, st>>>(wa, Q, dt, H, K, J, omega, B);
+    spectra_kernel<<<J, 256, 0, st>>>(wa, Q, dt, H, K, J, omega, B, Bf);
 }
 
 }  // namespace fh
