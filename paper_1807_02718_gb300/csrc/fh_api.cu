@@ -799,12 +799,16 @@ fh_status spectra_common(fh_ctx *ctx, Problem &pb, const double *d_a, int n_samp
 bool use_contract_tc(const fh_ctx *ctx, const Problem &pb) {
     return ctx->precision != FH_FP64 && ctx->tune.contract_tc && fh::contract_tc_ok(pb.J);
 }
+// ... unless the sums are so few that plain FP64 FMAs beat its five launches.
+bool use_contract_small(const fh_ctx *ctx, const Problem &pb, int n_x, int n_T) {
+    return use_contract_tc(ctx, pb) && fh::contract_small(pb.J, n_x, n_T);
+}
 
 fh_status synth_buffers(fh_ctx *ctx, Problem &pb, int n_x, int n_T) {
     if (ctx->precision == FH_FP64 || use_contract_tc(ctx, pb)) {
         FH_TRY(ensure(ctx, ctx->d_Gr, (size_t)pb.J * n_T * sizeof(double)));
         FH_TRY(ensure(ctx, ctx->d_Gm, (size_t)pb.J * n_T * sizeof(double)));
-        if (ctx->precision != FH_FP64) {
+        if (ctx->precision != FH_FP64 && !use_contract_small(ctx, pb, n_x, n_T)) {
             FH_TRY(ensure(ctx, ctx->d_ctc, fh::contract_tc_scratch_bytes(pb.J, n_x, n_T)));
             FH_TRY(ensure(ctx, ctx->d_ctc_err, sizeof(int)));
         }
@@ -841,10 +845,10 @@ fh_status weights_kernels(fh_ctx *ctx, Problem &pb, const double *d_T, int n_T) 
 }
 
 fh_status contract_kernels(fh_ctx *ctx, Problem &pb, int n_x, int n_T, double *d_u) {
-    const bool tcc = use_contract_tc(ctx, pb);
+    const bool tcc = use_contract_tc(ctx, pb), small = use_contract_small(ctx, pb, n_x, n_T);
     const bool mixed = ctx->precision != FH_FP64 && !tcc;
-    PhaseScope ps(ctx, FH_PH_CONTRACT, tcc ? 5 : mixed ? 2 : 1);
-    if (tcc) {
+    PhaseScope ps(ctx, FH_PH_CONTRACT, small ? 1 : tcc ? 5 : mixed ? 2 : 1);
+    if (tcc && !small) {
         FH_CUDA(ctx, cudaMemsetAsync(ctx->d_ctc_err.p, 0, sizeof(int), ctx->stream));
         const cudaError_t e = fh::launch_contract_tc(pb.J, n_x, n_T, ctx->d_V.as<double2>(),
                                                      ctx->d_Gr.as<double>(), ctx->d_Gm.as<double>(), d_u,

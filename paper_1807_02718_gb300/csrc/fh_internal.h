@@ -245,7 +245,9 @@ inline long long sinc_tab_entries(int J) {
     return G ? (2LL * G + 1) * J : 0;
 }
 void launch_sinc_table(int J, int M, const float4 *phase_tab, float4 *tab, cudaStream_t st);
-// FP64 contraction u = [Vr | Vi] [Gr ; Gm] (FP64 FMAs).
+// FP64 contraction u = [Vr | Vi] [Gr ; Gm] (FP64 FMAs).  contract_small: the
+// products are so few that this beats the tensor-core contraction's launches.
+inline bool contract_small(int J, int n_x, int n_T) { return 2LL * J * n_x * n_T <= (1LL << 24); }
 void launch_synth_contract(int J, int n_x, int n_T, const double2 *V, const double *Gr,
                            const double *Gm, double *u, cudaStream_t st);
 // Tensor-core contraction (mixed-precision paths, 2J <= kContractTcMaxK): the

@@ -617,21 +617,27 @@ __global__ void __launch_bounds__(256) weights_kernel(
 constexpr int BM = 64, BN = 64, BK = 16;
 
 // u[x][t] = sum_{kk < 2J} A[x][kk] Bm[kk][t], A = [Vr | Vi], Bm = [Gr ; Gm].
+// kTile x kTile outputs per CTA, (kTile / 16)^2 per thread.  Bound by the FP64
+// pipe (1.19 of 1.05 TFLOP/s measured by FMA chains at 1024 x 4096, 2J = 512), so
+// what matters is that every SM has a tile: tiles of 32 where tiles of 64 are
+// fewer than two per SM (333 x 1001, 2J = 402: 96 tiles, 0.50 ms).
+template <int kTile>
 __global__ void __launch_bounds__(256) contract_kernel(int J, int n_x, int n_T,
                                                        const double2 *__restrict__ V,
                                                        const double *__restrict__ Gr,
                                                        const double *__restrict__ Gm,
                                                        double *__restrict__ u) {
-    __shared__ double As[BK][BM];
-    __shared__ double Bs[BK][BN + 2];
-    const int x0 = blockIdx.y * BM, t0 = blockIdx.x * BN;
+    constexpr int kPer = kTile / 16;
+    __shared__ double As[BK][kTile];
+    __shared__ double Bs[BK][kTile + 2];
+    const int x0 = blockIdx.y * kTile, t0 = blockIdx.x * kTile;
     const int tid = threadIdx.x;
     const int tx = tid & 15, ty = tid >> 4;
-    double acc[4][4] = {};
+    double acc[kPer][kPer] = {};
     const int K2 = 2 * J;
     for (int k0 = 0; k0 < K2; k0 += BK) {
-        for (int e = tid; e < BK * BM; e += 256) {
-            const int kk = e / BM, xx = e % BM;
+        for (int e = tid; e < BK * kTile; e += 256) {
+            const int kk = e / kTile, xx = e % kTile;
             const int k = k0 + kk, x = x0 + xx;
             double v = 0.0;
             if (k < K2 && x < n_x) {
@@ -640,8 +646,8 @@ __global__ void __launch_bounds__(256) contract_kernel(int J, int n_x, int n_T,
             }
             As[kk][xx] = v;
         }
-        for (int e = tid; e < BK * BN; e += 256) {
-            const int kk = e / BN, tt = e % BN;
+        for (int e = tid; e < BK * kTile; e += 256) {
+            const int kk = e / kTile, tt = e % kTile;
             const int k = k0 + kk, t = t0 + tt;
             double v = 0.0;
             if (k < K2 && t < n_T) v = (k < J) ? Gr[(long long)k * n_T + t] : Gm[(long long)(k - J) * n_T + t];
@@ -650,27 +656,57 @@ __global__ void __launch_bounds__(256) contract_kernel(int J, int n_x, int n_T,
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
-            double a[4], b[4];
+            double a[kPer], b[kPer];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
+            for (int i = 0; i < kPer; ++i) a[i] = As[kk][ty * kPer + i];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
+            for (int j = 0; j < kPer; ++j) b[j] = Bs[kk][tx * kPer + j];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < kPer; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+                for (int j = 0; j < kPer; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int x = x0 + ty * 4 + i;
+    for (int i = 0; i < kPer; ++i) {
+        const int x = x0 + ty * kPer + i;
         if (x >= n_x) continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int t = t0 + tx * 4 + j;
+        for (int j = 0; j < kPer; ++j) {
+            const int t = t0 + tx * kPer + j;
             if (t < n_T) u[(long long)x * n_T + t] = acc[i][j];
         }
+    }
+}
+
+// The same sums for few outputs (contract_small): CTAs of 8 targets x 16 times,
+// a warp per four times, lane = (target, every fourth frequency), so that a few
+// thousand outputs spread over the chip and nothing is staged.  Measured
+// (GB300): 777 targets x 16 times, 2J = 256: 66 us through the tensor-core
+// contraction's scaling, slicing and product before.
+__global__ void __launch_bounds__(128) contract_small_kernel(int J, int n_x, int n_T, const double2 *__restrict__ V,
+                                                             const double *__restrict__ Gr,
+                                                             const double *__restrict__ Gm, double *__restrict__ u) {
+    const int lane = threadIdx.x & 31, x = blockIdx.x * 8 + (lane & 7);
+    const int t0 = blockIdx.y * 16 + 4 * (threadIdx.x >> 5);
+    if (t0 >= n_T) return;   // whole warps
+    int tt[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) tt[i] = min(t0 + i, n_T - 1);
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+    for (int p = lane >> 3; p < J; p += 4) {
+        const double2 v = x < n_x ? __ldg(V + (long long)p * n_x + x) : make_double2(0.0, 0.0);
+        const double *gr = Gr + (long long)p * n_T, *gm = Gm + (long long)p * n_T;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i] = fma(v.x, __ldg(gr + tt[i]), fma(v.y, __ldg(gm + tt[i]), acc[i]));
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 8);
+        acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
+        if (lane < 8 && x < n_x && t0 + i < n_T) u[(long long)x * n_T + t0 + i] = acc[i];
     }
 }
 
@@ -846,8 +882,14 @@ void launch_synth_weights(int J, int M, double W, int K, const double *s, const 
 void launch_synth_contract(int J, int n_x, int n_T, const double2 *V, const double *Gr,
                            const double *Gm, double *u, cudaStream_t st) {
     if (n_x <= 0 || n_T <= 0) return;
-    dim3 grid((n_T + BN - 1) / BN, (n_x + BM - 1) / BM);
-    contract_kernel<<<grid, 256, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
+    auto tiles = [&](int e) { return dim3((n_T + e - 1) / e, (n_x + e - 1) / e); };
+    const dim3 g64 = tiles(64);
+    if (contract_small(J, n_x, n_T))
+        contract_small_kernel<<<dim3((n_x + 7) / 8, (n_T + 15) / 16), 128, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
+    else if (g64.x * g64.y < 2 * 152)
+        contract_kernel<32><<<tiles(32), 256, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
+    else
+        contract_kernel<64><<<g64, 256, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
 }
 
 void launch_synth_contract_df(int J, int n_x, int n_T, const double2 *V, float2 *Vs,
