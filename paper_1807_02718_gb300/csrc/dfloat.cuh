@@ -297,6 +297,24 @@ __device__ __forceinline__ void df2_acc(float2 &sh, float2 &sl, df2 a, df2 b) { 
     sh = t;
 }
 
+// The same with the low part compensated too: the running sum is (sh, sl, sc),
+// and the product's error with the exact two-sum error of the high part enters
+// sl by a second two-sum.
+__device__ __forceinline__ void df2_acc_c(float2 &sh, float2 &sl, float2 &sc, df2 a, df2 b) {
+    float2 e;
+    const float2 p = p2_prod(a, b, e), t = p2_add(sh, p);
+    const float2 x = p2_add(p2_two_sum_err(sh, p, t), e), u = p2_add(sl, x);
+    sc = p2_add(sc, p2_two_sum_err(sl, x, u));
+    sl = u;
+    sh = t;
+}
+
+// The sum of df2_acc_c, renormalised.
+__device__ __forceinline__ df2 df2_sum3(float2 sh, float2 sl, float2 sc) {
+    const df2 t = df2_quick(sh, sl);
+    return df2_quick(t.h, p2_add(t.l, sc));
+}
+
 // Remainder polynomials of the Hankel form for two functions at a time (which
 // two: PQ0 = P0 with Q0; PP = P0 with P1 and QQ = Q0 with Q1), coefficients
 // interleaved: (c1 c1' c2 c2'), (c3 c3' c4 c4'), (c5 c5' c0.hi c0'.hi), (c0.lo

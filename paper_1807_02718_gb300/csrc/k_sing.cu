@@ -14,7 +14,7 @@
 // the subintervals [mu_{j-1}, mu_j], j = 2..4 (eq. gradedmeshIntRule): the
 // degree-7 interpolant times e^{-iwt} integrated exactly through the
 // Chebyshev moments rho_n(kappa) = int_{-1}^{1} T_n(x) e^{-i kappa x} dx
-// (32-point Gauss-Legendre for |kappa| < 12, the forward three-term
+// (power series, Gauss-Legendre for |kappa| < 12, the forward three-term
 // recurrence above, where it is stable).
 //
 // Everything is linear in the frequency samples, so, as in the periodic
@@ -26,12 +26,29 @@
 // D_p(t') = sum_m K_m(t') E[m][p] with E = (shifted DFT) o (FC extension) and
 // K_m(t') = e^{-i delta t'} 2A sinc((2A/P)(alpha t' - m)), alpha = P / (2 pi);
 // for the singular samples the FCC weights.
+//
+// The L-term sums.  E is a shifted DFT after an extension that is the identity
+// but for the 6 samples at either end, and with i = p - (n-1)/2, r = (n-1)/L
+//   D_p = (2A/L) e^{-i delta t'} [S_i(y) + sum_j Xc[j][p] S_(n+j-(n-1)/2)(y)],
+//   S_i(y) = sum_m sinc(r (y - m)) e^{-2 pi i m i / L},  y = alpha t',
+// the sum over j (the continuation) for the end samples only, i modulo L.  S_i
+// is the periodic synthesis's D_p with the kernel sinc(r .), band-limited to
+// [-r pi, r pi] in y, and S_-i is its conjugate, so for i = 0..h (h = L/2):
+//   |y| < 1.25 h: 42 samples of a table of S_i at the half-integers, built per
+//     call (sinc_interp.cuh);
+//   beyond: sin(pi r (y - m)) split into e^{+-i pi r (y - m)} and the Chebyshev
+//     expansion of 1/(y - m) (k_synth.cu): with F_l(rho) = sum_q rho^q sum_m T_q(m/h)
+//     e^{-2 pi i m l / L} (the far-field table of the periodic path, order L),
+//     S_i = a F_(i+(n-1)/2) + conj(a) F_(i-(n-1)/2).
+// Per (time, window) that is about 500 packed instructions for each of h + 1
+// values in place of L of them for each of n.
 #include <cmath>
 
 #include "dfloat.cuh"
 #include "fc_gram_table.h"
 #include "fh_internal.h"
 #include "scratch.cuh"
+#include "sinc_interp.cuh"
 
 namespace fh {
 namespace {
@@ -39,31 +56,13 @@ namespace {
 constexpr int kSM = 4, kSNq = 8;
 constexpr double kSQ = 9.1;
 constexpr int kNsing = (kSM - 1) * kSNq;
-constexpr int kGl = 32;
+constexpr int kGl = 24;    // Gauss-Legendre nodes, symmetric: the positive half is kept
+constexpr int kMom = 13;   // terms of the moments' power series in kappa^2
 
 __constant__ double c_cheb[kSNq][kSNq];   // interpolant coefficients a_n = sum_c c_cheb[n][c] f_c
-__constant__ double c_glx[kGl], c_glw[kGl];
+__constant__ double c_glx[kGl / 2], c_glw[kGl / 2];
+__constant__ double c_mom[kSNq][kMom];    // int T_n x^q dx / q!, q = 2 m + n mod 2
 __constant__ double c_mu[kSM];
-
-// acc += a * b (or -= when neg) with the low part compensated too: the
-// running sum is (sh, sl, sc), the product's FMA residual and cross terms
-// and the exact two-sum error of the high part enter sl by a second two-sum
-// (the smooth weights' sums cancel strongly).
-__device__ __forceinline__ void df_acc_c(float &sh, float &sl, float &sc, dfv a, dfv b, bool neg) {
-    float p = a.hi * b.hi;
-    float pe = fmaf(a.hi, b.hi, -p);
-    pe = fmaf(a.hi, b.lo, pe);
-    pe = fmaf(a.lo, b.hi, pe);
-    if (neg) { p = -p; pe = -pe; }
-    const float t = sh + p;
-    const float z = t - sh;
-    const float x = ((sh - (t - z)) + (p - z)) + pe;
-    const float u = sl + x;
-    const float w = u - sl;
-    sc += (sl - (u - w)) + (x - w);
-    sl = u;
-    sh = t;
-}
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -74,15 +73,6 @@ __device__ __forceinline__ double2 expi(double th) {
     sincos(th, &s, &c);
     return make_double2(c, s);
 }
-// e^{i pi r} for a rational phase r = num / den, num reduced modulo 2 den in integers
-__device__ __forceinline__ double2 expi_pi_ratio(long long num, long long den) {
-    long long r = num % (2 * den);
-    if (r < 0) r += 2 * den;
-    double s, c;
-    sincospi((double)r / (double)den, &s, &c);
-    return make_double2(c, s);
-}
-
 // Continuation rows: Xc[j * n + p] = d e_j / d f_p (right end blended to
 // zero, plus the left end read backwards, blended and reversed).
 __global__ void fc_rows_kernel(int n, double *__restrict__ Xc) {
@@ -100,156 +90,386 @@ __global__ void fc_rows_kernel(int n, double *__restrict__ Xc) {
     Xc[(long long)j * n + p] = v;
 }
 
-// E[mi * n + p] (mi = m + L/2): coefficient c'_m about the interval centre
-// per unit sample p:  (1/L) e^{i pi m (n-1)/L} sum_l e^{-2 pi i m l / L} X[l][p].
-__global__ void fc_dft_kernel(int n, int L, const double *__restrict__ Xc, float4 *__restrict__ E) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x, mi = blockIdx.y;
-    if (p >= n) return;
-    const long long m = mi - L / 2;
-    double2 acc = expi_pi_ratio(-2 * m * p, L);
-    for (int j = 0; j < kFcC; ++j) {
-        const double w = Xc[(long long)j * n + p];
-        const double2 e = expi_pi_ratio(-2 * m * (n + j), L);
-        acc.x += w * e.x;
-        acc.y += w * e.y;
-    }
-    const double2 sh = expi_pi_ratio(m * (n - 1), L);
-    const double2 r = cmul(acc, sh);
-    E[(long long)mi * n + p] = df_pack(r.x / L, r.y / L);   // double-float pairs for the weights
+// sinc(r v / 2) for integers v, r = num / L: the phase pi num v / (2 L) is reduced in integers.
+__device__ __forceinline__ double sinc_half(int num, int L, long long v) {
+    if (v == 0) return 1.0;
+    const long long k = (long long)num * v;
+    return sinpi((double)(k % (4LL * L)) / (2.0 * L)) * (2.0 * L) / (kPi * (double)k);
 }
 
-// Smooth-piece weights: one CTA per time; for every window the kernel row
-// K_m(t - s_k) goes to shared memory, then each thread forms D_p = sum_m K_m
-// E[m][p] for its samples and accumulates B_k(w_p) D_p.  Rows 0..n-1 of the
-// weight planes: Gr = Re G / pi, Gm = -Im G / pi.  The kernel row (FP64) and
-// E are held as double-float pairs and the L-term sums D_p run in
-// double-float on the FP32 pipe (exact products, compensated two-sum
-// accumulation); B_k D_p and the sum over windows stay FP64.  The pairs'
-// ~2^-48 rounding, amplified like any input rounding by the FC(Gram)
-// continuation, leaves ~1e-10 of u (measured 8.8e-11 on the small kite
-// against 3.8e-11 with FP64 sums), 50x below the split rule's own error.
-__global__ void __launch_bounds__(256) smooth_weights_kernel(
+// Table of S_i(g/2), |g| <= G, i = 0..h: tab[(g + G) hp + i] = (re hi, im hi, re
+// lo, im lo), hp = h + 1.  One CTA per kTabRows rows g >= 0 and 128 columns; m and
+// -m are paired, their sinc sums staged in chunks of kTabChunk for all columns;
+// the rows -g from S_i(-y) = conj S_i(y) + (-1)^i (sinc(r (y - h)) - sinc(r (y + h))).
+constexpr int kTabRows = 4, kTabChunk = 256;
+
+__global__ void __launch_bounds__(128) split_table_kernel(int num, int L, int G, const float4 *__restrict__ ph,
+                                                          float4 *__restrict__ tab) {
+    const int h = L / 2, hp = h + 1, i = blockIdx.y * 128 + threadIdx.x, g0 = kTabRows * blockIdx.x;
+    __shared__ float4 sc[kTabRows][kTabChunk];   // sinc(r (y - m)) +- sinc(r (y + m))
+    float2 ah[kTabRows], al[kTabRows], ac[kTabRows];   // (re, im), compensated
+#pragma unroll
+    for (int q = 0; q < kTabRows; ++q) {
+        const int g = g0 + q;
+        const double e = sinc_half(num, L, g + 2LL * h);
+        const dfv v = df_from(sinc_half(num, L, g) + ((i & 1) ? -e : e));
+        ah[q] = p2(v.hi, 0.f);
+        al[q] = p2(v.lo, 0.f);
+        ac[q] = p2(0.f, 0.f);
+    }
+    int k = 0;   // m i mod L
+    for (int m0 = 1; m0 < h; m0 += kTabChunk) {
+        const int mc = min(kTabChunk, h - m0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < kTabRows * mc; e += 128) {
+            const int q = e / mc, m = m0 + e % mc;
+            const double a = sinc_half(num, L, g0 + q - 2LL * m), b = sinc_half(num, L, g0 + q + 2LL * m);
+            sc[q][e % mc] = df_pack(a + b, a - b);
+        }
+        __syncthreads();
+        if (i < hp)
+            for (int m = 0; m < mc; ++m) {
+                k += i;
+                if (k >= L) k -= L;
+                const float4 e = __ldg(ph + k);   // e^{-2 pi i m i / L}
+#pragma unroll
+                for (int q = 0; q < kTabRows; ++q) {
+                    const float4 v = sc[q][m];
+                    df2_acc_c(ah[q], al[q], ac[q], {p2(e.x, e.z), p2(e.y, e.w)}, {p2(v.x, v.z), p2(v.y, v.w)});
+                }
+            }
+    }
+    if (i >= hp) return;
+#pragma unroll
+    for (int q = 0; q < kTabRows; ++q) {
+        const int g = g0 + q;
+        if (g > G) break;
+        const df2 t = df2_sum3(ah[q], al[q], ac[q]);
+        tab[(long long)(g + G) * hp + i] = make_float4(t.h.x, t.h.y, t.l.x, t.l.y);
+        const double c = sinc_half(num, L, g - 2LL * h) - sinc_half(num, L, g + 2LL * h);
+        const dfv re = df_add(df2_x(t), df_from((i & 1) ? -c : c));
+        if (g > 0) tab[(long long)(G - g) * hp + i] = make_float4(re.hi, -t.h.y, re.lo, -t.l.y);
+    }
+}
+
+// sinc(2u) E(u) of sample row g0 + i in FP64 (as sinc_weight).
+__device__ __forceinline__ double sinc_weight64(double uc, double s2, int gc, int g0, int i) {
+    const double u = uc + 0.5 * (double)(gc - g0 - i);
+    if (u == 0.0) return 1.0;
+    const double x = u * u * (1.0 / (kSincU * kSincU));
+    if (!(x < 1.0)) return 0.0;
+    const double e = exp(-kSincBeta * x / (1.0 + sqrt(1.0 - x)));
+    return (((g0 + i) & 1) ? -s2 : s2) * e / (2.0 * kPi * u);
+}
+
+// What a window contributes at one time (formed in FP64 by one thread).
+struct SplitWindow {
+    int R, R1;           // far terms and those taken in double-float; R = 0: near
+    int g0, gc;          // near: first and nearest sample, y - gc/2 and sin(2 pi y)
+    double uc, s2;
+    dfv rho, ar, ai;     // far: ratio and the factor a
+    dfv cr, ci;          // (2A/L) e^{-i delta t'} / pi
+};
+constexpr int kSplitChunk = 32;   // windows whose constants are held at once
+constexpr int kEdge = 2 * kFcD;   // end samples, whose weights take the continuation
+constexpr int kEdgeItems = kEdge * 32;   // end sample x (31 continuation points, the sample itself)
+constexpr int kSplitThreads = 256, kEdgePer = (kEdgeItems + 127) / 128;
+
+// Smooth-piece weights: one CTA per time.  Per window S_0 .. S_h go to shared
+// memory, then every interior sample adds B_k(w_p) D_p to its sum (shared memory,
+// its thread's own), and every (end sample p, continuation point j) adds B_k(w_p)
+// (2A/L) e^{-i delta t'} S to a sum of its own.  The interpolation weights are
+// FP64, all sums double-float with compensated low parts: the sum over j with Xc (entries up to 6e4 that cancel for smooth
+// fields) is taken once per time, in FP64.  Rows 0..n-1 of the weight planes: Gr =
+// Re G / pi, Gm = -Im G / pi.
+// Measured (GB300; 1024 x 4096 samples, n = 251, 29 windows): 21.0 -> 1.6 ms (L-term
+// double-float sums per sample before); the table takes 0.11 ms per call, the
+// whole synthesis 27.2 -> 6.0 ms (4.0 of it the FP64 contraction).  Error against
+// 64 bits over ten meshes of n = 25..230: 1.4e-12..6.7e-11 -> 4e-13..5.9e-11.
+__global__ void __launch_bounds__(kSplitThreads) smooth_weights_kernel(
     int n, int L, double A, double P, double delta, int K, const double *__restrict__ s,
-    const double2 *__restrict__ B, int J, int j_c, const float4 *__restrict__ E,
-    const double *__restrict__ T, int n_T, double *__restrict__ Gr, double *__restrict__ Gm) {
-    extern __shared__ float4 km[];   // L values (re hi, re lo, im hi, im lo)
-    const int it = blockIdx.x;
+    const double2 *__restrict__ B, int J, int j_c, const double *__restrict__ Xc, const float4 *__restrict__ tab, int G,
+    const float4 *__restrict__ nu, const double *__restrict__ T, int n_T, double *__restrict__ Gr,
+    double *__restrict__ Gm) {
+    extern __shared__ float4 sm[];
+    __shared__ SplitWindow win[kSplitChunk];
+    __shared__ float2 swt[kSincPts];
+    __shared__ double2 edge[kEdgeItems];
+    const int h = L / 2, hp = h + 1, nm = (n - 1) / 2, it = blockIdx.x, tid = threadIdx.x;
+    float4 *Ss = sm, *Fs = sm + hp, *acc = sm + 2 * hp;   // S_i, F_l, G_p: (re hi, im hi, re lo, im lo)
+    float2 *accc = reinterpret_cast<float2 *>(acc + n);   // G_p: third parts
     const double t = T[it];
-    const double alpha = P / (2.0 * kPi), r = 2.0 * A / P;
-    constexpr int kPer = 4;           // samples per thread and pass
-    for (int p0 = 0; p0 < n; p0 += kPer * blockDim.x) {
-        double2 acc[kPer];
-        for (int q = 0; q < kPer; ++q) acc[q] = make_double2(0.0, 0.0);
-        for (int k = 0; k < K; ++k) {
-            const double tp = t - s[k];
-            __syncthreads();
+    for (int p = tid; p < n; p += blockDim.x) {
+        acc[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+        accc[p] = p2(0.f, 0.f);
+    }
+    float2 eh[kEdgePer], el[kEdgePer], ec[kEdgePer];
+#pragma unroll
+    for (int e = 0; e < kEdgePer; ++e) eh[e] = el[e] = ec[e] = p2(0.f, 0.f);
+    const double r = (double)(n - 1) / (double)L;
+    for (int k0 = 0; k0 < K; k0 += kSplitChunk) {
+        __syncthreads();
+        for (int k = tid; k < min(kSplitChunk, K - k0); k += blockDim.x) {
+            SplitWindow w;
+            const double tp = t - s[k0 + k], y = P * tp * (0.5 / kPi), a = y / (double)h;
+            w.R = w.R1 = 0;
+            w.rho = w.ar = w.ai = df_make(0.f, 0.f);
+            w.g0 = w.gc = 0;
+            w.uc = w.s2 = 0.0;
+            if (fabs(a) < 1.25) {
+                w.gc = (int)rint(2.0 * y);
+                w.g0 = (int)floor(2.0 * y) - (kSincPts / 2 - 1);
+                w.uc = y - 0.5 * (double)w.gc;   // exact
+                double sn, cs;
+                sincospi(y, &sn, &cs);
+                w.s2 = 2.0 * sn * cs;
+            } else {
+                const double sq = copysign(sqrt((a - 1.0) * (a + 1.0)), a);
+                const double rho = 1.0 / (a + sq);
+                // truncation from binary32 logarithms (a term count, not a value)
+                const float lr = -logf(fabsf((float)rho));
+                w.R = max(1, min((int)ceilf(48.f * 0.693147181f / lr), kFarTerms));
+                w.R1 = max(1, min((int)ceilf((25.f * 0.693147181f + logf((float)w.R)) / lr), w.R));
+                w.rho = df_from(rho);
+                // a = e^{i pi r y} / (2 i) times 1/(pi r) and the expansion's factor 2/(h s)
+                double sn, cs;
+                sincospi(A * tp * (1.0 / kPi), &sn, &cs);   // r y = A t' / pi
+                const double f = 1.0 / (kPi * r * (double)h * sq);
+                w.ar = df_from(f * sn);
+                w.ai = df_from(-f * cs);
+            }
             const double2 ph = expi(-delta * tp);
-            for (int mi = threadIdx.x; mi < L; mi += blockDim.x) {
-                const double y = r * (alpha * tp - (double)(mi - L / 2));
-                const double sv = y == 0.0 ? 1.0 : sinpi(y) / (kPi * y);
-                km[mi] = df_pack(2.0 * A * sv * ph.x, 2.0 * A * sv * ph.y);
+            const double f = 2.0 * A / ((double)L * kPi);
+            w.cr = df_from(f * ph.x);
+            w.ci = df_from(f * ph.y);
+            win[k] = w;
+        }
+        for (int k = k0; k < min(k0 + kSplitChunk, K); ++k) {
+            __syncthreads();   // the window constants; the previous window's S is used
+            const SplitWindow &w = win[k - k0];
+            if (w.R == 0) {
+                if (tid < kSincPts) {
+                    const dfv v = df_from(sinc_weight64(w.uc, w.s2, w.gc, w.g0, tid));
+                    swt[tid] = p2(v.hi, v.lo);
+                }
+                __syncthreads();
+                const float4 *row = tab + (long long)(w.g0 + G) * hp;
+                for (int i = tid; i < hp; i += blockDim.x) {
+                    float2 sh = p2(0.f, 0.f), sl = sh, sc = sh;
+#pragma unroll 6
+                    for (int q = 0; q < kSincPts; ++q) {
+                        const float4 v = __ldg(row + (long long)q * hp + i);
+                        const float2 wt = swt[q];
+                        df2_acc_c(sh, sl, sc, {p2(wt.x, wt.x), p2(wt.y, wt.y)}, {p2(v.x, v.y), p2(v.z, v.w)});
+                    }
+                    const df2 v = df2_sum3(sh, sl, sc);
+                    Ss[i] = make_float4(v.h.x, v.h.y, v.l.x, v.l.y);
+                }
+            } else {
+                for (int l = tid; l < hp; l += blockDim.x) {   // F_(l + h)
+                    float2 a = p2(0.f, 0.f);
+                    const float2 rh = p2(w.rho.hi, w.rho.hi), rl = p2(w.rho.lo, w.rho.lo);
+                    for (int q = w.R - 1; q >= w.R1; --q) {    // binary32 tail
+                        const float4 v = __ldg(nu + (long long)q * hp + l);
+                        a = p2_fma(a, rh, p2(v.x, v.y));
+                    }
+                    df2 f = {a, p2(0.f, 0.f)};
+                    for (int q = w.R1 - 1; q >= 0; --q) {
+                        const float4 v = __ldg(nu + (long long)q * hp + l);
+                        float2 e;
+                        const float2 p = p2_prod(f, {rh, rl}, e), c = p2(v.x, v.y), x = p2_add(p, c);
+                        f = df2_quick(x, p2_add(p2_two_sum_err(p, c, x), p2_add(e, p2(v.z, v.w))));
+                    }
+                    Fs[l] = make_float4(f.h.x, f.h.y, f.l.x, f.l.y);
+                }
+                __syncthreads();
+                const df2 ar = df2_bcast(w.ar), ai = df2_make(df_neg(w.ai), w.ai);
+                for (int i = tid; i < hp; i += blockDim.x) {
+                    auto F = [&](int l) {   // F_l, 0 <= l < L: F_(h - l) = conj F_(h + l)
+                        const float4 v = Fs[l >= h ? l - h : h - l];
+                        const float sg = l >= h ? 1.f : -1.f;
+                        return df2{p2(v.x, sg * v.y), p2(v.z, sg * v.w)};
+                    };
+                    const df2 u = F(i + nm), v = F(i >= nm ? i - nm : i - nm + L);
+                    // a u + conj(a) v = ar (u + v) + i ai (u - v)
+                    const df2 sum = df2_add(u, v), dif = df2_add(u, {p2_neg(v.h), p2_neg(v.l)});
+                    const df2 S = df2_dot2(ar, sum, ai, df2_swap(dif));
+                    Ss[i] = make_float4(S.h.x, S.h.y, S.l.x, S.l.y);
+                }
             }
             __syncthreads();
-            for (int q = 0; q < kPer; ++q) {
-                const int p = p0 + q * blockDim.x + threadIdx.x;
-                if (p >= n) continue;
-                float rh = 0.f, rl = 0.f, rc = 0.f, ih = 0.f, il = 0.f, ic = 0.f;
-                for (int mi = 0; mi < L; ++mi) {
-                    const float4 e = __ldg(&E[(long long)mi * n + p]);
-                    const float4 kk = km[mi];
-                    const dfv kr = df_make(kk.x, kk.y), ki = df_make(kk.z, kk.w);
-                    const dfv er = df_make(e.x, e.y), ei = df_make(e.z, e.w);
-                    df_acc_c(rh, rl, rc, kr, er, false);   // Re: kr er - ki ei
-                    df_acc_c(rh, rl, rc, ki, ei, true);
-                    df_acc_c(ih, il, ic, kr, ei, false);   // Im: kr ei + ki er
-                    df_acc_c(ih, il, ic, ki, er, false);
-                }
-                const double2 d = make_double2((double)rh + (double)rl + (double)rc,
-                                               (double)ih + (double)il + (double)ic);
-                acc[q] = cadd(acc[q], cmul(B[(long long)k * J + j_c + p], d));
+            auto S = [&](int i) {   // S_i, |i| <= h
+                const float4 v = Ss[i < 0 ? -i : i];
+                const float sg = i < 0 ? -1.f : 1.f;
+                return df2{p2(v.x, sg * v.y), p2(v.z, sg * v.w)};
+            };
+            auto bc = [&](int p) {   // B_k(w_p) (2A/L) e^{-i delta t'} / pi
+                const double2 b = B[(long long)k * J + j_c + p];
+                const dfv br = df_from(b.x), bi = df_from(b.y);
+                return df2_dot2(df2_bcast(br), df2_make(w.cr, w.ci), df2_make(df_neg(bi), bi), df2_make(w.ci, w.cr));
+            };
+            for (int p = kFcD + tid; p < n - kFcD; p += blockDim.x) {
+                const df2 b = bc(p), x = S(p - nm), xs = df2_swap(x);
+                const float4 q = acc[p];
+                float2 gh = p2(q.x, q.y), gl = p2(q.z, q.w), gc = accc[p];
+                df2_acc_c(gh, gl, gc, df2_bcast(df2_x(b)), x);
+                df2_acc_c(gh, gl, gc, df2_make(df_neg(df2_y(b)), df2_y(b)), xs);
+                acc[p] = make_float4(gh.x, gh.y, gl.x, gl.y);
+                accc[p] = gc;
+            }
+#pragma unroll
+            for (int e = 0; e < kEdgePer; ++e) {
+                const int id = tid + e * blockDim.x;
+                if (id >= kEdgeItems) continue;
+                const int pe = id >> 5, j = id & 31, p = pe < kFcD ? pe : n - kEdge + pe;
+                int i = j < kFcC ? n + j - nm : p - nm;
+                if (i > h) i -= L;
+                const df2 b = bc(p), x = S(i), xs = df2_swap(x);
+                df2_acc_c(eh[e], el[e], ec[e], df2_bcast(df2_x(b)), x);
+                df2_acc_c(eh[e], el[e], ec[e], df2_make(df_neg(df2_y(b)), df2_y(b)), xs);
             }
         }
-        for (int q = 0; q < kPer; ++q) {
-            const int p = p0 + q * blockDim.x + threadIdx.x;
-            if (p >= n) continue;
-            Gr[(long long)p * n_T + it] = acc[q].x / kPi;
-            Gm[(long long)p * n_T + it] = -acc[q].y / kPi;
+    }
+#pragma unroll
+    for (int e = 0; e < kEdgePer; ++e) {
+        const int id = tid + e * blockDim.x;
+        if (id < kEdgeItems)
+            edge[id] = make_double2((double)eh[e].x + (double)el[e].x + (double)ec[e].x,
+                                    (double)eh[e].y + (double)el[e].y + (double)ec[e].y);
+    }
+    __syncthreads();
+    for (int p = tid; p < n; p += blockDim.x) {
+        double2 g;
+        if (p < kFcD || p >= n - kFcD) {
+            const double2 *z = edge + 32 * (p < kFcD ? p : p - n + kEdge);
+            g = z[kFcC];
+            for (int j = 0; j < kFcC; ++j) {
+                const double x = Xc[(long long)j * n + p];
+                g.x = fma(x, z[j].x, g.x);
+                g.y = fma(x, z[j].y, g.y);
+            }
+        } else {
+            const float4 q = acc[p];
+            const float2 c = accc[p];
+            g = make_double2((double)q.x + (double)q.z + (double)c.x, (double)q.y + (double)q.w + (double)c.y);
         }
+        Gr[(long long)p * n_T + it] = g.x;
+        Gm[(long long)p * n_T + it] = -g.y;
     }
 }
 
-// Chebyshev moments rho_n(kappa), n < 8.
-__device__ void cheb_moments(double kap, double2 (&rho)[kSNq]) {
-    if (fabs(kap) < 12.0) {
-        for (int q = 0; q < kSNq; ++q) rho[q] = make_double2(0.0, 0.0);
-        for (int g = 0; g < kGl; ++g) {
-            const double x = c_glx[g];
-            const double2 e = expi(-kap * x);
+// Chebyshev moments rho_n(kappa) = int_{-1}^{1} T_n(x) e^{-i kappa x} dx, n < 8: real
+// for even n, imaginary for odd n (rho[n] holds the real or imaginary part).
+//   |kappa| <= 2: their power series (c_mom[n][s] (-1)^s kappa^(2s), times -kappa
+//     for odd n; the remainder is below 3e-17);
+//   |kappa| < 12: 24-point Gauss-Legendre, x and -x together (error below 1e-17);
+//   beyond: the forward three-term recurrence, stable there.
+__device__ void cheb_moments(double kap, double (&rho)[kSNq]) {
+    const double ka = fabs(kap);
+    if (ka <= 2.0) {
+        const double z = -kap * kap;
+#pragma unroll
+        for (int q = 0; q < kSNq; ++q) {
+            double v = c_mom[q][kMom - 1];
+#pragma unroll
+            for (int m = kMom - 2; m >= 0; --m) v = fma(v, z, c_mom[q][m]);
+            rho[q] = (q & 1) ? -kap * v : v;
+        }
+        return;
+    }
+    if (ka < 12.0) {
+#pragma unroll
+        for (int q = 0; q < kSNq; ++q) rho[q] = 0.0;
+        for (int g = 0; g < kGl / 2; ++g) {
+            const double x = c_glx[g], x2 = 2.0 * x;
+            double s, c;
+            sincos(kap * x, &s, &c);
+            c *= c_glw[g];
+            s *= -c_glw[g];
             double t0 = 1.0, t1 = x;
-            for (int q = 0; q < kSNq; ++q) {
-                const double tq = q == 0 ? 1.0 : (q == 1 ? x : 2.0 * x * t1 - t0);
-                if (q >= 2) {
-                    t0 = t1;
-                    t1 = tq;
-                }
-                rho[q].x += c_glw[g] * tq * e.x;
-                rho[q].y += c_glw[g] * tq * e.y;
+#pragma unroll
+            for (int q = 0; q < kSNq; ++q) {   // T_q(x) times the even (cos) or odd (-sin) part
+                rho[q] = fma(t0, (q & 1) ? s : c, rho[q]);
+                const double t2 = fma(x2, t1, -t0);
+                t0 = t1;
+                t1 = t2;
             }
         }
         return;
     }
     double sn, cs;
     sincos(kap, &sn, &cs);
-    rho[0] = make_double2(2.0 * sn / kap, 0.0);
-    rho[1] = make_double2(0.0, -2.0 * (sn - kap * cs) / (kap * kap));
-    const double x2 = 2.0 * ((kap * kap - 2.0) * sn + 2.0 * kap * cs) / (kap * kap * kap);
-    rho[2] = make_double2(2.0 * x2 - rho[0].x, 0.0);
-    const double2 em = make_double2(cs, -sn), ep = make_double2(cs, sn);
+    const double ik = 1.0 / kap;
+    rho[0] = 2.0 * sn * ik;
+    rho[1] = -2.0 * (sn - kap * cs) * ik * ik;
+    const double x2 = 2.0 * ((kap * kap - 2.0) * sn + 2.0 * kap * cs) * ik * ik * ik;
+    rho[2] = 2.0 * x2 - rho[0];
+    // rho_{q+1} = (q+1)/(i kappa) [2 rho_q - (1/(q+1) - 1/(q-1)) sigma] + (q+1)/(q-1) rho_{q-1}, sigma =
+    // e^{-i kappa} - (-1)^(q+1) e^{i kappa} = -2 i sin kappa (q odd) or 2 cos kappa (q even)
+#pragma unroll
     for (int q = 2; q + 1 < kSNq; ++q) {
-        const double sgn = ((q + 1) & 1) ? -1.0 : 1.0;   // (-1)^(q+1)
-        const double2 sig = make_double2(em.x - sgn * ep.x, em.y - sgn * ep.y);
-        const double f = 1.0 / (q + 1) - 1.0 / (q - 1);
-        const double2 br = make_double2(2.0 * rho[q].x - f * sig.x, 2.0 * rho[q].y - f * sig.y);
-        // (q+1)/(i kap) * br = -i (q+1)/kap * br
-        const double a = (double)(q + 1) / kap;
-        rho[q + 1] = make_double2(a * br.y + (double)(q + 1) / (q - 1) * rho[q - 1].x,
-                                  -a * br.x + (double)(q + 1) / (q - 1) * rho[q - 1].y);
+        const double f = 1.0 / (q + 1) - 1.0 / (q - 1), a = (double)(q + 1) * ik, e = (double)(q + 1) / (q - 1);
+        // even q: rho_q real, bracket real b -> -i a b; odd q: bracket i b -> a b
+        rho[q + 1] = (q & 1) ? fma(a, 2.0 * rho[q] + 2.0 * f * sn, e * rho[q - 1])
+                             : fma(-a, 2.0 * rho[q] - 2.0 * f * cs, e * rho[q - 1]);
     }
 }
 
-// Singular-piece weights: one thread per (time, interval of the graded
-// mesh); the interval's eight Clenshaw-Curtis points share its Chebyshev
-// moments and phase, computed once per window.  Rows n .. n+23 of the weight
-// planes (row n + 8 (jv - 1) + c for point c of interval jv).
-__global__ void fcc_weights_kernel(int n, int K, const double *__restrict__ s, const double2 *__restrict__ Bs,
-                                   const double *__restrict__ T, int n_T, double *__restrict__ Gr,
-                                   double *__restrict__ Gm) {
-    const int it = blockIdx.x * blockDim.x + threadIdx.x, jv = blockIdx.y + 1;
-    if (it >= n_T) return;
+// Singular-piece weights: one thread per (time, interval of the graded mesh,
+// every kFccGroups-th window); the interval's eight Clenshaw-Curtis points
+// share its Chebyshev moments and phase, computed once per window, and the
+// window groups' sums are added in order.  Rows n .. n+23 of the weight planes
+// (row n + 8 (jv - 1) + c for point c of interval jv).  Bound by the FP64 pipe:
+// the moments took 32 sincos for |kappa| < 12 before
+// (1.94 -> 0.34 ms at 4096 times, 29 windows).
+constexpr int kFccTimes = 32, kFccGroups = 4;
+
+__global__ void __launch_bounds__(kFccTimes *kFccGroups) fcc_weights_kernel(
+    int n, int K, const double *__restrict__ s, const double2 *__restrict__ Bs, const double *__restrict__ T, int n_T,
+    double *__restrict__ Gr, double *__restrict__ Gm) {
+    __shared__ double2 sums[kFccGroups][kSNq][kFccTimes];
+    const int lane = threadIdx.x % kFccTimes, grp = threadIdx.x / kFccTimes;
+    const int it = blockIdx.x * kFccTimes + lane, jv = blockIdx.y + 1;
     const double a = c_mu[jv - 1], b = c_mu[jv];        // interval [mu_{jv-1}, mu_jv] (0-based c_mu)
     const double h = 0.5 * (b - a), dl = 0.5 * (a + b);
     const int i0 = (jv - 1) * kSNq;
     double2 acc[kSNq];
-    for (int c = 0; c < kSNq; ++c) acc[c] = make_double2(0.0, 0.0);
-    for (int k = 0; k < K; ++k) {
-        const double tp = T[it] - s[k];
-        double2 rho[kSNq];
-        cheb_moments(h * tp, rho);
-        const double2 ph = expi(-dl * tp);
 #pragma unroll
-        for (int c = 0; c < kSNq; ++c) {
-            double2 w = make_double2(0.0, 0.0);
-            for (int q = 0; q < kSNq; ++q) {
-                w.x += c_cheb[q][c] * rho[q].x;
-                w.y += c_cheb[q][c] * rho[q].y;
+    for (int c = 0; c < kSNq; ++c) acc[c] = make_double2(0.0, 0.0);
+    if (it < n_T) {
+        const double t = T[it];
+        for (int k = grp; k < K; k += kFccGroups) {
+            const double tp = t - s[k];
+            double rho[kSNq];
+            cheb_moments(h * tp, rho);
+            double2 ph = expi(-dl * tp);
+            ph.x *= h;
+            ph.y *= h;
+#pragma unroll
+            for (int c = 0; c < kSNq; ++c) {
+                double2 w = make_double2(0.0, 0.0);
+#pragma unroll
+                for (int q = 0; q < kSNq; q += 2) {
+                    w.x = fma(c_cheb[q][c], rho[q], w.x);
+                    w.y = fma(c_cheb[q + 1][c], rho[q + 1], w.y);
+                }
+                w = cmul(w, ph);
+                const double2 bb = Bs[(long long)k * kNsing + i0 + c];
+                acc[c].x = fma(bb.x, w.x, fma(-bb.y, w.y, acc[c].x));
+                acc[c].y = fma(bb.x, w.y, fma(bb.y, w.x, acc[c].y));
             }
-            w = cmul(w, ph);
-            acc[c] = cadd(acc[c], cmul(Bs[(long long)k * kNsing + i0 + c], make_double2(h * w.x, h * w.y)));
         }
     }
-    for (int c = 0; c < kSNq; ++c) {
-        Gr[(long long)(n + i0 + c) * n_T + it] = acc[c].x / kPi;
-        Gm[(long long)(n + i0 + c) * n_T + it] = -acc[c].y / kPi;
+#pragma unroll
+    for (int c = 0; c < kSNq; ++c) sums[grp][c][lane] = acc[c];
+    __syncthreads();
+    for (int e = threadIdx.x; e < kSNq * kFccTimes; e += kFccTimes * kFccGroups) {
+        const int c = e / kFccTimes, l = e % kFccTimes, ti = blockIdx.x * kFccTimes + l;
+        if (ti >= n_T) continue;
+        double2 v = sums[0][c][l];
+        for (int g = 1; g < kFccGroups; ++g) v = cadd(v, sums[g][c][l]);
+        Gr[(long long)(n + i0 + c) * n_T + ti] = v.x / kPi;
+        Gm[(long long)(n + i0 + c) * n_T + ti] = -v.y / kPi;
     }
 }
 
@@ -286,6 +506,24 @@ void gauss_legendre(int n, double *x, double *w) {
     }
 }
 
+// mom[n][m] = int_{-1}^{1} T_n(x) x^q dx / q! with q = 2 m + n mod 2 (extended
+// precision: the monomial terms of T_7 cancel by two digits).
+void cheb_power_moments(double (&mom)[kSNq][kMom]) {
+    long double c[kSNq][kSNq] = {};   // T_n = sum_k c[n][k] x^k
+    c[0][0] = c[1][1] = 1.0L;
+    for (int n = 2; n < kSNq; ++n)
+        for (int k = 0; k < kSNq; ++k) c[n][k] = (k ? 2.0L * c[n - 1][k - 1] : 0.0L) - c[n - 2][k];
+    for (int n = 0; n < kSNq; ++n)
+        for (int m = 0; m < kMom; ++m) {
+            const int q = 2 * m + (n & 1);
+            long double v = 0.0L, f = 1.0L;
+            for (int k = 0; k <= n; ++k)
+                if (!((k + q) & 1)) v += c[n][k] * 2.0L / (k + q + 1);
+            for (int k = 2; k <= q; ++k) f *= k;
+            mom[n][m] = (double)(v / f);
+        }
+}
+
 }  // namespace
 }  // namespace fh
 
@@ -315,7 +553,7 @@ extern "C" fh_status fh_synthesize_sing(int J, double W, int j_c, int K, const d
     const double dw = W / (J - 1), wc = j_c * dw;
     const int L = n + kFcC, ns = n + kNsing;
     // constants of the rule on this stream
-    double cheb[kSNq][kSNq], glx[kGl], glw[kGl], mu[kSM];
+    double cheb[kSNq][kSNq], glx[kGl], glw[kGl], mu[kSM], mom[kSNq][kMom];
     for (int q = 0; q < kSNq; ++q)
         for (int c = 0; c < kSNq; ++c) {
             const double wt = (c == 0 || c == kSNq - 1) ? 0.5 : 1.0;
@@ -324,34 +562,44 @@ extern "C" fh_status fh_synthesize_sing(int J, double W, int j_c, int K, const d
             cheb[q][c] = v;
         }
     gauss_legendre(kGl, glx, glw);
+    for (int g = 0; g < kGl / 2; ++g) glw[g] *= 2.0;   // node x and -x (the first half is positive)
+    cheb_power_moments(mom);
     for (int j = 0; j < kSM; ++j) mu[j] = wc * std::pow((double)(j + 1) / kSM, kSQ);
     if (cudaMemcpyToSymbolAsync(c_cheb, cheb, sizeof cheb, 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyToSymbolAsync(c_glx, glx, sizeof glx, 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyToSymbolAsync(c_glw, glw, sizeof glw, 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+        cudaMemcpyToSymbolAsync(c_glx, glx, sizeof glx / 2, 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+        cudaMemcpyToSymbolAsync(c_glw, glw, sizeof glw / 2, 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+        cudaMemcpyToSymbolAsync(c_mom, mom, sizeof mom, 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyToSymbolAsync(c_mu, mu, sizeof mu, 0, cudaMemcpyHostToDevice, st) != cudaSuccess)
         return FH_ECUDA;
     fh_status status = FH_OK;
     {
         Scratch sc{{}, st};
         double *Xc = sc.get<double>((size_t)kFcC * n);
-        float4 *E = sc.get<float4>((size_t)L * n);   // the FC operator as double-float pairs
+        // half-integer table of S_i, far-field table of order L with its phases and powers
+        const int h = L / 2, hp = h + 1, G = (5 * h + 1) / 2 + 24;
+        float4 *tab = sc.get<float4>((size_t)(2 * G + 1) * hp);
+        float4 *nu = sc.get<float4>((size_t)kFarTerms * hp);
+        float4 *ph = sc.get<float4>((size_t)L);
+        double *pw = sc.get<double>((size_t)L * kFarTerms);
         double2 *Vp = sc.get<double2>((size_t)ns * n_x);
         double *Gr = sc.get<double>((size_t)ns * n_T);
         double *Gm = sc.get<double>((size_t)ns * n_T);
-        if (!Xc || !E || !Vp || !Gr || !Gm) {
+        if (!Xc || !tab || !nu || !ph || !pw || !Vp || !Gr || !Gm) {
             cudaGetLastError();
             return FH_ENOMEM;
         }
         fc_rows_kernel<<<dim3(grid_of(n, 128), kFcC), 128, 0, st>>>(n, Xc);
-        fc_dft_kernel<<<dim3(grid_of(n, 128), L), 128, 0, st>>>(n, L, Xc, E);
+        launch_far_table(hp, L, pw, nullptr, nu, ph, st);
+        split_table_kernel<<<dim3(G / kTabRows + 1, grid_of(hp, 128)), 128, 0, st>>>(n - 1, L, G, ph, tab);
         const double A = 0.5 * (W - wc), P = L * dw, delta = 0.5 * (wc + W);
-        const size_t smem = (size_t)L * sizeof(float4);
-        if (smem > 48 * 1024)
-            cudaFuncSetAttribute(smooth_weights_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        smooth_weights_kernel<<<n_T, 256, smem, st>>>(n, L, A, P, delta, K, d_s,
-                                                      reinterpret_cast<const double2 *>(d_B), J, j_c, E, d_T, n_T,
-                                                      Gr, Gm);
-        fcc_weights_kernel<<<dim3(grid_of(n_T, 64), kSM - 1), 64, 0, st>>>(   // 3 n_T / 64 CTAs
+        const size_t smem = (size_t)(2 * hp + n) * sizeof(float4) + (size_t)n * sizeof(float2);
+        static std::atomic<unsigned long long> attr{0};
+        ensure_smem_attr((const void *)smooth_weights_kernel, 200 * 1024, attr);
+        // as many threads as values S_i (the longest loops), at least 128 for the end samples
+        const int threads = std::min(kSplitThreads, std::max(128, (hp + 31) / 32 * 32));
+        smooth_weights_kernel<<<n_T, threads, smem, st>>>(n, L, A, P, delta, K, d_s, reinterpret_cast<const double2 *>(d_B),
+                                                          J, j_c, Xc, tab, G, nu, d_T, n_T, Gr, Gm);
+        fcc_weights_kernel<<<dim3(grid_of(n_T, kFccTimes), kSM - 1), kFccTimes * kFccGroups, 0, st>>>(
             n, K, d_s, reinterpret_cast<const double2 *>(d_Bs), d_T, n_T, Gr, Gm);
         stack_fields_kernel<<<dim3(grid_of(n_x, 128), ns), 128, 0, st>>>(
             n, n_x, j_c, reinterpret_cast<const double2 *>(d_V), reinterpret_cast<const double2 *>(d_Vs), Vp);
