@@ -413,20 +413,49 @@ __global__ void __launch_bounds__(kThreads, 1) lu_factor_tc_kernel(
                 v[2 * h + 1] = make_float2(t.z, t.w);
             }
         };
-        auto store_row = [&](int i) {
-            float4 *dst = reinterpret_cast<float4 *>(a + (long long)(k0 + i) * n + k0);
+        // The fast path's rows go between global memory and the registers of
+        // their threads through this warp's 8 KiB of the B and C space (idle
+        // between the updates): half a warp per 256-byte row, so that a load
+        // touches four lines and not one per lane; 16-byte pieces exchanged
+        // (piece h of row r at h ^ (r mod 16)) so that neither side has bank
+        // conflicts.
+        float4 *xch = gbuf + warp * (32 * NB / 2);
+        const int frows = nb == NB ? ((m - NB + cs - 1) / cs + 1) & ~1 : 0;   // rows below the block, per CTA
+        const int frow = rank * frows + tid;                                 // this thread's, relative to k0 + NB
+        const bool lrow = tid < frows && frow < m - NB;
+        const int wrow0 = rank * frows + 32 * warp;                          // the warp's first row
+        const int wrows = min(min(frows - 32 * warp, m - NB - wrow0), 32);   // and how many (<= 0: none)
+        const int xr = lane >> 4, xh = lane & 15;
+        auto load_rows = [&](int col) {   // columns col .. col + 31 of the warp's rows into v
+            const float4 *src = reinterpret_cast<const float4 *>(a + (long long)(k0 + NB + wrow0 + xr) * n + col) + xh;
+#pragma unroll 1
+            for (int i0 = 0; i0 < 32; i0 += 16) {
+                float4 t[8];
 #pragma unroll
-            for (int h = 0; h < NB / 2; ++h)
-                if (2 * h < nb) __stcg(dst + h, make_float4(v[2 * h].x, v[2 * h].y, v[2 * h + 1].x, v[2 * h + 1].y));
-        };
-        auto load_first = [&](int i) {   // row k0 + i of the pair's first panel (L21)
-            const float4 *lp = reinterpret_cast<const float4 *>(a + (long long)(k0 + i) * n + (k0 - NB));
+                for (int i = 0; i < 8; ++i, src += n)
+                    t[i] = i0 + 2 * i + xr < wrows ? __ldcg(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) xch[16 * (i0 + 2 * i + xr) + (xh ^ (2 * i + xr))] = t[i];
+            }
+            __syncwarp();
 #pragma unroll
             for (int h = 0; h < NB / 2; ++h) {
-                const float4 t = __ldcg(lp + h);
-                v[2 * h] = make_float2(t.x, t.y);
-                v[2 * h + 1] = make_float2(t.z, t.w);
+                const float4 w = xch[16 * lane + (h ^ xh)];
+                v[2 * h] = make_float2(w.x, w.y);
+                v[2 * h + 1] = make_float2(w.z, w.w);
             }
+            __syncwarp();
+        };
+        auto store_rows = [&](int col) {
+#pragma unroll
+            for (int h = 0; h < NB / 2; ++h)
+                xch[16 * lane + (h ^ xh)] = make_float4(v[2 * h].x, v[2 * h].y, v[2 * h + 1].x, v[2 * h + 1].y);
+            __syncwarp();
+            float4 *dst = reinterpret_cast<float4 *>(a + (long long)(k0 + NB + wrow0 + xr) * n + col) + xh;
+#pragma unroll 4
+            for (int i = 0; i < 16; ++i, dst += n)
+                if (2 * i + xr < wrows) __stcg(dst, xch[16 * (2 * i + xr) + (xh ^ ((2 * i + xr) & 15))]);
+            __syncwarp();
         };
 
         // 1a. Checked fast path.  Partial pivoting keeps the diagonal row
@@ -448,21 +477,19 @@ __global__ void __launch_bounds__(kThreads, 1) lu_factor_tc_kernel(
         // 3 and 4, per-phase clocks of an instrumented copy): 256 k when one
         // warp eliminated the block, a row per lane, and copied its rows to
         // the other CTAs (50 k), when rows belonged to CTAs by 512 (29 k) and
-        // when the write-back waited for the cluster (37 k); 197 k now: load
-        // 13, block 19, rows 14, verdict and staging 8, write-back 13, U12 38,
-        // update 82.  Shared-memory reads bound the rows and U12 (a
+        // when the write-back waited for the cluster (37 k); 197 k with every
+        // thread moving its own row (load 13, write-back 13: a line per lane);
+        // 184 k now: load 5, block 19, rows 15, verdict and staging 5,
+        // write-back 7, U12 40, update 82.  Shared-memory reads bound the rows and U12 (a
         // warp-wide broadcast read takes a cycle per four bytes), so the
         // complex product is four FMAs and one 8-byte read; packed pairs with
         // 16-byte reads were slower (U12 37 -> 54 k).  Factor phase: 38.2 ->
-        // 29.3 ms (BF16, 511 systems of N 64..1920), 1.06 -> 0.88 ms (255, N to
+        // 28.4 ms (BF16, 511 systems of N 64..1920), 1.06 -> 0.82 ms (255, N to
         // 480), 8.9 -> 7.2 ms (TF32, 16 x 127 systems of N 64..832).
         bool fast = false;
-        const int frows = nb == NB ? ((m - NB + cs - 1) / cs + 1) & ~1 : 0;   // rows below the block, per CTA
-        const int frow = rank * frows + tid;                                 // this thread's, relative to k0 + NB
-        const bool lrow = tid < frows && frow < m - NB;
         {
             uint32_t fail = 0u;
-            load_row(lrow, NB + frow);
+            load_rows(k0);
             auto row_step = [&](auto rows_c, const int q0) {
                 constexpr int kRows = decltype(rows_c)::value;
 #pragma unroll
@@ -795,16 +822,19 @@ __global__ void __launch_bounds__(kThreads, 1) lu_factor_tc_kernel(
                     __stcg(reinterpret_cast<float4 *>(a + (long long)(k0 + r) * n + k0 + q), make_float4(e0.x, e0.y, e1.x, e1.y));
                 }
             }
-            if (lrow) {
-                store_row(NB + frow);
-                if (role == 2) {
-                    load_first(NB + frow);
-                    put_a_row<kKind, 2>(atiles, frow / TR, frow % TR, v, 0);
+            if (wrows > 0) {
+                store_rows(k0);
+                if (LT::kPair && role == 2) {
+                    load_rows(k0 - NB);
+                    if (lrow) put_a_row<kKind, 2>(atiles, frow / TR, frow % TR, v, 0);
                 }
             }
         } else {
             if (own) {
-                store_row(mypos);
+                float4 *dst = reinterpret_cast<float4 *>(a + (long long)(k0 + mypos) * n + k0);
+#pragma unroll
+                for (int h = 0; h < NB / 2; ++h)
+                    if (2 * h < nb) __stcg(dst + h, make_float4(v[2 * h].x, v[2 * h].y, v[2 * h + 1].x, v[2 * h + 1].y));
                 if (role != 2) {
                     if (mypos >= nb && nb == NB)
                         put_a_row<kKind, 1>(atiles, (mypos - NB) / TR, (mypos - NB) % TR, v, 0);
@@ -823,7 +853,13 @@ __global__ void __launch_bounds__(kThreads, 1) lu_factor_tc_kernel(
                     // place before the swaps of this panel: into slot 0 of the
                     // two-panel A tiles, or for a pivot row into row mypos of lpq
                     // at every CTA
-                    load_first(myslot);
+                    const float4 *lp = reinterpret_cast<const float4 *>(a + (long long)(k0 + myslot) * n + (k0 - NB));
+#pragma unroll
+                    for (int h = 0; h < NB / 2; ++h) {
+                        const float4 t = __ldcg(lp + h);
+                        v[2 * h] = make_float2(t.x, t.y);
+                        v[2 * h + 1] = make_float2(t.z, t.w);
+                    }
                     if (mypos >= NB) {
                         put_a_row<kKind, 2>(atiles, (mypos - NB) / TR, (mypos - NB) % TR, v, 0);
                     } else {
