@@ -792,25 +792,31 @@ fh_status spectra_common(fh_ctx *ctx, Problem &pb, const double *d_a, int n_samp
     return FH_OK;
 }
 
-// FP64: weight planes Gr, Gm; mixed: the double-float weights Gs and the
-// double-float copy Vs of the target fields (2J rows each, padded pitch).
-// The mixed paths contract on the tensor cores when the schedule asks for it
-// and 2J fits the exact-accumulation bound.
-bool use_contract_tc(const fh_ctx *ctx, const Problem &pb) {
-    return ctx->precision != FH_FP64 && ctx->tune.contract_tc && fh::contract_tc_ok(pb.J);
+// Weights as FP64 planes Gr, Gm (FP64, and the mixed paths when the schedule
+// asks for the tensor-core contraction) or else as the double-float weights Gs
+// beside the double-float copy Vs of the target fields (2J rows each, padded
+// pitch).
+bool use_planes(const fh_ctx *ctx, const Problem &pb) {
+    return ctx->precision == FH_FP64 || (ctx->tune.contract_tc && fh::contract_tc_ok(pb.J));
 }
-// ... unless the sums are so few that plain FP64 FMAs beat its five launches.
-bool use_contract_small(const fh_ctx *ctx, const Problem &pb, int n_x, int n_T) {
-    return use_contract_tc(ctx, pb) && fh::contract_small(pb.J, n_x, n_T);
+// From the planes: on the tensor cores, unless the sums are so few that plain
+// FP64 FMAs beat its five launches.  FP64 contexts ran without
+// the slices' scratch before: they do so still where it is large.
+bool use_contract_tc(const fh_ctx *ctx, const Problem &pb, int n_x, int n_T) {
+    if (!use_planes(ctx, pb) || !ctx->tune.contract_tc) return false;
+    return ctx->precision == FH_FP64 ? fh::contract_slices_fp64(pb.J, n_x, n_T)
+                                     : !fh::contract_small(pb.J, n_x, n_T);
 }
 
 fh_status synth_buffers(fh_ctx *ctx, Problem &pb, int n_x, int n_T) {
-    if (ctx->precision == FH_FP64 || use_contract_tc(ctx, pb)) {
+    if (use_planes(ctx, pb)) {
         FH_TRY(ensure(ctx, ctx->d_Gr, (size_t)pb.J * n_T * sizeof(double)));
         FH_TRY(ensure(ctx, ctx->d_Gm, (size_t)pb.J * n_T * sizeof(double)));
-        if (ctx->precision != FH_FP64 && !use_contract_small(ctx, pb, n_x, n_T)) {
-            FH_TRY(ensure(ctx, ctx->d_ctc, fh::contract_tc_scratch_bytes(pb.J, n_x, n_T)));
+        if (use_contract_tc(ctx, pb, n_x, n_T)) {
             FH_TRY(ensure(ctx, ctx->d_ctc_err, sizeof(int)));
+            const fh_status st = ensure(ctx, ctx->d_ctc, fh::contract_tc_scratch_bytes(pb.J, n_x, n_T));
+            if (st != FH_OK && ctx->precision != FH_FP64) return st;
+            if (st != FH_OK) ctx->err.clear();   // contract_kernels takes the plain FP64 kernel
         }
     } else {
         FH_TRY(ensure(ctx, ctx->d_Gs, (size_t)2 * pb.J * fh::synth_pitch(n_T) * sizeof(float2)));
@@ -829,8 +835,7 @@ struct OnStream {
 
 // Weights G_p(t) (buffers exist); contract_kernels: u = Re sum_p V_p G_p.
 fh_status weights_kernels(fh_ctx *ctx, Problem &pb, const double *d_T, int n_T) {
-    const bool tcc = use_contract_tc(ctx, pb);
-    const bool mixed = ctx->precision != FH_FP64 && !tcc;   // double-float weights and contraction
+    const bool mixed = !use_planes(ctx, pb);   // double-float weights and contraction
     {
         PhaseScope ps(ctx, FH_PH_WEIGHTS, 1);
         fh::launch_synth_weights(pb.J, pb.M, pb.W, pb.K, pb.d_s.as<double>(), pb.d_B.as<double2>(),
@@ -845,10 +850,11 @@ fh_status weights_kernels(fh_ctx *ctx, Problem &pb, const double *d_T, int n_T) 
 }
 
 fh_status contract_kernels(fh_ctx *ctx, Problem &pb, int n_x, int n_T, double *d_u) {
-    const bool tcc = use_contract_tc(ctx, pb), small = use_contract_small(ctx, pb, n_x, n_T);
-    const bool mixed = ctx->precision != FH_FP64 && !tcc;
-    PhaseScope ps(ctx, FH_PH_CONTRACT, small ? 1 : tcc ? 5 : mixed ? 2 : 1);
-    if (tcc && !small) {
+    const bool tcc = use_contract_tc(ctx, pb, n_x, n_T) &&
+                     ctx->d_ctc.cap >= fh::contract_tc_scratch_bytes(pb.J, n_x, n_T);
+    const bool mixed = !use_planes(ctx, pb);
+    PhaseScope ps(ctx, FH_PH_CONTRACT, tcc ? 5 : mixed ? 2 : 1);
+    if (tcc) {
         FH_CUDA(ctx, cudaMemsetAsync(ctx->d_ctc_err.p, 0, sizeof(int), ctx->stream));
         const cudaError_t e = fh::launch_contract_tc(pb.J, n_x, n_T, ctx->d_V.as<double2>(),
                                                      ctx->d_Gr.as<double>(), ctx->d_Gm.as<double>(), d_u,

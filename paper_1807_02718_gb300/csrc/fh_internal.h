@@ -245,20 +245,29 @@ inline long long sinc_tab_entries(int J) {
     return G ? (2LL * G + 1) * J : 0;
 }
 void launch_sinc_table(int J, int M, const float4 *phase_tab, float4 *tab, cudaStream_t st);
-// FP64 contraction u = [Vr | Vi] [Gr ; Gm] (FP64 FMAs).  contract_small: the
-// products are so few that this beats the tensor-core contraction's launches.
+// FP64 contraction u = [Vr | Vi] [Gr ; Gm] (FP64 FMAs).  contract_small: one
+// launch for few products.
 inline bool contract_small(int J, int n_x, int n_T) { return 2LL * J * n_x * n_T <= (1LL << 24); }
 void launch_synth_contract(int J, int n_x, int n_T, const double2 *V, const double *Gr,
                            const double *Gm, double *u, cudaStream_t st);
-// Tensor-core contraction (mixed-precision paths, 2J <= kContractTcMaxK): the
-// operands cut into eight 6-bit slices held exactly in BF16, every slice
-// product summed exactly in FP32 per level over K segments of 512, levels and
-// segments combined in double-float.
-// scratch: contract_tc_scratch_bytes(J, n_x, n_T) bytes; err set if an MMA
-// completion wait gave up.  Six launches.
+// Tensor-core contraction (2J <= kContractTcMaxK): the operands cut into eight
+// 7-bit slices held exactly in BF16, every slice product summed exactly in
+// FP32 per level over K segments of 512, levels joined as integers and summed
+// over the segments in FP64.
+// scratch: contract_tc_scratch_bytes(J, n_x, n_T) bytes; err (may be null) set
+// if an MMA completion wait gave up (the CTA's sums are then taken directly).
+// Five launches.
 constexpr int kContractTcMaxK = 8192;
 bool contract_tc_ok(int J);
 size_t contract_tc_scratch_bytes(int J, int n_x, int n_T);
+// FP64 callers: whether the slices pay (2^25 products, measured plain -> slices:
+// 64..82 -> 46..62 us, 320 -> 130 us for 100 x 330 outputs) and their scratch is
+// small beside the other buffers (the plain kernel has none).
+constexpr size_t kContractTcFp64Scratch = 1ull << 30;
+inline bool contract_slices_fp64(int J, int n_x, int n_T) {
+    return contract_tc_ok(J) && 2LL * J * n_x * n_T > (1LL << 25) &&
+           contract_tc_scratch_bytes(J, n_x, n_T) <= kContractTcFp64Scratch;
+}
 cudaError_t launch_contract_tc(int J, int n_x, int n_T, const double2 *V, const double *Gr,
                                const double *Gm, double *u, void *scratch, int *err, cudaStream_t st);
 int contract_tc_kpad(int J);

@@ -1,49 +1,68 @@
 // Step a7 on the tensor cores: u[x][t] = sum_{kk < 2J} A[x][kk] B[kk][t] with
 // A = [Vr | Vi] and B = [Gr ; Gm] (Sec. 4.1 eq. approx in collapsed form),
-// to FP64-class accuracy through exact BF16 products (an error-free slicing
-// of the operands, the "Ozaki scheme").
+// to FP64 accuracy through exact BF16 products (an error-free slicing of the
+// operands, the "Ozaki scheme").  Every precision contracts here, and so does
+// the split synthesis: the FP64 pipe bounds the plain FP64 kernel.  Measured,
+// plain -> slices (five launches): 1024 x 4096 outputs, 2J = 512 3.62 -> 0.23 ms
+// (MMAs at the measured BF16 rate 0.08 ms; the rest is slicing, 42 MB written
+// and read back, and the FP64 epilogue), 2J = 1024 7.2 -> 0.41 ms, 333 x 1001,
+// 2J = 402 334 -> 75 us.
 //
-// Each row x of A is scaled by a power of two sa_x >= max_kk |A[x][kk]| and
-// cut into kSlices = 8 slices of kSliceBits = 6 bits, A[x][kk] / sa_x =
-// sum_i a_i 2^-(6 (i + 1)) + O(2^-49), a_i integers with |a_i| <= 2^6;
-// likewise each column t of B with sb_t.  Integers of 7 bits are exact in
-// BF16, their products (<= 2^12) are exact in the FP32 accumulator, and a
-// level d = i + j sums at most kSlices pairs over a K segment of kSegK = 512
-// terms below 2^24 (8 x 512 x 2^12 = 2^24), so every level is an exact
-// integer sum: TMEM holds one FP32 accumulator per level (kSlices x 64 = 512
-// columns, all of it).  After each K segment the epilogue combines the
-// levels, scaled by 2^-(kSliceBits (d + 2)), into double-float sums (one per
-// output) and the next segment starts its levels afresh; at the end the sums
-// are multiplied by sa_x sb_t.  The result differs from the exact product by
-// the dropped slice pairs (i + j >= kSlices) and the remainders, ~K 2^-48
-// sa_x sb_t at worst.
+// Scaling.  Term kk is first balanced by a power of two, A[x][kk] 2^d_kk times
+// B[kk][t] 2^-d_kk, so that entries which meet small partners (the fields at
+// frequencies outside the signal's band) do not set the scales: d_kk is half
+// the difference of the exponents of the largest entries of B's row kk and of
+// A's column kk, every target's row of A and time's column of B taken relative
+// to its own largest entry.  Each row x is then scaled by 2^ea_x with ea_x the
+// exponent of its largest entry and cut into kSlices = 8 slices of kSliceBits
+// = 7 bits, A / 2^ea_x = sum_i a_i 2^-(7 (i + 1)) + O(2^-57), a_i integers with
+// |a_0| <= 2^7 and |a_i| <= 2^6; likewise each column t of B.  These integers
+// are exact in BF16 and their products in the FP32 accumulator; a level d =
+// i + j sums at most kSlices pairs over a K segment of kSegK = 512 terms: TMEM
+// holds one FP32 accumulator per level (kSlices x 64 = 512 columns, all of it).
+// Levels stay below 2^24 and exact, except levels 6 and 7 when nearly all 512
+// terms have one sign and both factors within 10 % of their maxima; they then
+// lose units of 2^-56 of a sum of some 2^8 of the same measure.  After each K
+// segment the epilogue joins the levels four by four as 64-bit integers and
+// adds the two to the FP64 sum of the output; at the end the sums take the
+// factor 2^(ea_x + eb_t - 14).  The result differs from the exact product by
+// the dropped slice pairs (i + j >= kSlices) and the remainders, about 2^-58 of
+// max|row| max|column| per term after balancing.  Measured against quadruple
+// precision (relative L2, 64 x 96 outputs, 2J = 80 .. 1024; plain FP64 sums in
+// brackets): random operands 0.7-0.9e-16 (1.7-5.3e-16), Gaussian spectra with
+// sigma of 5 % of the band 0.8-1.4e-16 (1.6-5.0e-16), those against fields that
+// grow by six decades over the band 0.9-1.8e-16 (1.6-4.9e-16).
 //
-// Kernels: ozaki_scale_kernel (the power-of-two scale of each row of A and
-// each column of B), ozaki_slice_kernel (slices in BF16, written directly in
-// the MMA's shared-memory layout: per 128-row (A) or 64-row (B) tile and K
-// chunk of 16, the eight slices' K-major core matrices in one contiguous
-// block), contract_tc_kernel (one CTA per 128 x 64 output tile, warp
+// Rows of A and columns of B with an infinity or NaN, and tiles whose waits
+// gave up, are summed directly in FP64.
+//
+// Kernels: ozaki_scale_kernel (ea, eb; once for the balance and once
+// after it), ozaki_balance_kernel (d_kk), ozaki_slice_kernel (slices in BF16, written directly in the MMA's
+// shared-memory layout: per 128-row (A) or 64-row (B) tile and K chunk of 16,
+// the eight slices' K-major core matrices in one contiguous block; A and B in
+// one launch each), contract_tc_kernel (one CTA per 128 x 64 output tile, warp
 // specialised over a four-stage pipeline: one thread bulk-copies each chunk's
 // A and B blocks (48 KB), one thread issues the kind::f16 MMAs of every slice
 // pair into its level's accumulator, eight epilogue warps combine the levels
 // after each segment; mbarriers with bounded waits hand the stages over).
 #include <cuda_bf16.h>
 
+#include <climits>
+
 #include "fh_internal.h"
-#include "dfloat.cuh"
 #include "tc_gemm.cuh"
 
 namespace fh {
 namespace {
 
 constexpr int kSlices = 8;
-constexpr int kSliceBits = 6;
+constexpr int kSliceBits = 7;
 constexpr int kTM = 128;                 // output rows (x) per CTA = TMEM lanes
 constexpr int kTN = 64;                  // output columns (t) per CTA
 constexpr int kKC = 16;                  // K elements per staged chunk: one MMA K step (32 bytes)
 constexpr int kKBytes = kKC * 2;
 constexpr int kKPad = 64;                // K padding of the slice arrays
-constexpr int kThr = 256;
+constexpr int kThr = 256, kScaleThr = 512;
 constexpr int kASlice = kTM * kKBytes;   // bytes of one A slice chunk (4 KiB)
 constexpr int kBSlice = kTN * kKBytes;   // bytes of one B slice chunk (2 KiB)
 constexpr int kABlock = kSlices * kASlice, kBBlock = kSlices * kBSlice;   // 32 + 16 KiB per chunk
@@ -52,43 +71,113 @@ constexpr int kStages = 4;
 constexpr int kSmem = 1024 + kStages * kStage;
 constexpr int kSegK = 512;                  // K per exact segment
 constexpr int kCtaThreads = 384;            // producer (warp 0), MMA (warp 1), epilogue (warps 4 .. 11)
+constexpr int kOutPitch = 33;               // output tile of an epilogue warp: 32 x 32, padded rows
 constexpr long long kWaitLimit = 1LL << 22;
+constexpr int kZeroExp = INT_MIN / 4;       // exponent of a zero; balance of a term that is zero throughout
+constexpr int kNonFinite = INT_MAX;         // scale of a row or column with an infinity or NaN
+static_assert(8 * 32 * kOutPitch * (int)sizeof(double) <= kStages * kStage, "output tiles fit the stages");
 
 // Element (r, kk) of the operand whose rows are r: A rows are targets x (from
 // V[kk][x] complex, real parts for kk < J, imaginary parts above), B rows are
 // times t (from Gr[kk][t] for kk < J, Gm[kk - J][t] above).
 struct Src {
-    const double2 *V;        // A: V[j * ld + r]
-    const double *G0, *G1;   // B: Gr, Gm [j * ld + r]
-    int J, ld, rows;
+    const double2 *V;        // A: V[j * rows + r]
+    const double *G0, *G1;   // B: Gr, Gm [j * rows + r]
+    int J, rows;
     __device__ __forceinline__ double at(int r, int kk) const {
         if (r >= rows || kk >= 2 * J) return 0.0;
         const int j = kk < J ? kk : kk - J;
         if (V) {
-            const double2 v = V[(long long)j * ld + r];
+            const double2 v = V[(long long)j * rows + r];
             return kk < J ? v.x : v.y;
         }
-        return (kk < J ? G0 : G1)[(long long)j * ld + r];
+        return (kk < J ? G0 : G1)[(long long)j * rows + r];
     }
 };
 
-// e[r] with max_kk |src(r, kk)| < 2^e[r] (0 for a zero row).  A CTA takes 32
-// rows: lane = row (consecutive rows are contiguous in both sources), the
-// eight warps stride over kk, then a shared-memory maximum.
-__global__ void __launch_bounds__(kThr) ozaki_scale_kernel(Src src, int K, int *__restrict__ e) {
-    __shared__ double part[kThr / 32][32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int r = blockIdx.x * 32 + lane;
-    double m = 0.0;
+// e with |v| < 2^e (the least such), kZeroExp for zero, kNonFinite for
+// infinities and NaN; integer operations (the FP64 pipe is the slow one).
+__device__ __forceinline__ int exp_of(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v) & ~(1ull << 63);
+    const int be = (int)(b >> 52);
+    if (be == 0x7FF) return kNonFinite;
+    if (be) return be - 1022;
+    return b ? 64 - __clzll((long long)b) - 1074 : kZeroExp;
+}
+
+// d[j], d[J + j]: the balance of the terms Vr Gr and Vi Gm of frequency j, with
+// ea, eb the exponents of the rows' largest entries (rows with an infinity or
+// NaN take no part).  One CTA per j reads its three rows.
+__global__ void __launch_bounds__(kThr) ozaki_balance_kernel(Src a, Src b, const int *__restrict__ ea,
+                                                             const int *__restrict__ eb, int *__restrict__ d) {
+    __shared__ int part[kThr / 32][4];
+    const int j = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int m[4] = {kZeroExp, kZeroExp, kZeroExp, kZeroExp};   // Vr, Vi, Gr, Gm
+    auto take = [](int &mx, double v, int e0) {
+        const int e = exp_of(v);
+        if (e0 != kNonFinite && e != kZeroExp) mx = max(mx, e - e0);
+    };
+#pragma unroll 4
+    for (int x = threadIdx.x; x < a.rows; x += kThr) {
+        const double2 v = a.V[(long long)j * a.rows + x];
+        const int e0 = ea[x];
+        take(m[0], v.x, e0);
+        take(m[1], v.y, e0);
+    }
+#pragma unroll 4
+    for (int t = threadIdx.x; t < b.rows; t += kThr) {
+        const int e0 = eb[t];
+        take(m[2], b.G0[(long long)j * b.rows + t], e0);
+        take(m[3], b.G1[(long long)j * b.rows + t], e0);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        m[i] = __reduce_max_sync(0xffffffffu, m[i]);
+        if (lane == 0) part[warp][i] = m[i];
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        int ma = kZeroExp, mb = kZeroExp;
+        for (int w = 0; w < kThr / 32; ++w) {
+            ma = max(ma, part[w][threadIdx.x]);
+            mb = max(mb, part[w][2 + threadIdx.x]);
+        }
+        d[threadIdx.x * a.J + j] = ma == kZeroExp || mb == kZeroExp ? kZeroExp : (mb - ma) >> 1;
+    }
+}
+
+// e[r] with max_kk |src(r, kk)| 2^(+-d[kk]) < 2^e[r] (0 for a zero row,
+// kNonFinite with an infinity or NaN); d may be null (no balance).  A CTA
+// takes 32 rows: lane = row (consecutive rows are contiguous in both sources),
+// the sixteen warps stride over the frequencies, two terms each (latency
+// bound), then a shared-memory maximum.  The first actas CTAs take A.
+__global__ void __launch_bounds__(kScaleThr) ozaki_scale_kernel(Src a, Src b, int actas, const int *__restrict__ d,
+                                                                int *__restrict__ ea, int *__restrict__ eb) {
+    __shared__ int part[kScaleThr / 32][32];
+    const bool left = (int)blockIdx.x < actas;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, J = a.J;
+    const int r = (left ? blockIdx.x : blockIdx.x - actas) * 32 + lane, rows = left ? a.rows : b.rows;
+    int m = kZeroExp;
+    auto take = [&](double v, int dk) {
+        const int e = exp_of(v);
+        if (e == kNonFinite) m = kNonFinite;
+        else if (e != kZeroExp && dk != kZeroExp) m = max(m, left ? e + dk : e - dk);
+    };
+    if (r < rows) {
 #pragma unroll 8
-    for (int kk = warp; kk < K; kk += kThr / 32) m = fmax(m, fabs(src.at(r, kk)));
+        for (int j = warp; j < J; j += kScaleThr / 32) {
+            const long long o = (long long)j * rows + r;
+            const double2 v = left ? __ldg(a.V + o) : make_double2(__ldg(b.G0 + o), __ldg(b.G1 + o));
+            take(v.x, d ? __ldg(d + j) : 0);
+            take(v.y, d ? __ldg(d + J + j) : 0);
+        }
+    }
     part[warp][lane] = m;
     __syncthreads();
     if (warp == 0) {
-        for (int w = 1; w < kThr / 32; ++w) m = fmax(m, part[w][lane]);
-        int ex = 0;
-        if (m > 0.0) frexp(m, &ex);   // m = f 2^ex, f in [1/2, 1)
-        e[r] = ex;
+#pragma unroll
+        for (int w = 1; w < kScaleThr / 32; ++w) m = max(m, part[w][lane]);
+        (left ? ea : eb)[r] = m == kZeroExp ? 0 : m;
     }
 }
 
@@ -98,42 +187,49 @@ __global__ void __launch_bounds__(kThr) ozaki_scale_kernel(Src src, int K, int *
 // one after the other, each tr rows of 32 bytes as K-major core matrices
 // (8 rows x 16 bytes; the two 16-byte halves of K 128 bytes apart, 8-row
 // groups 256 bytes apart).
-// In integer arithmetic on the FP64 bit pattern: V = round(src 2^(42 - e[r]))
-// (|V| <= 2^48) = sum_s a_s 2^(42 - 6 s) with balanced digits, each the
-// nearest multiple of the remainder (a_0 in [-64, 64], a_s in [-32, 32]), so
-// that the dropped slice products carry no common sign: src / 2^e[r] =
-// sum_s a_s 2^-(6 (s + 1)) to within 2^-49.
-__global__ void __launch_bounds__(kThr) ozaki_slice_kernel(Src src, const int *__restrict__ e,
-                                                           int kpad, int tr,
-                                                           __nv_bfloat16 *__restrict__ out) {
+// In integer arithmetic on the FP64 bit pattern: V = round(src 2^(+-d[kk] + 56
+// - e[r])) (|V| <= 2^56) = sum_s a_s 2^(49 - 7 s) with balanced digits, each the
+// nearest multiple of the remainder (|a_0| <= 128, |a_s| <= 64), so that the
+// dropped slice products carry no common sign.  The first ablocks blocks of x take A.
+__global__ void __launch_bounds__(kThr) ozaki_slice_kernel(Src sa, Src sb, int ablocks, const int *__restrict__ d,
+                                                           const int *__restrict__ ea, const int *__restrict__ eb,
+                                                           int kpad, __nv_bfloat16 *__restrict__ outa,
+                                                           __nv_bfloat16 *__restrict__ outb) {
     __shared__ __nv_bfloat16 t[kSlices][32][64 + 8];   // [slice][kk][r], padded rows
-    const int r0 = blockIdx.y * 64, k0 = blockIdx.x * 32;
+    const bool left = (int)blockIdx.x < ablocks;
+    const Src src = left ? sa : sb;
+    const int *e = left ? ea : eb;
+    const int r0 = (left ? blockIdx.x : blockIdx.x - ablocks) * 64, k0 = blockIdx.y * 32, tr = left ? kTM : kTN;
     for (int idx = threadIdx.x; idx < 64 * 32; idx += kThr) {
         const int rr = idx & 63, kk = idx >> 6;          // consecutive threads: consecutive rows
-        const int r = r0 + rr;
+        const int r = r0 + rr, er = e[r], dk = k0 + kk < 2 * src.J ? d[k0 + kk] : kZeroExp;
         const unsigned long long bits = (unsigned long long)__double_as_longlong(src.at(r, k0 + kk));
         const int bexp = (int)((bits >> 52) & 0x7FF);
         const unsigned long long mant = (bits & ((1ull << 52) - 1)) | (bexp ? (1ull << 52) : 0ull);
-        // |src| = mant 2^(E), E = bexp - 1075 (1 - 1075 for subnormals); V = mant 2^(E + 42 - e)
-        const int sh = (bexp ? bexp : 1) - 1075 + kSlices * kSliceBits - e[r];   // <= -5
         long long V = 0;
-        if (sh > -64) {
-            const int rs = -sh;
-            V = (long long)((mant + (1ull << (rs - 1))) >> rs);   // round half up on |V|
+        if (er != kNonFinite && dk != kZeroExp && mant) {
+            // |src| = mant 2^(bexp - 1075) (1 - 1075 for subnormals); mant 2^sh <= 2^56 by the choice of e[r]
+            const int sh = (bexp ? bexp : 1) - 1075 + (left ? dk : -dk) + kSlices * kSliceBits - er;
+            if (sh >= 0) V = (long long)(mant << sh);
+            else if (sh > -64) V = (long long)((mant + (1ull << (-sh - 1))) >> -sh);   // round half up on |V|
         }
         if (bits >> 63) V = -V;
+        // two halves of four digits each in 32-bit arithmetic
+        const int vh = (int)((V + (1ll << 27)) >> 28);
+        int v = vh;
 #pragma unroll
         for (int s = 0; s < kSlices; ++s) {
-            const int p = kSliceBits * (kSlices - 1 - s);   // 42, 36, ..., 0
-            const long long a = p ? (V + (1ll << (p - 1))) >> p : V;   // nearest, ties up
-            V -= a << p;                                    // |V| <= 2^(p - 1)
-            t[s][kk][rr] = __float2bfloat16_rn((float)a);   // |a| <= 64: exact
+            if (s == kSlices / 2) v = (int)(V - ((long long)vh << 28));
+            const int p = kSliceBits * (kSlices / 2 - 1 - s % (kSlices / 2));   // 21, 14, 7, 0
+            const int q = p ? (v + (1 << (p - 1))) >> p : v;    // nearest, ties up
+            v -= q << p;                                        // |v| <= 2^(p - 1)
+            t[s][kk][rr] = __float2bfloat16_rn((float)q);       // |q| <= 128: exact
         }
     }
     __syncthreads();
     // 16-byte pieces: 8 consecutive K of one row and slice
     const int nkc = kpad / kKC;
-    uint8_t *ob = reinterpret_cast<uint8_t *>(out);
+    uint8_t *ob = reinterpret_cast<uint8_t *>(left ? outa : outb);
     for (int idx = threadIdx.x; idx < kSlices * 64 * 4; idx += kThr) {
         const int rr = idx & 63, k8 = (idx >> 6) & 3, s = idx >> 8;
         const int r = r0 + rr, kk = k0 + 8 * k8;
@@ -146,9 +242,15 @@ __global__ void __launch_bounds__(kThr) ozaki_slice_kernel(Src src, const int *_
     }
 }
 
+// v 2^k
+__device__ __forceinline__ double scale_pow2(double v, int k) {
+    if (k > 1000 || k < -1000) return ldexp(v, k);
+    return v * __hiloint2double((k + 1023) << 20, 0);
+}
+
 __global__ void __launch_bounds__(kCtaThreads, 1) contract_tc_kernel(
     const uint8_t *__restrict__ As, const uint8_t *__restrict__ Bs, int kpad, const int *__restrict__ ea,
-    const int *__restrict__ eb, int n_x, int n_T, double *__restrict__ u, int *__restrict__ err) {
+    const int *__restrict__ eb, Src sa, Src sb, double *__restrict__ u, int *__restrict__ err) {
     extern __shared__ uint8_t dsm[];
     uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(dsm) + 1023) & ~(uintptr_t)1023);
     __shared__ uint64_t full[kStages], empty[kStages], lv_full, lv_empty;
@@ -172,6 +274,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) contract_tc_kernel(
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t taddr = tslot;
+    double acc[2][16] = {};   // epilogue threads: sums of row 32 (warp % 4) + lane
     const uint8_t *ablk = As + (size_t)blockIdx.y * nkc * kABlock;   // this tile's chunks, in K order
     const uint8_t *bblk = Bs + (size_t)blockIdx.x * nkc * kBBlock;
     if (tid == 0) {
@@ -218,14 +321,8 @@ __global__ void __launch_bounds__(kCtaThreads, 1) contract_tc_kernel(
         }
     } else if (warp >= 4) {
         // epilogue: warp w reads TMEM lanes 32 (w % 4) .. (rows), columns
-        // 32 ((w - 4) / 4) .. of each level; double-float sums across segments
+        // 32 ((w - 4) / 4) .. of each level
         const int q = warp & 3, ch = (warp - 4) >> 2;
-        const int x = x0 + 32 * q + lane;
-        float hi[2][16], lo[2][16];
-#pragma unroll
-        for (int g = 0; g < 2; ++g)
-#pragma unroll
-            for (int c = 0; c < 16; ++c) hi[g][c] = lo[g][c] = 0.f;
         bool ok = true;
         for (int sg = 0; sg < nseg && ok; ++sg) {
             ok = tc::mbar_wait(&lv_full, (uint32_t)(sg & 1), kWaitLimit);
@@ -237,27 +334,24 @@ __global__ void __launch_bounds__(kCtaThreads, 1) contract_tc_kernel(
 #pragma unroll
             for (int g = 0; g < 2; ++g) {
                 const int c0 = 32 * ch + 16 * g;
-                float h2[16], l2[16];
-#pragma unroll
-                for (int c = 0; c < 16; ++c) h2[c] = l2[c] = 0.f;
 #pragma unroll 1
-                for (int d = kSlices - 1; d >= 0; --d) {   // smallest levels first
-                    float v[16];
-                    tc::tmem_ld16(taddr + ((uint32_t)(32 * q) << 16) + (uint32_t)(d * kTN + c0), v);
-                    const float sc = ldexpf(1.f, -kSliceBits * d);   // level d relative to level 0
+                for (int half = 1; half >= 0; --half) {   // the smaller levels first
+                    long long h[16];
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) {          // (h2, l2) += v sc, two-sum
-                        const float p = v[c] * sc;           // exact: integer times a power of two
-                        const float t = h2[c] + p, bb = t - h2[c];
-                        l2[c] += (h2[c] - (t - bb)) + (p - bb);
-                        h2[c] = t;
+                    for (int c = 0; c < 16; ++c) h[c] = 0;
+#pragma unroll 1
+                    for (int d = 0; d < kSlices / 2; ++d) {
+                        float v[16];
+                        tc::tmem_ld16(taddr + ((uint32_t)(32 * q) << 16) +
+                                          (uint32_t)((half * (kSlices / 2) + d) * kTN + c0), v);
+#pragma unroll
+                        for (int c = 0; c < 16; ++c)   // below 2^47 in magnitude: exact in FP64 as well
+                            h[c] = h[c] * (1 << kSliceBits) + __float2int_rn(v[c]);
                     }
-                }
+                    // levels 4 half .. 4 half + 3 relative to level 0
+                    const double sc = half ? 0x1p-49 : 0x1p-21;
 #pragma unroll
-                for (int c = 0; c < 16; ++c) {   // segment sum into the running sum
-                    const dfv r = df_add(df_make(hi[g][c], lo[g][c]), df_make(h2[c], l2[c]));
-                    hi[g][c] = r.hi;
-                    lo[g][c] = r.lo;
+                    for (int c = 0; c < 16; ++c) acc[g][c] = fma((double)h[c], sc, acc[g][c]);
                 }
             }
             tc::tc_fence_before();
@@ -265,18 +359,6 @@ __global__ void __launch_bounds__(kCtaThreads, 1) contract_tc_kernel(
             if (lane == 0) tc::mbar_arrive(&lv_empty);   // the levels may be overwritten
         }
         if (!ok && lane == 0) failed = 1;
-        if (ok && x < n_x) {
-            const int ex = ea[x];
-#pragma unroll
-            for (int g = 0; g < 2; ++g)
-#pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    const int t = t0 + 32 * ch + 16 * g + c;
-                    if (t < n_T)
-                        u[(long long)x * n_T + t] =
-                            ldexp((double)hi[g][c] + (double)lo[g][c], ex + eb[t] - 2 * kSliceBits);
-                }
-        }
     }
     // drain: loads and MMAs in flight have landed before the CTA ends (a
     // no-op unless a wait gave up)
@@ -289,7 +371,35 @@ __global__ void __launch_bounds__(kCtaThreads, 1) contract_tc_kernel(
     }
     tc::tc_fence_before();
     __syncthreads();
-    if (failed && tid == 0) atomicOr(err, 1);
+    if (failed && err && tid == 0) atomicOr(err, 1);
+    if (warp >= 4) {
+        // through shared memory (the stages are idle now), so that rows are
+        // stored 256 bytes at a time
+        const int q = warp & 3, ch = (warp - 4) >> 2;
+        double *tile = reinterpret_cast<double *>(sm) + (warp - 4) * 32 * kOutPitch;
+#pragma unroll
+        for (int g = 0; g < 2; ++g)
+#pragma unroll
+            for (int c = 0; c < 16; ++c) tile[lane * kOutPitch + 16 * g + c] = acc[g][c];
+        __syncwarp();
+        const int t = t0 + 32 * ch + lane, J = sa.J, n_x = sa.rows, n_T = sb.rows;
+        const int et = eb[t], rows = min(32, n_x - (x0 + 32 * q));
+        if (t < n_T)
+            for (int r = 0; r < rows; ++r) {
+                const int x = x0 + 32 * q + r, ex = ea[x];
+                double v;
+                if (failed || ex == kNonFinite || et == kNonFinite) {
+                    v = 0.0;
+                    for (int j = 0; j < J; ++j) v = fma(sa.V[(long long)j * n_x + x].x, sb.G0[(long long)j * n_T + t], v);
+                    for (int j = 0; j < J; ++j) v = fma(sa.V[(long long)j * n_x + x].y, sb.G1[(long long)j * n_T + t], v);
+                } else {
+                    v = scale_pow2(tile[r * kOutPitch + lane], ex + et - 2 * kSliceBits);
+                }
+                u[(long long)x * n_T + t] = v;
+            }
+    }
+    tc::tc_fence_before();
+    __syncthreads();
     if (warp == 0) tc::tmem_free(taddr, 512);
 }
 
@@ -303,7 +413,7 @@ bool contract_tc_ok(int J) { return 2 * J <= kContractTcMaxK; }
 size_t contract_tc_scratch_bytes(int J, int n_x, int n_T) {
     const size_t kp = (size_t)contract_tc_kpad(J);
     const size_t rx = (size_t)contract_tc_rows(n_x), rt = (size_t)contract_tc_cols(n_T);
-    return (size_t)kSlices * (rx + rt) * kp * sizeof(__nv_bfloat16) + (rx + rt) * sizeof(int);
+    return (size_t)kSlices * (rx + rt) * kp * sizeof(__nv_bfloat16) + (rx + rt + kp) * sizeof(int);
 }
 
 cudaError_t launch_contract_tc(int J, int n_x, int n_T, const double2 *V, const double *Gr,
@@ -318,15 +428,14 @@ cudaError_t launch_contract_tc(int J, int n_x, int n_T, const double2 *V, const 
     __nv_bfloat16 *As = static_cast<__nv_bfloat16 *>(scratch);
     __nv_bfloat16 *Bs = As + (size_t)kSlices * rx * kp;
     int *ea = reinterpret_cast<int *>(Bs + (size_t)kSlices * rt * kp);
-    int *eb = ea + rx;
-    const Src sa{V, nullptr, nullptr, J, n_x, n_x};
-    const Src sbt{nullptr, Gr, Gm, J, n_T, n_T};
-    ozaki_scale_kernel<<<rx / 32, kThr, 0, st>>>(sa, 2 * J, ea);
-    ozaki_scale_kernel<<<rt / 32, kThr, 0, st>>>(sbt, 2 * J, eb);
-    ozaki_slice_kernel<<<dim3(kp / 32, rx / 64), kThr, 0, st>>>(sa, ea, kp, kTM, As);
-    ozaki_slice_kernel<<<dim3(kp / 32, rt / 64), kThr, 0, st>>>(sbt, eb, kp, kTN, Bs);
+    int *eb = ea + rx, *d = eb + rt;
+    const Src sa{V, nullptr, nullptr, J, n_x}, sb{nullptr, Gr, Gm, J, n_T};
+    ozaki_scale_kernel<<<(rx + rt) / 32, kScaleThr, 0, st>>>(sa, sb, rx / 32, nullptr, ea, eb);
+    ozaki_balance_kernel<<<J, kThr, 0, st>>>(sa, sb, ea, eb, d);
+    ozaki_scale_kernel<<<(rx + rt) / 32, kScaleThr, 0, st>>>(sa, sb, rx / 32, d, ea, eb);
+    ozaki_slice_kernel<<<dim3((rx + rt) / 64, kp / 32), kThr, 0, st>>>(sa, sb, rx / 64, d, ea, eb, kp, As, Bs);
     contract_tc_kernel<<<dim3(rt / kTN, rx / kTM), kCtaThreads, kSmem, st>>>(
-        reinterpret_cast<const uint8_t *>(As), reinterpret_cast<const uint8_t *>(Bs), kp, ea, eb, n_x, n_T, u, err);
+        reinterpret_cast<const uint8_t *>(As), reinterpret_cast<const uint8_t *>(Bs), kp, ea, eb, sa, sb, u, err);
     return cudaGetLastError();
 }
 

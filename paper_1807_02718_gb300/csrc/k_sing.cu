@@ -184,7 +184,7 @@ constexpr int kSplitThreads = 256, kEdgePer = (kEdgeItems + 127) / 128;
 // Re G / pi, Gm = -Im G / pi.
 // Measured (GB300; 1024 x 4096 samples, n = 251, 29 windows): 21.0 -> 1.6 ms (L-term
 // double-float sums per sample before); the table takes 0.11 ms per call, the
-// whole synthesis 27.2 -> 6.0 ms (4.0 of it the FP64 contraction).  Error against
+// whole synthesis 27.2 -> 6.0 ms (2.4 ms with the contraction on the tensor cores).  Error against
 // 64 bits over ten meshes of n = 25..230: 1.4e-12..6.7e-11 -> 4e-13..5.9e-11.
 __global__ void __launch_bounds__(kSplitThreads) smooth_weights_kernel(
     int n, int L, double A, double P, double delta, int K, const double *__restrict__ s,
@@ -603,7 +603,14 @@ extern "C" fh_status fh_synthesize_sing(int J, double W, int j_c, int K, const d
             n, K, d_s, reinterpret_cast<const double2 *>(d_Bs), d_T, n_T, Gr, Gm);
         stack_fields_kernel<<<dim3(grid_of(n_x, 128), ns), 128, 0, st>>>(
             n, n_x, j_c, reinterpret_cast<const double2 *>(d_V), reinterpret_cast<const double2 *>(d_Vs), Vp);
-        launch_synth_contract(ns, n_x, n_T, Vp, Gr, Gm, d_u, st);
+        unsigned char *slices = contract_slices_fp64(ns, n_x, n_T)
+                                    ? sc.get<unsigned char>(contract_tc_scratch_bytes(ns, n_x, n_T)) : nullptr;
+        if (slices) {
+            if (launch_contract_tc(ns, n_x, n_T, Vp, Gr, Gm, d_u, slices, nullptr, st) != cudaSuccess) status = FH_ECUDA;
+        } else {
+            if (cudaPeekAtLastError() == cudaErrorMemoryAllocation) cudaGetLastError();   // no room for the slices
+            launch_synth_contract(ns, n_x, n_T, Vp, Gr, Gm, d_u, st);
+        }
         if (cudaGetLastError() != cudaSuccess) status = FH_ECUDA;
     }
     return status;
