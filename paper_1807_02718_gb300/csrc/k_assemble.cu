@@ -356,60 +356,61 @@ __global__ void __launch_bounds__(256, 3) assemble_group_df_kernel(
 // matrices of solves list[0 .. gridDim.y - 1] for the mixed paths, in
 // FP64 with the FP64 kernel's formulas: there r is of the order of the node
 // spacing and ln r nearly cancels against the Kress log table.  One thread
-// per entry, so that no warp of assemble_group_df_kernel runs FP64 Bessel
+// per diagonal entry and per node pair (i, i + o), whose Bessel values serve
+// both entries, so that no warp of assemble_group_df_kernel runs FP64 Bessel
 // series for a few lanes.  A32 (may be null): the hi parts, row-major.
+// Bound by the FP64 pipe: 16 x 127 systems of N 64..832 1175 -> 518 us, 511 of
+// N 64..1920 1056 -> 471 us (one thread per entry before).
 __global__ void __launch_bounds__(256) assemble_band_kernel(
     SolveTables t, const int *__restrict__ list, const double2 *__restrict__ z, const double2 *__restrict__ dz,
     const double2 *__restrict__ ddz, const double *__restrict__ kress,
     const double *__restrict__ logsin, float4 *__restrict__ A, float2 *__restrict__ A32, long long out_shift) {
-    constexpr int kW = 2 * kNearBand + 1;
     const int s = list[blockIdx.y];
     const int N = t.N[s];
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= N * kW) return;
-    const int i = e / kW, o = e % kW - kNearBand;
+    if (e >= N * (kNearBand + 1)) return;
+    const int o = e / N, i = e - o * N;   // o = 0: the diagonal (whole warps take one branch)
     int l = i + o;
-    if (l < 0) l += N;
     if (l >= N) l -= N;
-    int d = i - l;
-    if (d < 0) d += N;
     const int vo = t.vec_off[s], to = t.tab_off[t.tab[s]];
     const double kappa = t.kappa[s], et = t.eta[s];
     const double pin = 2.0 * kPi / (double)N;   // pi / n
     const double inv4pi = 1.0 / (4.0 * kPi);
     const double2 zi = z[vo + i], dzi = dz[vo + i];
     const double si = sqrt(dzi.x * dzi.x + dzi.y * dzi.y);
-    const double Rw = kress[to + d];
-    double ar, ai;
-    if (l == i) {
+    auto put = [&](int row, int col, double ar, double ai) {
+        const float4 v = df_pack(ar, ai);
+        A[t.mat_off[s] + out_shift + (long long)col * N + row] = v;
+        if (A32) A32[t.mat_off[s] + out_shift + (long long)row * N + col] = make_float2(v.x, v.z);
+    };
+    if (o == 0) {
+        const double Rw = kress[to];
         const double2 dd = ddz[vo + i];
         const double M1 = -si * inv4pi;
         const double L2r = (dd.x * dzi.y - dd.y * dzi.x) * inv4pi / (si * si);
         const double M2r = (-kEulerGamma / (2.0 * kPi) - log(kappa * si * 0.5) / (2.0 * kPi)) * si;
         const double M2i = 0.25 * si;
-        ar = 0.5 + pin * (L2r + et * M2i);
-        ai = Rw * (-et * M1) + pin * (0.0 - et * M2r);
+        put(i, i, 0.5 + pin * (L2r + et * M2i), Rw * (-et * M1) + pin * (0.0 - et * M2r));
     } else {
-        const double ls = logsin[to + d];
         const double2 zl = z[vo + l], dzl = dz[vo + l];
         const double e1 = zl.x - zi.x, e2 = zl.y - zi.y;
         const double r = sqrt(e1 * e1 + e2 * e2);
         const double sl = sqrt(dzl.x * dzl.x + dzl.y * dzl.y);
-        const double gg = (dzi.y * e1 - dzi.x * e2) * sl / (si * r);
         double J0, Y0, J1, Y1;
         bessel_j0y0j1y1(kappa * r, J0, Y0, J1, Y1);
-        const double Mr = -0.25 * Y0 * sl, Mi = 0.25 * J0 * sl;
-        const double M1 = -J0 * sl * inv4pi;
-        const double M2r = Mr - M1 * ls;
-        const double Lr = -0.25 * kappa * Y1 * gg, Li = 0.25 * kappa * J1 * gg;
-        const double L1 = -kappa * inv4pi * J1 * gg;
-        const double L2r = Lr - L1 * ls;
-        ar = Rw * L1 + pin * (L2r + et * Mi);
-        ai = Rw * (-et * M1) + pin * (Li - et * M2r);
+        // the entry with weights Rw, ls at its index difference, source length s and normal factor gg
+        auto entry = [&](int row, int col, double Rw, double ls, double sc, double gg) {
+            const double Mr = -0.25 * Y0 * sc, Mi = 0.25 * J0 * sc;
+            const double M1 = -J0 * sc * inv4pi;
+            const double M2r = Mr - M1 * ls;
+            const double Lr = -0.25 * kappa * Y1 * gg, Li = 0.25 * kappa * J1 * gg;
+            const double L1 = -kappa * inv4pi * J1 * gg;
+            const double L2r = Lr - L1 * ls;
+            put(row, col, Rw * L1 + pin * (L2r + et * Mi), Rw * (-et * M1) + pin * (Li - et * M2r));
+        };
+        entry(i, l, kress[to + N - o], logsin[to + N - o], sl, (dzi.y * e1 - dzi.x * e2) * sl / (si * r));
+        entry(l, i, kress[to + o], logsin[to + o], si, (dzl.x * e2 - dzl.y * e1) * si / (sl * r));
     }
-    const float4 v = df_pack(ar, ai);
-    A[t.mat_off[s] + out_shift + (long long)l * N + i] = v;
-    if (A32) A32[t.mat_off[s] + out_shift + (long long)i * N + l] = make_float2(v.x, v.z);
 }
 
 // g_i = dB/dn - i eta B = i (kappa p.nu_i - eta) e^{i kappa p.z_i}
@@ -446,7 +447,7 @@ void launch_assemble_groups(const SolveTables &t, const Subgroups &g, int n_grou
     if (n_tiles <= 0 || n_groups <= 0) return;
     if (Af) {
         if (band_count > 0) {
-            const dim3 grid((maxN * (2 * kNearBand + 1) + 255) / 256, band_count);
+            const dim3 grid((maxN * (kNearBand + 1) + 255) / 256, band_count);
             assemble_band_kernel<<<grid, 256, 0, band_st>>>(t, band_list, z, dz, ddz, kress, logsin, Af,
                                                             A32, out_shift);
         }
