@@ -347,11 +347,11 @@ __global__ void __launch_bounds__(64) diag_inverse_kernel(const int2 *__restrict
     }
 }
 
-// Row-major factors (tensor-core LU), blockDim = 512: blocked substitution
+// Row-major factors (tensor-core LU), blockDim = 256 or 512: blocked substitution
 // over 32-row blocks, forward (L) then backward (U).  The last warp forms each
 // diagonal block's values as the product with its precomputed inverse (one
-// warp, no dependent chain).  The other 15 warps own the 32-row chunks w, w +
-// 15, ... and update every active row by its 32-column segment of the block:
+// warp, no dependent chain).  The other nw warps own the 32-row chunks w, w +
+// nw, ... and update every active row by its 32-column segment of the block:
 // eight lanes per row, lane h holding columns 2h, 2h + 1, 16 + 2h, 17 + 2h
 // (two 16-byte loads, so that one warp load covers four rows in four
 // 128-byte lines), then the eight partial sums of a lane group's eight rows
@@ -693,9 +693,15 @@ void launch_lu_refine(bool row_major, const int *order, int S, const int *N,
     if (row_major)
         diag_inverse_kernel<<<n_blocks, 64, 0, st>>>(blocks, N, mat_off, blk_off, LU32, inv);
     refine_setup_kernel<<<S, 256, 0, st>>>(order, N, vec_off, piv, g, x, y32, rs, iters, info);
+    // One CTA of 512 threads fills an SM and waits at two barriers per block of
+    // 32 rows; with several systems per SM to come and few rows each (a warp
+    // takes 32), two of 256 overlap.  Measured refinement, 512 -> 256 threads:
+    // 2032 systems of N <= 832 3.70 -> 3.10 ms, 1016 1.98 -> 1.73, 508 1.07 ->
+    // 1.08; 511 of N <= 1920 7.65 -> 8.09.  The sums are the same, bit for bit.
+    const int rt = S > 4 * 152 && maxN <= 1024 ? 256 : 512;
     for (int it = 1; it <= max_iters; ++it) {
         if (row_major)
-            refine_solve_kernel<true><<<S, 512, (size_t)maxN * sizeof(float2), st>>>(
+            refine_solve_kernel<true><<<S, rt, (size_t)maxN * sizeof(float2), st>>>(
                 order, N, mat_off, vec_off, LU32, inv, blk_off, x, y32, rs, it, tol, iters);
         else
             refine_solve_kernel<false><<<S, 256, (size_t)maxN * sizeof(float2), st>>>(
