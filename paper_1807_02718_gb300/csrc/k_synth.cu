@@ -683,32 +683,47 @@ __global__ void __launch_bounds__(256) contract_kernel(int J, int n_x, int n_T,
 }
 
 // The same sums for few outputs (contract_small): CTAs of 8 targets x 16 times,
-// a warp per four times, lane = (target, every fourth frequency), so that a few
-// thousand outputs spread over the chip and nothing is staged.  Measured
-// (GB300): 777 targets x 16 times, 2J = 256: 66 us through the tensor-core
-// contraction's scaling, slicing and product before.
-__global__ void __launch_bounds__(128) contract_small_kernel(int J, int n_x, int n_T, const double2 *__restrict__ V,
-                                                             const double *__restrict__ Gr,
-                                                             const double *__restrict__ Gm, double *__restrict__ u) {
+// a warp per four times and slice of the frequencies, lane = (target, every
+// fourth frequency of the slice), so that a few thousand outputs spread over
+// the chip and nothing is staged; the slices are summed in order.  With fewer
+// than two CTAs per SM the latency of a lane's loads bounds it: four slices, a
+// quarter of the loads in a row.  Measured (GB300), one slice -> four: 777
+// targets x 16 times, 2J = 256 18.5 -> 12.4 us (66 us through the tensor-core
+// contraction's launches), 30 x 64, 2J = 1024 59.6 -> 37.0 us; 4000 x 16, 2J =
+// 128 (500 CTAs, FP64 pipe) 20.6 -> 24.7 us.
+template <int kSmallSlices>
+__global__ void __launch_bounds__(128 * kSmallSlices) contract_small_kernel(
+    int J, int n_x, int n_T, const double2 *__restrict__ V, const double *__restrict__ Gr,
+    const double *__restrict__ Gm, double *__restrict__ u) {
+    __shared__ double part[kSmallSlices][16][8 + 1];
     const int lane = threadIdx.x & 31, x = blockIdx.x * 8 + (lane & 7);
-    const int t0 = blockIdx.y * 16 + 4 * (threadIdx.x >> 5);
-    if (t0 >= n_T) return;   // whole warps
+    const int tg = (threadIdx.x >> 5) & 3, slice = threadIdx.x >> 7, t0 = blockIdx.y * 16;
     int tt[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) tt[i] = min(t0 + i, n_T - 1);
+    for (int i = 0; i < 4; ++i) tt[i] = min(t0 + 4 * tg + i, n_T - 1);
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    if (t0 + 4 * tg < n_T) {   // whole warps
 #pragma unroll 4
-    for (int p = lane >> 3; p < J; p += 4) {
-        const double2 v = x < n_x ? __ldg(V + (long long)p * n_x + x) : make_double2(0.0, 0.0);
-        const double *gr = Gr + (long long)p * n_T, *gm = Gm + (long long)p * n_T;
+        for (int p = 4 * slice + (lane >> 3); p < J; p += 4 * kSmallSlices) {
+            const double2 v = x < n_x ? __ldg(V + (long long)p * n_x + x) : make_double2(0.0, 0.0);
+            const double *gr = Gr + (long long)p * n_T, *gm = Gm + (long long)p * n_T;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i] = fma(v.x, __ldg(gr + tt[i]), fma(v.y, __ldg(gm + tt[i]), acc[i]));
+            for (int i = 0; i < 4; ++i) acc[i] = fma(v.x, __ldg(gr + tt[i]), fma(v.y, __ldg(gm + tt[i]), acc[i]));
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 8);
+            acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
+            if (lane < 8) part[slice][4 * tg + i][lane] = acc[i];
+        }
     }
+    __syncthreads();
+    const int q = threadIdx.x & 15, r = threadIdx.x >> 4;   // time, target (the first 128 threads)
+    if (r < 8 && blockIdx.x * 8 + r < n_x && t0 + q < n_T) {
+        double v = part[0][q][r];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 8);
-        acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
-        if (lane < 8 && x < n_x && t0 + i < n_T) u[(long long)x * n_T + t0 + i] = acc[i];
+        for (int i = 1; i < kSmallSlices; ++i) v += part[i][q][r];
+        u[(long long)(blockIdx.x * 8 + r) * n_T + t0 + q] = v;
     }
 }
 
@@ -886,9 +901,13 @@ void launch_synth_contract(int J, int n_x, int n_T, const double2 *V, const doub
     if (n_x <= 0 || n_T <= 0) return;
     auto tiles = [&](int e) { return dim3((n_T + e - 1) / e, (n_x + e - 1) / e); };
     const dim3 g64 = tiles(64);
-    if (contract_small(J, n_x, n_T))
-        contract_small_kernel<<<dim3((n_x + 7) / 8, (n_T + 15) / 16), 128, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
-    else if (g64.x * g64.y < 2 * 152)
+    if (contract_small(J, n_x, n_T)) {
+        const dim3 grid((n_x + 7) / 8, (n_T + 15) / 16);
+        if (grid.x * grid.y < 2 * 152)
+            contract_small_kernel<4><<<grid, 4 * 128, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
+        else
+            contract_small_kernel<1><<<grid, 128, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
+    } else if (g64.x * g64.y < 2 * 152)
         contract_kernel<32><<<tiles(32), 256, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
     else
         contract_kernel<64><<<g64, 256, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
