@@ -84,41 +84,48 @@ __device__ __forceinline__ void hankel_pq_r8(double x, double r8, double &P0, do
     }
 }
 
-// Horner form of P0, Q0 (and P1, Q1) for x >= 8 on the intervals of kPQ:
-// the table is staged in shared memory by pq_stage() (threads of a warp may
-// fall into different intervals).
+// Horner form of P0, Q0 (and P1, Q1) for x >= 8 on 32 equal intervals of u =
+// (8/x)^2, five terms each to below 1e-17 (the FP64 pipe bounds the callers, so
+// short polynomials: with six intervals of x they took eight terms; fields of
+// 333 targets and 200 frequencies with their synthesis 1249 -> 1120 us, FP64 kite
+// of 255 systems 28.77 -> 27.93 ms, same errors).  The table
+// is staged in shared memory by pq_stage() (threads of a warp may fall into
+// different intervals).
 struct PQShared {
-    double c[kPQ_NI * 4 * kPQ_TERMS];
-    double uc[kPQ_NI], iuh[kPQ_NI];
+    double2 c[kPU_NI * kPU_TERMS * 2];   // [interval][power of t][(P0, q0), (P1, q1)]
+    double off[kPU_NI];                  // -(2 k + 1)
 };
 
 __device__ __forceinline__ void pq_stage(PQShared &tb) {
-    for (int i = threadIdx.x; i < kPQ_NI * 4 * kPQ_TERMS; i += blockDim.x) tb.c[i] = kPQ[i];
-    for (int i = threadIdx.x; i < kPQ_NI; i += blockDim.x) {
-        tb.uc[i] = kPQ_UC[i];
-        tb.iuh[i] = 1.0 / kPQ_UH[i];
-    }
-}
-
-__device__ __forceinline__ double horner8(const double *c, double t) {
-    double a = c[7];
-#pragma unroll
-    for (int k = 6; k >= 0; --k) a = fma(a, t, c[k]);
-    return a;
+    const double2 *src = reinterpret_cast<const double2 *>(kPU);
+    for (int i = threadIdx.x; i < kPU_NI * kPU_TERMS * 2; i += blockDim.x) tb.c[i] = src[i];
+    for (int i = threadIdx.x; i < kPU_NI; i += blockDim.x) tb.off[i] = -(double)(2 * i + 1);
 }
 
 template <bool want1>
 __device__ __forceinline__ void pq_horner(const PQShared &tb, float xf, double r8, double &P0,
                                           double &Q0, double &P1, double &Q1) {
-    // (the interval from binary32 comparisons: FP64 ones would take five issues of the FP64 pipe)
-    const int k = (xf >= 10.f) + (xf >= 13.f) + (xf >= 18.f) + (xf >= 28.f) + (xf >= 60.f);
-    const double t = (r8 * r8 - tb.uc[k]) * tb.iuh[k];
-    const double *c = tb.c + k * 4 * kPQ_TERMS;
-    P0 = horner8(c, t);
-    Q0 = r8 * horner8(c + kPQ_TERMS, t);
+    // (the interval in binary32: off by one at its ends is as good)
+    const int k = min((int)__fdividef(64.f * kPU_NI, xf * xf), kPU_NI - 1);
+    const double t = fma(r8 * r8, 2.0 * kPU_NI, tb.off[k]);
+    const double2 *c = tb.c + k * kPU_TERMS * 2;
+    double2 a = c[2 * (kPU_TERMS - 1)], b = want1 ? c[2 * (kPU_TERMS - 1) + 1] : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int p = kPU_TERMS - 2; p >= 0; --p) {
+        const double2 v = c[2 * p];
+        a.x = fma(a.x, t, v.x);
+        a.y = fma(a.y, t, v.y);
+        if (want1) {
+            const double2 w = c[2 * p + 1];
+            b.x = fma(b.x, t, w.x);
+            b.y = fma(b.y, t, w.y);
+        }
+    }
+    P0 = a.x;
+    Q0 = r8 * a.y;
     if (want1) {
-        P1 = horner8(c + 2 * kPQ_TERMS, t);
-        Q1 = r8 * horner8(c + 3 * kPQ_TERMS, t);
+        P1 = b.x;
+        Q1 = r8 * b.y;
     }
 }
 

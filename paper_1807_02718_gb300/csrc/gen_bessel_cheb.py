@@ -11,7 +11,8 @@ The device routine (bessel.cuh) evaluates the four functions together:
   x >= 8 (Hankel's asymptotic form, H_nu = sqrt(2/(pi x)) (P_nu + i Q_nu) e^{i chi_nu},
           chi_nu = x - (2 nu + 1) pi/4; variable u = (x0/x)^2 on each piece):
       P0 = B0(t), Q0 = (8/x) B1(t), P1 = B2(t), Q1 = (8/x) B3(t)
-  on the pieces x in [8, 20] and [20, inf).
+  on the pieces x in [8, 20] and [20, inf); the FP64 assembly and field kernels
+  take Horner forms on 32 equal intervals of u = (8/x)^2.
 
 Each function is interpolated at Chebyshev points of the first kind with
 mpmath at 40 digits and its Chebyshev series truncated once the remaining
@@ -135,8 +136,8 @@ def large(x0, x1):
     return [cheb(f) for f in fs], u0
 
 
-PQ_BREAKS = [8, 10, 13, 18, 28, 60]   # x intervals [8,10), ..., [60, inf)
-PQ_TERMS = 8
+PQ_BREAKS = [8, 10, 13, 18, 28, 60]   # x intervals [8,10), ..., [60, inf) of the double-float path
+PU_NI, PU_TERMS = 32, 5               # intervals of u = (8/x)^2 in [0, 1] and terms of the FP64 path
 
 
 def cheb_to_monomial(c):
@@ -158,29 +159,30 @@ def cheb_to_monomial(c):
 
 
 def pq_table():
-    """Horner tables for P0, q0, P1, q1 (Q = (8/x) q) on each x interval, in the
-    variable t = (u - uc)/uh of u = (8/x)^2 mapped to [-1, 1]."""
-    rows, ucs, uhs = [], [], []
+    """Horner tables for P0, q0, P1, q1 (Q = (8/x) q) on each interval k of u, in t = 64 u - (2 k + 1):
+    [interval][power][function]."""
+    out = []
+    for k in range(PU_NI):
+        def x_of(t, k=k):
+            u = (2 * k + 1 + t) / (2 * PU_NI)
+            return 8 / mp.sqrt(u)
+
+        row = []
+        for f in (lambda t: pq(0, x_of(t))[0], lambda t: pq(0, x_of(t))[1] * x_of(t) / 8,
+                  lambda t: pq(1, x_of(t))[0], lambda t: pq(1, x_of(t))[1] * x_of(t) / 8):
+            c = cheb(f, 16)
+            if len(c) > PU_TERMS:
+                raise SystemExit(f"interval {k} of u needs {len(c)} terms")
+            row.append(cheb_to_monomial(c + [mp.mpf(0)] * (PU_TERMS - len(c))))
+        out += [row[f][p] for p in range(PU_TERMS) for f in range(4)]
+    return out
+
+
+def g_intervals():
+    """Centre and half-width in u of the intervals PQ_BREAKS."""
     bounds = PQ_BREAKS + [mp.inf]
-    for x0, x1 in zip(bounds[:-1], bounds[1:]):
-        u_hi = (mp.mpf(8) / x0) ** 2
-        u_lo = mp.mpf(0) if x1 == mp.inf else (mp.mpf(8) / x1) ** 2
-        uc, uh = (u_hi + u_lo) / 2, (u_hi - u_lo) / 2
-
-        def x_of(t, uc=uc, uh=uh):
-            return 8 / mp.sqrt(uc + uh * t)
-
-        fs = [lambda t: pq(0, x_of(t))[0], lambda t: pq(0, x_of(t))[1] * x_of(t) / 8,
-              lambda t: pq(1, x_of(t))[0], lambda t: pq(1, x_of(t))[1] * x_of(t) / 8]
-        for f in fs:
-            c = cheb(f)
-            if len(c) > PQ_TERMS:
-                raise SystemExit(f"interval [{x0},{x1}) needs {len(c)} terms")
-            c = c + [mp.mpf(0)] * (PQ_TERMS - len(c))
-            rows.append(cheb_to_monomial(c))
-        ucs.append(uc)
-        uhs.append(uh)
-    return rows, ucs, uhs
+    us = [((mp.mpf(8) / a) ** 2, mp.mpf(0) if b == mp.inf else (mp.mpf(8) / b) ** 2) for a, b in zip(bounds[:-1], bounds[1:])]
+    return [(h + l) / 2 for h, l in us], [(h - l) / 2 for h, l in us]
 
 
 # Double-float evaluation (mixed-precision paths) writes each function as its
@@ -197,7 +199,7 @@ G_EVAL = 6    # nonzero terms the device sums
 
 
 def g_table():
-    """Horner tables (binary32) of G0..G3 per x interval, variable t as in pq_table."""
+    """Horner tables (binary32) of G0..G3 per x interval, t = (u - uc)/uh."""
     rows = []
     bounds = PQ_BREAKS + [mp.inf]
     for x0, x1 in zip(bounds[:-1], bounds[1:]):
@@ -267,15 +269,14 @@ def main():
         out.append(emit(f"kBLo{k}", c))
     for k, c in enumerate(b_hi):
         out.append(emit(f"kBHi{k}", c))
-    rows, ucs, uhs = pq_table()
-    ni = len(ucs)
-    out.append(f"constexpr int kPQ_NI = {ni};          // x intervals {PQ_BREAKS} .. inf")
-    out.append(f"constexpr int kPQ_TERMS = {PQ_TERMS};")
-    out.append("// Horner coefficients [interval][P0, q0, P1, q1][power of t], t = (u - uc)/uh, u = (8/x)^2")
-    flat = [v for r in rows for v in r]
-    out.append(emit("kPQ", flat))
-    out.append(emit("kPQ_UC", ucs))
-    out.append(emit("kPQ_UH", uhs))
+    ucs, uhs = g_intervals()
+    out.append("// P0, q0, P1, q1 (Q = (8/x) q) at x >= 8: Horner coefficients [interval][power of t][function],")
+    out.append(f"// t = {2 * PU_NI} u - (2 k + 1), u = (8/x)^2, k = floor({PU_NI} u)")
+    out.append(f"constexpr int kPU_NI = {PU_NI}, kPU_TERMS = {PU_TERMS};")
+    pu = [mp.nstr(v, 20, min_fixed=-1, max_fixed=-1) for v in pq_table()]
+    out.append(f"static __device__ const __align__(16) double kPU[{len(pu)}] = {{\n    " +
+               ",\n    ".join(", ".join(pu[i:i + 4]) for i in range(0, len(pu), 4)) + "};")
+    out.append(f"constexpr int kPQ_NI = {len(ucs)};          // double-float path: x intervals {PQ_BREAKS} .. inf")
     out.append("// binary32 remainder polynomials G0..G3 [interval][function][power of t] (double-float path)")
     out.append(f"constexpr int kG_TERMS = {G_TERMS};")
     g_rows = g_table()

@@ -39,7 +39,8 @@ constexpr int kChunk = kFieldChunk;   // largest number of source nodes per work
 // hundred targets made less than three waves of them.  Measured (GB300): 16
 // targets x 63 frequencies, N = 256: 2.60 -> 0.20 ms; 1024 x 255, N 64..480:
 // 8.44 -> 5.61 ms; spectra, fields and synthesis at 333 targets x 1001 times,
-// 200 frequencies: 4.77 -> 1.9 ms.
+// 200 frequencies: 4.77 -> 1.9 ms (1.12 ms with the contraction's and the
+// Hankel polynomials' later changes).
 constexpr int kTileF64 = 16, kSlicesF64 = kTgt / kTileF64;
 
 __global__ void __launch_bounds__(kTgt) field_partial_kernel(

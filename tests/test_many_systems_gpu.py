@@ -53,3 +53,29 @@ def test_many_systems_equal_each_problem_alone(precision):
         assert np.array_equal(F.fh_sample_p(ctx, q, x, T), alone.sample(x, T))
         alone.close()
     F.fh_destroy(ctx)
+
+
+@pytest.mark.parametrize("omega", [0.9, 7.0, 61.0])
+def test_fp64_fields_over_the_argument_range(omega):
+    """FP64 target fields of a random density with kappa r from below 8 to past 1e4, the first and last intervals of
+    the Hankel polynomials among them, against the oracle: 1e-13 of the largest covers 64 sums and phases of 1e4
+    (2^-53 1e4 = 1e-12 at the far targets, whose fields are the smallest)."""
+    N = 64
+    wl = fi.circle_gauss(J=2, W=omega, N=N, n_x=3, n_T=4)
+    rng = np.random.default_rng(3)
+    psi = rng.standard_normal(N) + 1j * rng.standard_normal(N)
+    d = np.concatenate([np.geomspace(7.9, 2e4, 200) / omega, 8.0 / np.sqrt(np.arange(1, 33) / 32.0) / omega])
+    d = 1.5 + d[d > 0.2]
+    x = np.stack([d * np.cos(0.3), d * np.sin(0.3)], axis=1)
+    pr = F.Problem(0, F.FH_FP64)
+    pr.discretize(wl.curve, wl.omega, np.full(2, N, dtype=np.int32), 1.0, wl.p)
+    F.fh_set_densities(pr.ctx, psi)
+    pr.window_spectra(wl.a, wl.t0, wl.dt, wl.H)
+    pr.sample(x, np.array([1.0]))
+    V = F.fh_get_target_field(pr.ctx, len(x), 2)[:, 1]
+    ref = O.target_field(wl.curve, N // 2, omega, psi, x, 1.0)
+    near = omega * d < 100.0
+    if near.any():
+        assert np.max(np.abs(V - ref)[near]) <= 1e-13 * np.max(np.abs(ref))
+    assert np.max(np.abs(V - ref)) <= 1e-12 * np.max(np.abs(ref))
+    pr.close()
