@@ -226,7 +226,7 @@ def phase_rooflines(wl, precision, ms, iters, peaks, contract_tc=False):
     put("assemble", "assemble_group_df_kernel" if mixed else "assemble_group_kernel", "alu",
         float(np.sum(N * N)), "entries/s")
     if precision == "fp64":
-        put("factor", "lu_solve_fp64_kernel", "alu", lu_flops(N), "TFLOP/s", peaks.get("fp64_tflops"),
+        put("factor", "lu_strip_fp64_kernel", "alu", lu_flops(N), "TFLOP/s", peaks.get("fp64_tflops"),
             "measured FP64 FMA-chain rate of this GPU (fh_probe_fma_peak)", 1e12)
     elif precision == "mixed":
         put("factor", "lu_factor_fp32_kernel", "alu", lu_flops(N), "TFLOP/s", peaks.get("fp32_tflops"),
@@ -243,7 +243,7 @@ def phase_rooflines(wl, precision, ms, iters, peaks, contract_tc=False):
             "per sweep x the largest sweep count", 1e9)
     put("field", "field_partial_df_kernel" if mixed else "field_partial_kernel", "alu",
         float(wl.n_x) * float(np.sum(N)), "pairs/s")
-    put("weights", "weights_kernel", "alu", float(window_pairs(wl)), "(t,k) pairs/s",
+    put("weights", "weights_tab_kernel", "alu", float(window_pairs(wl)), "(t,k) pairs/s",
         extra={"frequencies": wl.J})
     cf = contract_flops(wl.n_x, wl.T.size, wl.J)
     if contract_tc:
@@ -761,8 +761,7 @@ def run_gpu(args, world, rank, local):
     dominant = max(phase_ms, key=phase_ms.get)
     e2e_times, h2d, d2h = leg.e2e(args.steps, flush)
     e2e_total = max_over_ranks(sum(e2e_times), world, dev)
-    contract_tc = (args.precision != "fp64" and bool(leg.tuning["setting"].get("contract_tc"))
-                   and 2 * wl.J <= 8192)
+    contract_tc = bool(leg.tuning["setting"].get("contract_tc")) and 2 * wl.J <= 8192
     roofs = phase_rooflines(wl, args.precision, phase_ms, leg.stats.get("iters", 0), peaks,
                             contract_tc)
     roof = dict(roofs.get(dominant) or {"bound": "alu", "achieved": None, "peak": None,
