@@ -3,10 +3,10 @@
 // to FP64 accuracy through exact BF16 products (an error-free slicing of the
 // operands, the "Ozaki scheme").  Every precision contracts here, and so does
 // the split synthesis: the FP64 pipe bounds the plain FP64 kernel.  Measured,
-// plain -> slices (five launches): 1024 x 4096 outputs, 2J = 512 3.62 -> 0.23 ms
+// plain -> slices (five launches): 1024 x 4096 outputs, 2J = 512 3.62 -> 0.21 ms
 // (MMAs at the measured BF16 rate 0.08 ms; the rest is slicing, 42 MB written
-// and read back, and the FP64 epilogue), 2J = 1024 7.2 -> 0.41 ms, 333 x 1001,
-// 2J = 402 334 -> 75 us.
+// and read back, and the epilogue, which cannot overlap the MMAs: TMEM holds
+// one tile's levels), 2J = 1024 7.2 -> 0.37 ms, 333 x 1001, 2J = 402 334 -> 74 us.
 //
 // Scaling.  Term kk is first balanced by a power of two, A[x][kk] 2^d_kk times
 // B[kk][t] 2^-d_kk, so that entries which meet small partners (the fields at
@@ -23,8 +23,8 @@
 // Levels stay below 2^24 and exact, except levels 6 and 7 when nearly all 512
 // terms have one sign and both factors within 10 % of their maxima; they then
 // lose units of 2^-56 of a sum of some 2^8 of the same measure.  After each K
-// segment the epilogue joins the levels four by four as 64-bit integers and
-// adds the two to the FP64 sum of the output; at the end the sums take the
+// segment the epilogue joins the levels as integers, rounds once to FP64 and
+// adds up the segments; at the end the sums take the
 // factor 2^(ea_x + eb_t - 14).  The result differs from the exact product by
 // the dropped slice pairs (i + j >= kSlices) and the remainders, about 2^-58 of
 // max|row| max|column| per term after balancing.  Measured against quadruple
@@ -242,6 +242,25 @@ __global__ void __launch_bounds__(kThr) ozaki_slice_kernel(Src sa, Src sb, int a
     }
 }
 
+// hi 2^-21 + lo 2^-49 (|hi|, |lo| < 2^47) rounded to FP64, on integers (the FP64
+// pipe, two lanes a clock, held a quarter of the kernel with conversions and
+// multiply-adds): the sum as a 28 + 48 bit number, its leading 53 bits rounded.
+// 1024 x 4096 outputs, 2J = 512, 550 and 1024: 231, 290, 408 -> 214, 255, 374 us.
+__device__ __forceinline__ double join_levels(long long hi, long long lo) {
+    constexpr unsigned int kLow = (1u << 28) - 1;
+    const long long s = hi + (lo >> 28);
+    const unsigned int r = (unsigned int)lo & kLow;
+    const bool neg = s < 0;
+    const unsigned long long a = neg ? (unsigned long long)(-s - (r != 0u)) : (unsigned long long)s;
+    const unsigned long long b = neg ? (0u - r) & kLow : r;
+    if (a == 0ull) return fma((double)hi, 0x1p-21, (double)lo * 0x1p-49);
+    const int c = __clzll((long long)a);   // 15 .. 63
+    const unsigned long long y = (a << c) | (c >= 28 ? b << (c - 28) : b >> (28 - c));
+    const unsigned long long m = (y >> 11) + ((y >> 10) & 1ull);   // 2^52 .. 2^53
+    const unsigned long long e = (unsigned long long)(neg ? 2048 + 1064 - c : 1064 - c);
+    return __longlong_as_double((long long)((e << 52) + m));
+}
+
 // v 2^k
 __device__ __forceinline__ double scale_pow2(double v, int k) {
     if (k > 1000 || k < -1000) return ldexp(v, k);
@@ -334,24 +353,25 @@ __global__ void __launch_bounds__(kCtaThreads, 1) contract_tc_kernel(
 #pragma unroll
             for (int g = 0; g < 2; ++g) {
                 const int c0 = 32 * ch + 16 * g;
-#pragma unroll 1
-                for (int half = 1; half >= 0; --half) {   // the smaller levels first
-                    long long h[16];
+long long hi[16], lo[16];   // levels 0 .. 3 and 4 .. 7
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) h[c] = 0;
+                for (int c = 0; c < 16; ++c) hi[c] = lo[c] = 0;
+                auto join = [&](long long (&h)[16], int d0) {
 #pragma unroll 1
-                    for (int d = 0; d < kSlices / 2; ++d) {
+                    for (int d = d0; d < d0 + kSlices / 2; ++d) {
                         float v[16];
-                        tc::tmem_ld16(taddr + ((uint32_t)(32 * q) << 16) +
-                                          (uint32_t)((half * (kSlices / 2) + d) * kTN + c0), v);
+                        tc::tmem_ld16(taddr + ((uint32_t)(32 * q) << 16) + (uint32_t)(d * kTN + c0), v);
 #pragma unroll
-                        for (int c = 0; c < 16; ++c)   // below 2^47 in magnitude: exact in FP64 as well
+                        for (int c = 0; c < 16; ++c)   // below 2^47 in magnitude
                             h[c] = h[c] * (1 << kSliceBits) + __float2int_rn(v[c]);
                     }
-                    // levels 4 half .. 4 half + 3 relative to level 0
-                    const double sc = half ? 0x1p-49 : 0x1p-21;
+                };
+                join(hi, 0);
+                join(lo, kSlices / 2);
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) acc[g][c] = fma((double)h[c], sc, acc[g][c]);
+                for (int c = 0; c < 16; ++c) {
+                    const double v = join_levels(hi[c], lo[c]);
+                    acc[g][c] = sg == 0 ? v : acc[g][c] + v;
                 }
             }
             tc::tc_fence_before();
