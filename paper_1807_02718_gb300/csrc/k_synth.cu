@@ -696,8 +696,9 @@ __global__ void __launch_bounds__(128 * kSmallSlices) contract_small_kernel(
     int J, int n_x, int n_T, const double2 *__restrict__ V, const double *__restrict__ Gr,
     const double *__restrict__ Gm, double *__restrict__ u) {
     __shared__ double part[kSmallSlices][16][8 + 1];
-    const int lane = threadIdx.x & 31, x = blockIdx.x * 8 + (lane & 7);
-    const int tg = (threadIdx.x >> 5) & 3, slice = threadIdx.x >> 7, t0 = blockIdx.y * 16;
+    const int x_tiles = (n_x + 7) / 8, x0 = (int)(blockIdx.x % x_tiles) * 8, t0 = (int)(blockIdx.x / x_tiles) * 16;
+    const int lane = threadIdx.x & 31, x = x0 + (lane & 7);
+    const int tg = (threadIdx.x >> 5) & 3, slice = threadIdx.x >> 7;
     int tt[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) tt[i] = min(t0 + 4 * tg + i, n_T - 1);
@@ -719,11 +720,11 @@ __global__ void __launch_bounds__(128 * kSmallSlices) contract_small_kernel(
     }
     __syncthreads();
     const int q = threadIdx.x & 15, r = threadIdx.x >> 4;   // time, target (the first 128 threads)
-    if (r < 8 && blockIdx.x * 8 + r < n_x && t0 + q < n_T) {
+    if (r < 8 && x0 + r < n_x && t0 + q < n_T) {
         double v = part[0][q][r];
 #pragma unroll
         for (int i = 1; i < kSmallSlices; ++i) v += part[i][q][r];
-        u[(long long)(blockIdx.x * 8 + r) * n_T + t0 + q] = v;
+        u[(long long)(x0 + r) * n_T + t0 + q] = v;
     }
 }
 
@@ -902,11 +903,12 @@ void launch_synth_contract(int J, int n_x, int n_T, const double2 *V, const doub
     auto tiles = [&](int e) { return dim3((n_T + e - 1) / e, (n_x + e - 1) / e); };
     const dim3 g64 = tiles(64);
     if (contract_small(J, n_x, n_T)) {
-        const dim3 grid((n_x + 7) / 8, (n_T + 15) / 16);
-        if (grid.x * grid.y < 2 * 152)
-            contract_small_kernel<4><<<grid, 4 * 128, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
+        // all tiles in grid.x: J = 2 leaves 2^22 outputs, which for one target are more than 65535 tiles of 16 times
+        const unsigned ctas = (unsigned)((n_x + 7) / 8) * (unsigned)((n_T + 15) / 16);
+        if (ctas < 2 * 152)
+            contract_small_kernel<4><<<ctas, 4 * 128, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
         else
-            contract_small_kernel<1><<<grid, 128, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
+            contract_small_kernel<1><<<ctas, 128, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
     } else if (g64.x * g64.y < 2 * 152)
         contract_kernel<32><<<tiles(32), 256, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
     else
