@@ -302,7 +302,8 @@ fh_status fh_sing_frequencies(double omega_c, double *out);
  * j_c .. J-1; the singular piece on (0, w_c] is the Filon-Clenshaw-Curtis rule
  * on the points of fh_sing_frequencies(w_c).  The smooth piece's weights run in
  * compensated double-float on the FP32 pipe (the sums over the Fourier index
- * interpolated from a table or expanded, as in the periodic synthesis),
+ * interpolated from a table or expanded, as in the periodic synthesis), those
+ * of the six samples at either end, which the continuation amplifies, and
  * everything else in FP64: u agrees with the FP64 oracle's split synthesis to ~1e-10
  * relative (measured 8.8e-11 on a small kite, 1.1e-12 on the circle).
  *   J, W       uniform mesh omega_j = j W/(J-1); n = J - j_c >= 12 and n + 31 even

@@ -74,9 +74,15 @@ __device__ __forceinline__ double2 expi(double th) {
     return make_double2(c, s);
 }
 // Continuation rows: Xc[j * n + p] = d e_j / d f_p (right end blended to
-// zero, plus the left end read backwards, blended and reversed).
-__global__ void fc_rows_kernel(int n, double *__restrict__ Xc) {
+// zero, plus the left end read backwards, blended and reversed); and the FP64
+// phases ph[q] = e^{-2 pi i q / L}, q < L = n + kFcC.
+__global__ void fc_rows_kernel(int n, double *__restrict__ Xc, double2 *__restrict__ ph) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+    if (j == 0 && p < n + kFcC) {
+        double sn, cs;
+        sincospi(-2.0 * (double)p / (double)(n + kFcC), &sn, &cs);
+        ph[p] = make_double2(cs, sn);
+    }
     if (p >= n) return;
     double v = 0.0;
     if (p >= n - kFcD) {
@@ -97,16 +103,29 @@ __device__ __forceinline__ double sinc_half(int num, int L, long long v) {
     return sinpi((double)(k % (4LL * L)) / (2.0 * L)) * (2.0 * L) / (kPi * (double)k);
 }
 
+constexpr int kMid = kFcC / 2;    // continuation point kMid has the frequency index h
+constexpr int kTop = kMid + 1 + kFcD;        // S_(h - kTop + 1) .. S_h enter the end samples' weights
+
 // Table of S_i(g/2), |g| <= G, i = 0..h: tab[(g + G) hp + i] = (re hi, im hi, re
 // lo, im lo), hp = h + 1.  One CTA per kTabRows rows g >= 0 and 128 columns; m and
 // -m are paired, their sinc sums staged in chunks of kTabChunk for all columns;
 // the rows -g from S_i(-y) = conj S_i(y) + (-1)^i (sinc(r (y - h)) - sinc(r (y + h))).
+// The CTAs of the first columns also form top[(g + G) kTop + q] = S_(h-q)(g/2),
+// q < kTop, in FP64 (one thread per row and q; 1 % of the sums).
 constexpr int kTabRows = 4, kTabChunk = 256;
 
 __global__ void __launch_bounds__(128) split_table_kernel(int num, int L, int G, const float4 *__restrict__ ph,
-                                                          float4 *__restrict__ tab) {
+                                                          const double2 *__restrict__ ph64, float4 *__restrict__ tab,
+                                                          double2 *__restrict__ top) {
     const int h = L / 2, hp = h + 1, i = blockIdx.y * 128 + threadIdx.x, g0 = kTabRows * blockIdx.x;
     __shared__ float4 sc[kTabRows][kTabChunk];   // sinc(r (y - m)) +- sinc(r (y + m))
+    __shared__ double2 sd[kTabRows][kTabChunk];
+    static_assert(kTabRows * kTop <= 128, "a thread per row and top column");
+    const bool first = blockIdx.y == 0, fp64 = first && threadIdx.x < kTabRows * kTop;
+    const int tq = fp64 ? threadIdx.x / kTop : 0, ti = h - (fp64 ? threadIdx.x % kTop : 0), tg = g0 + tq;
+    double2 td = make_double2(0.0, 0.0);
+    int tk = 0;
+    if (fp64) td.x = sinc_half(num, L, tg) + ((ti & 1) ? -1.0 : 1.0) * sinc_half(num, L, tg + 2LL * h);
     float2 ah[kTabRows], al[kTabRows], ac[kTabRows];   // (re, im), compensated
 #pragma unroll
     for (int q = 0; q < kTabRows; ++q) {
@@ -125,8 +144,18 @@ __global__ void __launch_bounds__(128) split_table_kernel(int num, int L, int G,
             const int q = e / mc, m = m0 + e % mc;
             const double a = sinc_half(num, L, g0 + q - 2LL * m), b = sinc_half(num, L, g0 + q + 2LL * m);
             sc[q][e % mc] = df_pack(a + b, a - b);
+            if (first) sd[q][e % mc] = make_double2(a + b, a - b);
         }
         __syncthreads();
+        if (fp64)
+#pragma unroll 4
+            for (int m = 0; m < mc; ++m) {
+                tk += ti;
+                if (tk >= L) tk -= L;
+                const double2 e = __ldg(ph64 + tk), v = sd[tq][m];
+                td.x = fma(e.x, v.x, td.x);
+                td.y = fma(e.y, v.y, td.y);
+            }
         if (i < hp)
             for (int m = 0; m < mc; ++m) {
                 k += i;
@@ -138,6 +167,12 @@ __global__ void __launch_bounds__(128) split_table_kernel(int num, int L, int G,
                     df2_acc_c(ah[q], al[q], ac[q], {p2(e.x, e.z), p2(e.y, e.w)}, {p2(v.x, v.z), p2(v.y, v.w)});
                 }
             }
+    }
+    if (fp64 && tg <= G) {
+        double2 *row = top + threadIdx.x % kTop;
+        row[(long long)(tg + G) * kTop] = td;
+        const double c = sinc_half(num, L, tg - 2LL * h) - sinc_half(num, L, tg + 2LL * h);
+        if (tg > 0) row[(long long)(G - tg) * kTop] = make_double2(td.x + ((ti & 1) ? -c : c), -td.y);
     }
     if (i >= hp) return;
 #pragma unroll
@@ -168,33 +203,46 @@ struct SplitWindow {
     int g0, gc;          // near: first and nearest sample, y - gc/2 and sin(2 pi y)
     double uc, s2;
     dfv rho, ar, ai;     // far: ratio and the factor a
-    dfv cr, ci;          // (2A/L) e^{-i delta t'} / pi
+    double2 c;           // (2A/L) e^{-i delta t'} / pi, and in double-float
+    dfv cr, ci;
 };
 constexpr int kSplitChunk = 32;   // windows whose constants are held at once
-constexpr int kEdge = 2 * kFcD;   // end samples, whose weights take the continuation
-constexpr int kEdgeItems = kEdge * 32;   // end sample x (31 continuation points, the sample itself)
-constexpr int kSplitThreads = 256, kEdgePer = (kEdgeItems + 127) / 128;
+constexpr int kSplitThreads = 256;
+constexpr int kEndPer = (kMid + 1) / 2;      // folded continuation terms per lane
+constexpr int kTopParts = 4;      // interpolations of a top value side by side
+static_assert(kFcC == 2 * kMid + 1 && 2 * kEndPer == kMid + 1, "continuation points in pairs about the middle one");
+static_assert(4 * kFcD <= 32 && kTop <= 32, "one warp takes the end samples");
 
 // Smooth-piece weights: one CTA per time.  Per window S_0 .. S_h go to shared
 // memory, then every interior sample adds B_k(w_p) D_p to its sum (shared memory,
-// its thread's own), and every (end sample p, continuation point j) adds B_k(w_p)
-// (2A/L) e^{-i delta t'} S to a sum of its own.  The interpolation weights are
-// FP64, all sums double-float with compensated low parts: the sum over j with Xc (entries up to 6e4 that cancel for smooth
-// fields) is taken once per time, in FP64.  Rows 0..n-1 of the weight planes: Gr =
-// Re G / pi, Gm = -Im G / pi.
-// Measured (GB300; 1024 x 4096 samples, n = 251, 29 windows): 21.0 -> 1.6 ms (L-term
-// double-float sums per sample before); the table takes 0.11 ms per call, the
-// whole synthesis 27.2 -> 6.0 ms (2.4 ms with the contraction on the tensor cores).  Error against
-// 64 bits over ten meshes of n = 25..230: 1.4e-12..6.7e-11 -> 4e-13..5.9e-11.
+// its thread's own; double-float with compensated low parts).
+// The end samples: the continuation point j has index i = h - kMid + j modulo L, so
+// that points kMid - q and kMid + q carry S_(h-q) and its conjugate, and sample n -
+// kFcD + s (index h - kTop + 1 + s) has
+//   Re D = Re S + Xc[kMid] Re S_h + sum_q (Xc[kMid - q] + Xc[kMid + q]) Re S_(h-q),
+//   Im D = Im S + Xc[kMid] Im S_h + sum_q (Xc[kMid - q] - Xc[kMid + q]) Im S_(h-q),
+// sample kFcD - 1 - s the conjugate.  The entries of Xc reach 6e4; they cancel for
+// fields that are smooth from sample to sample, and for others every rounding
+// before them shows in u.  So the S of near windows that enter here are FP64 (table,
+// weights and sums), and the sums and products with B_k(w_p), one warp per window:
+// 24 lanes (sample, part, half of the terms), then 12 lanes (end sample).
+// Rows 0..n-1 of the weight planes: Gr = Re G / pi, Gm = -Im G / pi.
+// Measured (GB300; 1024 x 4096 samples, n = 251, 29 windows): whole call 2.34 ms with 384
+// double-float products (end sample, continuation point) per window, each splitting
+// its B in FP64, 1.86 ms so.  Error against extended precision over 28 meshes of
+// n = 20..110: geometric mean 4.8e-12 -> 6.6e-13, largest 6.6e-11 -> 1.7e-11 (L-term
+// double-float sums per sample: 2.0e-11 and 1.3e-10).
 __global__ void __launch_bounds__(kSplitThreads) smooth_weights_kernel(
     int n, int L, double A, double P, double delta, int K, const double *__restrict__ s,
-    const double2 *__restrict__ B, int J, int j_c, const double *__restrict__ Xc, const float4 *__restrict__ tab, int G,
-    const float4 *__restrict__ nu, const double *__restrict__ T, int n_T, double *__restrict__ Gr,
+    const double2 *__restrict__ B, int J, int j_c, const double *__restrict__ Xc, const float4 *__restrict__ tab,
+    const double2 *__restrict__ top_tab, int G, const float4 *__restrict__ nu, const double *__restrict__ T, int n_T, double *__restrict__ Gr,
     double *__restrict__ Gm) {
     extern __shared__ float4 sm[];
     __shared__ SplitWindow win[kSplitChunk];
     __shared__ float2 swt[kSincPts];
-    __shared__ double2 edge[kEdgeItems];
+    __shared__ double swd[kSincPts];
+    __shared__ double2 tops[kTopParts][kTop];
+    __shared__ double top[2][kTop];   // Re, Im S_(h-q)
     const int h = L / 2, hp = h + 1, nm = (n - 1) / 2, it = blockIdx.x, tid = threadIdx.x;
     float4 *Ss = sm, *Fs = sm + hp, *acc = sm + 2 * hp;   // S_i, F_l, G_p: (re hi, im hi, re lo, im lo)
     float2 *accc = reinterpret_cast<float2 *>(acc + n);   // G_p: third parts
@@ -203,9 +251,22 @@ __global__ void __launch_bounds__(kSplitThreads) smooth_weights_kernel(
         acc[p] = make_float4(0.f, 0.f, 0.f, 0.f);
         accc[p] = p2(0.f, 0.f);
     }
-    float2 eh[kEdgePer], el[kEdgePer], ec[kEdgePer];
+    // the last warp (it has the fewest interior samples): the folded
+    // continuation terms of its lanes, and sums of end sample `lane`
+    const bool ends = tid >= (int)blockDim.x - 32;
+    const int lane = tid & 31, smp = min(lane >> 2, kFcD - 1), part = (lane >> 1) & 1, q0 = (lane & 1) * kEndPer;
+    double xf[kEndPer];
+    const int pe = lane < kFcD ? n - kFcD + lane : 2 * kFcD - 1 - min(lane, 2 * kFcD - 1);
+    double2 ge = make_double2(0.0, 0.0);
+    if (ends) {
+        const double *x = Xc + n - kFcD + smp;
 #pragma unroll
-    for (int e = 0; e < kEdgePer; ++e) eh[e] = el[e] = ec[e] = p2(0.f, 0.f);
+        for (int e = 0; e < kEndPer; ++e) {
+            const int q = q0 + e;
+            const double lo = x[(long long)(kMid - q) * n], hi = q ? x[(long long)(kMid + q) * n] : 0.0;
+            xf[e] = part ? lo - hi : lo + hi;
+        }
+    }
     const double r = (double)(n - 1) / (double)L;
     for (int k0 = 0; k0 < K; k0 += kSplitChunk) {
         __syncthreads();
@@ -240,8 +301,9 @@ __global__ void __launch_bounds__(kSplitThreads) smooth_weights_kernel(
             }
             const double2 ph = expi(-delta * tp);
             const double f = 2.0 * A / ((double)L * kPi);
-            w.cr = df_from(f * ph.x);
-            w.ci = df_from(f * ph.y);
+            w.c = make_double2(f * ph.x, f * ph.y);
+            w.cr = df_from(w.c.x);
+            w.ci = df_from(w.c.y);
             win[k] = w;
         }
         for (int k = k0; k < min(k0 + kSplitChunk, K); ++k) {
@@ -249,12 +311,27 @@ __global__ void __launch_bounds__(kSplitThreads) smooth_weights_kernel(
             const SplitWindow &w = win[k - k0];
             if (w.R == 0) {
                 if (tid < kSincPts) {
-                    const dfv v = df_from(sinc_weight64(w.uc, w.s2, w.gc, w.g0, tid));
+                    const double v64 = sinc_weight64(w.uc, w.s2, w.gc, w.g0, tid);
+                    const dfv v = df_from(v64);
                     swt[tid] = p2(v.hi, v.lo);
+                    swd[tid] = v64;
                 }
                 __syncthreads();
+                const int te = (int)blockDim.x - 1 - tid;   // the top values: the last threads
+                if (te < kTopParts * kTop) {
+                    const int c = te / kTop, e = te % kTop;
+                    const double2 *col = top_tab + (long long)(w.g0 + G) * kTop + e;
+                    double2 v = make_double2(0.0, 0.0);
+#pragma unroll 4
+                    for (int q = c; q < kSincPts; q += kTopParts) {
+                        const double2 x = __ldg(col + q * kTop);
+                        v.x = fma(swd[q], x.x, v.x);
+                        v.y = fma(swd[q], x.y, v.y);
+                    }
+                    tops[c][e] = v;
+                }
                 const float4 *row = tab + (long long)(w.g0 + G) * hp;
-                for (int i = tid; i < hp; i += blockDim.x) {
+                for (int i = tid; i < hp - kTop; i += blockDim.x) {
                     float2 sh = p2(0.f, 0.f), sl = sh, sc = sh;
 #pragma unroll 6
                     for (int q = 0; q < kSincPts; ++q) {
@@ -317,44 +394,43 @@ __global__ void __launch_bounds__(kSplitThreads) smooth_weights_kernel(
                 acc[p] = make_float4(gh.x, gh.y, gl.x, gl.y);
                 accc[p] = gc;
             }
+            if (ends) {   // FP64
+                if (lane < kTop) {
+                    double2 v;
+                    if (w.R == 0) {
+                        v = tops[0][lane];
+                        for (int c = 1; c < kTopParts; ++c) v = cadd(v, tops[c][lane]);
+                    } else {
+                        const float4 f = Ss[h - lane];
+                        v = make_double2((double)f.x + (double)f.z, (double)f.y + (double)f.w);
+                    }
+                    top[0][lane] = v.x;
+                    top[1][lane] = v.y;
+                }
+                const double2 b = B[(long long)k * J + j_c + pe], c = w.c;
+                __syncwarp();
+                double d = q0 ? 0.0 : top[part][kTop - 1 - smp];
 #pragma unroll
-            for (int e = 0; e < kEdgePer; ++e) {
-                const int id = tid + e * blockDim.x;
-                if (id >= kEdgeItems) continue;
-                const int pe = id >> 5, j = id & 31, p = pe < kFcD ? pe : n - kEdge + pe;
-                int i = j < kFcC ? n + j - nm : p - nm;
-                if (i > h) i -= L;
-                const df2 b = bc(p), x = S(i), xs = df2_swap(x);
-                df2_acc_c(eh[e], el[e], ec[e], df2_bcast(df2_x(b)), x);
-                df2_acc_c(eh[e], el[e], ec[e], df2_make(df_neg(df2_y(b)), df2_y(b)), xs);
+                for (int e = 0; e < kEndPer; ++e) d = fma(xf[e], top[part][q0 + e], d);
+                d += __shfl_xor_sync(0xffffffffu, d, 1);
+                const int src = 4 * (lane < kFcD ? lane : min(lane, 2 * kFcD - 1) - kFcD);
+                const double dr = __shfl_sync(0xffffffffu, d, src), di = __shfl_sync(0xffffffffu, d, src + 2);
+                const double2 bw = cmul(b, c), v = cmul(bw, make_double2(dr, lane < kFcD ? di : -di));
+                ge.x += v.x;
+                ge.y += v.y;
             }
         }
-    }
-#pragma unroll
-    for (int e = 0; e < kEdgePer; ++e) {
-        const int id = tid + e * blockDim.x;
-        if (id < kEdgeItems)
-            edge[id] = make_double2((double)eh[e].x + (double)el[e].x + (double)ec[e].x,
-                                    (double)eh[e].y + (double)el[e].y + (double)ec[e].y);
     }
     __syncthreads();
-    for (int p = tid; p < n; p += blockDim.x) {
-        double2 g;
-        if (p < kFcD || p >= n - kFcD) {
-            const double2 *z = edge + 32 * (p < kFcD ? p : p - n + kEdge);
-            g = z[kFcC];
-            for (int j = 0; j < kFcC; ++j) {
-                const double x = Xc[(long long)j * n + p];
-                g.x = fma(x, z[j].x, g.x);
-                g.y = fma(x, z[j].y, g.y);
-            }
-        } else {
-            const float4 q = acc[p];
-            const float2 c = accc[p];
-            g = make_double2((double)q.x + (double)q.z + (double)c.x, (double)q.y + (double)q.w + (double)c.y);
-        }
-        Gr[(long long)p * n_T + it] = g.x;
-        Gm[(long long)p * n_T + it] = -g.y;
+    for (int p = kFcD + tid; p < n - kFcD; p += blockDim.x) {
+        const float4 q = acc[p];
+        const float2 c = accc[p];
+        Gr[(long long)p * n_T + it] = (double)q.x + (double)q.z + (double)c.x;
+        Gm[(long long)p * n_T + it] = -((double)q.y + (double)q.w + (double)c.y);
+    }
+    if (ends && lane < 2 * kFcD) {
+        Gr[(long long)pe * n_T + it] = ge.x;
+        Gm[(long long)pe * n_T + it] = -ge.y;
     }
 }
 
@@ -578,19 +654,21 @@ extern "C" fh_status fh_synthesize_sing(int J, double W, int j_c, int K, const d
         // half-integer table of S_i, far-field table of order L with its phases and powers
         const int h = L / 2, hp = h + 1, G = (5 * h + 1) / 2 + 24;
         float4 *tab = sc.get<float4>((size_t)(2 * G + 1) * hp);
+        double2 *top = sc.get<double2>((size_t)(2 * G + 1) * kTop);
+        double2 *ph64 = sc.get<double2>((size_t)L);
         float4 *nu = sc.get<float4>((size_t)kFarTerms * hp);
         float4 *ph = sc.get<float4>((size_t)L);
         double *pw = sc.get<double>((size_t)L * kFarTerms);
         double2 *Vp = sc.get<double2>((size_t)ns * n_x);
         double *Gr = sc.get<double>((size_t)ns * n_T);
         double *Gm = sc.get<double>((size_t)ns * n_T);
-        if (!Xc || !tab || !nu || !ph || !pw || !Vp || !Gr || !Gm) {
+        if (!Xc || !tab || !top || !ph64 || !nu || !ph || !pw || !Vp || !Gr || !Gm) {
             cudaGetLastError();
             return FH_ENOMEM;
         }
-        fc_rows_kernel<<<dim3(grid_of(n, 128), kFcC), 128, 0, st>>>(n, Xc);
+        fc_rows_kernel<<<dim3(grid_of(L, 128), kFcC), 128, 0, st>>>(n, Xc, ph64);
         launch_far_table(hp, L, pw, nullptr, nu, ph, st);
-        split_table_kernel<<<dim3(G / kTabRows + 1, grid_of(hp, 128)), 128, 0, st>>>(n - 1, L, G, ph, tab);
+        split_table_kernel<<<dim3(G / kTabRows + 1, grid_of(hp, 128)), 128, 0, st>>>(n - 1, L, G, ph, ph64, tab, top);
         const double A = 0.5 * (W - wc), P = L * dw, delta = 0.5 * (wc + W);
         const size_t smem = (size_t)(2 * hp + n) * sizeof(float4) + (size_t)n * sizeof(float2);
         static std::atomic<unsigned long long> attr{0};
@@ -598,7 +676,7 @@ extern "C" fh_status fh_synthesize_sing(int J, double W, int j_c, int K, const d
         // as many threads as values S_i (the longest loops), at least 128 for the end samples
         const int threads = std::min(kSplitThreads, std::max(128, (hp + 31) / 32 * 32));
         smooth_weights_kernel<<<n_T, threads, smem, st>>>(n, L, A, P, delta, K, d_s, reinterpret_cast<const double2 *>(d_B),
-                                                          J, j_c, Xc, tab, G, nu, d_T, n_T, Gr, Gm);
+                                                          J, j_c, Xc, tab, top, G, nu, d_T, n_T, Gr, Gm);
         fcc_weights_kernel<<<dim3(grid_of(n_T, kFccTimes), kSM - 1), kFccTimes * kFccGroups, 0, st>>>(
             n, K, d_s, reinterpret_cast<const double2 *>(d_Bs), d_T, n_T, Gr, Gm);
         stack_fields_kernel<<<dim3(grid_of(n_x, 128), ns), 128, 0, st>>>(
