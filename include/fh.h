@@ -306,7 +306,8 @@ fh_status fh_sing_frequencies(double omega_c, double *out);
  * of the six samples at either end, which the continuation amplifies, and
  * everything else in FP64: u agrees with the FP64 oracle's split synthesis to ~1e-10
  * relative (measured 8.8e-11 on a small kite, 1.1e-12 on the circle).
- *   J, W       uniform mesh omega_j = j W/(J-1); n = J - j_c >= 12 and n + 31 even
+ *   J, W       uniform mesh omega_j = j W/(J-1); 12 <= n = J - j_c <= 65511 and n + 31 even
+ *              (work space ~20 n^2 bytes)
  *   j_c        index of w_c (>= 1)
  *   K, d_s     window centres (device, K doubles)
  *   d_B        B_k^slow(omega_j), K*J complex, B[k*J + j] (device)

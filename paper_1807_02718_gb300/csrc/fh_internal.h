@@ -29,6 +29,8 @@ inline cudaError_t ensure_smem_attr(const void *fn, int bytes,
     return e;
 }
 
+constexpr int kSms = 152;   // streaming multiprocessors of the GPU these kernels are written for
+
 constexpr double kPi = 3.14159265358979323846;
 constexpr double kEulerGamma = 0.57721566490153286061;
 

@@ -212,6 +212,13 @@ constexpr int kEndPer = (kMid + 1) / 2;      // folded continuation terms per la
 constexpr int kTopParts = 4;      // interpolations of a top value side by side
 static_assert(kFcC == 2 * kMid + 1 && 2 * kEndPer == kMid + 1, "continuation points in pairs about the middle one");
 static_assert(4 * kFcD <= 32 && kTop <= 32, "one warp takes the end samples");
+// The values a CTA keeps for its time: S_0 .. S_h, F_0 .. F_h and the sums of n samples.
+constexpr int kSplitSmem = 200 * 1024;
+constexpr int kSplitCtas = 4 * kSms;   // times per launch where they are in device memory
+__host__ __device__ inline size_t split_work_bytes(int n) {
+    const size_t hp = (size_t)(n + kFcC) / 2 + 1;
+    return ((2 * hp + n) * sizeof(float4) + n * sizeof(float2) + 15) & ~(size_t)15;
+}
 
 // Smooth-piece weights: one CTA per time.  Per window S_0 .. S_h go to shared
 // memory, then every interior sample adds B_k(w_p) D_p to its sum (shared memory,
@@ -227,13 +234,17 @@ static_assert(4 * kFcD <= 32 && kTop <= 32, "one warp takes the end samples");
 // weights and sums), and the sums and products with B_k(w_p), one warp per window:
 // 24 lanes (sample, part, half of the terms), then 12 lanes (end sample).
 // Rows 0..n-1 of the weight planes: Gr = Re G / pi, Gm = -Im G / pi.
+// kShared: the values of a time in shared memory (split_work_bytes(n) = 40 n + 528
+// bytes, n <= 5106 at kSplitSmem); otherwise in `work`, the launch's CTAs taking
+// the times from it0 on.
 // Measured (GB300; 1024 x 4096 samples, n = 251, 29 windows): whole call 2.34 ms with 384
 // double-float products (end sample, continuation point) per window, each splitting
-// its B in FP64, 1.86 ms so.  Error against extended precision over 28 meshes of
+// its B in FP64, 1.74 ms so.  Error against extended precision over 28 meshes of
 // n = 20..110: geometric mean 4.8e-12 -> 6.6e-13, largest 6.6e-11 -> 1.7e-11 (L-term
 // double-float sums per sample: 2.0e-11 and 1.3e-10).
+template <bool kShared>
 __global__ void __launch_bounds__(kSplitThreads) smooth_weights_kernel(
-    int n, int L, double A, double P, double delta, int K, const double *__restrict__ s,
+    int it0, float4 *work, int n, int L, double A, double P, double delta, int K, const double *__restrict__ s,
     const double2 *__restrict__ B, int J, int j_c, const double *__restrict__ Xc, const float4 *__restrict__ tab,
     const double2 *__restrict__ top_tab, int G, const float4 *__restrict__ nu, const double *__restrict__ T, int n_T, double *__restrict__ Gr,
     double *__restrict__ Gm) {
@@ -243,8 +254,9 @@ __global__ void __launch_bounds__(kSplitThreads) smooth_weights_kernel(
     __shared__ double swd[kSincPts];
     __shared__ double2 tops[kTopParts][kTop];
     __shared__ double top[2][kTop];   // Re, Im S_(h-q)
-    const int h = L / 2, hp = h + 1, nm = (n - 1) / 2, it = blockIdx.x, tid = threadIdx.x;
-    float4 *Ss = sm, *Fs = sm + hp, *acc = sm + 2 * hp;   // S_i, F_l, G_p: (re hi, im hi, re lo, im lo)
+    const int h = L / 2, hp = h + 1, nm = (n - 1) / 2, it = it0 + blockIdx.x, tid = threadIdx.x;
+    float4 *Ss = kShared ? sm : work + blockIdx.x * (split_work_bytes(n) / sizeof(float4));
+    float4 *Fs = Ss + hp, *acc = Ss + 2 * hp;   // S_i, F_l, G_p: (re hi, im hi, re lo, im lo)
     float2 *accc = reinterpret_cast<float2 *>(acc + n);   // G_p: third parts
     const double t = T[it];
     for (int p = tid; p < n; p += blockDim.x) {
@@ -622,6 +634,7 @@ extern "C" fh_status fh_synthesize_sing(int J, double W, int j_c, int K, const d
     if (J < 2 || !(W > 0.0) || K < 1 || n_x < 0 || n_T < 0 || j_c < 1) return FH_EINVAL;
     const int n = J - j_c;
     if (n < 2 * kFcD || ((n + kFcC) & 1)) return FH_EINVAL;   // FC needs 2d samples; n + C even
+    if (n + kNsing > 65535) return FH_EINVAL;                  // rows of the stacked fields are in grid.y
     if (n_x == 0 || n_T == 0) return FH_OK;
     if (!d_s || !d_B || !d_Bs || !d_V || !d_Vs || !d_T || !d_u) return FH_EINVAL;
     if (cudaPeekAtLastError() != cudaSuccess) return FH_ECUDA;
@@ -662,7 +675,10 @@ extern "C" fh_status fh_synthesize_sing(int J, double W, int j_c, int K, const d
         double2 *Vp = sc.get<double2>((size_t)ns * n_x);
         double *Gr = sc.get<double>((size_t)ns * n_T);
         double *Gm = sc.get<double>((size_t)ns * n_T);
-        if (!Xc || !tab || !top || !ph64 || !nu || !ph || !pw || !Vp || !Gr || !Gm) {
+        const size_t work_bytes = split_work_bytes(n);
+        const bool in_memory = work_bytes > kSplitSmem;
+        float4 *work = in_memory ? sc.get<float4>(work_bytes / sizeof(float4) * std::min(kSplitCtas, n_T)) : nullptr;
+        if ((in_memory && !work) || !Xc || !tab || !top || !ph64 || !nu || !ph || !pw || !Vp || !Gr || !Gm) {
             cudaGetLastError();
             return FH_ENOMEM;
         }
@@ -670,13 +686,20 @@ extern "C" fh_status fh_synthesize_sing(int J, double W, int j_c, int K, const d
         launch_far_table(hp, L, pw, nullptr, nu, ph, st);
         split_table_kernel<<<dim3(G / kTabRows + 1, grid_of(hp, 128)), 128, 0, st>>>(n - 1, L, G, ph, ph64, tab, top);
         const double A = 0.5 * (W - wc), P = L * dw, delta = 0.5 * (wc + W);
-        const size_t smem = (size_t)(2 * hp + n) * sizeof(float4) + (size_t)n * sizeof(float2);
-        static std::atomic<unsigned long long> attr{0};
-        ensure_smem_attr((const void *)smooth_weights_kernel, 200 * 1024, attr);
         // as many threads as values S_i (the longest loops), at least 128 for the end samples
         const int threads = std::min(kSplitThreads, std::max(128, (hp + 31) / 32 * 32));
-        smooth_weights_kernel<<<n_T, threads, smem, st>>>(n, L, A, P, delta, K, d_s, reinterpret_cast<const double2 *>(d_B),
-                                                          J, j_c, Xc, tab, top, G, nu, d_T, n_T, Gr, Gm);
+        if (!work) {
+            static std::atomic<unsigned long long> attr{0};
+            ensure_smem_attr((const void *)smooth_weights_kernel<true>, kSplitSmem, attr);
+            smooth_weights_kernel<true><<<n_T, threads, work_bytes, st>>>(
+                0, nullptr, n, L, A, P, delta, K, d_s, reinterpret_cast<const double2 *>(d_B), J, j_c, Xc, tab, top, G,
+                nu, d_T, n_T, Gr, Gm);
+        } else {
+            for (int it0 = 0; it0 < n_T; it0 += kSplitCtas)
+                smooth_weights_kernel<false><<<std::min(kSplitCtas, n_T - it0), threads, 0, st>>>(
+                    it0, work, n, L, A, P, delta, K, d_s, reinterpret_cast<const double2 *>(d_B), J, j_c, Xc, tab, top,
+                    G, nu, d_T, n_T, Gr, Gm);
+        }
         fcc_weights_kernel<<<dim3(grid_of(n_T, kFccTimes), kSM - 1), kFccTimes * kFccGroups, 0, st>>>(
             n, K, d_s, reinterpret_cast<const double2 *>(d_Bs), d_T, n_T, Gr, Gm);
         stack_fields_kernel<<<dim3(grid_of(n_x, 128), ns), 128, 0, st>>>(
