@@ -59,10 +59,14 @@ constexpr int kNsing = (kSM - 1) * kSNq;
 constexpr int kGl = 24;    // Gauss-Legendre nodes, symmetric: the positive half is kept
 constexpr int kMom = 13;   // terms of the moments' power series in kappa^2
 
-__constant__ double c_cheb[kSNq][kSNq];   // interpolant coefficients a_n = sum_c c_cheb[n][c] f_c
-__constant__ double c_glx[kGl / 2], c_glw[kGl / 2];
-__constant__ double c_mom[kSNq][kMom];    // int T_n x^q dx / q!, q = 2 m + n mod 2
-__constant__ double c_mu[kSM];
+// Constants of the rule: an argument of the launch (constant memory), so that calls
+// with other meshes on other streams keep theirs.
+struct FccRule {
+    double cheb[kSNq][kSNq];   // interpolant coefficients a_n = sum_c cheb[n][c] f_c
+    double glx[kGl / 2], glw[kGl / 2];
+    double mom[kSNq][kMom];    // int T_n x^q dx / q!, q = 2 m + n mod 2
+    double mu[kSM];            // graded mesh
+};
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -448,19 +452,19 @@ __global__ void __launch_bounds__(kSplitThreads) smooth_weights_kernel(
 
 // Chebyshev moments rho_n(kappa) = int_{-1}^{1} T_n(x) e^{-i kappa x} dx, n < 8: real
 // for even n, imaginary for odd n (rho[n] holds the real or imaginary part).
-//   |kappa| <= 2: their power series (c_mom[n][s] (-1)^s kappa^(2s), times -kappa
+//   |kappa| <= 2: their power series (mom[n][s] (-1)^s kappa^(2s), times -kappa
 //     for odd n; the remainder is below 3e-17);
 //   |kappa| < 12: 24-point Gauss-Legendre, x and -x together (error below 1e-17);
 //   beyond: the forward three-term recurrence, stable there.
-__device__ void cheb_moments(double kap, double (&rho)[kSNq]) {
+__device__ __forceinline__ void cheb_moments(const FccRule &rule, double kap, double (&rho)[kSNq]) {
     const double ka = fabs(kap);
     if (ka <= 2.0) {
         const double z = -kap * kap;
 #pragma unroll
         for (int q = 0; q < kSNq; ++q) {
-            double v = c_mom[q][kMom - 1];
+            double v = rule.mom[q][kMom - 1];
 #pragma unroll
-            for (int m = kMom - 2; m >= 0; --m) v = fma(v, z, c_mom[q][m]);
+            for (int m = kMom - 2; m >= 0; --m) v = fma(v, z, rule.mom[q][m]);
             rho[q] = (q & 1) ? -kap * v : v;
         }
         return;
@@ -469,11 +473,11 @@ __device__ void cheb_moments(double kap, double (&rho)[kSNq]) {
 #pragma unroll
         for (int q = 0; q < kSNq; ++q) rho[q] = 0.0;
         for (int g = 0; g < kGl / 2; ++g) {
-            const double x = c_glx[g], x2 = 2.0 * x;
+            const double x = rule.glx[g], x2 = 2.0 * x;
             double s, c;
             sincos(kap * x, &s, &c);
-            c *= c_glw[g];
-            s *= -c_glw[g];
+            c *= rule.glw[g];
+            s *= -rule.glw[g];
             double t0 = 1.0, t1 = x;
 #pragma unroll
             for (int q = 0; q < kSNq; ++q) {   // T_q(x) times the even (cos) or odd (-sin) part
@@ -513,12 +517,12 @@ __device__ void cheb_moments(double kap, double (&rho)[kSNq]) {
 constexpr int kFccTimes = 32, kFccGroups = 4;
 
 __global__ void __launch_bounds__(kFccTimes *kFccGroups) fcc_weights_kernel(
-    int n, int K, const double *__restrict__ s, const double2 *__restrict__ Bs, const double *__restrict__ T, int n_T,
-    double *__restrict__ Gr, double *__restrict__ Gm) {
+    const __grid_constant__ FccRule rule, int n, int K, const double *__restrict__ s, const double2 *__restrict__ Bs,
+    const double *__restrict__ T, int n_T, double *__restrict__ Gr, double *__restrict__ Gm) {
     __shared__ double2 sums[kFccGroups][kSNq][kFccTimes];
     const int lane = threadIdx.x % kFccTimes, grp = threadIdx.x / kFccTimes;
     const int it = blockIdx.x * kFccTimes + lane, jv = blockIdx.y + 1;
-    const double a = c_mu[jv - 1], b = c_mu[jv];        // interval [mu_{jv-1}, mu_jv] (0-based c_mu)
+    const double a = rule.mu[jv - 1], b = rule.mu[jv];        // interval [mu_{jv-1}, mu_jv] (0-based)
     const double h = 0.5 * (b - a), dl = 0.5 * (a + b);
     const int i0 = (jv - 1) * kSNq;
     double2 acc[kSNq];
@@ -529,7 +533,7 @@ __global__ void __launch_bounds__(kFccTimes *kFccGroups) fcc_weights_kernel(
         for (int k = grp; k < K; k += kFccGroups) {
             const double tp = t - s[k];
             double rho[kSNq];
-            cheb_moments(h * tp, rho);
+            cheb_moments(rule, h * tp, rho);
             double2 ph = expi(-dl * tp);
             ph.x *= h;
             ph.y *= h;
@@ -538,8 +542,8 @@ __global__ void __launch_bounds__(kFccTimes *kFccGroups) fcc_weights_kernel(
                 double2 w = make_double2(0.0, 0.0);
 #pragma unroll
                 for (int q = 0; q < kSNq; q += 2) {
-                    w.x = fma(c_cheb[q][c], rho[q], w.x);
-                    w.y = fma(c_cheb[q + 1][c], rho[q + 1], w.y);
+                    w.x = fma(rule.cheb[q][c], rho[q], w.x);
+                    w.y = fma(rule.cheb[q + 1][c], rho[q + 1], w.y);
                 }
                 w = cmul(w, ph);
                 const double2 bb = Bs[(long long)k * kNsing + i0 + c];
@@ -641,25 +645,22 @@ extern "C" fh_status fh_synthesize_sing(int J, double W, int j_c, int K, const d
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const double dw = W / (J - 1), wc = j_c * dw;
     const int L = n + kFcC, ns = n + kNsing;
-    // constants of the rule on this stream
-    double cheb[kSNq][kSNq], glx[kGl], glw[kGl], mu[kSM], mom[kSNq][kMom];
+    FccRule rule;
+    double glx[kGl], glw[kGl];
     for (int q = 0; q < kSNq; ++q)
         for (int c = 0; c < kSNq; ++c) {
             const double wt = (c == 0 || c == kSNq - 1) ? 0.5 : 1.0;
             double v = 2.0 / (kSNq - 1) * wt * std::cos(kPi * q * c / (kSNq - 1));
             if (q == 0 || q == kSNq - 1) v *= 0.5;
-            cheb[q][c] = v;
+            rule.cheb[q][c] = v;
         }
     gauss_legendre(kGl, glx, glw);
-    for (int g = 0; g < kGl / 2; ++g) glw[g] *= 2.0;   // node x and -x (the first half is positive)
-    cheb_power_moments(mom);
-    for (int j = 0; j < kSM; ++j) mu[j] = wc * std::pow((double)(j + 1) / kSM, kSQ);
-    if (cudaMemcpyToSymbolAsync(c_cheb, cheb, sizeof cheb, 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyToSymbolAsync(c_glx, glx, sizeof glx / 2, 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyToSymbolAsync(c_glw, glw, sizeof glw / 2, 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyToSymbolAsync(c_mom, mom, sizeof mom, 0, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyToSymbolAsync(c_mu, mu, sizeof mu, 0, cudaMemcpyHostToDevice, st) != cudaSuccess)
-        return FH_ECUDA;
+    for (int g = 0; g < kGl / 2; ++g) {   // node x and -x (the first half is positive)
+        rule.glx[g] = glx[g];
+        rule.glw[g] = 2.0 * glw[g];
+    }
+    cheb_power_moments(rule.mom);
+    for (int j = 0; j < kSM; ++j) rule.mu[j] = wc * std::pow((double)(j + 1) / kSM, kSQ);
     fh_status status = FH_OK;
     {
         Scratch sc{{}, st};
@@ -701,7 +702,7 @@ extern "C" fh_status fh_synthesize_sing(int J, double W, int j_c, int K, const d
                     G, nu, d_T, n_T, Gr, Gm);
         }
         fcc_weights_kernel<<<dim3(grid_of(n_T, kFccTimes), kSM - 1), kFccTimes * kFccGroups, 0, st>>>(
-            n, K, d_s, reinterpret_cast<const double2 *>(d_Bs), d_T, n_T, Gr, Gm);
+            rule, n, K, d_s, reinterpret_cast<const double2 *>(d_Bs), d_T, n_T, Gr, Gm);
         stack_fields_kernel<<<dim3(grid_of(n_x, 128), ns), 128, 0, st>>>(
             n, n_x, j_c, reinterpret_cast<const double2 *>(d_V), reinterpret_cast<const double2 *>(d_Vs), Vp);
         unsigned char *slices = contract_slices_fp64(ns, n_x, n_T)
