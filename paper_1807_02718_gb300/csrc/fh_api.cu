@@ -18,15 +18,12 @@
 #include <string>
 #include <vector>
 
+#include "devbuf.h"
 #include "fh_internal.h"
 
 namespace {
 
-struct DevBuf {
-    void *p = nullptr;
-    size_t cap = 0;
-    template <class T> T *as() const { return reinterpret_cast<T *>(p); }
-};
+using fh::DevBuf;
 
 void free_buf(DevBuf &b) {
     if (b.p) cudaFree(b.p);
@@ -221,19 +218,19 @@ fh_status fail(fh_ctx *ctx, fh_status st, const char *fmt, ...) {
         if (s_ != FH_OK) return s_;     \
     } while (0)
 
+struct DeviceMemory {
+    int alloc(void **p, size_t n) { return (int)cudaMalloc(p, n); }
+    void release(void *p) { cudaFree(p); }
+};
+
 fh_status ensure(fh_ctx *ctx, DevBuf &b, size_t bytes) {
-    if (b.cap >= bytes && b.p) return FH_OK;
-    free_buf(b);
-    size_t want = std::max<size_t>(bytes, 256);
-    cudaError_t e = cudaMalloc(&b.p, want);
+    DeviceMemory mem;
+    const cudaError_t e = (cudaError_t)fh::grow(mem, b, bytes, ctx->buf_gen);
     if (e != cudaSuccess) {
-        b.p = nullptr;
         cudaGetLastError();
         return fail(ctx, e == cudaErrorMemoryAllocation ? FH_ENOMEM : FH_ECUDA,
-                    "device allocation of %zu bytes failed: %s", want, cudaGetErrorString(e));
+                    "device allocation of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
     }
-    b.cap = want;
-    ++ctx->buf_gen;
     return FH_OK;
 }
 
