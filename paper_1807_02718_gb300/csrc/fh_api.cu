@@ -786,6 +786,7 @@ fh_status spectra_common(fh_ctx *ctx, Problem &pb, const double *d_a, int n_samp
             return fail(ctx, FH_EINVAL, "window starts are not equispaced on the sample grid");
     }
     const size_t wa_bytes = (size_t)K * (size_t)(Q + 1) * sizeof(double);
+    pb.spectra = false;   // the buffers below may be released and not come back
     FH_TRY(ensure(ctx, ctx->d_wa, wa_bytes));
     FH_TRY(ensure(ctx, pb.d_B, (size_t)K * pb.J * sizeof(double2)));
     FH_TRY(ensure(ctx, pb.d_Bf, (size_t)K * pb.J * sizeof(float4)));
@@ -905,9 +906,12 @@ fh_status field_kernels(fh_ctx *ctx, Problem &pb, const double *d_x, int n_x) {
     return check_launch(ctx, "target field");
 }
 
-// Scratch of the target fields of one problem at n_x targets.
+// Scratch of the target fields of one problem at n_x targets.  Fields resident
+// in d_V are gone once it has to grow, also if that fails.
 fh_status field_buffers(fh_ctx *ctx, const Problem &pb, int n_x) {
-    FH_TRY(ensure(ctx, ctx->d_V, (size_t)pb.J * n_x * sizeof(double2)));
+    const size_t bytes = (size_t)pb.J * n_x * sizeof(double2);
+    if (ctx->d_V.cap < bytes) ctx->have_V = false;
+    FH_TRY(ensure(ctx, ctx->d_V, bytes));
     const int n_items = pb.item_end - pb.item_begin;
     return ensure(ctx, ctx->d_part, (size_t)n_items * fh::kGroup * (size_t)n_x * sizeof(double2));
 }
@@ -942,6 +946,7 @@ fh_status sample_common(fh_ctx *ctx, int q, const double *d_x, int n_x, const do
     const long long key = graph_key(ctx, q + ((long long)pb.K << 24), n_x + ((long long)n_T << 32),
                                     (long long)(uintptr_t)d_x, (long long)(uintptr_t)d_T,
                                     (long long)(uintptr_t)d_u);
+    ctx->have_V = false;   // until the launches below have been issued
     FH_TRY(run_captured(ctx, ctx->sample_graph, key,
                         [&]() { return sample_kernels(ctx, pb, d_x, n_x, d_T, n_T, d_u); }));
     ctx->n_x_last = n_x;
@@ -1681,6 +1686,7 @@ fh_status fh_synthesize(fh_ctx *ctx, const double *V, int n_x, const double *T, 
     for (int i = 0; i < n_x; ++i)
         for (int j = 0; j < J; ++j)
             h[(size_t)j * n_x + i] = make_double2(V[2 * ((size_t)i * J + j)], V[2 * ((size_t)i * J + j) + 1]);
+    ctx->have_V = false;
     FH_TRY(upload(ctx, ctx->d_V, h));
     ctx->n_x_last = n_x;
     ctx->v_problem = 0;
