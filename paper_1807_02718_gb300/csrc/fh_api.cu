@@ -137,7 +137,7 @@ struct fh_ctx {
     DevBuf d_wa, d_a;
     int n_x_last = 0;
     DevBuf d_x, d_T, d_u, d_V, d_Gr, d_Gm, d_Gs, d_Vs, d_ctc, d_ctc_err;
-    bool ctc_pending = false;   // a tensor-core contraction ran since its flag was last read
+    bool ctc_pending = false;   // the last contraction ran on the tensor cores: d_ctc_err is its flag
     DevBuf d_tmpA, d_tmpg, d_tmp_ll, d_tmp_d, d_tmp_i;
 
     // timing: pending (phase, start, stop) event triples and totals
@@ -860,9 +860,13 @@ fh_status weights_kernels(fh_ctx *ctx, Problem &pb, const double *d_T, int n_T) 
     return FH_OK;
 }
 
+// The route of a call whose buffers exist (FP64 contexts may have had no room for the slices).
+bool on_slices(const fh_ctx *ctx, const Problem &pb, int n_x, int n_T) {
+    return use_contract_tc(ctx, pb, n_x, n_T) && ctx->d_ctc.cap >= fh::contract_tc_scratch_bytes(pb.J, n_x, n_T);
+}
+
 fh_status contract_kernels(fh_ctx *ctx, Problem &pb, int n_x, int n_T, double *d_u) {
-    const bool tcc = use_contract_tc(ctx, pb, n_x, n_T) &&
-                     ctx->d_ctc.cap >= fh::contract_tc_scratch_bytes(pb.J, n_x, n_T);
+    const bool tcc = on_slices(ctx, pb, n_x, n_T);
     const bool mixed = !use_planes(ctx, pb);
     PhaseScope ps(ctx, FH_PH_CONTRACT, tcc ? 5 : mixed ? 2 : 1);
     if (tcc) {
@@ -871,7 +875,6 @@ fh_status contract_kernels(fh_ctx *ctx, Problem &pb, int n_x, int n_T, double *d
                                                      ctx->d_Gr.as<double>(), ctx->d_Gm.as<double>(), d_u,
                                                      ctx->d_ctc.p, ctx->d_ctc_err.as<int>(), ctx->stream);
         if (e != cudaSuccess) return fail(ctx, FH_ECUDA, "tensor-core contraction: %s", cudaGetErrorString(e));
-        ctx->ctc_pending = true;
         return FH_OK;
     }
     if (mixed)
@@ -890,6 +893,7 @@ fh_status synth_kernels(fh_ctx *ctx, Problem &pb, int n_x, const double *d_T, in
 
 fh_status synth_common(fh_ctx *ctx, Problem &pb, int n_x, const double *d_T, int n_T, double *d_u) {
     FH_TRY(synth_buffers(ctx, pb, n_x, n_T));
+    ctx->ctc_pending = on_slices(ctx, pb, n_x, n_T);
     return synth_kernels(ctx, pb, n_x, d_T, n_T, d_u);
 }
 
@@ -947,6 +951,7 @@ fh_status sample_common(fh_ctx *ctx, int q, const double *d_x, int n_x, const do
                                     (long long)(uintptr_t)d_x, (long long)(uintptr_t)d_T,
                                     (long long)(uintptr_t)d_u);
     ctx->have_V = false;   // until the launches below have been issued
+    ctx->ctc_pending = on_slices(ctx, pb, n_x, n_T);   // (a replayed graph too)
     FH_TRY(run_captured(ctx, ctx->sample_graph, key,
                         [&]() { return sample_kernels(ctx, pb, d_x, n_x, d_T, n_T, d_u); }));
     ctx->n_x_last = n_x;
@@ -964,8 +969,8 @@ fh_status check_sample_args(fh_ctx *ctx, int q, int n_x, int n_T) {
     return FH_OK;
 }
 
-// Waits for a host-pointer sample; reports a tensor-core contraction that gave
-// up waiting (its flag is read with the result).
+// Waits for a host-pointer sample; reports that its tensor-core contraction gave
+// up waiting (the flag is read with the result; a call on another route has none).
 fh_status finish_sample(fh_ctx *ctx) {
     int ctc_err = 0;
     if (ctx->ctc_pending)
