@@ -219,18 +219,22 @@ fh_status fail(fh_ctx *ctx, fh_status st, const char *fmt, ...) {
     } while (0)
 
 struct DeviceMemory {
-    int alloc(void **p, size_t n) { return (int)cudaMalloc(p, n); }
+    int alloc(void **p, size_t n) {
+        const cudaError_t e = cudaMalloc(p, n);
+        if (e != cudaSuccess) cudaGetLastError();
+        return (int)e;
+    }
     void release(void *p) { cudaFree(p); }
 };
 
+// (The contraction's slices are ensured last in a call that uses them, and an
+// FP64 context, which ran without them once, may hold 1 GiB of them.)
 fh_status ensure(fh_ctx *ctx, DevBuf &b, size_t bytes) {
     DeviceMemory mem;
-    const cudaError_t e = (cudaError_t)fh::grow(mem, b, bytes, ctx->buf_gen);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
+    const cudaError_t e = (cudaError_t)fh::grow(mem, b, bytes, ctx->buf_gen, &ctx->d_ctc);
+    if (e != cudaSuccess)
         return fail(ctx, e == cudaErrorMemoryAllocation ? FH_ENOMEM : FH_ECUDA,
                     "device allocation of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
-    }
     return FH_OK;
 }
 

@@ -54,6 +54,15 @@ CASES = {
     m.room = 1 << 20;
     CHECK(fh::grow(m, b, 1000, g) == 0 && b.p && g != captured);
 ''',
+    # a buffer that can be done without makes room for one that cannot, and its address is given up with it
+    "spare": r'''
+    Memory m; fh::DevBuf b, c, spare; long long g = 0;
+    CHECK(fh::grow(m, spare, 600000, g, &spare) == 0 && fh::grow(m, b, 300000, g, &spare) == 0 && spare.p && g == 2);
+    CHECK(fh::grow(m, c, 500000, g, &spare) == 0 && c.p && b.p && !spare.p && spare.cap == 0 && g == 4);
+    CHECK(fh::grow(m, spare, 600000, g, &spare) == 2 && !spare.p && b.p && c.p && g == 4);
+    CHECK(fh::grow(m, spare, 100000, g, &spare) == 0 && fh::grow(m, b, 1 << 21, g, &spare) == 2);
+    CHECK(!b.p && !spare.p && c.p && g == 7 && m.live == 1);
+''',
 }
 
 
