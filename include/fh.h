@@ -208,8 +208,11 @@ fh_status fh_resample_p_dev(fh_ctx *ctx, int problem, const double *d_T, int n_T
 fh_status fh_get_density_p(fh_ctx *ctx, int problem, int j, double *psi);
 
 /* Device bytes a context needs for P problems with J[q] frequencies and sizes
- * N (laid out as in fh_discretize_batch) at `precision`, excluding the
- * per-call sampling work space (about 16 (J + n_items) n_x + 16 J n_T bytes).
+ * N (laid out as in fh_discretize_batch) at `precision`, excluding what a
+ * call's sizes decide: the spectra (32 J bytes per window and problem), the
+ * sampling work space (about 16 (J + n_items) n_x + 16 J n_T bytes) and the
+ * tensor-core contraction's slices (32 J (n_x + n_T) bytes, rounded up to its
+ * tiles; FP64 contexts take them up to 1 GiB and only where there is room).
  * Used for admission by memory footprint.  No device is touched. */
 fh_status fh_footprint(const int *J, const int *N, int P, int precision, long long *bytes);
 

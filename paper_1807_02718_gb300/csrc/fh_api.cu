@@ -15,6 +15,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <set>
 #include <string>
 #include <vector>
 
@@ -1732,11 +1733,13 @@ fh_status fh_device_memory(int device, long long *free_bytes, long long *total_b
 fh_status fh_footprint(const int *J, const int *N, int P, int precision, long long *bytes) {
     if (!J || !N || !bytes || P < 1) return FH_EINVAL;
     long long b = 0, jo = 0;
+    std::set<int> tables;   // problems of equal J share their synthesis tables
     for (int q = 0; q < P; ++q) {
         if (J[q] < 2) return FH_EINVAL;
         for (int j = 1; j < J[q]; ++j) {
             const long long n = N[jo + j];
             b += n * n * 16 + n * (16 * 4 + 16 + 8);          // matrix, nodes, density, tables
+            b += (long long)fh::lu_fp64_scratch_bytes(1);     // row moves; the mixed paths' states are smaller
             if (precision != FH_FP64) b += n * n * 8 + n * (16 + 4 + 8);   // FP32 copy, rhs, perm, FP32 rhs
             if (precision == FH_MIXED_TF32 || precision == FH_MIXED_BF16) {
                 b += (n + 31) / 32 * 2048 * 8;                            // diagonal-block inverses
@@ -1745,7 +1748,8 @@ fh_status fh_footprint(const int *J, const int *N, int P, int precision, long lo
                      (long long)fh::lu_tc_map_bytes(1);
             }
         }
-        b += (long long)fh::kFarTerms * J[q] * 16 + 2LL * (J[q] - 1) * 16 + fh::sinc_tab_entries(J[q]) * 16;
+        if (tables.insert(J[q]).second)
+            b += (long long)fh::kFarTerms * J[q] * 16 + 2LL * (J[q] - 1) * 16 + fh::sinc_tab_entries(J[q]) * 16;
         jo += J[q];
     }
     *bytes = b;
