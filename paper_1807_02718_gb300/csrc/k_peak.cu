@@ -1,7 +1,10 @@
 // Arithmetic-peak probes, used to state the rooflines of the path's kernels
 // on the device they run on:
 //  * a long chain of independent FP64 (or FP32) FMAs per thread, enough warps
-//    to fill every SM (the FP64 and double-float kernels);
+//    to fill every SM (the FP64 and double-float kernels).  All three operands
+//    are registers: with a factor and an addend known at compile time an FP64
+//    FMA holds the pipe for 19 clocks in place of 16 (as do FP64 additions and
+//    products), 1.06 TFLOP/s in place of 1.25 at 2070 MHz;
 //  * back-to-back tcgen05 MMAs (M = 128, N = 256, one K step) from operands
 //    resident in shared memory, one CTA per SM (the TF32 / BF16 tensor-core
 //    kernels): the tensor pipe's own rate, without operand traffic.
@@ -22,7 +25,7 @@ __global__ void __launch_bounds__(256) fma_chain_kernel(T *out, int iters, T see
     T a[kChains];
 #pragma unroll
     for (int c = 0; c < kChains; ++c) a[c] = seed + (T)(threadIdx.x + c);
-    const T m = (T)0.999999, k = (T)1e-7;
+    const T m = (T)0.999999 - (T)1e-6 * (T)threadIdx.x, k = (T)1e-7 * (T)(threadIdx.x + 1);   // registers
     for (int i = 0; i < iters; ++i) {
 #pragma unroll
         for (int c = 0; c < kChains; ++c) a[c] = fma(a[c], m, k);
