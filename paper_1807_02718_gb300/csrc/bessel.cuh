@@ -60,30 +60,6 @@ __device__ __forceinline__ void hankel_pq(double x, double &P0, double &Q0, doub
     }
 }
 
-// P0, Q0, P1, Q1 at x >= 8 given r8 = 8/x (shared by the grouped kernels).
-template <bool want1>
-__device__ __forceinline__ void hankel_pq_r8(double x, double r8, double &P0, double &Q0,
-                                             double &P1, double &Q1) {
-    if (x < 20.0) {
-        const double t = (r8 * r8 - kBLoU0) * (2.0 / (1.0 - kBLoU0)) - 1.0;
-        P0 = clenshaw<kBLo0_N>(kBLo0, t);
-        Q0 = r8 * clenshaw<kBLo1_N>(kBLo1, t);
-        if (want1) {
-            P1 = clenshaw<kBLo2_N>(kBLo2, t);
-            Q1 = r8 * clenshaw<kBLo3_N>(kBLo3, t);
-        }
-    } else {
-        const double r20 = 2.5 * r8;
-        const double t = 2.0 * r20 * r20 - 1.0;
-        P0 = clenshaw<kBHi0_N>(kBHi0, t);
-        Q0 = r8 * clenshaw<kBHi1_N>(kBHi1, t);
-        if (want1) {
-            P1 = clenshaw<kBHi2_N>(kBHi2, t);
-            Q1 = r8 * clenshaw<kBHi3_N>(kBHi3, t);
-        }
-    }
-}
-
 // Horner form of P0, Q0 (and P1, Q1) for x >= 8 on 32 equal intervals of u =
 // (8/x)^2, five terms each to below 1e-17 (the FP64 pipe bounds the callers, so
 // short polynomials: with six intervals of x they took eight terms; fields of

@@ -76,7 +76,6 @@ __device__ __forceinline__ dfv df_mul_f(dfv a, float b) {
 }
 
 // a * b + c
-__device__ __forceinline__ dfv df_fma(dfv a, dfv b, dfv c) { return df_add(df_mul(a, b), c); }
 
 // a * b + c with one renormalisation: the exact product of the hi parts (FMA
 // residual) and the cross terms, the sum of the two leading parts by two-sum,
@@ -104,21 +103,6 @@ __device__ __forceinline__ dfv df_dot2(dfv a, dfv b, dfv c, dfv d) {
     const float s = p + q;
     const float bb = s - p;
     return df_quick(s, ((p - (s - bb)) + (q - bb)) + (e + f));
-}
-
-// acc += a * b (or -= when neg): exact FP32 product hi*hi with its FMA
-// residual and the cross terms; the running sum (sh, sl) is a two-sum pair
-// that the caller renormalises (df_quick) every few terms.
-__device__ __forceinline__ void df_acc(float &sh, float &sl, dfv a, dfv b, bool neg) {
-    float p = a.hi * b.hi;
-    float pe = fmaf(a.hi, b.hi, -p);
-    pe = fmaf(a.hi, b.lo, pe);
-    pe = fmaf(a.lo, b.hi, pe);
-    if (neg) { p = -p; pe = -pe; }
-    const float t = sh + p;
-    const float z = t - sh;
-    sl += ((sh - (t - z)) + (p - z)) + pe;
-    sh = t;
 }
 
 __device__ __forceinline__ dfv df_sqrt(dfv a) {
@@ -290,7 +274,10 @@ __device__ __forceinline__ df2 df2_dot3(df2 a, df2 b, df2 c, df2 d, df2 u, df2 v
     return df2_quick(t, p2_add(err, p2_add(p2_add(e, f), g)));
 }
 
-__device__ __forceinline__ void df2_acc(float2 &sh, float2 &sl, df2 a, df2 b) {   // as df_acc
+// sum += a b: the product's error and the cross terms enter the low part with
+// the exact two-sum error of the high part; the running sum (sh, sl) is a pair
+// that the caller renormalises (df2_quick) every few terms.
+__device__ __forceinline__ void df2_acc(float2 &sh, float2 &sl, df2 a, df2 b) {
     float2 e;
     const float2 p = p2_prod(a, b, e), t = p2_add(sh, p);
     sl = p2_add(sl, p2_add(p2_two_sum_err(sh, p, t), e));

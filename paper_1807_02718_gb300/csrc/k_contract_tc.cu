@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1) contract_tc_kernel(
 #pragma unroll
             for (int g = 0; g < 2; ++g) {
                 const int c0 = 32 * ch + 16 * g;
-long long hi[16], lo[16];   // levels 0 .. 3 and 4 .. 7
+                long long hi[16], lo[16];   // levels 0 .. 3 and 4 .. 7
 #pragma unroll
                 for (int c = 0; c < 16; ++c) hi[c] = lo[c] = 0;
                 auto join = [&](long long (&h)[16], int d0) {

@@ -663,7 +663,7 @@ __global__ void convert_kernel(const float4 *__restrict__ A, float2 *__restrict_
 
 void launch_convert_fp32(const float4 *A, float2 *A32, long long n, cudaStream_t st) {
     if (n <= 0) return;
-    convert_kernel<<<152 * 8, 256, 0, st>>>(A, A32, n);
+    convert_kernel<<<kSms * 8, 256, 0, st>>>(A, A32, n);
 }
 
 void launch_lu_factor_fp32(const int *order, int S, const int *N, const long long *mat_off,
@@ -698,7 +698,7 @@ void launch_lu_refine(bool row_major, const int *order, int S, const int *N,
     // takes 32), two of 256 overlap.  Measured refinement, 512 -> 256 threads:
     // 2032 systems of N <= 832 3.70 -> 3.10 ms, 1016 1.98 -> 1.73, 508 1.07 ->
     // 1.08; 511 of N <= 1920 7.65 -> 8.09.  The sums are the same, bit for bit.
-    const int rt = S > 4 * 152 && maxN <= 1024 ? 256 : 512;
+    const int rt = S > 4 * kSms && maxN <= 1024 ? 256 : 512;
     for (int it = 1; it <= max_iters; ++it) {
         if (row_major)
             refine_solve_kernel<true><<<S, rt, (size_t)maxN * sizeof(float2), st>>>(

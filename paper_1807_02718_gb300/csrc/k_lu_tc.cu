@@ -420,6 +420,7 @@ __global__ void __launch_bounds__(kThreads, 1) lu_factor_tc_kernel(
         // (piece h of row r at h ^ (r mod 16)) so that neither side has bank
         // conflicts.
         float4 *xch = gbuf + warp * (32 * NB / 2);
+        static_assert(kWarps * 32 * NB / 2 <= kGather, "the warps' exchange buffers fit the B and C space");
         const int frows = nb == NB ? ((m - NB + cs - 1) / cs + 1) & ~1 : 0;   // rows below the block, per CTA
         const int frow = rank * frows + tid;                                 // this thread's, relative to k0 + NB
         const bool lrow = tid < frows && frow < m - NB;

@@ -905,11 +905,11 @@ void launch_synth_contract(int J, int n_x, int n_T, const double2 *V, const doub
     if (contract_small(J, n_x, n_T)) {
         // all tiles in grid.x: J = 2 leaves 2^22 outputs, which for one target are more than 65535 tiles of 16 times
         const unsigned ctas = (unsigned)((n_x + 7) / 8) * (unsigned)((n_T + 15) / 16);
-        if (ctas < 2 * 152)
+        if (ctas < 2 * kSms)
             contract_small_kernel<4><<<ctas, 4 * 128, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
         else
             contract_small_kernel<1><<<ctas, 128, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
-    } else if (g64.x * g64.y < 2 * 152)
+    } else if (g64.x * g64.y < 2 * kSms)
         contract_kernel<32><<<tiles(32), 256, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
     else
         contract_kernel<64><<<g64, 256, 0, st>>>(J, n_x, n_T, V, Gr, Gm, u);
