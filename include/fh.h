@@ -376,9 +376,8 @@ fh_status fh_set_graphs(fh_ctx *ctx, int enable);
  *                    (1..8; they share the geometry of each node pair)
  *   field_group      frequencies of equal N per target-field work item (1..8)
  *   field_chunk      source nodes per target-field work item (16, 32 or 64)
- *   lu_rows_per_cta  tensor-core LU: a system of order N is factored by the
- *                    smallest power of two of CTAs, at most 8, that is
- *                    >= N / lu_rows_per_cta (128, 256 or 512)
+ *   lu_rows_per_cta  tensor-core LU: a system of order N is factored by
+ *                    ceil(N / lu_rows_per_cta) CTAs, at most 8 (128, 256 or 512)
  *   lu_early         tensor-core LU: the largest systems, at least this
  *                    percentage of them (0..50, whole assembly subgroups), are
  *                    assembled and factored on a second stream while the
@@ -386,10 +385,15 @@ fh_status fh_set_graphs(fh_ctx *ctx, int enable);
  *                    (fh_set_timing) runs the single sequence.
  *   contract_tc      2J <= 8192: 1 contracts u = [Vr | Vi][Gr ; Gm] on the
  *                    tensor cores (operands cut into eight 7-bit slices held
- *                    exactly in BF16, FP32 sums per slice level, levels
- *                    combined in FP64; ~2^-58 of max|row| max|column| per
- *                    term; few outputs take FP64 FMAs), 0 on the FP32 pipe in
- *                    double-float (mixed paths) or on the FP64 pipe (FP64).
+ *                    exactly in BF16, FP32 sums per slice level, levels joined
+ *                    as integers and rounded to FP64; ~2^-58 of max|row|
+ *                    max|column| per term after a balance of the terms that
+ *                    all targets and times of the call share), 0 on the FP32
+ *                    pipe in double-float (mixed paths) or on the FP64 pipe
+ *                    (FP64).  Few outputs take FP64 FMAs either way, and an
+ *                    FP64 context does where the slices find no room.  So the
+ *                    last bits of a sample may differ between calls with other
+ *                    targets or times beside it (not with contract_tc = 0).
  *                    fh_sample and fh_synthesize (host pointers)
  *                    report a tensor-core completion wait that gave up as
  *                    FH_ETIMEOUT.

@@ -253,9 +253,9 @@ inline bool contract_small(int J, int n_x, int n_T) { return 2LL * J * n_x * n_T
 void launch_synth_contract(int J, int n_x, int n_T, const double2 *V, const double *Gr,
                            const double *Gm, double *u, cudaStream_t st);
 // Tensor-core contraction (2J <= kContractTcMaxK): the operands cut into eight
-// 7-bit slices held exactly in BF16, every slice product summed exactly in
-// FP32 per level over K segments of 512, levels joined as integers and summed
-// over the segments in FP64.
+// 7-bit slices held exactly in BF16, the slice products of a level summed in FP32
+// over K segments of 512 (exactly, but for rare sums of the two lowest levels),
+// levels joined as integers and summed over the segments in FP64.
 // scratch: contract_tc_scratch_bytes(J, n_x, n_T) bytes; err (may be null) set
 // if an MMA completion wait gave up (the CTA's sums are then taken directly).
 // Five launches.

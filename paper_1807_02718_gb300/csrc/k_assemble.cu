@@ -61,9 +61,9 @@ __device__ __forceinline__ void triangle_tile(long long lt, int &tr, int &tc) {
 // Bound by the FP64 pipe (2 FMAs per clock and SM): about 75 FP64 instructions
 // per entry, the small-argument series of the near-diagonal warps included,
 // against 168 for one thread per entry with M1, M2, L1, L2 formed separately.
-// Measured (GB300): 255 systems of N 64..480: 5.75 -> 2.55 ms (3.56 with Clenshaw
-// sums below x = 8 and FP64 interval comparisons); 63 systems of N = 256: 1.77
-// -> 0.65 ms.
+// Measured (GB300): 255 systems of N 64..480: 5.75 -> 2.32 ms (FP64 pipe active 90 %
+// of the cycles; 3.56 ms with Clenshaw sums below x = 8 and FP64 interval
+// comparisons); 63 systems of N = 256: 1.77 -> 0.65 ms.
 __global__ void __launch_bounds__(256, 2) assemble_group_kernel(
     SolveTables t, Subgroups grp, int n_groups, const double2 *__restrict__ z,
     const double2 *__restrict__ dz, const double2 *__restrict__ ddz,

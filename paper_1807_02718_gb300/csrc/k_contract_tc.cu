@@ -2,11 +2,17 @@
 // A = [Vr | Vi] and B = [Gr ; Gm] (Sec. 4.1 eq. approx in collapsed form),
 // to FP64 accuracy through exact BF16 products (an error-free slicing of the
 // operands, the "Ozaki scheme").  Every precision contracts here, and so does
-// the split synthesis: the FP64 pipe bounds the plain FP64 kernel.  Measured,
+// the split synthesis, unless the outputs are few (contract_small,
+// contract_slices_fp64) or may not allocate: the FP64 pipe bounds the plain FP64
+// kernel.  Measured,
 // plain -> slices (five launches): 1024 x 4096 outputs, 2J = 512 3.62 -> 0.21 ms
 // (MMAs at the measured BF16 rate 0.08 ms; the rest is slicing, 42 MB written
 // and read back, and the epilogue, which cannot overlap the MMAs: TMEM holds
 // one tile's levels), 2J = 1024 7.2 -> 0.37 ms, 333 x 1001, 2J = 402 334 -> 74 us.
+//
+// The balance below is taken over all targets and times of the call, and the call's
+// size decides between this kernel and the FP64 ones: a sample's last bits depend on
+// what else the call asks for (the fields and weights that enter do not).
 //
 // Scaling.  Term kk is first balanced by a power of two, A[x][kk] 2^d_kk times
 // B[kk][t] 2^-d_kk, so that entries which meet small partners (the fields at

@@ -30,7 +30,8 @@
 // Measured (GB300; out-of-place radix-2 stages with a sincospi per butterfly
 // before): 64 traces of L = 16384, M = 1000: 7.38 -> 0.71 ms; one trace of L =
 // 10^6, M = 5000: 20.2 -> 3.12 ms (eight FFTs of 2^21 points, 1.2e9 FP64
-// instructions: 2.3 ms at the measured 1.0 TFLOP/s).
+// instructions: 2.3 ms where a warp's addition or product holds the pipe for 19
+// clocks, as measured; an FMA holds it for 16).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>

@@ -38,7 +38,7 @@ constexpr int kChunk = kFieldChunk;   // largest number of source nodes per work
 // (64 nodes x 8 frequencies) held an SM for a millisecond, so that a few
 // hundred targets made less than three waves of them.  Measured (GB300): 16
 // targets x 63 frequencies, N = 256: 2.60 -> 0.20 ms; 1024 x 255, N 64..480:
-// 8.44 -> 5.61 ms; spectra, fields and synthesis at 333 targets x 1001 times,
+// 8.44 -> 4.96 ms (FP64 pipe active 90 % of the cycles); spectra, fields and synthesis at 333 targets x 1001 times,
 // 200 frequencies: 4.77 -> 1.9 ms (1.12 ms with the contraction's and the
 // Hankel polynomials' later changes).
 constexpr int kTileF64 = 16, kSlicesF64 = kTgt / kTileF64;
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(kTgt) field_partial_kernel(
 // grid has four times the CTAs of one target per thread, each a quarter as
 // long, which is what a few hundred targets (one problem of a batch) need.
 // Measured (GB300): 1024 targets x 511 frequencies, N up to 1920: 7.6 -> 6.7 ms;
-// x 255, N up to 480: 1.21 -> 0.96 ms; 256 targets of each of 16 obstacles (127
+// x 255, N up to 480: 1.21 -> 0.93 ms (FMA pipe 69 %); 256 targets of each of 16 obstacles (127
 // frequencies, N 64..832): 8.3 -> 3.5 ms.
 constexpr int kTileDf = 32, kSlicesDf = kTgt / kTileDf;
 

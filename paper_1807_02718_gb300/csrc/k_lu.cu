@@ -15,13 +15,13 @@
 // (short dependent steps that leave most of the chip idle) overlap with the
 // other half's strips.
 //
-// Bound: the FP64 pipe, two FMAs per clock and SM (1.05 TFLOP/s measured), so
+// Bound: the FP64 pipe, two FMAs per clock and SM (1.25 TFLOP/s measured), so
 // that one warp's FMA occupies an SM for 16 clocks: loads, shared memory and
 // launches are nearly free, and what counts is that every SM has FMAs to
 // issue.  One CTA per system, as before, leaves the largest system on one SM
-// (N = 480: 43 ms at the SM's peak) and 63 systems on 63 SMs; strips of SW = 8
+// (N = 480: 36 ms at the SM's peak) and 63 systems on 63 SMs; strips of SW = 8
 // columns spread each system over N / 8 CTAs.
-// Measured (GB300, LU phase; the flops at peak take 2.7 and 20 ms): 63 systems
+// Measured (GB300, LU phase; the flops at peak take 2.3 and 17 ms): 63 systems
 // of N = 256: 14.3 -> 3.5 ms; 255 systems of N = 64..480: 78.0 -> 20.5 ms
 // (strips of 16 columns: 3.8 and 21.1 ms).
 #include <algorithm>

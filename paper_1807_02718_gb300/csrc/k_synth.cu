@@ -620,7 +620,7 @@ constexpr int BM = 64, BN = 64, BK = 16;
 // For sums that contract_slices_fp64 does not take (up to 2^25 products, 2J >
 // 8192, scratch) and the synthesis without allocation.
 // kTile x kTile outputs per CTA, (kTile / 16)^2 per thread.  Bound by the FP64
-// pipe (1.19 of 1.05 TFLOP/s measured by FMA chains at 1024 x 4096, 2J = 512), so
+// pipe (1.19 of the 1.25 TFLOP/s that FMA chains reach at 1024 x 4096, 2J = 512), so
 // what matters is that every SM has a tile: tiles of 32 where tiles of 64 are
 // fewer than two per SM (333 x 1001, 2J = 402: 96 tiles, 0.50 ms).
 template <int kTile>
