@@ -115,7 +115,7 @@ constexpr int kTop = kMid + 1 + kFcD;        // S_(h - kTop + 1) .. S_h enter th
 // -m are paired, their sinc sums staged in chunks of kTabChunk for all columns;
 // the rows -g from S_i(-y) = conj S_i(y) + (-1)^i (sinc(r (y - h)) - sinc(r (y + h))).
 // The CTAs of the first columns also form top[(g + G) kTop + q] = S_(h-q)(g/2),
-// q < kTop, in FP64 (one thread per row and q; 1 % of the sums).
+// q < kTop, in FP64 (one thread per row and q).  0.13 ms for n = 251, 0.11 without.
 constexpr int kTabRows = 4, kTabChunk = 256;
 
 __global__ void __launch_bounds__(128) split_table_kernel(int num, int L, int G, const float4 *__restrict__ ph,
@@ -241,8 +241,10 @@ __host__ __device__ inline size_t split_work_bytes(int n) {
 // kShared: the values of a time in shared memory (split_work_bytes(n) = 40 n + 528
 // bytes, n <= 5106 at kSplitSmem); otherwise in `work`, the launch's CTAs taking
 // the times from it0 on.
-// Measured (GB300; 1024 x 4096 samples, n = 251, 29 windows): whole call 2.34 ms with 384
-// double-float products (end sample, continuation point) per window, each splitting
+// Bound by the FP64 pipe (active 73 % of the cycles, the FMA pipe 36 %): splits of B for the
+// interior samples, interpolation weights and constants per window, end samples.
+// Measured (GB300; 1024 x 4096 samples, n = 251, 29 windows): 1.58 -> 0.99 ms, whole call
+// 2.34 ms with 384 double-float products (end sample, continuation point) per window, each splitting
 // its B in FP64, 1.74 ms so.  Error against extended precision over 28 meshes of
 // n = 20..110: geometric mean 4.8e-12 -> 6.6e-13, largest 6.6e-11 -> 1.7e-11 (L-term
 // double-float sums per sample: 2.0e-11 and 1.3e-10).

@@ -392,8 +392,9 @@ __device__ __forceinline__ void store_weight(int J, int p, int t, int n_T, int p
 // Near windows: 42 samples around y, their weights (with 2W/M) formed by the
 // group's first threads; far windows: Horner's rule over the far table, the
 // terms past R1 in binary32.  (re, im) are one packed pair throughout.
-// Bound by FP32 issue with many times; with few, by the dependent steps of a
-// window (weights, barrier, loads from L2), which the groups take side by side.
+// With many times the FMA pipe is active 60 % of the cycles and most other stalls
+// wait for the table's rows out of L2; with few, the dependent steps of a window
+// (weights, barrier, loads) bound it, which the groups take side by side.
 // (Four groups, 512 threads, were 4 % slower with many times: fewer CTAs hide
 // the FP64 set-up.)  Measured (GB300): 4096 times, J = 256, 29 windows: 0.63 ms before; 16
 // times, J = 128, 7 windows: 56 us before (one window after another, re and im
