@@ -666,12 +666,12 @@ extern "C" fh_status fh_synthesize_sing(int J, double W, int j_c, int K, const d
     fh_status status = FH_OK;
     {
         Scratch sc{{}, st};
-        double *Xc = sc.get<double>((size_t)kFcC * n);
         // half-integer table of S_i, far-field table of order L with its phases and powers
         const int h = L / 2, hp = h + 1, G = (5 * h + 1) / 2 + 24;
         float4 *tab = sc.get<float4>((size_t)(2 * G + 1) * hp);
-        double2 *top = sc.get<double2>((size_t)(2 * G + 1) * kTop);
-        double2 *ph64 = sc.get<double2>((size_t)L);
+        double2 *top = sc.get<double2>((size_t)(2 * G + 1) * kTop + L + ((size_t)kFcC * n + 1) / 2);
+        double2 *ph64 = top + (size_t)(2 * G + 1) * kTop;             // and the continuation rows, one allocation
+        double *Xc = reinterpret_cast<double *>(ph64 + L);
         float4 *nu = sc.get<float4>((size_t)kFarTerms * hp);
         float4 *ph = sc.get<float4>((size_t)L);
         double *pw = sc.get<double>((size_t)L * kFarTerms);
@@ -681,7 +681,7 @@ extern "C" fh_status fh_synthesize_sing(int J, double W, int j_c, int K, const d
         const size_t work_bytes = split_work_bytes(n);
         const bool in_memory = work_bytes > kSplitSmem;
         float4 *work = in_memory ? sc.get<float4>(work_bytes / sizeof(float4) * std::min(kSplitCtas, n_T)) : nullptr;
-        if ((in_memory && !work) || !Xc || !tab || !top || !ph64 || !nu || !ph || !pw || !Vp || !Gr || !Gm) {
+        if ((in_memory && !work) || !tab || !top || !nu || !ph || !pw || !Vp || !Gr || !Gm) {
             cudaGetLastError();
             return FH_ENOMEM;
         }
