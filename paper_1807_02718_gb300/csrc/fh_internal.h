@@ -223,6 +223,8 @@ void launch_synth_weights(int J, int M, double W, int K, const double *s, const 
 // kWeightsMaxSmem bytes are available (so K and J are bounded; callers
 // reject larger problems before launching).
 constexpr size_t kWeightsMaxSmem = 200 * 1024;
+// (with the table the kernel takes the windows in chunks and needs none: there
+// the value only keeps the number of windows that a context accepts).
 size_t synth_weights_smem(int J, int K, bool table);
 // Near-window sums by interpolation.  The near sums
 //   D_p(y) = sum_{m=-h}^{h-1} e^{-2 pi i m p / M} sinc(y - m)
